@@ -65,19 +65,18 @@ typedef enum elutq_status {
                                    indices with the top bit clear and the other half is obtained by
                                    negation; same product up to fp32 rounding                              */
 
-#define ELUTQ_TENSOR_MIN_M 9      /* batches of this many rows or more take the tensor-core path (G = 128, no
-                                     look-up variant flag): the batched look-up kernel needs one pass per 4 rows,
-                                     the tensor-core kernel's time does not depend on M up to 128              */
-#define ELUTQ_TENSOR_MIN_M_NARROW 5   /* ... and so do batches of 5 to 8 rows when N <= ELUTQ_TENSOR_NARROW_N: there  */
-#define ELUTQ_TENSOR_NARROW_N 8192    /* the second look-up pass already costs more than the tensor-core call (measured
-                                         on the 8B shapes at M = 8, q = 2 / 3, us: qkv 6144 x 4096 17.1 / 20.8 against
-                                         15.4 / 17.7, o 4096 x 4096 13.4 / 16.8 against 11.7 / 13.3, down 4096 x 14336
-                                         27.3 / 36.3 against 26.3 / 32.0; gate_up 28672 x 4096 43.9 / 60.6 against
-                                         48.8 / 66.5 stays on the look-up kernel).  elutq_takes_tensor_path says which
-                                         path a call takes.                                                    */
+#define ELUTQ_TENSOR_MIN_M 3      /* batches of this many rows or more run on the tensor cores (G = 128 or 64, no look-up
+                                     variant flag).  Two rows stay on the batched look-up kernel: one pass, 17.3 us
+                                     on 8B gate_up 28672 x 4096 at q = 2 against 25.6; from three rows on it needs a
+                                     wider pass (M = 4: 26.2 / 25.9, 4096 x 4096 9.5 / 7.6, M = 8: 43.9 / 26.8)        */
+#define ELUTQ_FRAGMENT_MAX_M 16   /* G = 128: up to this many rows the bit-planes are contracted as they are (scales
+                                     applied to fp32 sums, as exact as the look-up kernels); larger batches rebuild
+                                     W_hat in fp16 tiles (8B gate_up at q = 2, us: M = 16 37 / 48, M = 32 82 / 48).
+                                     At G = 64 every batch takes the former, 32 rows at a time
+                                     (elutq_takes_tensor_path is 1 for both)                                        */
 
-#define ELUTQ_FLAG_LUT_ONLY 0x80u /* M >= 9: stay on the look-up-table kernels.  Without this flag batches of
-                                     ELUTQ_TENSOR_MIN_M rows or more (G = 128) take the dequantise-and-contract path: the
+#define ELUTQ_FLAG_LUT_ONLY 0x80u /* M > 1: stay on the look-up-table kernels.  Without this flag batches of more than
+                                     ELUTQ_FRAGMENT_MAX_M rows (G = 128) take the dequantise-and-contract path: the
                                      weight tile is rebuilt in fp16 from the bit-planes (BCQ form of
                                      Appendix D) and contracted on the tensor cores with fp32 accumulation;
                                      its results carry the fp16 rounding of W_hat (about 3e-4 relative)     */
@@ -253,13 +252,14 @@ int elutq_lut_gemm_host(const void* X_host, const void* packed, void* Y_host,
  *     needs clearing: every value read was written by the same call).  Calls that overlap on the
  *     GPU, e.g. on different streams, race on it: keep them stream-ordered.
  *   - Every M stays on the look-up kernels here (the tensor-core path needs more scratch than the array
- *     holds), so from M = 9 on the result differs from elutq_lut_gemm's in rounding (it is the more
+ *     holds), so above ELUTQ_FRAGMENT_MAX_M rows the result differs from elutq_lut_gemm's in rounding (it is the more
  *     accurate of the two: W_hat is never rounded to fp16) and the call is slower.
  *   - `packed` must be known to the library (packed or described in this process) before a capture
  *     begins: an unknown address makes the call read the header with a synchronous copy.
  */
 /* 1 when elutq_lut_gemm (and _f32, _ws, _host, _bias) runs a call of this shape on the tensor-core path, 0 when on the
- * look-up kernels; host-only, launches nothing.  (The tensor-core path's results carry the fp16 rounding of W_hat.) */
+ * look-up kernels; host-only, launches nothing.  (Above ELUTQ_FRAGMENT_MAX_M rows at G = 128 its results carry the fp16
+ * rounding of W_hat.) */
 int elutq_takes_tensor_path(int M, int N, int K, int G, unsigned flags);
 
 int elutq_lut_gemm_static(const void* X, const void* packed, void* Y, int M, int N, int K, void* stream);
@@ -380,8 +380,8 @@ int elutq_hlq_fit(const void* W, int q, int G, int N, int K, int t_max, uint8_t*
 int elutq_device_status(void* stream, int* status);
 
 /*
- * Test entry for the bounded waits of the tensor-core kernel (9 <= M <= 128, G = 128, K >= 384): the call is
- * launched with the issuing thread told to issue no MMA and no completion signal and with the poll limit of the
+ * Test entry for the bounded waits of the tensor-core kernels (9 <= M <= 128, G = 128, K >= 384): the call is
+ * launched with the issuing thread told to issue no MMA and no completion signal (up to ELUTQ_FRAGMENT_MAX_M rows: no load) and with the poll limit of the
  * device-side waits set to `wait_limit`, so that the waits for MMA completion run out: the kernel gives up
  * waiting, still joins every barrier, frees its tensor memory and returns; elutq_device_status then reads
  * ELUTQ_DEVICE_WAIT_EXPIRED.  Y (float [M][N]) receives undefined values.  Nothing faults and nothing waits

@@ -61,7 +61,8 @@ int num_sms() {
 }
 
 // Workspace layout: a 256-byte control area (word 0 = device status), then the partial sums.
-size_t counters_bytes(int, int) { return 256; }
+// Batches: plus one ticket per 128 output rows (hlq_frag.cu).
+size_t counters_bytes(int M, int N) { return 256 + (M == 1 ? 0 : ((size_t)(N + 127) / 128 * sizeof(unsigned) + 255) / 256 * 256); }
 size_t partials_bytes(int M, int N, int K) {
     const size_t n_rb = (size_t)(N + kTileRows - 1) / kTileRows;
     const size_t n_kc = (size_t)(K + kChunkK - 1) / kChunkK;
@@ -163,12 +164,11 @@ int launch_copy_in(const void* src, void* dst, size_t bytes, cudaStream_t stream
     return (int)e;
 }
 
-// Which kernel family a batched call runs on (the crossover depends on the shape: see ELUTQ_TENSOR_MIN_M_NARROW).
-bool takes_tensor_path(int M, int N, int G, unsigned flags) {
+// Whether a batched call runs on the tensor cores.
+bool takes_tensor_path(int M, int G, unsigned flags) {
     const unsigned lut_variants = ELUTQ_FLAG_PLAIN_G4 | ELUTQ_FLAG_CLUSTER_REDUCE | ELUTQ_FLAG_MIRROR | ELUTQ_FLAG_LUT_ONLY |
                                   ELUTQ_FLAG_TABLE_F16 | ELUTQ_FLAG_TABLE_I8;
-    if (G != 128 || (flags & lut_variants)) return false;
-    return M >= ELUTQ_TENSOR_MIN_M || (M >= ELUTQ_TENSOR_MIN_M_NARROW && N <= ELUTQ_TENSOR_NARROW_N);
+    return M >= ELUTQ_TENSOR_MIN_M && G != 32 && !(flags & lut_variants);
 }
 
 int run_gemm(const void* X, const void* packed, void* Y, int M, int N, int K, unsigned flags,
@@ -217,8 +217,9 @@ int run_gemm(const void* X, const void* packed, void* Y, int M, int N, int K, un
     const int sms = num_sms();
     int ce;
     if (M == 1) ce = launch_lut_gemv(a, m.q, m.G, sms, (cudaStream_t)stream);
-    else if (takes_tensor_path(M, N, m.G, flags)) ce = launch_hlq_mma(a, m.q, m.G, sms, (cudaStream_t)stream);
-    else ce = launch_lut_gemm(a, m.q, m.G, sms, (cudaStream_t)stream);
+    else if (!takes_tensor_path(M, m.G, flags)) ce = launch_lut_gemm(a, m.q, m.G, sms, (cudaStream_t)stream);
+    else if (m.G == 128 && M > ELUTQ_FRAGMENT_MAX_M) ce = launch_hlq_mma(a, m.q, m.G, sms, (cudaStream_t)stream);
+    else ce = launch_hlq_frag(a, m.q, m.G, sms, (cudaStream_t)stream);
     if (ce == (int)cudaErrorNotSupported) return ELUTQ_ERR_UNSUPPORTED;
     if (ce != 0) return cuda_fail((cudaError_t)ce);
     return ELUTQ_OK;
@@ -383,7 +384,7 @@ int elutq_lut_gemm_host(const void* X_host, const void* packed, void* Y_host, in
 }
 
 int elutq_test_wait_expiry(const void* X, const void* packed, float* Y, int M, int N, int K, unsigned wait_limit, void* stream) {
-    if (M < ELUTQ_TENSOR_MIN_M || M > 128 || wait_limit == 0) return ELUTQ_ERR_UNSUPPORTED;   // the one-token-tile schedule only
+    if (M < 9 || M > 128 || wait_limit == 0) return ELUTQ_ERR_UNSUPPORTED;   // the one-token-tile schedule only
     if (K < 3 * 128) return ELUTQ_ERR_UNSUPPORTED;                                           // a wait needs a third K step
     g_test_flags = kFlagTestNoMma;
     g_test_wait_limit = wait_limit;
@@ -435,8 +436,9 @@ int elutq_release_scratch(void) {
 }
 
 int elutq_takes_tensor_path(int M, int N, int K, int G, unsigned flags) {
+    (void)N;
     (void)K;
-    return M > 1 && takes_tensor_path(M, N, G, flags) ? 1 : 0;
+    return takes_tensor_path(M, G, flags) ? 1 : 0;
 }
 
 int elutq_reserve(int M, int N, int K, void* stream) {

@@ -1,0 +1,626 @@
+// Batches of up to ELUTQ_FRAGMENT_MAX_M rows (any at G = 64): bit-planes as MMA fragments, without dequantising.
+//
+// A warp forms the A fragments of mma.sync (16 weight rows x 16 k) in the registers that the MMA reads, with ONE logic
+// operation per two weights: of a register with two weight bytes, one in each half, a mask leaves one bit of each half, at
+// one of the lowest four bits of the fp16 exponent: 0 or 2^-14, 2^-13, 2^-11, 2^-7.  (The mantissa's bits would do, as
+// subnormal numbers, but the tensor core aligns those by their exponent field and loses up to ten bits.)  The activations
+// carry the other factor: scaled by 2^c, 2^(c-1), 2^(c-3), 2^(c-7), c such that the largest |x| of the batch row and step
+// (128 k) lies just below 2^15.  The scaled values are exact except for elements 2^-22 times smaller than that largest
+// one, whose error is at most 2^-33 of it: less than the rounding of the fp32 sums.  So
+//
+//   Y = sum_g [ sum_j s_j 2^(14-c) D_j + z sum_{k in g} x ],   D_j = the MMAs' sum over the group for plane j,
+//
+// with the scales applied to the sums in fp32: W_hat is never formed, as in the look-up kernels, and as exact.  (The MMAs'
+// running sums are truncated, not rounded; a sum runs over one group.)
+//
+//   k order  an MMA sums over k, so A and B only have to agree on which k a lane holds.  Lane c of a quad takes the bytes of word c
+//            of the row's 128 k (at G = 64: bytes 2c, 2c+1 of each group) as two sub-words with one byte in each half, twice: a
+//            left shift by 2 brings the upper copy's bits 0-3 to the four positions, one by 6 the lower copy's bits 4-7 (as
+//            multiplications: the logic pipe is the busy one).
+//   unit     128 weight rows x 512 k (eight packed tiles, contiguous in the blob: one bulk copy).  The units of a call, row tile
+//            by row tile, are dealt to the CTAs (one per SM) in equal contiguous runs, so no SM idles for a wave.  A row
+//            tile that several CTAs share is summed in ascending k order (bit-reproducible) by the CTA that finishes it last
+//            (a ticket per row tile, no CTA waits for another).
+//   warps    16 compute warps: warp 4 s + r takes step s (128 k) of every unit and rows 32 r .. 32 r + 31 of the tile, so each
+//            activation fragment serves two MMAs.  Four activation warps, one per step: scale the unit's activations and
+//            lay them out as B fragments, form the group sums; the first of them also loads the weights.
+//
+// Every wait is bounded; a thread whose wait runs out raises the status word and a CTA-wide flag that ends the other
+// warps' waits; copies in flight are waited for (bounded) and the kernel returns.
+#include "common.cuh"
+
+namespace elutq {
+
+namespace {
+
+constexpr int kComputeWarps = 16, kComputeThreads = 32 * kComputeWarps;
+constexpr int kFragThreads = kComputeThreads + 128;
+constexpr int kUnitRows = 128;
+constexpr uint32_t kFragWaitLimit = 1u << 22;
+constexpr int kMaxRing = 8, kXSlots = 2;        // weight units (at most), units of prepared activations
+constexpr int kSumStride = kUnitRows + 4;       // floats per batch row of the sum buffer (conflict-free for fragments)
+
+struct FragArgs {
+    GemmArgs g;
+    int n_steps;                // 128-k steps of the whole K
+    int chunks;                 // units per row tile (512-k chunks)
+    int units, per_cta;         // all units; units of one CTA
+    int ws;                     // weight units in flight
+    unsigned* tickets;          // one per row tile, zero between calls
+};
+
+enum { kBarWFull = 0, kBarXFull = kBarWFull + kMaxRing, kBarXEmpty = kBarXFull + kXSlots, kNumBars = kBarXEmpty + kXSlots };
+
+template <int Q, int G>
+struct FragCfg {
+    static constexpr int W = G / 8, NSG = 128 / G;
+    static constexpr int PLANE_BYTES = 1024 * Q;
+    static constexpr int TILE_BYTES = PLANE_BYTES + 128 * (NSG * (Q + 1));
+    static constexpr int UNIT_BYTES = 8 * TILE_BYTES;
+};
+
+__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(bar) : "memory");
+}
+__device__ __forceinline__ void mbar_expect(uint32_t bar, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(bar), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    return ok != 0;
+}
+__device__ __forceinline__ bool elect_one() {
+    uint32_t e;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
+    return e != 0;
+}
+__device__ __forceinline__ uint32_t lds32(uint32_t addr) {
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
+    return v;
+}
+__device__ __forceinline__ uint32_t lds16(uint32_t addr) {
+    unsigned short v;
+    asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(addr));
+    return v;
+}
+__device__ __forceinline__ uint4 lds128(uint32_t addr) {
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
+    return v;
+}
+__device__ __forceinline__ void mma_16816(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ float half_bits(uint32_t v) { return __half2float(__ushort_as_half((unsigned short)v)); }
+
+// slot and parity of the n-th use of a ring, advanced without divisions
+struct Ring {
+    int len, i;
+    uint32_t phase;
+    __device__ __forceinline__ Ring(int n) : len(n), i(0), phase(0) {}
+    __device__ __forceinline__ void next() {
+        if (++i == len) { i = 0; phase ^= 1u; }
+    }
+};
+
+// NB = blocks of 8 batch rows (MMA N).
+template <int Q, int G, int NB>
+__global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArgs a) {
+    using C = FragCfg<Q, G>;
+    static_assert(G == 128 || G == 64, "");
+    constexpr int NSG = C::NSG;                               // groups per step: 1 or 2
+    constexpr int MP = 8 * NB;
+    constexpr int XF_BYTES = MP * 1024;                       // B fragments of a unit: [step][block][4][lane] 16 bytes
+    constexpr int XM_FLOATS = 4 * (1 + NSG) * MP;             // per step: factor 2^(14-c) and group sums of every batch row
+    extern __shared__ __align__(1024) uint8_t smem[];
+    uint8_t* sX = smem;
+    uint8_t* sW = sX + kXSlots * XF_BYTES;
+    float* sM = reinterpret_cast<float*>(sW + a.ws * C::UNIT_BYTES);
+    float* sSum = sM + kXSlots * XM_FLOATS;                   // [step][MP][kSumStride]
+    uint64_t* bars = reinterpret_cast<uint64_t*>(sSum + 4 * MP * kSumStride);
+    volatile uint32_t* give_up = reinterpret_cast<uint32_t*>(bars + kNumBars);
+    volatile uint32_t* ticket_box = give_up + 1;
+    volatile uint32_t* stop = give_up + 2;                    // a compute warp gave up (read behind their barrier)
+    const uint32_t bar0 = smem_addr(bars);
+    auto bar = [&](int i) { return bar0 + 8u * (uint32_t)i; };
+
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // warp-uniform for the compiler too
+    uint4 h0;
+    uint2 h1;
+    blob_header_load(a.g.tiles, h0, h1);
+    if (tid == 0) {
+        auto init = [&](int i, int n) { asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(bar(i)), "r"(n) : "memory"); };
+        for (int i = 0; i < kMaxRing; ++i) init(kBarWFull + i, 1);
+        for (int i = 0; i < kXSlots; ++i) {
+            init(kBarXFull + i, 4);
+            init(kBarXEmpty + i, kComputeWarps);              // a unit is done with: its activations and its weights
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        *give_up = 0;
+        *stop = 0;
+    }
+    __syncthreads();
+
+    const int b = blockIdx.x, C_ = a.chunks;
+    const int u0 = b * a.per_cta;
+    int u1 = min(a.units, u0 + a.per_cta);
+    if (!blob_header_ok(h0, h1, Q, G, a.g.N, a.g.K)) {         // before any tile is read; the same answer in every thread: no work
+        u1 = u0;
+        if (tid == 0 && a.g.counters != nullptr) atomicExch(a.g.counters, kStatusBlobMismatch);
+    }
+    const uint32_t limit = a.g.wait_limit ? a.g.wait_limit : kFragWaitLimit;
+    // Bounded wait; false once this CTA has given up.
+    auto wait_many = [&](auto poll) {
+        for (uint32_t n = 0; n < limit; ++n) {
+            if (poll()) return true;
+            if (*give_up) return false;
+        }
+        *give_up = 1;
+        if (a.g.counters != nullptr) atomicExch(a.g.counters, kStatusWaitExpired);
+        return false;
+    };
+    auto steps_of = [&](int chunk) { return min(4, a.n_steps - 4 * chunk); };
+    const int gq = lane >> 2, c = lane & 3;                   // fragment row (and batch row of B), position in the quad
+    const int M = a.g.M, N = a.g.N;
+    grid_launch_dependents();
+
+    if (warp >= kComputeWarps) {
+        // ---- activation warps ------------------------------------------------------------------------------------------------
+        const int step = warp - kComputeWarps;
+        const bool loads = !(a.g.flags & kFlagTestNoMma);     // (test flag: nothing is loaded, the waits run out)
+        int wu = u0;                                          // next unit whose weights are to be loaded
+        auto load_weights = [&](int upto) {                   // by one elected lane; slot = unit number in the CTA mod ws
+            for (; wu < upto; ++wu) {
+                const int tile = wu / C_, rb0 = tile * 8, slot = (wu - u0) % a.ws;
+                const uint32_t bytes = (uint32_t)(min(8, a.g.n_rb - rb0) * C::TILE_BYTES);
+                if (elect_one()) {
+                    mbar_expect(bar(kBarWFull + slot), bytes);
+                    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                                 :: "r"(smem_addr(sW) + (uint32_t)(slot * C::UNIT_BYTES)),
+                                    "l"(a.g.tiles + ((size_t)(wu - tile * C_) * a.g.n_rb + rb0) * C::TILE_BYTES), "r"(bytes), "r"(bar(kBarWFull + slot))
+                                 : "memory");
+                }
+                __syncwarp();
+            }
+        };
+        // weights do not depend on the previous kernel: the first units are requested before the dependency wait
+        if (step == 0 && loads) load_weights(min(u1, u0 + a.ws));
+        grid_dependency_wait();
+
+        // The lane's four 16-byte pieces (8 k each) of a batch row and step: the low and the high bytes of the two sub-words.
+        const int piece[2][2] = {{G == 128 ? 4 * c : 2 * c, G == 128 ? 4 * c + 2 : 2 * c + 1},
+                                 {G == 128 ? 4 * c + 1 : 8 + 2 * c, G == 128 ? 4 * c + 3 : 8 + 2 * c + 1}};
+        constexpr int RB = NB <= 2 ? NB : 2;                  // blocks of 8 rows fetched at a time
+        uint4 raw[RB][2][2];
+        auto fetch = [&](int chunk, int nb0) {
+#pragma unroll
+            for (int nb = 0; nb < RB; ++nb)
+#pragma unroll
+                for (int q = 0; q < 2; ++q)
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const int m = 8 * (nb0 + nb) + gq, k = chunk * kChunkK + step * 128 + piece[q][e] * 8;
+                        raw[nb][q][e] = (m < M && k < a.g.K) ? __ldg(reinterpret_cast<const uint4*>(a.g.X + (size_t)m * a.g.K + k)) : make_uint4(0, 0, 0, 0);
+                    }
+        };
+        int chunk = u0 % C_;
+        if (u0 < u1) fetch(chunk, 0);
+        for (int u = u0; u < u1; ++u) {
+            const int t = u - u0, slot = t & 1;
+            if (!__all_sync(0xffffffffu, wait_many([&]() { return mbar_try(bar(kBarXEmpty + slot), (uint32_t)((t >> 1) & 1) ^ 1u); }))) break;
+            if (step == 0 && t >= 2 && loads) load_weights(min(u1, u - 2 + a.ws + 1));      // the unit two back has been read
+            if (step < steps_of(chunk)) {
+                uint4* frag = reinterpret_cast<uint4*>(sX + slot * XF_BYTES) + step * (NB * 128) + lane;
+                float* meta = sM + slot * XM_FLOATS + step * ((1 + NSG) * MP);
+#pragma unroll 1
+                for (int nb0 = 0; nb0 < NB; nb0 += RB) {
+                if (nb0 > 0) fetch(chunk, nb0);
+#pragma unroll
+                for (int r8 = 0; r8 < RB; ++r8) {
+                    const int nb = nb0 + r8;
+                    __half2 v[2][2][4];
+#pragma unroll
+                    for (int q = 0; q < 2; ++q)
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            const uint32_t r[4] = {raw[r8][q][e].x, raw[r8][q][e].y, raw[r8][q][e].z, raw[r8][q][e].w};
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) v[q][e][i] = *reinterpret_cast<const __half2*>(&r[i]);
+                        }
+                    // group sums: the batch rows as A rows, times ones; a sub-word's activations belong to one group
+                    float sum[2][4] = {};
+                    __half2 mx = __habs2(v[0][0][0]);         // largest |x| of the row's step
+#pragma unroll
+                    for (int q = 0; q < 2; ++q)
+#pragma unroll
+                        for (int e = 0; e < 2; ++e)
+#pragma unroll
+                            for (int i = 0; i < 4; i += 2) {
+                                mma_16816(sum[q], *reinterpret_cast<const uint32_t*>(&v[q][e][i]), 0u,
+                                          *reinterpret_cast<const uint32_t*>(&v[q][e][i + 1]), 0u, 0x3c003c00u, 0x3c003c00u);
+                                mx = __hmax2(mx, __hmax2(__habs2(v[q][e][i]), __habs2(v[q][e][i + 1])));
+                            }
+                    uint32_t top = __half_as_ushort(__hmax(__low2half(mx), __high2half(mx)));
+                    top = max(top, __shfl_xor_sync(0xffffffffu, top, 1));
+                    top = max(top, __shfl_xor_sync(0xffffffffu, top, 2));
+                    const int ex = max(1, (int)(top >> 10)), cx = 29 - ex, c1 = min(cx, 14);      // x 2^cx < 2^15
+                    if (c == 0) {
+                        meta[8 * nb + gq] = __uint_as_float((uint32_t)(127 + 14 - cx) << 23);
+                        if (NSG == 1) {
+                            meta[MP + 8 * nb + gq] = sum[0][0] + sum[1][0];
+                        } else {
+                            meta[MP + 8 * nb + gq] = sum[0][0];
+                            meta[2 * MP + 8 * nb + gq] = sum[1][0];
+                        }
+                    }
+                    // x 2^c1 exactly, then 2^(cx - c1) and what the bit's mask leaves to do (2^cx may exceed fp16)
+                    const uint32_t f1b = (uint32_t)(15 + c1) * 0x04000400u, f2b = (uint32_t)(15 + cx - c1) * 0x04000400u;
+                    const __half2 f1 = *reinterpret_cast<const __half2*>(&f1b);
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        uint32_t o[8];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const __half2 lo = __hmul2(v[q][0][i], f1), hi = __hmul2(v[q][1][i], f1);
+                            const uint32_t l = *reinterpret_cast<const uint32_t*>(&lo), h = *reinterpret_cast<const uint32_t*>(&hi);
+                            const uint32_t pr[2] = {__byte_perm(l, h, 0x5410), __byte_perm(l, h, 0x7632)};
+#pragma unroll
+                            for (int e = 0; e < 2; ++e) {
+                                constexpr uint32_t kDown[4] = {0u, 1u, 3u, 7u};
+                                const uint32_t fb = f2b - kDown[(2 * i + e) & 3] * 0x04000400u;
+                                const __half2 r = __hmul2(*reinterpret_cast<const __half2*>(&pr[e]), *reinterpret_cast<const __half2*>(&fb));
+                                o[2 * i + e] = *reinterpret_cast<const uint32_t*>(&r);
+                            }
+                        }
+                        frag[(nb * 4 + 2 * q) * 32] = make_uint4(o[0], o[1], o[2], o[3]);
+                        frag[(nb * 4 + 2 * q + 1) * 32] = make_uint4(o[4], o[5], o[6], o[7]);
+                    }
+                }
+                }
+            }
+            if (++chunk == C_) chunk = 0;
+            if (u + 1 < u1) fetch(chunk, 0);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(kBarXFull + slot));
+        }
+        if (step == 0)                                        // copies in flight land before the CTA may leave (given up or not)
+            for (int n = max(u0, wu - a.ws); n < wu; ++n)
+                for (uint32_t t = 0; t < kFragWaitLimit && !mbar_try(bar(kBarWFull + (n - u0) % a.ws), (uint32_t)((n - u0) / a.ws) & 1u); ++t) {}
+        __syncthreads();
+        return;
+    }
+
+    // ---- compute warps -------------------------------------------------------------------------------------------------------
+    const int step = warp >> 2, rp = warp & 3;                // the warp's 128 k of every chunk, its 32 rows of the tile
+    const bool use_planes = !(a.g.flags & ELUTQ_FLAG_OFFSET_ONLY), use_offset = !(a.g.flags & ELUTQ_FLAG_SKIP_OFFSET);
+    const uint32_t offset_mask = use_offset ? 0xffffffffu : 0u;
+
+    // Where the lane finds its bytes of rows gq and gq + 8 of a packed tile (the layout rotates groups and bytes by the row):
+    // two 32-bit words at off0 / off1 (G = 64: per group), of which the selectors pick the bytes of a sub-word.
+    uint32_t off0[2], off1[2], sel[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const int l = gq + 8 * e;
+        const uint32_t vec = (uint32_t)((2 * rp) * C::TILE_BYTES + ((step >> 1) * Q * 32 + 16 * (step & 1) + l) * 16);
+        const int ii = G == 128 ? (4 * c - l) & 15 : (2 * c - l) & 7;
+        off0[e] = vec + (uint32_t)(ii & ~3);
+        off1[e] = vec + (uint32_t)(((ii & ~3) + 4) & (C::W - 1));
+    }
+    {   // a sub-word's low byte goes to bytes 0 and 1, its high byte to bytes 2 and 3
+        const uint32_t s = (uint32_t)((G == 128 ? 4 * c - gq : 2 * c - gq) & 3);
+        sel[0] = s * 0x0011u + (s + (G == 128 ? 2u : 1u)) * 0x1100u;
+        sel[1] = G == 128 ? sel[0] + 0x1111u : sel[0];
+    }
+    uint32_t by4 = 4u, by64 = 64u;                            // opaque, so that the products stay products
+    asm volatile("" : "+r"(by4), "+r"(by64));
+    const uint32_t poff = (uint32_t)((2 * rp) * C::TILE_BYTES + C::PLANE_BYTES + (16 * (step & 1) + gq) * 4);
+    // fp16 bits of component `comp` of the group at position p, row r (gq + 8 r of the warp's 32); tb = the unit's weights
+    auto parameter = [&](uint32_t tb, int r, int p, int comp) {
+        const int v = NSG == 1 ? 0 : (p - (r & 1)) & 1;       // (rows gq + 8 start with the other group)
+        const int rec = ((step >> 1) * NSG + v) * (Q + 1) + comp;
+        return lds16(tb + poff + (uint32_t)((r >> 1) * C::TILE_BYTES + (r & 1) * 32 + (rec >> 1) * 128 + (rec & 1) * 2));
+    };
+
+    grid_dependency_wait();
+    const size_t n_pad = (size_t)a.g.n_rb * kTileRows;
+    const bool plain = !(a.g.flags & (ELUTQ_FLAG_OUT_F32 | ELUTQ_FLAG_ACCUMULATE));
+    auto put = [&](int m, int n, float y) {
+        if (plain) reinterpret_cast<__half*>(a.g.Y)[(size_t)m * N + n] = __float2half_rn(y);
+        else store_out(a.g, (size_t)m * N + n, y);
+    };
+    auto compute_sync = []() { asm volatile("bar.sync 1, 512;" ::: "memory"); };
+    // The CTA that came last to a shared row tile adds the parts in ascending k order (all compute threads call this).
+    auto finish_tile = [&](int tile) {
+        if (tile < 0 || *ticket_box == 0u) return;
+        const int n = tile * kUnitRows + (tid & (kUnitRows - 1));
+        const int parts = (tile * C_ + C_ - 1) / a.per_cta - tile * C_ / a.per_cta + 1;
+        if (n >= N) return;
+        const float* p0 = a.g.partials + n;
+        for (int m0 = tid >> 7; m0 < M; m0 += 16) {
+            float y[4] = {0.f, 0.f, 0.f, 0.f};
+            for (int p = 0; p < parts; p += 4) {
+                float v[4][4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        v[e][i] = (p + e < parts && m0 + 4 * i < M) ? __ldcg(p0 + ((size_t)(p + e) * M + m0 + 4 * i) * n_pad) : 0.f;
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) y[i] += v[e][i];
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (m0 + 4 * i < M) put(m0 + 4 * i, n, y[i]);
+        }
+    };
+
+    Ring w(a.ws), x(kXSlots);
+    bool live = true;
+    int pending = -1;                                         // row tile whose ticket has been taken and not looked at
+    for (int u = u0; u < u1 && live;) {
+        const int tile = u / C_, chunk0 = u - tile * C_;
+        const int n_units = min(C_ - chunk0, u1 - u);
+        u += n_units;
+        float acc[2][NB][4];
+#pragma unroll
+        for (int t = 0; t < 2; ++t)
+#pragma unroll
+            for (int nb = 0; nb < NB; ++nb)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) acc[t][nb][i] = 0.f;
+
+        for (int cu = 0; cu < n_units; ++cu) {
+            live = __all_sync(0xffffffffu, wait_many([&]() {
+                return mbar_try(bar(kBarWFull + w.i), w.phase) & mbar_try(bar(kBarXFull + x.i), x.phase);
+            }));
+            if (!live) break;
+            if (step < steps_of(chunk0 + cu)) {
+                const uint32_t wb = smem_addr(sW) + (uint32_t)(w.i * C::UNIT_BYTES);
+                const uint32_t xb = smem_addr(sX) + (uint32_t)(x.i * XF_BYTES + step * (NB * 2048) + lane * 16);
+                const float* meta = sM + x.i * XM_FLOATS + step * ((1 + NSG) * MP) + 2 * c;
+                // B fragments: held over the planes where they fit the registers
+                constexpr bool HOLD = NB <= 2;
+                uint4 xh[HOLD ? NB : 1][4];
+                if constexpr (HOLD) {
+#pragma unroll
+                    for (int nb = 0; nb < NB; ++nb)
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) xh[nb][i] = lds128(xb + (uint32_t)((nb * 4 + i) * 512));
+                }
+                float2 fac[NB];
+#pragma unroll
+                for (int nb = 0; nb < NB; ++nb) fac[nb] = *reinterpret_cast<const float2*>(meta + 8 * nb);
+                if (use_planes) {
+#pragma unroll(NB <= 2 ? Q : 1)
+                for (int j = 0; j < Q; ++j) {
+                    uint32_t sub[2][4];                       // sub-words of the four rows
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        const uint32_t tb = wb + (uint32_t)((r >> 1) * C::TILE_BYTES + j * 512);
+                        if constexpr (G == 128) {
+                            const uint32_t w0 = lds32(tb + off0[r & 1]), w1 = lds32(tb + off1[r & 1]);
+                            sub[0][r] = __byte_perm(w0, w1, sel[0]);
+                            sub[1][r] = __byte_perm(w0, w1, sel[1]);
+                        } else {
+#pragma unroll
+                            for (int p = 0; p < 2; ++p) {
+                                const uint32_t go = (uint32_t)(((p - (r & 1)) & 1) * 8);
+                                sub[p][r] = __byte_perm(lds32(tb + off0[r & 1] + go), lds32(tb + off1[r & 1] + go), sel[0]);
+                            }
+                        }
+                    }
+                    float d[2][NB][4];
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        if (q == 0 || NSG == 2) {
+#pragma unroll
+                            for (int t = 0; t < 2; ++t)
+#pragma unroll
+                                for (int nb = 0; nb < NB; ++nb)
+#pragma unroll
+                                    for (int i = 0; i < 4; ++i) d[t][nb][i] = 0.f;
+                        }
+#pragma unroll
+                        for (int i2 = 0; i2 < 2; ++i2) {      // bits 4 i2 .. 4 i2 + 3 of the sub-word's bytes: two MMAs
+                            uint32_t f[4][4];
+#pragma unroll
+                            for (int r = 0; r < 4; ++r) {
+                                const uint32_t v = sub[q][r] * (i2 ? by64 : by4);
+#pragma unroll
+                                for (int i = 0; i < 4; ++i) f[r][i] = v & (0x04000400u << i);
+                            }
+#pragma unroll
+                            for (int nb = 0; nb < NB; ++nb) {
+                                const uint4 xv = HOLD ? xh[HOLD ? nb : 0][2 * q + i2] : lds128(xb + (uint32_t)((nb * 4 + 2 * q + i2) * 512));
+#pragma unroll
+                                for (int t = 0; t < 2; ++t) {
+                                    mma_16816(d[t][nb], f[2 * t][0], f[2 * t + 1][0], f[2 * t][1], f[2 * t + 1][1], xv.x, xv.y);
+                                    mma_16816(d[t][nb], f[2 * t][2], f[2 * t + 1][2], f[2 * t][3], f[2 * t + 1][3], xv.z, xv.w);
+                                }
+                            }
+                        }
+                        if (q == 1 || NSG == 2) {             // the group is complete: its scale
+                            const int p = NSG == 2 ? q : 0;
+                            float sc[4];
+#pragma unroll
+                            for (int r = 0; r < 4; ++r) sc[r] = half_bits(parameter(wb, r, p, j));
+#pragma unroll
+                            for (int t = 0; t < 2; ++t)
+#pragma unroll
+                                for (int nb = 0; nb < NB; ++nb) {
+                                    acc[t][nb][0] = fmaf(sc[2 * t], d[t][nb][0] * fac[nb].x, acc[t][nb][0]);
+                                    acc[t][nb][1] = fmaf(sc[2 * t], d[t][nb][1] * fac[nb].y, acc[t][nb][1]);
+                                    acc[t][nb][2] = fmaf(sc[2 * t + 1], d[t][nb][2] * fac[nb].x, acc[t][nb][2]);
+                                    acc[t][nb][3] = fmaf(sc[2 * t + 1], d[t][nb][3] * fac[nb].y, acc[t][nb][3]);
+                                }
+                        }
+                    }
+                }
+                }
+                // offsets times the groups' activation sums
+#pragma unroll
+                for (int p = 0; p < NSG; ++p) {
+                    float z[4];
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) z[r] = half_bits(parameter(wb, r, p, Q) & offset_mask);
+#pragma unroll
+                    for (int nb = 0; nb < NB; ++nb) {
+                        const float2 s = *reinterpret_cast<const float2*>(meta + (1 + p) * MP + 8 * nb);
+#pragma unroll
+                        for (int t = 0; t < 2; ++t) {
+                            acc[t][nb][0] = fmaf(z[2 * t], s.x, acc[t][nb][0]);
+                            acc[t][nb][1] = fmaf(z[2 * t], s.y, acc[t][nb][1]);
+                            acc[t][nb][2] = fmaf(z[2 * t + 1], s.x, acc[t][nb][2]);
+                            acc[t][nb][3] = fmaf(z[2 * t + 1], s.y, acc[t][nb][3]);
+                        }
+                    }
+                }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(kBarXEmpty + x.i));
+            w.next();
+            x.next();
+        }
+
+        // The four steps' sums meet in shared memory and are added and written out row by row.  (A warp that gave up still joins
+        // the barriers, and all leave together.)
+        if (!live) *stop = 1;
+        compute_sync();                                       // the buffer has been read; the ticket of the run before is there
+        finish_tile(pending);
+        pending = -1;
+        {
+            float* p = sSum + (step * MP + 2 * c) * kSumStride + 32 * rp + gq;
+#pragma unroll
+            for (int nb = 0; nb < NB; ++nb)
+#pragma unroll
+                for (int t = 0; t < 2; ++t)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) p[(8 * nb + (i & 1)) * kSumStride + 16 * t + 8 * (i >> 1)] = acc[t][nb][i];
+        }
+        compute_sync();
+        if (*stop) break;
+        const int row = tid & (kUnitRows - 1), n = tile * kUnitRows + row;
+        const bool whole = n_units == C_;
+        const int first = tile * C_ / a.per_cta;
+        float* part = a.g.partials + (size_t)(b - first) * M * n_pad + n;
+        for (int m = tid >> 7; m < M; m += kComputeThreads / kUnitRows) {
+            float y = sSum[m * kSumStride + row];
+#pragma unroll
+            for (int s = 1; s < 4; ++s) y += sSum[(s * MP + m) * kSumStride + row];
+            if (whole) {
+                if (n < N) put(m, n, y);
+            } else if ((size_t)n < n_pad) {
+                part[(size_t)m * n_pad] = y;
+            }
+        }
+        if (!whole) {                                         // a ticket; what it says is looked at after the next run of units
+            compute_sync();
+            if (tid == 0) {
+                const int parts = (tile * C_ + C_ - 1) / a.per_cta - first + 1;
+                __threadfence();
+                const unsigned t = atomicAdd(a.tickets + tile, 1u);
+                const bool last = t == (unsigned)(parts - 1);
+                if (last) a.tickets[tile] = 0;                // zero again for the next call
+                __threadfence();
+                *ticket_box = last ? 1u : 0u;
+            }
+            pending = tile;
+        }
+    }
+    compute_sync();
+    if (!*stop) finish_tile(pending);
+    __syncthreads();                                          // nobody leaves while copies are in flight
+}
+
+template <int Q, int G, int NB>
+int launch_frag_cfg(const GemmArgs& g, int num_sms, cudaStream_t stream) {
+    using C = FragCfg<Q, G>;
+    constexpr int kMaxSmem = 232448, MP = 8 * NB;
+    constexpr int kFixed = kXSlots * (MP * 1024 + 4 * (1 + C::NSG) * MP * 4) + 4 * MP * kSumStride * 4 + kNumBars * 8 + 64;
+    static bool configured[64] = {};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev >= 0 && dev < 64 && !configured[dev]) {
+        cudaError_t e = cudaFuncSetAttribute(hlq_frag_kernel<Q, G, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+        if (e != cudaSuccess) return (int)e;
+        configured[dev] = true;
+    }
+    FragArgs a;
+    a.g = g;
+    const int n_tiles = (g.N + kUnitRows - 1) / kUnitRows;
+    a.n_steps = (g.K + 127) / 128;
+    a.chunks = g.n_kc;
+    const long long units = (long long)n_tiles * g.n_kc;
+    if (units >= (1LL << 30)) return (int)cudaErrorInvalidValue;
+    a.units = (int)units;
+    a.per_cta = (a.units + num_sms - 1) / num_sms;
+    const int grid = (a.units + a.per_cta - 1) / a.per_cta;
+    a.tickets = g.counters + 64;
+    static_assert((kMaxSmem - kFixed) / C::UNIT_BYTES >= 2, "shared memory");
+    a.ws = (kMaxSmem - kFixed) / C::UNIT_BYTES;
+    if (a.ws > 5) a.ws = 5;
+
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(kFragThreads);
+    cfg.dynamicSmemBytes = a.ws * C::UNIT_BYTES + kFixed;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, hlq_frag_kernel<Q, G, NB>, a);
+    count_launch(1);
+    return (int)e;
+}
+
+template <int Q, int G>
+int launch_frag_qg(const GemmArgs& g, int num_sms, cudaStream_t stream) {
+    if (g.M <= 8) return launch_frag_cfg<Q, G, 1>(g, num_sms, stream);
+    if (g.M <= 16) return launch_frag_cfg<Q, G, 2>(g, num_sms, stream);
+    if constexpr (G == 64) return launch_frag_cfg<Q, G, 4>(g, num_sms, stream);
+    return (int)cudaErrorInvalidValue;
+}
+
+template <int Q>
+int launch_frag_q(const GemmArgs& g, int G, int num_sms, cudaStream_t stream) {
+    switch (G) {
+        case 64: return launch_frag_qg<Q, 64>(g, num_sms, stream);
+        case 128: return launch_frag_qg<Q, 128>(g, num_sms, stream);
+        default: return (int)cudaErrorNotSupported;
+    }
+}
+
+}  // namespace
+
+// Up to ELUTQ_FRAGMENT_MAX_M rows at G = 128, any number at G = 64 (32 rows to a launch; the launches follow one another on
+// the stream and share the partial sums).
+int launch_hlq_frag(const GemmArgs& g, int q, int G, int num_sms, cudaStream_t stream) {
+    const size_t out = (g.flags & ELUTQ_FLAG_OUT_F32) ? sizeof(float) : sizeof(__half);
+    int ce = 0;
+    for (int m0 = 0; m0 < g.M && ce == 0; m0 += 32) {
+        GemmArgs p = g;
+        p.X = g.X + (size_t)m0 * g.K;
+        p.Y = reinterpret_cast<uint8_t*>(g.Y) + (size_t)m0 * g.N * out;
+        p.M = g.M - m0 < 32 ? g.M - m0 : 32;
+        switch (q) {
+            case 1: ce = launch_frag_q<1>(p, G, num_sms, stream); break;
+            case 2: ce = launch_frag_q<2>(p, G, num_sms, stream); break;
+            case 3: ce = launch_frag_q<3>(p, G, num_sms, stream); break;
+            case 4: ce = launch_frag_q<4>(p, G, num_sms, stream); break;
+            default: ce = (int)cudaErrorInvalidValue;
+        }
+    }
+    return ce;
+}
+
+}  // namespace elutq

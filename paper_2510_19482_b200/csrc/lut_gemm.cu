@@ -1,4 +1,4 @@
-// 2 <= M < ELUTQ_TENSOR_MIN_M (or any M > 1 on request): batched look-up GEMM over the same packed layout.
+// 2 <= M < ELUTQ_TENSOR_MIN_M (any M > 1 at G = 32 or on request): batched look-up GEMM over the same packed layout.
 //
 // MB activation rows are processed per pass: a table entry holds the partial sums of all MB rows for one
 // (byte value, column), so one weight byte costs one byte-permute, one shared-memory load and the adds of MB

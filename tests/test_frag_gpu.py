@@ -1,0 +1,61 @@
+"""GPU parity of the fragment kernel (batches of 3 to 16 rows at G = 128, any from 3 rows on at G = 64): bit-planes contracted
+on the tensor cores as they are, scales applied to fp32 sums.
+
+Tolerance: activations are scaled by powers of two (exact but for 2^-33 of the row's largest), products are exact, the
+MMAs' fp32 sums run over one group and are truncated (at most 2^-23 per step of 16 k), the groups are added in fp32: the same
+order as the look-up kernels' K * 2^-24 * A per element, doubled for the truncation, and 5e-6 in norm.
+"""
+
+import numpy as np
+import pytest
+import torch
+
+import paper_2510_19482_b200 as elutq
+import workloads
+from oracle import hlq
+from workloads import synth
+
+pytestmark = pytest.mark.gpu
+
+from gpu_util import gemm_f32, pack_layer, x_dev  # noqa: E402
+
+# (q, G, N, K, M): edges of the 8- and 16-row fragments, the 32-row launch and the 128-row tile, K ending inside a 512-k chunk and
+# a 64-k half step, one tile and one chunk, row tiles shared by several CTAs, every q
+CASES = [(2, 128, 128, 512, 3), (1, 128, 17, 128, 8), (3, 128, 129, 640, 9), (4, 128, 1000, 1408, 16), (2, 128, 4096, 4096, 5),
+         (4, 128, 300, 4224, 16), (3, 64, 127, 64, 3), (2, 64, 256, 1088, 16), (4, 64, 333, 2880, 17), (3, 64, 1000, 1984, 33),
+         (1, 64, 2048, 4096, 32)]
+
+
+@pytest.mark.parametrize("q,G,N,K,M", CASES)
+def test_fragment_kernel_matches_oracle(q, G, N, K, M):
+    layer = workloads.hlq_layer(60, f"frag/{q}/{G}/{N}/{K}", q, G, N, K, signed_scales=(q % 2 == 1))
+    X = synth.activations(60, f"frag/x/{M}/{K}", M, K, outliers=True)
+    X[0] *= np.float16(2.0 ** -12)                       # rows of very different size: each has its own exponent
+    X[-1] *= np.float16(100.0)
+    packed = pack_layer(layer)
+    ref = hlq.matmul(X, layer.planes, layer.scales, layer.offsets, G)
+    y = gemm_f32(X, packed, N, K)
+    assert elutq.elutq_device_status() == 0
+    assert max(hlq.rel_fro_error(y[m], ref[m]) for m in range(M)) <= 5e-6
+    A = hlq.magnitude_bound(X, layer.scales, layer.offsets, G)
+    assert np.all(np.abs(y - ref) <= 2 * K * 2.0 ** -24 * A)
+    assert np.array_equal(y.view(np.uint32), gemm_f32(X, packed, N, K).view(np.uint32))       # and the tickets are zero again
+    ys = gemm_f32(X, packed, N, K, elutq.FLAG_SKIP_OFFSET)
+    yb = gemm_f32(X, packed, N, K, elutq.FLAG_OFFSET_ONLY)
+    assert max(hlq.rel_fro_error(ys[m], hlq.scale_term(X, layer.planes, layer.scales, G)[m]) for m in range(M)) <= 5e-6
+    assert max(hlq.rel_fro_error(yb[m], hlq.offset_term(X, layer.offsets, G)[m]) for m in range(M)) <= 5e-6
+
+
+def test_fragment_kernel_reports_a_wait_that_runs_out():
+    q, G, N, K, M = 2, 128, 512, 2048, 12
+    layer = workloads.hlq_layer(61, "frag/expiry", q, G, N, K)
+    X = synth.activations(61, "frag/expiry/x", M, K)
+    packed = pack_layer(layer)
+    elutq.elutq_release_scratch()
+    Y = torch.zeros((M, N), dtype=torch.float32, device="cuda")
+    elutq.elutq_test_wait_expiry(x_dev(X), packed, Y, M, N, K, 4096)
+    assert elutq.elutq_device_status() == 0x7C05
+    elutq.elutq_release_scratch()
+    y = gemm_f32(X, packed, N, K)
+    assert elutq.elutq_device_status() == 0
+    assert hlq.rel_fro_error(y, hlq.matmul(X, layer.planes, layer.scales, layer.offsets, G)) <= 5e-6
