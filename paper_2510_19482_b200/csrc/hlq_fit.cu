@@ -1,8 +1,19 @@
-// Algorithm 1 on the GPU: alternating bit-pattern selection and least squares, one warp per weight group.
+// Algorithm 1 on the GPU: alternating bit-pattern selection and least squares.
 //
 // The step before the hot path: it turns unquantised fp16 weights into the (B, s, z) that elutq_pack
-// consumes.  Groups are independent, so a warp owns one group of G weights (G / 32 per lane) and keeps
-// everything in registers:
+// consumes.  Groups are independent.  Two forms with the same results bit for bit:
+//
+//   sorted   a lane per group.  The nearest candidate of a weight only depends on between which candidates it lies, so once
+//            a group's weights are sorted a round needs the 2^q - 1 places where the choice changes, not a look at every
+//            weight: a binary search on an estimate of each place, settled by the exact comparison of the two candidates at the
+//            neighbouring weights; bit counts and right-hand sides follow from the places and prefix sums.  A warp sorts its 32
+//            groups (two at a time in the halves of a register), then every lane runs its group's rounds, then
+//            the warp writes the bits.  A round's instructions are shared by 32 groups.  4096 x 4096, G = 128, ten rounds:
+//            q = 2 688 us direct (561 with the stop at unchanged bits), 113 sorted; q = 4 2293 (1616), 605.
+//   direct   a warp per group (G / 32 weights per lane) that evaluates every candidate for every weight: for few groups, for the error
+//            trace, and for groups with two candidates so close that rounding decides between them.
+//
+// The direct form:
 //
 //   initialisation   Delta = (max - min) / (2^q - 1), s = [Delta, 2 Delta, ...], z = min   (warp min / max)
 //   selection        every lane evaluates the 2^q candidate values for its weights, first minimum wins
@@ -24,6 +35,9 @@ namespace elutq {
 namespace {
 
 constexpr int kFitWarps = 8;      // warps (groups) per CTA
+// Fewer groups than this (q <= 2; 16384 above) leave the sorted form waiting on its own latencies: 8192 groups of 128, q = 2, ten rounds:
+// 45 us sorted, 46 direct; q = 4: 142 / 127, at 16384 of 64 121 / 122, at 32768 of 128 199 / 423.
+constexpr long long kSortedMinGroups = 8192;
 
 __device__ __forceinline__ long long warp_sum_ll(long long v) {
 #pragma unroll
@@ -36,17 +50,14 @@ __device__ __forceinline__ double warp_sum_d(double v) {
     return v;
 }
 
+// The direct form for one group, by a whole warp.
 template <int Q, int EPL>
-__global__ void __launch_bounds__(kFitWarps * 32) hlq_fit_kernel(const __half* __restrict__ W, int N, int K, int t_max,
-                                                                 uint8_t* __restrict__ planes, __half* __restrict__ scales,
-                                                                 __half* __restrict__ offsets, double* __restrict__ trace) {
+__device__ __forceinline__ void fit_group(const __half* __restrict__ W, long long grp, long long n_groups, int t_max,
+                                          uint8_t* __restrict__ planes, __half* __restrict__ scales, __half* __restrict__ offsets,
+                                          double* __restrict__ trace) {
     constexpr int G = 32 * EPL, NC = 1 << Q, NV = Q + 1;
     const int lane = threadIdx.x & 31;
-    const long long n_groups = (long long)N * (K / G);
-    const long long grp = (long long)blockIdx.x * kFitWarps + (threadIdx.x >> 5);
-    if (grp >= n_groups) return;
-    const int n = (int)(grp / (K / G)), kg = (int)(grp % (K / G));
-    const size_t base = (size_t)n * K + (size_t)kg * G;
+    const size_t base = (size_t)grp * G, plane_stride = (size_t)n_groups * G;      // (groups are contiguous: K is a multiple of G)
 
     double w[EPL];
     long long wfix[EPL];
@@ -74,7 +85,9 @@ __global__ void __launch_bounds__(kFitWarps * 32) hlq_fit_kernel(const __half* _
 #pragma unroll
     for (int j = 0; j < Q; ++j) s[j] = delta * (double)(1 << j);      // exact scaling
 
-    int code[EPL];
+    int code[EPL], before[EPL];
+#pragma unroll
+    for (int e = 0; e < EPL; ++e) before[e] = -1;
     auto select = [&]() {
         double V[NC];
 #pragma unroll
@@ -120,6 +133,20 @@ __global__ void __launch_bounds__(kFitWarps * 32) hlq_fit_kernel(const __half* _
 
     for (int t = 1; t <= t_max; ++t) {
         select();
+        // the same bits as in the round before: the parameters are theirs already, and so on in every later round
+        bool same = true;
+#pragma unroll
+        for (int e = 0; e < EPL; ++e) {
+            same &= code[e] == before[e];
+            before[e] = code[e];
+        }
+        if (__all_sync(0xffffffffu, same)) {
+            if (trace == nullptr) break;
+            const double et = group_sse();
+            if (lane == 0)
+                for (int r = t; r <= t_max; ++r) trace[(size_t)r * n_groups + grp] = et;
+            break;
+        }
 
         // ---- normal equations: bit counts (exact) and fixed-point weight sums (exact) -----------------
         long long A[NV][NV];
@@ -227,7 +254,7 @@ __global__ void __launch_bounds__(kFitWarps * 32) hlq_fit_kernel(const __half* _
 #pragma unroll
     for (int j = 0; j < Q; ++j)
 #pragma unroll
-        for (int e = 0; e < EPL; ++e) planes[(size_t)j * N * K + base + lane + 32 * e] = (uint8_t)((code[e] >> j) & 1);
+        for (int e = 0; e < EPL; ++e) planes[j * plane_stride + base + lane + 32 * e] = (uint8_t)((code[e] >> j) & 1);
     if (lane < Q) {
         double v = s[0];
 #pragma unroll
@@ -237,19 +264,393 @@ __global__ void __launch_bounds__(kFitWarps * 32) hlq_fit_kernel(const __half* _
     if (lane == Q) offsets[grp] = __double2half(z);
 }
 
-template <int Q>
-int launch_fit_q(const __half* W, int G, int N, int K, int t_max, uint8_t* planes, __half* scales, __half* offsets,
-                 double* trace, cudaStream_t stream) {
+template <int Q, int EPL>
+__global__ void __launch_bounds__(kFitWarps * 32) hlq_fit_kernel(const __half* __restrict__ W, long long n_groups, int t_max,
+                                                                 uint8_t* __restrict__ planes, __half* __restrict__ scales,
+                                                                 __half* __restrict__ offsets, double* __restrict__ trace) {
+    const long long grp = (long long)blockIdx.x * kFitWarps + (threadIdx.x >> 5);
+    if (grp < n_groups) fit_group<Q, EPL>(W, grp, n_groups, t_max, planes, scales, offsets, trace);
+}
+
+constexpr int kSortWarps = 4;     // warps (of 32 groups) per CTA of the sorted form
+// Bytes of a group's record.  It bounds the warps on an SM, and with them the latencies hidden: prefix sums of every 8 weights instead
+// of 4 took G = 128 from 146 to 113 us (q = 2, 4096 x 4096); at G = 32 the longer remainders cost more (1027 / 1083 us, q = 4).
+__host__ __device__ constexpr int sorted_step(int G) { return G == 32 ? 4 : 8; }
+__host__ __device__ constexpr int sorted_record(int G) { return 2 * G + 8 * (G / sorted_step(G) + 1); }
+
+// Determinant of [B 1]^T [B 1] (bit counts of at most 128): minors of order 4 stay below 2^30 in every partial sum.
+template <int NV>
+__device__ __forceinline__ bool gram_singular(const int (&m)[NV][NV]) {
+    if constexpr (NV == 2) {
+        return m[0][0] * m[1][1] - m[0][1] * m[1][0] == 0;
+    } else {
+        // minors of the first two rows by column pair, then row by row
+        int d2[NV][NV];
+#pragma unroll
+        for (int a = 0; a < NV; ++a)
+#pragma unroll
+            for (int b = a + 1; b < NV; ++b) d2[a][b] = m[0][a] * m[1][b] - m[0][b] * m[1][a];
+        auto d3 = [&](int a, int b, int c) { return m[2][a] * d2[b][c] - m[2][b] * d2[a][c] + m[2][c] * d2[a][b]; };
+        if constexpr (NV == 3) {
+            return d3(0, 1, 2) == 0;
+        } else if constexpr (NV == 4) {
+            return m[3][0] * d3(1, 2, 3) - m[3][1] * d3(0, 2, 3) + m[3][2] * d3(0, 1, 3) - m[3][3] * d3(0, 1, 2) == 0;
+        } else {
+            auto d4 = [&](int a, int b, int c, int d) {
+                return m[3][a] * d3(b, c, d) - m[3][b] * d3(a, c, d) + m[3][c] * d3(a, b, d) - m[3][d] * d3(a, b, c);
+            };
+            return (long long)m[4][0] * d4(1, 2, 3, 4) - (long long)m[4][1] * d4(0, 2, 3, 4) + (long long)m[4][2] * d4(0, 1, 3, 4) -
+                   (long long)m[4][3] * d4(0, 1, 2, 4) + (long long)m[4][4] * d4(0, 1, 2, 3) == 0;
+        }
+    }
+}
+
+template <int Q, int G>
+__global__ void __launch_bounds__(kSortWarps * 32) hlq_fit_sorted_kernel(const __half* __restrict__ W, long long n_groups, int t_max,
+                                                                         uint8_t* __restrict__ planes, __half* __restrict__ scales,
+                                                                         __half* __restrict__ offsets, const bool aligned) {
+    constexpr int NC = 1 << Q, NV = Q + 1, NB = 32 * G / 128;     // NB: blocks of 128 weights of a warp's 32 groups
+    constexpr int PS = sorted_step(G), REC = sorted_record(G);    // a group's sorted weights, and prefix sums of every PS of them
+    extern __shared__ __align__(16) uint8_t smem[];
+    const int lane = threadIdx.x & 31;
+    uint8_t* recs = smem + (threadIdx.x >> 5) * (32 * REC);
+    const long long grp0 = ((long long)blockIdx.x * kSortWarps + (threadIdx.x >> 5)) * 32;
+    if (grp0 >= n_groups) return;
+    const long long total = n_groups * G, w0 = grp0 * G;          // weights in all; the warp's first
+    const size_t plane_stride = (size_t)total;
+
+    auto load4 = [&](int block, __half (&h)[4]) {                 // weights 4 lane .. 4 lane + 3 of a block (zeros behind the end)
+        const long long i = w0 + block * 128 + 4 * lane;
+        if (aligned && i < total) {                               // (G is a multiple of 32: four weights are inside or outside)
+            const uint2 r = *reinterpret_cast<const uint2*>(W + i);
+            *reinterpret_cast<uint2*>(h) = r;
+        } else {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) h[e] = i + e < total ? W[i + e] : __ushort_as_half(0);
+        }
+    };
+
+    // ---- sort: bitonic over runs of G, two blocks at a time in the halves of a register.  Every merge begins against the mirrored
+    // half, so that all exchanges are ascending. -----------------------------------------------------------------------------
+    auto exchange = [&](__half2 mine, __half2 other, bool low) {  // the smaller for the lower index, the larger for the higher
+        const __half2 mn = __hmin2(mine, other), mx = __hmax2(mine, other);
+        return low ? mn : mx;
+    };
+    for (int blk = 0; blk < NB; blk += 2) {
+        __half ha[4], hb[4];
+        load4(blk, ha);
+        load4(blk + 1, hb);
+        __half2 v[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) v[e] = __halves2half2(ha[e], hb[e]);
+        auto in_lane = [&](int a, int b) {
+            const __half2 mn = __hmin2(v[a], v[b]), mx = __hmax2(v[a], v[b]);
+            v[a] = mn;
+            v[b] = mx;
+        };
+#pragma unroll
+        for (int size = 2; size <= G; size <<= 1) {
+            if (size == 2) {
+                in_lane(0, 1);
+                in_lane(2, 3);
+                continue;
+            }
+            if (size == 4) {
+                in_lane(0, 3);
+                in_lane(1, 2);
+            } else {                                              // against index ^ (size - 1)
+                const bool low = (lane & (size / 8)) == 0;
+                __half2 o[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) o[e] = __shfl_xor_sync(0xffffffffu, v[3 - e], size / 4 - 1);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) v[e] = exchange(v[e], o[e], low);
+            }
+#pragma unroll
+            for (int stride = size / 4; stride >= 4; stride >>= 1) {
+                const bool low = (lane & (stride / 4)) == 0;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) v[e] = exchange(v[e], __shfl_xor_sync(0xffffffffu, v[e], stride / 4), low);
+            }
+            if (size >= 8) {
+                in_lane(0, 2);
+                in_lane(1, 3);
+            }
+            in_lane(0, 1);
+            in_lane(2, 3);
+        }
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            __half h[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) h[e] = half ? __high2half(v[e]) : __low2half(v[e]);
+            // sums of fp16 values are exact in fp64
+            const double own = (double)__half2float(h[0]) + (double)__half2float(h[1]) + (double)__half2float(h[2]) + (double)__half2float(h[3]);
+            double incl = own;
+#pragma unroll
+            for (int o = 1; o < G / 4; o <<= 1) {
+                const double below = __shfl_up_sync(0xffffffffu, incl, o, G / 4);
+                if ((lane & (G / 4 - 1)) >= o) incl += below;
+            }
+            const int i = (blk + half) * 128 + 4 * lane, g = i / G, pos = i % G;
+            uint8_t* rec = recs + g * REC;
+            *reinterpret_cast<uint2*>(rec + 2 * pos) = *reinterpret_cast<const uint2*>(h);
+            double* pre = reinterpret_cast<double*>(rec + 2 * G);
+            if (pos % PS == 0) pre[pos / PS] = incl - own;
+            if (pos == G - 4) pre[G / PS] = incl;
+        }
+    }
+    __syncwarp();
+
+    // ---- rounds: lane = group --------------------------------------------------------------------------------------------------
+    uint8_t* rec = recs + lane * REC;
+    const __half* sorted = reinterpret_cast<const __half*>(rec);
+    double* pre = reinterpret_cast<double*>(rec + 2 * G);
+    const long long grp = grp0 + lane;
+    const bool valid = grp < n_groups;
+    auto weight = [&](int i) { return __half2float(sorted[i]); };
+    const double wmin = (double)weight(0), wmax = (double)weight(G - 1);
+    double s[Q], z = wmin;
+    const double delta = __ddiv_rn(__dsub_rn(wmax, wmin), (double)(NC - 1));
+#pragma unroll
+    for (int j = 0; j < Q; ++j) s[j] = delta * (double)(1 << j);      // exact scaling
+
+    int cut[NC - 1];                                              // first weight above the r-th place
+#pragma unroll
+    for (int r = 0; r < NC - 1; ++r) cut[r] = -1;
+    unsigned long long map = 0;                                   // nibble r: code of the r-th smallest candidate
+    bool active = valid, direct = false;
+    for (int t = 1; t <= t_max && __any_sync(0xffffffffu, active); ++t) {
+        if (!active) continue;
+        double V[NC];
+        int code[NC];
+#pragma unroll
+        for (int k = 0; k < NC; ++k) {
+            double v = 0.0;
+#pragma unroll
+            for (int j = 0; j < Q; ++j)
+                if ((k >> j) & 1) v = __dadd_rn(v, s[j]);
+            V[k] = v;
+            code[k] = k;
+        }
+        // candidates in ascending order (odd-even merge exchanges)
+#pragma unroll
+        for (int p = 1; p < NC; p <<= 1)
+#pragma unroll
+            for (int k = p; k >= 1; k >>= 1)
+#pragma unroll
+                for (int j = k % p; j <= NC - 1 - k; j += 2 * k)
+#pragma unroll
+                    for (int i = 0; i < k; ++i) {
+                        const int x = i + j, y = i + j + k;
+                        if (y < NC && x / (2 * p) == y / (2 * p)) {
+                            const bool swap = V[y] < V[x];
+                            const double lo = swap ? V[y] : V[x], hi = swap ? V[x] : V[y];
+                            const int cl = swap ? code[y] : code[x], ch = swap ? code[x] : code[y];
+                            V[x] = lo;
+                            V[y] = hi;
+                            code[x] = cl;
+                            code[y] = ch;
+                        }
+                    }
+        // Only the two candidates around a weight are in question as long as no two are within rounding of each other.
+        const double gap = 9.094947017729282e-13 /* 2^-40 */ * (fmax(fabs(wmin), fabs(wmax)) + fabs(z) + fmax(fabs(V[0]), fabs(V[NC - 1])));
+        bool apart = true;
+#pragma unroll
+        for (int r = 0; r < NC - 1; ++r) apart &= V[r + 1] - V[r] > gap;
+        if (!apart) {                                             // (also for values that are not finite)
+            direct = true;
+            active = false;
+            continue;
+        }
+        unsigned long long new_map = 0;
+#pragma unroll
+        for (int r = 0; r < NC; ++r) new_map |= (unsigned long long)code[r] << (4 * r);
+        bool changed = new_map != map;
+        map = new_map;
+#pragma unroll
+        for (int r = 0; r < NC - 1; ++r) {
+            const float guess = (float)(z + 0.5 * (V[r] + V[r + 1]));
+            int pos = 0;
+#pragma unroll
+            for (int st = G / 2; st >= 1; st >>= 1)
+                if (weight(pos + st - 1) < guess) pos += st;
+            if (weight(pos) < guess) ++pos;
+            auto above = [&](int i) {                             // the exact choice between candidates r and r + 1
+                const double shifted = __dsub_rn((double)weight(i), z);
+                const double da = fabs(__dsub_rn(shifted, V[r])), db = fabs(__dsub_rn(shifted, V[r + 1]));
+                return db < da || (db == da && code[r + 1] < code[r]);
+            };
+            while (pos > 0 && above(pos - 1)) --pos;
+            while (pos < G && !above(pos)) ++pos;
+            changed |= pos != cut[r];
+            cut[r] = pos;
+        }
+        // the same bits as in the round before: the parameters are theirs already, and so on in every later round
+        if (!changed) {
+            active = false;
+            continue;
+        }
+        int A[NV][NV];
+        double b[NV];
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {
+            b[i] = 0.0;
+#pragma unroll
+            for (int j = 0; j < NV; ++j) A[i][j] = 0;
+        }
+        A[Q][Q] = G;
+        b[Q] = 0.0 + pre[G / PS];                                // (never a negative zero)
+        {
+            int from = 0;
+            double below = 0.0;
+#pragma unroll
+            for (int r = 0; r < NC; ++r) {
+                const int to = r < NC - 1 ? cut[r < NC - 1 ? r : 0] : G;
+                double upto = pre[to / PS];
+#pragma unroll
+                for (int e = 0; e < PS - 1; ++e)
+                    if (e < to % PS) upto += (double)weight(to / PS * PS + e);
+                const int cnt = to - from;
+                const double part = upto - below;                 // exact
+                from = to;
+                below = upto;
+#pragma unroll
+                for (int i = 0; i < Q; ++i) {
+                    if ((code[r] >> i) & 1) {
+                        b[i] += part;
+                        A[i][Q] += cnt;
+                    }
+#pragma unroll
+                    for (int j = i; j < Q; ++j)
+                        if (((code[r] >> i) & (code[r] >> j)) & 1) A[i][j] += cnt;
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < NV; ++i)
+#pragma unroll
+                for (int j = 0; j < i; ++j) A[i][j] = A[j][i];
+        }
+        // fp64, elimination without pivoting, one rounding per operation (the direct form's order)
+        if (!gram_singular(A)) {
+            double a[NV][NV], x[NV];
+#pragma unroll
+            for (int i = 0; i < NV; ++i)
+#pragma unroll
+                for (int j = 0; j < NV; ++j) a[i][j] = (double)A[i][j];
+#pragma unroll
+            for (int c = 0; c < NV; ++c) {
+#pragma unroll
+                for (int i = c + 1; i < NV; ++i) {
+                    const double f = __ddiv_rn(a[i][c], a[c][c]);
+#pragma unroll
+                    for (int j = c + 1; j < NV; ++j) a[i][j] = __dsub_rn(a[i][j], __dmul_rn(f, a[c][j]));
+                    b[i] = __dsub_rn(b[i], __dmul_rn(f, b[c]));
+                }
+            }
+#pragma unroll
+            for (int i = NV - 1; i >= 0; --i) {
+                double acc = b[i];
+#pragma unroll
+                for (int j = i + 1; j < NV; ++j) acc = __dsub_rn(acc, __dmul_rn(a[i][j], x[j]));
+                x[i] = __ddiv_rn(acc, a[i][i]);
+            }
+#pragma unroll
+            for (int j = 0; j < Q; ++j) s[j] = x[j];
+            z = x[Q];
+        }
+    }
+
+    // ---- results: parameters by lane; per group the weights at the places and the codes, then the bits by the warp -----------
+    __half place[NC - 1];
+#pragma unroll
+    for (int r = 0; r < NC - 1; ++r) place[r] = cut[r] < G ? sorted[max(cut[r], 0)] : __ushort_as_half(0x7c00);      // (infinity: none)
+    __syncwarp();
+    __half* places = reinterpret_cast<__half*>(rec + 8);
+    *reinterpret_cast<unsigned long long*>(rec) = map;
+#pragma unroll
+    for (int r = 0; r < NC - 1; ++r) places[r] = place[r];
+    if (valid && !direct) {
+#pragma unroll
+        for (int j = 0; j < Q; ++j) scales[(size_t)grp * Q + j] = __double2half(s[j]);
+        offsets[grp] = __double2half(z);
+    }
+    const unsigned directs = __ballot_sync(0xffffffffu, direct);
+    __syncwarp();
+    for (int blk = 0; blk < NB; ++blk) {
+        __half h[4];
+        load4(blk, h);
+        const int g = (blk * 128 + 4 * lane) / G;
+        const long long i = w0 + blk * 128 + 4 * lane;
+        const uint8_t* gr = recs + g * REC;
+        const __half* pl = reinterpret_cast<const __half*>(gr + 8);
+        const unsigned long long codes = *reinterpret_cast<const unsigned long long*>(gr);
+        __half2 rank[2] = {__float2half2_rn(1024.f), __float2half2_rn(1024.f)};      // (1024 + rank: the rank in the low bits)
+        const __half2 w2[2] = {__halves2half2(h[0], h[1]), __halves2half2(h[2], h[3])};
+#pragma unroll
+        for (int r = 0; r < NC - 1; ++r) {
+            const __half2 p2 = __half2half2(pl[r]);
+            rank[0] = __hadd2(rank[0], __hge2(w2[0], p2));
+            rank[1] = __hadd2(rank[1], __hge2(w2[1], p2));
+        }
+        uint32_t four = 0;                                        // the codes of four weights, a byte each
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const __half rk = (e & 1) ? __high2half(rank[e >> 1]) : __low2half(rank[e >> 1]);
+            four |= (uint32_t)((codes >> (4 * (__half_as_ushort(rk) & 15))) & 15u) << (8 * e);
+        }
+        if (i < total && !((directs >> g) & 1u)) {
+#pragma unroll
+            for (int j = 0; j < Q; ++j) {
+                const uint32_t bits = (four >> j) & 0x01010101u;
+                uint8_t* dst = planes + j * plane_stride + i;
+                if (aligned) {
+                    *reinterpret_cast<uint32_t*>(dst) = bits;
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) dst[e] = (uint8_t)(bits >> (8 * e));
+                }
+            }
+        }
+    }
+    for (unsigned left = directs; left != 0; left &= left - 1)
+        fit_group<Q, G / 32>(W, grp0 + __ffs(left) - 1, n_groups, t_max, planes, scales, offsets, nullptr);
+}
+
+template <int Q, int G>
+int launch_fit_qg(const __half* W, int N, int K, int t_max, uint8_t* planes, __half* scales, __half* offsets, double* trace,
+                  cudaStream_t stream) {
     const long long n_groups = (long long)N * (K / G);
-    const unsigned grid = (unsigned)((n_groups + kFitWarps - 1) / kFitWarps);
-    switch (G) {
-        case 32: hlq_fit_kernel<Q, 1><<<grid, kFitWarps * 32, 0, stream>>>(W, N, K, t_max, planes, scales, offsets, trace); break;
-        case 64: hlq_fit_kernel<Q, 2><<<grid, kFitWarps * 32, 0, stream>>>(W, N, K, t_max, planes, scales, offsets, trace); break;
-        case 128: hlq_fit_kernel<Q, 4><<<grid, kFitWarps * 32, 0, stream>>>(W, N, K, t_max, planes, scales, offsets, trace); break;
-        default: return (int)cudaErrorInvalidValue;
+    if (trace == nullptr && n_groups >= (Q <= 2 ? 1 : 2) * kSortedMinGroups) {
+        constexpr int kSmem = kSortWarps * 32 * sorted_record(G);
+        static bool configured[64] = {};
+        int dev = 0;
+        cudaGetDevice(&dev);
+        if (dev >= 0 && dev < 64 && !configured[dev]) {
+            cudaError_t e = cudaFuncSetAttribute(hlq_fit_sorted_kernel<Q, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+            if (e != cudaSuccess) return (int)e;
+            configured[dev] = true;
+        }
+        const bool aligned = ((reinterpret_cast<uintptr_t>(W) & 7) | (reinterpret_cast<uintptr_t>(planes) & 3)) == 0;
+        const unsigned grid = (unsigned)((n_groups + 32 * kSortWarps - 1) / (32 * kSortWarps));
+        hlq_fit_sorted_kernel<Q, G><<<grid, kSortWarps * 32, kSmem, stream>>>(W, n_groups, t_max, planes, scales, offsets, aligned);
+    } else {
+        const unsigned grid = (unsigned)((n_groups + kFitWarps - 1) / kFitWarps);
+        hlq_fit_kernel<Q, G / 32><<<grid, kFitWarps * 32, 0, stream>>>(W, n_groups, t_max, planes, scales, offsets, trace);
     }
     count_launch(1);
     return (int)cudaGetLastError();
+}
+
+template <int Q>
+int launch_fit_q(const __half* W, int G, int N, int K, int t_max, uint8_t* planes, __half* scales, __half* offsets,
+                 double* trace, cudaStream_t stream) {
+    switch (G) {
+        case 32: return launch_fit_qg<Q, 32>(W, N, K, t_max, planes, scales, offsets, trace, stream);
+        case 64: return launch_fit_qg<Q, 64>(W, N, K, t_max, planes, scales, offsets, trace, stream);
+        case 128: return launch_fit_qg<Q, 128>(W, N, K, t_max, planes, scales, offsets, trace, stream);
+        default: return (int)cudaErrorInvalidValue;
+    }
 }
 
 }  // namespace

@@ -11,6 +11,8 @@ from tests.gpu_util import gemm_f32, to_dev
 
 pytestmark = pytest.mark.gpu
 
+SORTED_MIN_GROUPS = 16384        # from this many groups on elutq_hlq_fit sorts the groups for every q (without a trace)
+
 
 def _fit_gpu(W, q, G, t_max=10, trace=False):
     Wd = to_dev(W.view(np.int16)).view(torch.float16)
@@ -83,3 +85,34 @@ def test_fit_then_pack_then_product():
     # and the fitted layer approximates the dense product far better than its energy
     Y_dense = X.astype(np.float64) @ W.astype(np.float64).T
     assert hlq.rel_fro_error(Y_ref, Y_dense) < 0.5
+
+
+# (q, G, N, K): the last warp of 32 groups ragged, fewer than 32 groups, a block of 128 weights cut in two by the end
+@pytest.mark.parametrize("q,G,N,K", [(1, 128, 37, 1024), (2, 128, 1, 384), (2, 64, 33, 320), (3, 32, 7, 160), (3, 128, 65, 512), (4, 64, 50, 1088),
+                                     (4, 32, 129, 96), (4, 128, 64, 2048)])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_fit_of_sorted_groups_matches_oracle_bit_for_bit(q, G, N, K, shift):
+    """Without a trace the groups' sorted form runs (from a number of groups on: tiled here to reach it); `shift` = an input that
+    starts two bytes after an aligned address.  Groups on a grid, with few values, with equal or very different magnitudes."""
+    rng = np.random.default_rng(41)
+    W = workloads.dense_weights(41, f"fit-sorted{q}{G}{N}", N, K)
+    flat = W.reshape(-1, G)
+    n = flat.shape[0]
+    flat[0] = np.float16(0.25)
+    flat[n // 2] = rng.choice(np.array([-3.0, 0.0, -0.0, 5.0], dtype=np.float16), G)
+    flat[n // 3] = (0.5 * rng.integers(-2 ** (q - 1), 2 ** (q - 1), G)).astype(np.float16)
+    flat[n - 1] = (flat[n - 1].astype(np.float64) * 1e4).astype(np.float16)
+    flat[n // 4] = (flat[n // 4].astype(np.float64) * 2.0 ** -13).astype(np.float16)      # subnormal values
+    copies = -(-SORTED_MIN_GROUPS // n)
+    Wall = np.concatenate([W] * copies)
+    buf = torch.zeros(Wall.size + 8, dtype=torch.int16, device="cuda")
+    Wd = buf[shift: shift + Wall.size].view(Wall.shape)
+    Wd.copy_(to_dev(Wall.view(np.int16)))
+    p, s, z = elutq.elutq_hlq_fit(Wd.view(torch.float16), q, G, 10)
+    p = p.cpu().numpy()
+    s, z = (t.cpu().view(torch.int16).numpy().view(np.float16) for t in (s, z))
+    p_ref, s_ref, z_ref = ofit.fit(W, q, G, 10)
+    for c in range(copies):
+        rows = slice(c * N, (c + 1) * N)
+        assert np.array_equal(p[:, rows], p_ref)
+        assert _same_bits(s[rows], s_ref) and _same_bits(z[rows], z_ref)
