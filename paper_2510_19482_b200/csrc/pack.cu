@@ -9,30 +9,31 @@ namespace elutq {
 
 namespace {
 
-__global__ void write_header_kernel(uint32_t* hdr, Geo g) {
-    const int i = threadIdx.x;
-    if (i >= ELUTQ_HEADER_BYTES / 4) return;
-    uint32_t v = 0;
+__device__ __forceinline__ uint32_t header_word(const Geo& g, int i) {
     switch (i) {
-        case 0: v = (uint32_t)kMagic; break;
-        case 1: v = (uint32_t)kVersion; break;
-        case 2: v = (uint32_t)g.q; break;
-        case 3: v = (uint32_t)g.G; break;
-        case 4: v = (uint32_t)g.N; break;
-        case 5: v = (uint32_t)g.K; break;
-        case 6: v = (uint32_t)g.n_rb; break;
-        case 7: v = (uint32_t)g.n_kc; break;
-        case 8: v = (uint32_t)g.tile_bytes; break;
-        default: break;
+        case 0: return (uint32_t)kMagic;
+        case 1: return (uint32_t)kVersion;
+        case 2: return (uint32_t)g.q;
+        case 3: return (uint32_t)g.G;
+        case 4: return (uint32_t)g.N;
+        case 5: return (uint32_t)g.K;
+        case 6: return (uint32_t)g.n_rb;
+        case 7: return (uint32_t)g.n_kc;
+        case 8: return (uint32_t)g.tile_bytes;
+        default: return 0u;
     }
-    hdr[i] = v;
 }
 
-// One thread per plane vector: (tile, vec = u*q + j, lane) -> 16 bytes, byte i = column tau(l,i).
-__global__ void pack_planes_kernel(const uint8_t* __restrict__ planes, uint8_t* __restrict__ tiles, Geo g) {
-    const long long nvec = (long long)g.n_kc * g.n_rb * 2 * g.q * 32;
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= nvec) return;
+// Bit b of the result: byte b of x is not zero.
+__device__ __forceinline__ uint32_t nonzero_bytes(uint32_t x) {
+    // the bytes' top bits from any bit below them, then the four together: copies shifted by 7, 14, 21, 28 do not overlap
+    const uint32_t m = ((((x & 0x7f7f7f7fu) + 0x7f7f7f7fu) | x) >> 7) & 0x01010101u;
+    return (m * 0x10204080u) >> 28;
+}
+
+// One thread per plane vector: (tile, vec = u*q + j, lane) -> 16 bytes, byte i = column tau(l,i).  The lanes' 128 input bytes each
+// are whole lines, so sixteen 8-byte loads in flight per thread read every byte from memory once.
+__device__ __forceinline__ void pack_plane_vector(const uint8_t* __restrict__ planes, uint8_t* __restrict__ tiles, const Geo& g, long long idx) {
     const int lane = (int)(idx & 31);
     const int vec = (int)((idx >> 5) % (2 * g.q));
     const long long tile = idx / (64LL * g.q);
@@ -44,28 +45,23 @@ __global__ void pack_planes_kernel(const uint8_t* __restrict__ planes, uint8_t* 
     uint32_t out[4] = {0u, 0u, 0u, 0u};
     if (n < g.N) {
         const uint8_t* row = planes + ((size_t)j * g.N + n) * g.K;
+        uint2 x[16];
+#pragma unroll
         for (int i = 0; i < 16; ++i) {
             const int k0 = kc * kChunkK + (16 * sigma + tau_of(l, i, g.w, g.nsg)) * 8;
-            uint32_t byte = 0;
-            if (k0 < g.K) {
-                const uint64_t x = *reinterpret_cast<const uint64_t*>(row + k0);
-#pragma unroll
-                for (int b = 0; b < 8; ++b) byte |= (((x >> (8 * b)) & 0xffull) != 0ull ? 1u : 0u) << b;
-            }
-            out[i >> 2] |= byte << (8 * (i & 3));
+            x[i] = k0 < g.K ? __ldg(reinterpret_cast<const uint2*>(row + k0)) : make_uint2(0u, 0u);
         }
+#pragma unroll
+        for (int i = 0; i < 16; ++i) out[i >> 2] |= (nonzero_bytes(x[i].x) | nonzero_bytes(x[i].y) << 4) << (8 * (i & 3));
     }
     uint4* dst = reinterpret_cast<uint4*>(tiles + (size_t)tile * g.tile_bytes) + vec * 32 + lane;
     *dst = make_uint4(out[0], out[1], out[2], out[3]);
 }
 
 // One thread per parameter word: (tile, word, lane) -> two fp16 values of the lane's record.
-__global__ void pack_params_kernel(const uint16_t* __restrict__ scales, const uint16_t* __restrict__ offsets,
-                                   uint8_t* __restrict__ tiles, Geo g) {
+__device__ __forceinline__ void pack_param_word(const uint16_t* __restrict__ scales, const uint16_t* __restrict__ offsets,
+                                                uint8_t* __restrict__ tiles, const Geo& g, long long idx) {
     const int words = g.gl * (g.q + 1) / 2;
-    const long long total = (long long)g.n_kc * g.n_rb * words * 32;
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= total) return;
     const int lane = (int)(idx & 31);
     const int word = (int)((idx >> 5) % words);
     const long long tile = idx / (32LL * words);
@@ -89,6 +85,21 @@ __global__ void pack_params_kernel(const uint16_t* __restrict__ scales, const ui
     }
     uint32_t* dst = reinterpret_cast<uint32_t*>(tiles + (size_t)tile * g.tile_bytes + g.plane_bytes) + word * 32 + lane;
     *dst = packed;
+}
+
+// The whole blob in one launch: plane vectors, parameter words (blocks from plane_blocks on), the header.
+__global__ void __launch_bounds__(256) pack_kernel(const uint8_t* __restrict__ planes, const uint16_t* __restrict__ scales,
+                                                   const uint16_t* __restrict__ offsets, uint8_t* __restrict__ packed, const Geo g,
+                                                   const unsigned plane_blocks) {
+    uint8_t* tiles = packed + ELUTQ_HEADER_BYTES;
+    if (blockIdx.x < plane_blocks) {
+        const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+        if (idx < (long long)g.n_kc * g.n_rb * 2 * g.q * 32) pack_plane_vector(planes, tiles, g, idx);
+    } else {
+        const long long idx = (long long)(blockIdx.x - plane_blocks) * blockDim.x + threadIdx.x;
+        if (idx < (long long)g.n_kc * g.n_rb * (g.gl * (g.q + 1) / 2) * 32) pack_param_word(scales, offsets, tiles, g, idx);
+        if (idx < ELUTQ_HEADER_BYTES / 4) reinterpret_cast<uint32_t*>(packed)[idx] = header_word(g, (int)idx);
+    }
 }
 
 // One thread per (plane j, row n, byte-column cg): expands a packed byte to 8 uint8 {0,1}.
@@ -149,14 +160,12 @@ inline unsigned blocks_for(long long total, int threads) { return (unsigned)((to
 
 int launch_pack(const uint8_t* planes, const __half* scales, const __half* offsets, const Geo& g,
                 uint8_t* packed, cudaStream_t stream) {
-    uint8_t* tiles = packed + ELUTQ_HEADER_BYTES;
-    write_header_kernel<<<1, 32, 0, stream>>>(reinterpret_cast<uint32_t*>(packed), g);
     const long long nvec = (long long)g.n_kc * g.n_rb * 2 * g.q * 32;
-    pack_planes_kernel<<<blocks_for(nvec, 256), 256, 0, stream>>>(planes, tiles, g);
     const long long nwords = (long long)g.n_kc * g.n_rb * (g.gl * (g.q + 1) / 2) * 32;
-    pack_params_kernel<<<blocks_for(nwords, 256), 256, 0, stream>>>(
-        reinterpret_cast<const uint16_t*>(scales), reinterpret_cast<const uint16_t*>(offsets), tiles, g);
-    count_launch(3);
+    const unsigned plane_blocks = blocks_for(nvec, 256);
+    pack_kernel<<<plane_blocks + blocks_for(nwords, 256), 256, 0, stream>>>(
+        planes, reinterpret_cast<const uint16_t*>(scales), reinterpret_cast<const uint16_t*>(offsets), packed, g, plane_blocks);
+    count_launch(1);
     return (int)cudaGetLastError();
 }
 
