@@ -78,6 +78,24 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_
     return false;
 }
 
+// True in one lane of the (converged) warp.  The condition around tcgen05 instructions has to be this alone: only then does the
+// compiler know that one lane issues them, and an MMA takes about 10 cycles to issue; behind `tid == 0` it takes 50 to 90
+// (8B gate_up, M = 2048, q = 2: 446 -> 431 us; 4096 x 4096 55.5 -> 52.7; M = 512 110.4 -> 105.1).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t e;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
+    return e != 0;
+}
+template <int CG>
+__device__ __forceinline__ void mma_f16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
+    if constexpr (CG == 2)
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+                     :: "r"(d), "l"(a), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
+    else
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+                     :: "r"(d), "l"(a), "l"(b), "r"(idesc), "r"(accumulate) : "memory");
+}
+
 // 32 consecutive outputs of one token row: Y (fp16 or fp32, optionally accumulating) or the fp32 partials.
 __device__ __forceinline__ void store_row32(const GemmArgs& a, int m, int n0, const uint32_t (&r)[32], int splits,
                                             int split, size_t n_pad, bool y_vec_ok) {
@@ -143,7 +161,7 @@ __global__ void __launch_bounds__(kMmaThreads + (WS ? 32 : 0), 1) hlq_mma_kernel
                                                                             //      or per weight tile (TT = 1)
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mbar + 8);            // WS: mbar[2], mbar[3] = "half is ready"; pair form: [0..3] done, [4..7] ready
 
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);     // (warp-uniform for the compiler too)
     const int l = lane & 15;
     // CTA pairs are neighbours in x, so the pair form puts the token tiles there
     const int n_tile = n_tile0 + (CG == 2 ? blockIdx.y : blockIdx.x), m_tile = (CG == 2 ? blockIdx.x : blockIdx.y), split = blockIdx.z;
@@ -381,23 +399,22 @@ __global__ void __launch_bounds__(kMmaThreads + (WS ? 32 : 0), 1) hlq_mma_kernel
     // MMAs of one half step (64 k = 4 slices per token tile), issued by one thread; completion arrives on barrier hb.
     // (Single-CTA schedules; the pair form issues its own in the ring loop below.)
     auto issue_mma = [&](int step, int stage, int hb) {
-        if (tid != (WS ? kMmaThreads : 0)) return;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        if (warp != (WS ? kMmaThreads / 32 : 0)) return;
+        if (elect_one()) {
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
-        for (int tt = 0; tt < TT; ++tt) {
+            for (int tt = 0; tt < TT; ++tt) {
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {
-                const uint64_t da = desc_swizzle128(x_addr + stage * X_STAGE_BYTES + tt * kXTileBytes + hb * (kTileM * 128) + kk * 32);
-                const uint64_t db = desc_noswizzle(w_addr + hb * W_HALF_BYTES + kk * 256);
-                const uint32_t accumulate = (step != step0 || hb != 0 || kk != 0) ? 1u : 0u;
-                asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                             "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, {%5, %5, %5, %5}, p;\n\t}"
-                             :: "r"(tmem_d + (uint32_t)(tt * NW)), "l"(da), "l"(db), "r"(idesc), "r"(accumulate), "r"(0u)
-                             : "memory");
+                for (int kk = 0; kk < 4; ++kk) {
+                    const uint64_t da = desc_swizzle128(x_addr + stage * X_STAGE_BYTES + tt * kXTileBytes + hb * (kTileM * 128)) + kk * 2;
+                    const uint64_t db = desc_noswizzle(w_addr + hb * W_HALF_BYTES) + kk * 16;
+                    mma_f16<1>(tmem_d + (uint32_t)(tt * NW), da, db, idesc, (step != step0 || hb != 0 || kk != 0) ? 1u : 0u);
+                }
             }
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
+                         :: "r"(bar_addr + 8u * hb) : "memory");
         }
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                     :: "r"(bar_addr + 8u * hb) : "memory");
+        __syncwarp();
     };
     auto publish = [&]() {     // generic-proxy writes of this thread -> visible to the tensor core, then CTA barrier
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -411,20 +428,19 @@ __global__ void __launch_bounds__(kMmaThreads + (WS ? 32 : 0), 1) hlq_mma_kernel
         // MMAs of step s - 2, long finished), publish, issue the MMAs of step s, go on with step s + 1.  Three
         // activation stages, so the copy for step s + 1 never waits for the MMAs of step s - 1 either.
         auto issue_step = [&](int step, int stage, int wt) {
-            if (tid != 0) return;
+            if (warp != 0) return;
             if (a.flags & kFlagTestNoMma) return;      // test only: nothing is issued, nothing completes, the waits run out
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            if (elect_one()) {
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint64_t da0 = desc_swizzle128(x_addr + stage * X_STAGE_BYTES), db0 = desc_noswizzle(w_addr + wt * W_BYTES);
 #pragma unroll
-            for (int kk = 0; kk < kStepK / 16; ++kk) {
-                const uint64_t da = desc_swizzle128(x_addr + stage * X_STAGE_BYTES + (kk >> 2) * (kTileM * 128) + (kk & 3) * 32);
-                const uint64_t db = desc_noswizzle(w_addr + wt * W_BYTES + (kk >> 2) * W_HALF_BYTES + (kk & 3) * 256);
-                const uint32_t accumulate = (step != step0 || kk != 0) ? 1u : 0u;
-                asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                             "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, {%5, %5, %5, %5}, p;\n\t}"
-                             :: "r"(tmem_d), "l"(da), "l"(db), "r"(idesc), "r"(accumulate), "r"(0u) : "memory");
+                for (int kk = 0; kk < kStepK / 16; ++kk)
+                    mma_f16<1>(tmem_d, da0 + (kk >> 2) * (kTileM * 128 / 16) + (kk & 3) * 2, db0 + (kk >> 2) * (W_HALF_BYTES / 16) + (kk & 3) * 16,
+                               idesc, (step != step0 || kk != 0) ? 1u : 0u);
+                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
+                             :: "r"(bar_addr + 8u * wt) : "memory");
             }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                         :: "r"(bar_addr + 8u * wt) : "memory");
+            __syncwarp();
         };
         if (step0 < step1) copy_x(step0, 0);
         asm volatile("cp.async.commit_group;" ::: "memory");
@@ -523,27 +539,24 @@ __global__ void __launch_bounds__(kMmaThreads + (WS ? 32 : 0), 1) hlq_mma_kernel
                 }
                 asm volatile("cp.async.wait_group 0;" ::: "memory");
                 if (n_half > 0) wait_mma((n_half - 1) & 3, (uint32_t)(((n_half - 1) >> 2) & 1));   // commits complete in order
-            } else if (cta_rank == 0 && lane == 0) {
-                for (int i = 0; i < n_half; ++i) {
-                    const int slot = i & 3;
-                    wait_ready(4 + slot, (uint32_t)((i >> 2) & 1));
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            } else if (cta_rank == 0) {
+                if (elect_one()) {
+                    for (int i = 0; i < n_half; ++i) {
+                        const int slot = i & 3;
+                        wait_ready(4 + slot, (uint32_t)((i >> 2) & 1));
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                        const uint64_t da0 = desc_swizzle128(x_addr + slot * XH_BYTES), db0 = desc_noswizzle(w_addr + slot * WH_BYTES);
 #pragma unroll
-                    for (int tt = 0; tt < TT; ++tt) {
+                        for (int tt = 0; tt < TT; ++tt)
 #pragma unroll
-                        for (int kk = 0; kk < 4; ++kk) {
-                            const uint64_t da = desc_swizzle128(x_addr + slot * XH_BYTES + tt * (kTileM * 128) + kk * 32);
-                            const uint64_t db = desc_noswizzle(w_addr + slot * WH_BYTES + kk * 256);
-                            const uint32_t accumulate = (i != 0 || kk != 0) ? 1u : 0u;
-                            asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                                         "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, {%5, %5, %5, %5, %5, %5, %5, %5}, p;\n\t}"
-                                         :: "r"(tmem_d + (uint32_t)(tt * NW)), "l"(da), "l"(db), "r"(idesc), "r"(accumulate), "r"(0u)
-                                         : "memory");
-                        }
+                            for (int kk = 0; kk < 4; ++kk)
+                                mma_f16<2>(tmem_d + (uint32_t)(tt * NW), da0 + tt * (kTileM * 128 / 16) + kk * 2, db0 + kk * 16, idesc,
+                                           (i != 0 || kk != 0) ? 1u : 0u);
+                        asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+                                     :: "r"(bar_addr + 8u * slot), "h"((unsigned short)3) : "memory");
                     }
-                    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-                                 :: "r"(bar_addr + 8u * slot), "h"((unsigned short)3) : "memory");
                 }
+                __syncwarp();
             }
         } else {
             uint32_t phase = 0;                                   // every barrier completes once per step
