@@ -100,10 +100,19 @@ def _ptr(t) -> int:
     return 0 if t is None else t.data_ptr()
 
 
+_CURRENT = None      # torch's current device, and its current stream's address
+
+
 def _stream(stream) -> int:
+    """Address of a stream; None = torch's current one (its raw handle: building a torch.cuda.Stream takes 3 us a call)."""
+    global _CURRENT
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        if _CURRENT is None:
+            import torch
+            raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+            _CURRENT = (torch.cuda.current_device, raw or (lambda device: torch.cuda.current_stream(device).cuda_stream))
+        device, raw = _CURRENT
+        return raw(device())
     return stream if isinstance(stream, int) else stream.cuda_stream
 
 
