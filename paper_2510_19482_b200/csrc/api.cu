@@ -61,8 +61,12 @@ int num_sms() {
 }
 
 // Workspace layout: a 256-byte control area (word 0 = device status), then the partial sums.
-// Batches: plus one ticket per 128 output rows (hlq_frag.cu).
-size_t counters_bytes(int M, int N) { return 256 + (M == 1 ? 0 : ((size_t)(N + 127) / 128 * sizeof(unsigned) + 255) / 256 * 256); }
+// From word 64 of the control area on: tickets.  Batches: one per 128 output rows (hlq_frag.cu); M = 1 with a K split: one per row range
+// of CTAs (lut_gemv.cu).
+size_t counters_bytes(int M, int N, int K) {
+    const size_t n = M > 1 ? ((size_t)N + 127) / 128 : K > kChunkK ? kGemvTickets : 0;
+    return 256 + (n * sizeof(unsigned) + 255) / 256 * 256;
+}
 size_t partials_bytes(int M, int N, int K) {
     const size_t n_rb = (size_t)(N + kTileRows - 1) / kTileRows;
     const size_t n_kc = (size_t)(K + kChunkK - 1) / kChunkK;
@@ -187,7 +191,7 @@ int run_gemm(const void* X, const void* packed, void* Y, int M, int N, int K, un
     // decode-kernel variants exist for M = 1 only
     if ((flags & (ELUTQ_FLAG_PLAIN_G4 | ELUTQ_FLAG_MIRROR | ELUTQ_FLAG_CLUSTER_REDUCE)) && M > 1) return ELUTQ_ERR_UNSUPPORTED;
 
-    const size_t cb = counters_bytes(M, N), pb = partials_bytes(M, N, K);
+    const size_t cb = counters_bytes(M, N, K), pb = partials_bytes(M, N, K);
     void* counters = workspace;
     void* partials = nullptr;
     if (own_workspace) {
@@ -213,6 +217,7 @@ int run_gemm(const void* X, const void* packed, void* Y, int M, int N, int K, un
     a.n_rb = g.n_rb; a.n_kc = g.n_kc;
     a.flags = flags | g_test_flags;
     a.wait_limit = g_test_wait_limit;
+    a.tickets = a.counters + 64;
     a.items_q = 0; a.items_r = 0; a.active_warps = 0; a.ranges = 0; a.rb_q = 0; a.rb_r = 0; a.cpc = 1; a.cluster_reduce = 0;
     const int sms = num_sms();
     int ce;
@@ -321,7 +326,7 @@ int elutq_forget(const void* packed) {
 
 int elutq_workspace_bytes(int M, int N, int K, size_t* bytes) {
     if (!bytes || M <= 0 || N <= 0 || K <= 0) return ELUTQ_ERR_INVALID_ARG;
-    *bytes = counters_bytes(M, N) + partials_bytes(M, N, K);
+    *bytes = counters_bytes(M, N, K) + partials_bytes(M, N, K);
     return ELUTQ_OK;
 }
 
@@ -444,7 +449,7 @@ int elutq_takes_tensor_path(int M, int N, int K, int G, unsigned flags) {
 int elutq_reserve(int M, int N, int K, void* stream) {
     if (M <= 0 || N <= 0 || K <= 0) return ELUTQ_ERR_INVALID_ARG;
     void* p = nullptr;
-    int st = get_scratch(stream, 0, counters_bytes(M, N), true, &p);
+    int st = get_scratch(stream, 0, counters_bytes(M, N, K), true, &p);
     if (st != ELUTQ_OK) return st;
     const size_t pb = partials_bytes(M, N, K);
     st = get_scratch(stream, 3, pb ? pb : 16, false, &p);

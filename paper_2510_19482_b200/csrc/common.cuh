@@ -11,6 +11,7 @@ namespace elutq {
 
 constexpr int kTileRows = 16;     // output rows per tile (one per lane of a half-warp)
 constexpr int kChunkK = 512;      // input columns per tile (64 byte-columns)
+constexpr int kGemvTickets = 256;        // row ranges of the M = 1 kernel that can have a ticket
 constexpr int kMagic = 0x51544C45;
 constexpr int kVersion = 1;
 
@@ -64,6 +65,7 @@ struct GemmArgs {
     int cpc;                 // chunks per CTA in the aligned partition
     int cluster_reduce;      // 1: launched as clusters of n_kc CTAs (one per chunk, same row range): partials stay in
                              //    shared memory and are reduced through distributed shared memory
+    unsigned* tickets;       // zero between calls: M = 1 one per row range, batches one per 128 rows (null: none to use)
     unsigned wait_limit;     // poll limit of the tensor-core kernel's bounded waits (0: the default)
 };
 

@@ -563,7 +563,7 @@ int launch_frag_cfg(const GemmArgs& g, int num_sms, cudaStream_t stream) {
     a.units = (int)units;
     a.per_cta = (a.units + num_sms - 1) / num_sms;
     const int grid = (a.units + a.per_cta - 1) / a.per_cta;
-    a.tickets = g.counters + 64;
+    a.tickets = g.tickets;
     static_assert((kMaxSmem - kFixed) / C::UNIT_BYTES >= 2, "shared memory");
     a.ws = (kMaxSmem - kFixed) / C::UNIT_BYTES;
     if (a.ws > 5) a.ws = 5;
