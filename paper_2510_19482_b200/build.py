@@ -8,7 +8,7 @@ import sys
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
-SOURCES = ["api.cu", "pack.cu", "lut_gemv.cu", "lut_gemm.cu", "hlq_mma.cu", "hlq_frag.cu", "hlq_fit.cu", "static_scratch.cu", "lut_chain.cu"]
+SOURCES = ["api.cu", "pack.cu", "lut_gemv.cu", "lut_gemm.cu", "hlq_mma.cu", "hlq_tmem.cu", "hlq_frag.cu", "hlq_fit.cu", "static_scratch.cu", "lut_chain.cu"]
 LIB = os.path.join(HERE, "libelutq.so")
 
 

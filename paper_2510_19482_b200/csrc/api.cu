@@ -64,7 +64,8 @@ int num_sms() {
 // From word 64 of the control area on: tickets.  Batches: one per 128 output rows (hlq_frag.cu); M = 1 with a K split: one per row range
 // of CTAs (lut_gemv.cu).
 size_t counters_bytes(int M, int N, int K) {
-    const size_t n = M > 1 ? ((size_t)N + 127) / 128 : K > kChunkK ? kGemvTickets : 0;
+    const size_t rows = ((size_t)N + 127) / 128;
+    const size_t n = M > ELUTQ_FRAGMENT_MAX_M ? (rows > kTmemTickets ? rows : kTmemTickets) : M > 1 ? rows : K > kChunkK ? kGemvTickets : 0;
     return 256 + (n * sizeof(unsigned) + 255) / 256 * 256;
 }
 size_t partials_bytes(int M, int N, int K) {
@@ -74,6 +75,22 @@ size_t partials_bytes(int M, int N, int K) {
     // M > 1: one per 256-column half chunk
     const size_t chunks = (M == 1) ? (n_kc > 1 ? n_kc : 0) : 2 * n_kc;
     return chunks * (size_t)M * n_rb * kTileRows * sizeof(float);
+}
+
+// Which kernel takes more than ELUTQ_FRAGMENT_MAX_M rows at G = 128: true = hlq_mma.cu (weights rebuilt in shared memory), false =
+// hlq_tmem.cu (in tensor memory).  In output tiles of 256 rows x 128 tokens, us of hlq_mma and hlq_tmem:
+//   few tiles          deep K splits: hlq_mma's smaller parts (1000 x 4096, q = 3, M = 64 9.7 and 13.6; 2048 x 4096, M = 128 16 and 20;
+//                      against 4096 x 4096, M = 64, 16.0 and 15.4)
+//   many tokens        its CTA pairs rebuild a weight once per 512 tokens and need no split where they fill the GPU (28672 x 4096,
+//                      q = 2: M = 512 108 and 117, M = 2048 422 and 473; against M = 384 106 and 95, M = 128 54 and 33, and where
+//                      they do not, 4096 x 4096, M = 1024, 66 and 32).  They take an even number of 256-token tiles; 2 * 256 tokens
+//                      cost them as much as 3.5 * 128 cost hlq_tmem.
+//   q = 4, 193 to 256  (28672 x 4096, M = 256, 79 and 87; q = 2 63 and 62)
+bool rebuilds_in_shared_memory(int M, int N, int K, int q, int sms) {
+    const long long rows = ((long long)N + 255) / 256, m128 = (M + 127) / 128, m256 = (M + 255) / 256, tiles = rows * m128;
+    if (tiles <= 8 || (tiles <= 16 && tiles * (K / 128) <= 256)) return true;
+    if (m256 % 2 == 0 && 4 * m128 >= 7 * m256 && rows * m256 * 20 >= 17LL * sms) return true;
+    return q == 4 && M > 192 && M <= 256;
 }
 
 int lookup_blob(const void* packed, int N, int K, BlobMeta* out, bool force_read = false) {
@@ -223,8 +240,10 @@ int run_gemm(const void* X, const void* packed, void* Y, int M, int N, int K, un
     int ce;
     if (M == 1) ce = launch_lut_gemv(a, m.q, m.G, sms, (cudaStream_t)stream);
     else if (!takes_tensor_path(M, m.G, flags)) ce = launch_lut_gemm(a, m.q, m.G, sms, (cudaStream_t)stream);
-    else if (m.G == 128 && M > ELUTQ_FRAGMENT_MAX_M) ce = launch_hlq_mma(a, m.q, m.G, sms, (cudaStream_t)stream);
-    else ce = launch_hlq_frag(a, m.q, m.G, sms, (cudaStream_t)stream);
+    else if (m.G == 128 && M > ELUTQ_FRAGMENT_MAX_M) {
+        ce = rebuilds_in_shared_memory(M, N, K, m.q, sms) ? (int)cudaErrorNotSupported : launch_hlq_tmem(a, m.q, sms, (cudaStream_t)stream);
+        if (ce == (int)cudaErrorNotSupported) ce = launch_hlq_mma(a, m.q, m.G, sms, (cudaStream_t)stream);
+    } else ce = launch_hlq_frag(a, m.q, m.G, sms, (cudaStream_t)stream);
     if (ce == (int)cudaErrorNotSupported) return ELUTQ_ERR_UNSUPPORTED;
     if (ce != 0) return cuda_fail((cudaError_t)ce);
     return ELUTQ_OK;

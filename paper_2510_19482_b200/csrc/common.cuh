@@ -12,6 +12,7 @@ namespace elutq {
 constexpr int kTileRows = 16;     // output rows per tile (one per lane of a half-warp)
 constexpr int kChunkK = 512;      // input columns per tile (64 byte-columns)
 constexpr int kGemvTickets = 256;        // row ranges of the M = 1 kernel that can have a ticket
+constexpr int kTmemTickets = 16 * 256;   // hlq_tmem.cu: 16 per CTA
 constexpr int kMagic = 0x51544C45;
 constexpr int kVersion = 1;
 
@@ -78,6 +79,7 @@ int launch_lut_gemv(const GemmArgs& a, int q, int G, int num_sms, cudaStream_t s
 int launch_lut_gemm(const GemmArgs& a, int q, int G, int num_sms, cudaStream_t stream);
 int launch_hlq_frag(const GemmArgs& a, int q, int G, int num_sms, cudaStream_t stream);
 int launch_hlq_mma(const GemmArgs& a, int q, int G, int num_sms, cudaStream_t stream);
+int launch_hlq_tmem(const GemmArgs& a, int q, int num_sms, cudaStream_t stream);
 
 // col0 / cols restrict the reduction to output columns [col0, col0 + cols) (cols = 0: all N columns).
 int launch_finalize(const GemmArgs& a, int n_chunks, bool pdl, cudaStream_t stream, int col0 = 0, int cols = 0);

@@ -1,4 +1,5 @@
-// Batches of more than ELUTQ_FRAGMENT_MAX_M rows at G = 128: dequantise-and-contract on the 5th-generation tensor cores.
+// Large batches (and any of more than ELUTQ_FRAGMENT_MAX_M rows where there are few weight rows) at G = 128: dequantise-and-contract
+// on the 5th-generation tensor cores, the rebuilt weights in shared memory.  (In tensor memory: hlq_tmem.cu.)
 //
 // For large M the look-up path is bound by the shared-memory look-up rate (it does M look-ups per
 // weight byte), while Y = X W_hat^T is then a genuine dense contraction.  This kernel rebuilds each
@@ -761,7 +762,7 @@ int launch_mma_q(const GemmArgs& a, int num_sms, cudaStream_t stream) {
     // number of 256-token tiles
     if (two && !narrow && m_tiles % 2 == 0) return launch_mma_cfg<Q, 256, 2, true, 2>(a, num_sms, stream);
     if (two && !narrow) return launch_mma_cfg<Q, 256, 2, true>(a, num_sms, stream);
-    if (two) return narrow ? launch_mma_cfg<Q, 128, 2>(a, num_sms, stream) : launch_mma_cfg<Q, 256, 2>(a, num_sms, stream);
+    if (two) return launch_mma_cfg<Q, 128, 2>(a, num_sms, stream);
     return narrow ? launch_mma_cfg<Q, 128, 1>(a, num_sms, stream) : launch_mma_cfg<Q, 256, 1>(a, num_sms, stream);
 }
 

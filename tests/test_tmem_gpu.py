@@ -1,0 +1,80 @@
+"""GPU parity of the kernel that rebuilds weights in tensor memory (batches of more than 16 rows at G = 128 with enough weight rows).
+
+Tolerance: W_hat = z + sum_j b_j s_j is formed with one fp16 fma per plane (exact products, each sum rounded at 2^-11 relative; weight 7
+of a byte starts from z^ = z + (1/2) sum_j s_j, rounded once, and adds +-s_j / 2), products are exact and the sums fp32.  The
+weights' rounding errors are independent across k: a relative error of about 2^-12 .. 2^-11 in norm, bar 1e-3; per element
+the worst-case bound of gpu_util.assert_elementwise.
+"""
+
+import numpy as np
+import pytest
+import torch
+
+import paper_2510_19482_b200 as elutq
+import workloads
+from oracle import hlq
+from workloads import synth
+
+pytestmark = pytest.mark.gpu
+
+from gpu_util import assert_elementwise, gemm_f32, pack_layer, x_dev  # noqa: E402
+
+G, TOL = 128, 1e-3
+
+# (q, N, K, M): one step of K, a K that ends inside a 512-k chunk, ragged rows and tokens, one and several token tiles (17 -> 32 tokens,
+# 200 -> 2 x 112); whole tiles per CTA, shared tiles of two or three parts, of many parts
+CASES = [(2, 4621, 128, 17), (1, 4480, 1152, 128), (3, 4600, 640, 200), (4, 5000, 2944, 100), (4, 12800, 2048, 384), (2, 38000, 256, 33),
+         (3, 10240, 1024, 130)]
+
+
+@pytest.mark.parametrize("q,N,K,M", CASES)
+def test_tensor_memory_kernel_matches_oracle(q, N, K, M):
+    layer = workloads.hlq_layer(70, f"tmem/{q}/{N}/{K}", q, G, N, K, signed_scales=(q == 3))
+    X = synth.activations(70, f"tmem/x/{M}/{K}", M, K, outliers=True)
+    packed = pack_layer(layer)
+    ref = hlq.matmul(X, layer.planes, layer.scales, layer.offsets, G)
+    y = gemm_f32(X, packed, N, K)
+    assert elutq.elutq_device_status() == 0
+    assert max(hlq.rel_fro_error(y[m], ref[m]) for m in range(M)) <= TOL
+    assert_elementwise(y, ref, hlq.magnitude_bound(X, layer.scales, layer.offsets, G), q, K, True, False, "fp32 out")
+    assert np.array_equal(y.view(np.uint32), gemm_f32(X, packed, N, K).view(np.uint32))       # and the tickets are zero again
+    ys = gemm_f32(X, packed, N, K, elutq.FLAG_SKIP_OFFSET)
+    yb = gemm_f32(X, packed, N, K, elutq.FLAG_OFFSET_ONLY)
+    assert hlq.rel_fro_error(ys, hlq.scale_term(X, layer.planes, layer.scales, G)) <= TOL
+    assert hlq.rel_fro_error(yb, hlq.offset_term(X, layer.offsets, G)) <= TOL
+    Y = torch.full((M, N), 1.5, dtype=torch.float32, device="cuda")
+    elutq.elutq_lut_gemm_f32(x_dev(X), packed, Y, M, N, K, elutq.FLAG_ACCUMULATE)
+    np.testing.assert_allclose(Y.cpu().numpy(), y + 1.5, rtol=0, atol=1e-5 * np.abs(y).max())
+
+
+@pytest.mark.parametrize("q", [1, 2, 4])
+def test_scales_of_one_and_more(q):
+    N, K, M = 4700, 256, 40
+    layer = workloads.hlq_layer(71, f"tmem/scales/{q}", q, G, N, K)
+    s = layer.scales.astype(np.float32)
+    s[1::4] *= 64.0                                      # around 1: only some groups of a row
+    s[2::4] *= 8192.0
+    s[3::4, :, 0] = 30000.0 + 2000.0 * np.arange(s[3::4].shape[0])[:, None] % 10000.0         # the largest exponent
+    layer.scales[...] = s.astype(np.float16)
+    X = synth.activations(71, "tmem/scales/x", M, K)
+    packed = pack_layer(layer)
+    ref = hlq.matmul(X, layer.planes, layer.scales, layer.offsets, G)
+    y = gemm_f32(X, packed, N, K)
+    assert elutq.elutq_device_status() == 0
+    for first in range(4):
+        assert hlq.rel_fro_error(y[:, first::4], ref[:, first::4]) <= TOL
+
+
+def test_a_wait_that_runs_out_is_reported():
+    q, N, K, M = 2, 8192, 2048, 64
+    layer = workloads.hlq_layer(72, "tmem/expiry", q, G, N, K)
+    X = synth.activations(72, "tmem/expiry/x", M, K)
+    packed = pack_layer(layer)
+    elutq.elutq_release_scratch()
+    Y = torch.zeros((M, N), dtype=torch.float32, device="cuda")
+    elutq.elutq_test_wait_expiry(x_dev(X), packed, Y, M, N, K, 4096)
+    assert elutq.elutq_device_status() == 0x7C05
+    elutq.elutq_release_scratch()
+    y = gemm_f32(X, packed, N, K)
+    assert elutq.elutq_device_status() == 0
+    assert hlq.rel_fro_error(y, hlq.matmul(X, layer.planes, layer.scales, layer.offsets, G)) <= TOL
