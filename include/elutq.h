@@ -69,9 +69,10 @@ typedef enum elutq_status {
                                      variant flag).  Two rows stay on the batched look-up kernel: one pass, 17.3 us
                                      on 8B gate_up 28672 x 4096 at q = 2 against 25.6; from three rows on it needs a
                                      wider pass (M = 4: 26.2 / 25.9, 4096 x 4096 9.5 / 7.6, M = 8: 43.9 / 26.8)        */
-#define ELUTQ_FRAGMENT_MAX_M 16   /* G = 128: up to this many rows the bit-planes are contracted as they are (scales
+#define ELUTQ_FRAGMENT_MAX_M 8    /* G = 128: up to this many rows the bit-planes are contracted as they are (scales
                                      applied to fp32 sums, as exact as the look-up kernels); larger batches rebuild
-                                     W_hat in fp16 tiles (8B gate_up at q = 2, us: M = 16 37 / 48, M = 32 82 / 48).
+                                     W_hat in fp16 tiles (8B gate_up / down at q = 2, us: M = 8 26.9 / 15.9 and
+                                     24.9 / 18.9, M = 12 36.6 / 21.2 and 25.0 / 19.3).
                                      At G = 64 every batch takes the former, 32 rows at a time
                                      (elutq_takes_tensor_path is 1 for both)                                        */
 
@@ -380,8 +381,8 @@ int elutq_hlq_fit(const void* W, int q, int G, int N, int K, int t_max, uint8_t*
 int elutq_device_status(void* stream, int* status);
 
 /*
- * Test entry for the bounded waits of the tensor-core kernels (9 <= M <= 128, G = 128, K >= 384): the call is
- * launched with the issuing thread told to issue no MMA and no completion signal (up to ELUTQ_FRAGMENT_MAX_M rows: no load) and with the poll limit of the
+ * Test entry for the bounded waits of the tensor-core kernels (9 <= M <= 128, K >= 384): the call is
+ * launched with the issuing thread told to issue no MMA and no completion signal (G = 64: no load) and with the poll limit of the
  * device-side waits set to `wait_limit`, so that the waits for MMA completion run out: the kernel gives up
  * waiting, still joins every barrier, frees its tensor memory and returns; elutq_device_status then reads
  * ELUTQ_DEVICE_WAIT_EXPIRED.  Y (float [M][N]) receives undefined values.  Nothing faults and nothing waits

@@ -586,8 +586,7 @@ int launch_frag_cfg(const GemmArgs& g, int num_sms, cudaStream_t stream) {
 template <int Q, int G>
 int launch_frag_qg(const GemmArgs& g, int num_sms, cudaStream_t stream) {
     if (g.M <= 8) return launch_frag_cfg<Q, G, 1>(g, num_sms, stream);
-    if (g.M <= 16) return launch_frag_cfg<Q, G, 2>(g, num_sms, stream);
-    if constexpr (G == 64) return launch_frag_cfg<Q, G, 4>(g, num_sms, stream);
+    if constexpr (G == 64) return g.M <= 16 ? launch_frag_cfg<Q, G, 2>(g, num_sms, stream) : launch_frag_cfg<Q, G, 4>(g, num_sms, stream);
     return (int)cudaErrorInvalidValue;
 }
 

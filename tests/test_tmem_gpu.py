@@ -1,4 +1,4 @@
-"""GPU parity of the kernel that rebuilds weights in tensor memory (batches of more than 16 rows at G = 128 with enough weight rows).
+"""GPU parity of the kernel that rebuilds weights in tensor memory (batches of more than 8 rows at G = 128 with enough weight rows).
 
 Tolerance: W_hat = z + sum_j b_j s_j is formed with one fp16 fma per plane (exact products, each sum rounded at 2^-11 relative; weight 7
 of a byte starts from z^ = z + (1/2) sum_j s_j, rounded once, and adds +-s_j / 2), products are exact and the sums fp32.  The
@@ -21,9 +21,9 @@ from gpu_util import assert_elementwise, gemm_f32, pack_layer, x_dev  # noqa: E4
 
 G, TOL = 128, 1e-3
 
-# (q, N, K, M): one step of K, a K that ends inside a 512-k chunk, ragged rows and tokens, one and several token tiles (17 -> 32 tokens,
+# (q, N, K, M): one step of K, a K that ends inside a 512-k chunk, ragged rows and tokens, one and several token tiles (9 -> 16 tokens,
 # 200 -> 2 x 112); whole tiles per CTA, shared tiles of two or three parts, of many parts
-CASES = [(2, 4621, 128, 17), (1, 4480, 1152, 128), (3, 4600, 640, 200), (4, 5000, 2944, 100), (4, 12800, 2048, 384), (2, 38000, 256, 33),
+CASES = [(2, 4621, 128, 9), (1, 4480, 1152, 128), (3, 4600, 640, 200), (4, 5000, 2944, 100), (4, 12800, 2048, 384), (2, 38000, 256, 33),
          (3, 10240, 1024, 130)]
 
 
