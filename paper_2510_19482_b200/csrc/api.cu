@@ -79,18 +79,18 @@ size_t partials_bytes(int M, int N, int K) {
 
 // Which kernel takes more than ELUTQ_FRAGMENT_MAX_M rows at G = 128: true = hlq_mma.cu (weights rebuilt in shared memory), false =
 // hlq_tmem.cu (in tensor memory).  In output tiles of 256 rows x 128 tokens, us of hlq_mma and hlq_tmem:
-//   few tiles          deep K splits: hlq_mma's smaller parts (1000 x 4096, q = 3, M = 64 9.7 and 13.6; 2048 x 4096, M = 128 16 and 20;
-//                      against 4096 x 4096, M = 64, 16.0 and 15.4)
+//   few row tiles      its deeper K splits (1000 x 8192, q = 3, M = 64 12.9 and 20.7; against 1000 x 4096, M = 64 9.5 and 8.3), and
+//                      little work for more than 96 tokens (2048 x 2048, M = 128 10.9 and 11.7; against 2048 x 4096 16.2 and 14.4)
 //   many tokens        its CTA pairs rebuild a weight once per 512 tokens and need no split where they fill the GPU (28672 x 4096,
 //                      q = 2: M = 512 108 and 117, M = 2048 422 and 473; against M = 384 106 and 95, M = 128 54 and 33, and where
 //                      they do not, 4096 x 4096, M = 1024, 66 and 32).  They take an even number of 256-token tiles; 2 * 256 tokens
 //                      cost them as much as 3.5 * 128 cost hlq_tmem.
-//   q = 4, 193 to 256  (28672 x 4096, M = 256, 79 and 87; q = 2 63 and 62)
+//   q = 4, 193 to 256  with too many tiles for clusters (28672 x 4096, M = 256, 82 and 87; q = 2 63 and 62; 6144 x 4096, q = 4, 47 and 28)
 bool rebuilds_in_shared_memory(int M, int N, int K, int q, int sms) {
-    const long long rows = ((long long)N + 255) / 256, m128 = (M + 127) / 128, m256 = (M + 255) / 256, tiles = rows * m128;
-    if (tiles <= 8 || (tiles <= 16 && tiles * (K / 128) <= 256)) return true;
+    const long long rows = ((long long)N + 255) / 256, m128 = (M + 127) / 128, m256 = (M + 255) / 256;
+    if (rows <= 8 && m128 == 1 && (K / 128 >= 16 * rows || (M > 96 && rows * (K / 128) <= 128))) return true;
     if (m256 % 2 == 0 && 4 * m128 >= 7 * m256 && rows * m256 * 20 >= 17LL * sms) return true;
-    return q == 4 && M > 192 && M <= 256;
+    return q == 4 && M > 192 && M <= 256 && 4 * rows > 3LL * sms;
 }
 
 int lookup_blob(const void* packed, int N, int K, BlobMeta* out, bool force_read = false) {

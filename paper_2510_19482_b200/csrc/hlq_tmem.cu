@@ -8,8 +8,9 @@
 //   step       256 weight rows (two row blocks, UMMA M = 128 each) x 128 k x one token tile of up to 128 rows.  The two
 //              blocks share the activation tile, which is what the L2 has to feed again and again.  The steps of a call,
 //              tile by tile, are dealt to the CTAs (one per SM) in equal contiguous runs, so no SM idles for a wave.  The
-//              parts of a tile that several CTAs share go to the workspace and a second kernel adds them in ascending k order
-//              (bit-reproducible).
+//              parts of a tile that several CTAs share go to the workspace and are added in ascending k order (bit-reproducible)
+//              by the CTA that comes last or, where there are many, by a second kernel.  Or the CTAs of a cluster share the K of a
+//              tile and add up through their shared memory (a rule on costs: plan_of).
 //   warps      0 and 3 weight loaders (one bulk copy per row block and 512 k: eight packed tiles, contiguous in the blob), 1 MMA
 //              issuer, 2 activation loader (TMA, 128-byte swizzle), 4-19 producers: two warpgroups per row block, which take
 //              the steps in turn, rebuild the weights, and at the end of a tile write out half of its tokens each.  (Four warps
@@ -23,7 +24,7 @@
 //   bound      the producers' integer logic pipe (q = 4: 320 of a slot's 470 operations are the dequantisation itself, 65 to 75 % of
 //              the pipe's cycles); from 96 tokens also the activations' way from the L2.  Against weights rebuilt in shared memory with one
 //              barrier per step, us: 57344 x 8192, q = 4, M = 64 277 -> 127; 28672 x 4096, q = 2, M = 32 / 128 / 384
-//              49 / 51 / 110 -> 25 / 33 / 95; 4096 x 14336, q = 3, M = 64 37 -> 29.
+//              49 / 51 / 110 -> 25 / 33 / 95; 4096 x 14336, q = 3, M = 64 34 -> 24; 4096 x 4096, q = 2, M = 256 30 -> 18.
 //
 // Every wait is bounded; a thread whose wait runs out raises the status word and a CTA-wide flag that ends the other
 // roles' waits; copies and MMAs in flight are waited for (bounded), tensor memory is freed, the kernel returns.
@@ -43,6 +44,7 @@ constexpr int kSlotCols = 64;                   // TMEM columns of a slot: 128 k
 constexpr int kTmemCols = 512;
 constexpr int kMaxTokens = 128;                 // tokens per tile (UMMA N)
 constexpr uint32_t kTmWaitLimit = 1u << 20, kPollNs = 60;
+constexpr int kMaxSplit = 8;                    // CTAs of a cluster
 constexpr int kMaxX = 8, kMaxW = 4, kMaxSlots = 3;
 
 struct TmemArgs {
@@ -50,6 +52,7 @@ struct TmemArgs {
     int mp, m_tiles;            // tokens per tile (a multiple of 16), token tiles
     int n_steps;                // 128-k steps of the whole K: steps of a tile
     int steps, per_cta;         // all steps; steps of one CTA
+    int split;                  // CTAs of a cluster, which share a tile's K (1: no cluster)
     int reduce;                 // the CTAs add the parts of shared tiles themselves
     int xs, ws, ss;             // ring lengths: activation steps, weight chunks and slots (of a row block)
 };
@@ -149,6 +152,12 @@ __device__ __forceinline__ uint32_t opaque(uint32_t v) {
     return v;
 }
 
+__device__ __forceinline__ void st_cluster_u32(uint32_t addr, uint32_t rank, uint32_t v) {
+    uint32_t remote;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr), "r"(rank));
+    asm volatile("st.shared::cluster.u32 [%0], %1;" :: "r"(remote), "r"(v) : "memory");
+}
+
 // How many warps before this one took the ticket: read, or (take) announced behind the warp's own writes.
 __device__ __forceinline__ unsigned ticket_seen(unsigned* ticket, int lane, bool take) {
     unsigned t = 0;
@@ -162,7 +171,8 @@ __device__ __forceinline__ unsigned ticket_seen(unsigned* ticket, int lane, bool
 
 __device__ __forceinline__ __half2 as_half2(uint32_t v) { return *reinterpret_cast<const __half2*>(&v); }
 
-template <int Q>
+// CLUSTER: a tile's K is shared by the CTAs of a cluster.
+template <int Q, bool CLUSTER>
 __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_constant__ CUtensorMap xmap, const TmemArgs a) {
     using C = TmCfg<Q>;
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -203,12 +213,17 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
     const uint32_t slot_col0 = (uint32_t)(kTmemCols - kBlocks * a.ss * kSlotCols);   // accumulators below, slots above
 
     const int b = blockIdx.x;
-    const int t0 = b * a.per_cta;
-    int t1 = min(a.steps, t0 + a.per_cta);
+    int t0 = b * a.per_cta, t1 = min(a.steps, t0 + a.per_cta);
+    if constexpr (CLUSTER) {
+        const int tile = b / a.split, r = b - tile * a.split;
+        t0 = tile * a.n_steps + a.n_steps * r / a.split;
+        t1 = tile * a.n_steps + a.n_steps * (r + 1) / a.split;
+    }
     if (!blob_header_ok(h0, h1, Q, 128, a.g.N, a.g.K)) {      // before any tile is read; the same answer in every thread: no work
         t1 = t0;
         if (tid == 0 && a.g.counters != nullptr) atomicExch(a.g.counters, kStatusBlobMismatch);
     }
+    [[maybe_unused]] bool have_part = false;                 // CLUSTER: this warp's sums are in tensor memory
     const uint32_t limit = a.g.wait_limit ? a.g.wait_limit : kTmWaitLimit;
 
     // Bounded wait; false once this CTA has given up.  (Sleeping between polls: the waiting warps' instructions cost the
@@ -476,7 +491,7 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
                 // This warp's 32 rows and every other 16 tokens to Y, or to the workspace.  (A last part that its CTA adds up
                 // itself: below.)
                 const bool to_end = r.end == a.n_steps, whole = to_end && r.tile * a.n_steps >= t0;
-                if (a.reduce && !to_end) {
+                if (CLUSTER || (a.reduce && !to_end)) {
                     tail = r.tile;
                     break;
                 }
@@ -503,46 +518,101 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
                 if (lane == 0) mbar_arrive(bar(kBarDEmpty + blk));
             }
         }
-        // Shared tiles: the warp that finds all other parts in the workspace adds them to its own in ascending k order (no warp
-        // waits for another; a tile's other parts are mostly those that their CTAs began with, long written).
-        if (live && tail >= 0) {
-            const int mine = b - tail * a.n_steps / a.per_cta, m0 = (tail % a.m_tiles) * a.mp, m_count = min(a.mp, M - m0), n = row_of(tail);
-            if (ticket_seen(ticket_of(tail), lane, false) != (unsigned)(parts_of(tail) - 1)) {
-                float* part = a.g.partials + ((size_t)mine * M + m0) * n_pad + n;
+        if constexpr (CLUSTER) have_part = live && tail >= 0;
+        else {
+            // Shared tiles: the warp that finds all other parts in the workspace adds them to its own in ascending k order (no
+            // warp waits for another; a tile's other parts are mostly those that their CTAs began with, long written).
+            if (live && tail >= 0) {
+                const int mine = b - tail * a.n_steps / a.per_cta, m0 = (tail % a.m_tiles) * a.mp, m_count = min(a.mp, M - m0), n = row_of(tail);
+                if (ticket_seen(ticket_of(tail), lane, false) != (unsigned)(parts_of(tail) - 1)) {
+                    float* part = a.g.partials + ((size_t)mine * M + m0) * n_pad + n;
+                    for (int c0 = 16 * turn; c0 < m_count; c0 += 16 * kTurns) {
+                        uint32_t v[16];
+                        tmem_ld16(v, acc + (uint32_t)c0);
+                        tmem_ld_wait(v);
+#pragma unroll
+                        for (int i = 0; i < 16; ++i)
+                            if (c0 + i < m_count && (size_t)n < n_pad) part[(size_t)(c0 + i) * n_pad] = __uint_as_float(v[i]);
+                    }
+                    if (!announce(tail)) tail = -1;
+                }
+            }
+            for (int e = 0; e < 2 && live; ++e) {
+                const int tile = e ? head : tail;
+                if (tile < 0) continue;
+                const int parts = parts_of(tile), mine = e ? -1 : b - tile * a.n_steps / a.per_cta;
+                const int m0 = (tile % a.m_tiles) * a.mp, m_count = min(a.mp, M - m0), n = row_of(tile);
                 for (int c0 = 16 * turn; c0 < m_count; c0 += 16 * kTurns) {
                     uint32_t v[16];
+                    float y[16];
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) y[i] = 0.f;
                     tmem_ld16(v, acc + (uint32_t)c0);
                     tmem_ld_wait(v);
+                    for (int q = 0; q < parts; ++q) {
+                        const float* part = a.g.partials + ((size_t)q * M + m0 + c0) * n_pad + n;
 #pragma unroll
-                    for (int i = 0; i < 16; ++i)
-                        if (c0 + i < m_count && (size_t)n < n_pad) part[(size_t)(c0 + i) * n_pad] = __uint_as_float(v[i]);
+                        for (int i = 0; i < 16; ++i)
+                            y[i] += q == mine ? __uint_as_float(v[i]) : c0 + i < m_count && n < N ? __ldcg(part + (size_t)i * n_pad) : 0.f;
+                    }
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) v[i] = __float_as_uint(y[i]);
+                    if (n < N) put16(m0 + c0, n, m_count - c0, v);
                 }
-                if (!announce(tail)) tail = -1;
+                if (lane == 0) *ticket_of(tile) = 0;               // zero again for the next call
             }
         }
-        for (int e = 0; e < 2 && live; ++e) {
-            const int tile = e ? head : tail;
-            if (tile < 0) continue;
-            const int parts = parts_of(tile), mine = e ? -1 : b - tile * a.n_steps / a.per_cta;
-            const int m0 = (tile % a.m_tiles) * a.mp, m_count = min(a.mp, M - m0), n = row_of(tile);
-            for (int c0 = 16 * turn; c0 < m_count; c0 += 16 * kTurns) {
+    }
+    if constexpr (CLUSTER) {
+        // Each CTA of the cluster adds up its share of the tile's tokens, in ascending k order: the others' parts come into its shared
+        // memory as [rank][token][256 rows].  (Written there, not read from there: 4096 x 4096, q = 2, M = 64 13.0 -> 11.3 us.)
+        const int tile = b / a.split, rank = b - tile * a.split, share = (a.mp + a.split - 1) / a.split;
+        __syncwarp();
+        cluster_barrier();                                     // every CTA has read its weights and activations
+        if (warp >= kCtrlWarps && have_part) {
+            const int blk = ((warp - kCtrlWarps) >> 2) & 1, turn = (warp - kCtrlWarps) >> 3, quad = warp & 3;
+            const uint32_t mine = smem_addr(smem) + (uint32_t)((rank * share * kTileRowsN + blk * kBlockRows + quad * 32 + lane) * 4);
+            for (int c0 = 16 * turn; c0 < a.mp; c0 += 16 * kTurns) {
                 uint32_t v[16];
-                float y[16];
-#pragma unroll
-                for (int i = 0; i < 16; ++i) y[i] = 0.f;
-                tmem_ld16(v, acc + (uint32_t)c0);
+                tmem_ld16(v, tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(blk * a.mp + c0));
                 tmem_ld_wait(v);
-                for (int q = 0; q < parts; ++q) {
-                    const float* part = a.g.partials + ((size_t)q * M + m0 + c0) * n_pad + n;
+                int owner = c0 / share, token = c0 - owner * share;
 #pragma unroll
-                    for (int i = 0; i < 16; ++i)
-                        y[i] += q == mine ? __uint_as_float(v[i]) : c0 + i < m_count && n < N ? __ldcg(part + (size_t)i * n_pad) : 0.f;
+                for (int i = 0; i < 16; ++i) {
+                    if (owner == rank) reinterpret_cast<uint32_t*>(smem)[(mine - smem_addr(smem)) / 4 + token * kTileRowsN] = v[i];
+                    else st_cluster_u32(mine + (uint32_t)(token * kTileRowsN * 4), (uint32_t)owner, v[i]);
+                    if (++token == share) { token = 0; ++owner; }
                 }
-#pragma unroll
-                for (int i = 0; i < 16; ++i) v[i] = __float_as_uint(y[i]);
-                if (n < N) put16(m0 + c0, n, m_count - c0, v);
             }
-            if (lane == 0) *ticket_of(tile) = 0;               // zero again for the next call
+        }
+        __syncwarp();
+        cluster_barrier();                                     // the parts are there
+        const int m0 = (tile % a.m_tiles) * a.mp + rank * share, count = min(min(share, a.mp - rank * share), a.g.M - m0);
+        const int row = (tid & 63) * 4, n = (tile / a.m_tiles) * kTileRowsN + row;
+        if (warp >= kCtrlWarps && t1 > t0 && n < a.g.N) {
+            grid_dependency_wait();
+            const bool plain = !(a.g.flags & (ELUTQ_FLAG_OUT_F32 | ELUTQ_FLAG_ACCUMULATE)) && a.g.N % 4 == 0;
+            for (int m = (tid - 32 * kCtrlWarps) / 64; m < count; m += 4 * kBlocks * kTurns * 32 / 64) {
+                float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int q = 0; q < a.split; ++q) {
+                    const float4 v = *reinterpret_cast<const float4*>(smem + ((q * share + m) * kTileRowsN + row) * 4);
+                    y.x += v.x;
+                    y.y += v.y;
+                    y.z += v.z;
+                    y.w += v.w;
+                }
+                const size_t at = (size_t)(m0 + m) * a.g.N + n;
+                if (plain) {
+                    const __half2 lo = __floats2half2_rn(y.x, y.y), hi = __floats2half2_rn(y.z, y.w);
+                    *reinterpret_cast<uint2*>(reinterpret_cast<__half*>(a.g.Y) + at) =
+                        make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+                } else {
+                    const float t[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        if (n + i < a.g.N) store_out(a.g, at + i, t[i]);
+                }
+            }
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -599,17 +669,31 @@ EncodeFn encode_fn() {
     return fn;
 }
 
-// Steps per CTA: equal shares of all steps, which leaves tiles to be added up from parts, or whole tiles, which leaves SMs idle.  In us:
-// a step takes c when the other SMs do not fight for the L2, 10 % more when all do, the parts 5 and their fp32 bytes at 2.2 TB/s.
+// How the steps of a call are dealt to the SMs: equal shares of all steps, which leaves tiles to be added up from parts; whole tiles,
+// which leaves SMs idle; or each tile's K over a cluster of CTAs, which add up through their shared memory.  In us: a step takes
+// c when the other SMs do not fight for the L2, 10 % more when all do, the parts 5 (a second kernel 8) and their fp32 bytes at 2.2 TB/s, a cluster's
+// sums 1 and 0.035 a token.
 // (Measured, equal shares against whole tiles: 28672 x 4096, q = 2, 112 tiles, M = 32: 27 and 25, M = 128: 45 and 32; 57344 x 8192, q = 4,
-// 224 tiles, M = 64: 127 and 157; 4096 x 14336, q = 3, M = 768, 96 tiles: 99 and 117, M = 1024, 128 tiles: 127 and 120.)
-int runs_of(int q, int mp, int steps, int n_steps, int num_sms) {
+// 224 tiles, M = 64: 127 and 157; 4096 x 14336, q = 3, M = 768, 96 tiles: 99 and 117, M = 1024, 128 tiles: 127 and 120.  Equal
+// shares against clusters: 4096 x 4096, q = 2, M = 16 / 64 / 384 11.0 / 14.4 / 31 and 9.3 / 11.3 / 21; 6144 x 4096, q = 4, M = 128 28.5 and
+// 19.8; 4096 x 14336, q = 3, M = 64 28.2 and 24.3.)
+struct Plan { int per_cta, split; };
+Plan plan_of(int q, int mp, int steps, int n_steps, int num_sms, const int (&max_clusters)[kMaxSplit + 1]) {
     const double c = 0.25 + 0.2 * q + 0.0016 * mp;
     const int tiles = steps / n_steps, whole = (tiles + num_sms - 1) / num_sms * n_steps;
     int share = (steps + num_sms - 1) / num_sms;
     if (share < 2) share = 2;                                 // the partial buffer holds 2 * n_kc slices
     const double ctas = (double)steps / share;
-    return 1.1 * c * share + 5.0 + ctas * kTileRowsN * mp * 4.0 / 2.2e6 < c * whole ? share : whole;
+    Plan best = {whole, 1};
+    double cost = c * whole;
+    const double shared = 1.1 * c * share + (2 * share >= n_steps ? 5.0 : 8.0) + ctas * kTileRowsN * mp * 4.0 / 2.2e6;
+    if (shared < cost) { best = {share, 1}; cost = shared; }
+    for (int s = 2; s <= kMaxSplit && s <= n_steps; ++s) {
+        if (max_clusters[s] < tiles) continue;
+        const double t = 1.1 * c * ((n_steps + s - 1) / s) + 1.0 + 0.035 * mp;
+        if (t < cost) { best = {n_steps, s}; cost = t; }
+    }
+    return best;
 }
 
 template <int Q>
@@ -617,11 +701,30 @@ int launch_tmem_q(const GemmArgs& g, int num_sms, cudaStream_t stream) {
     using C = TmCfg<Q>;
     constexpr int kMaxSmem = 232448, kFixed = kNumBars * 8 + 64;
     static bool configured[64] = {};
+    static int max_clusters[64][kMaxSplit + 1] = {};          // of each size, resident together
     int dev = 0;
     cudaGetDevice(&dev);
-    if (dev >= 0 && dev < 64 && !configured[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(hlq_tmem_kernel<Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+    if (dev < 0 || dev >= 64) return (int)cudaErrorNotSupported;
+    if (!configured[dev]) {
+        cudaError_t e = cudaFuncSetAttribute(hlq_tmem_kernel<Q, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(hlq_tmem_kernel<Q, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
         if (e != cudaSuccess) return (int)e;
+        for (int n = 2; n <= kMaxSplit; ++n) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3((unsigned)(n * num_sms));
+            cfg.blockDim = dim3(kTmThreads);
+            cfg.dynamicSmemBytes = kMaxSmem;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = (unsigned)n;
+            attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            if (cudaOccupancyMaxActiveClusters(&max_clusters[dev][n], hlq_tmem_kernel<Q, true>, &cfg) != cudaSuccess) {
+                max_clusters[dev][n] = 0;
+                (void)cudaGetLastError();
+            }
+        }
         configured[dev] = true;
     }
     TmemArgs a;
@@ -632,8 +735,10 @@ int launch_tmem_q(const GemmArgs& g, int num_sms, cudaStream_t stream) {
     const long long steps = (long long)((g.N + kTileRowsN - 1) / kTileRowsN) * a.m_tiles * a.n_steps;
     if (steps >= (1LL << 30)) return (int)cudaErrorNotSupported;
     a.steps = (int)steps;
-    a.per_cta = runs_of(Q, a.mp, a.steps, a.n_steps, num_sms);
-    const int grid = (a.steps + a.per_cta - 1) / a.per_cta;
+    const Plan plan = plan_of(Q, a.mp, a.steps, a.n_steps, num_sms, max_clusters[dev]);
+    a.per_cta = plan.per_cta;
+    a.split = plan.split;
+    const int grid = (a.steps + a.per_cta - 1) / a.per_cta * a.split;
     a.reduce = a.per_cta % a.n_steps != 0 && 2 * a.per_cta >= a.n_steps && grid <= kTmemTickets / (4 * kBlocks * kTurns);      // up to three parts
     a.ss = (kTmemCols - kBlocks * a.mp) / (kBlocks * kSlotCols);
     if (a.ss > kMaxSlots) a.ss = kMaxSlots;
@@ -661,17 +766,21 @@ int launch_tmem_q(const GemmArgs& g, int num_sms, cudaStream_t stream) {
     cfg.blockDim = dim3(kTmThreads);
     cfg.dynamicSmemBytes = a.xs * x_bytes + a.ws * w_bytes + kFixed;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)a.split;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, hlq_tmem_kernel<Q>, map, a);
+    cfg.numAttrs = a.split > 1 ? 2 : 1;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, a.split > 1 ? hlq_tmem_kernel<Q, true> : hlq_tmem_kernel<Q, false>, map, a);
     count_launch(1);
     if (e != cudaSuccess || a.reduce || a.per_cta % a.n_steps == 0 || grid == 1) return (int)e;
     cfg.gridDim = dim3((unsigned)(grid - 1), (unsigned)((a.mp + 7) / 8));
     cfg.blockDim = dim3(256);
     cfg.dynamicSmemBytes = 0;
+    cfg.numAttrs = 1;
     e = cudaLaunchKernelEx(&cfg, hlq_tmem_finalize_kernel, a);
     count_launch(1);
     return (int)e;
