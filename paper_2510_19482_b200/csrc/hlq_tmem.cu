@@ -51,6 +51,7 @@ struct TmemArgs {
     GemmArgs g;
     int mp, m_tiles;            // tokens per tile (a multiple of 16), token tiles
     int n_steps;                // 128-k steps of the whole K: steps of a tile
+    int tile0;                  // first tile of this launch (0 but for clusters)
     int steps, per_cta;         // all steps; steps of one CTA
     int split;                  // CTAs of a cluster, which share a tile's K (1: no cluster)
     int reduce;                 // the CTAs add the parts of shared tiles themselves
@@ -212,7 +213,7 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
     const uint32_t tmem = *tmem_slot;
     const uint32_t slot_col0 = (uint32_t)(kTmemCols - kBlocks * a.ss * kSlotCols);   // accumulators below, slots above
 
-    const int b = blockIdx.x;
+    const int b = blockIdx.x, base_tile = CLUSTER ? a.tile0 : 0;
     int t0 = b * a.per_cta, t1 = min(a.steps, t0 + a.per_cta);
     if constexpr (CLUSTER) {
         const int tile = b / a.split, r = b - tile * a.split;
@@ -257,7 +258,7 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
             for (Walk r(t0, t1, a.n_steps); r.more(); r.next()) {
                 ok = wait(kBarWEmpty + blk * kMaxW + w.i, w.phase ^ 1u);
                 if (!ok) break;
-                const int rb0 = (r.tile / a.m_tiles) * (kBlocks * 8) + blk * 8, nrb = max(0, min(8, a.g.n_rb - rb0));
+                const int rb0 = ((r.tile + base_tile) / a.m_tiles) * (kBlocks * 8) + blk * 8, nrb = max(0, min(8, a.g.n_rb - rb0));
                 const uint32_t bytes = (uint32_t)(nrb * C::TILE_BYTES), mb = bar(kBarWFull + blk * kMaxW + w.i);
                 mbar_expect(mb, bytes);
                 if (nrb > 0)
@@ -277,7 +278,7 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
             int issued = 0;
             bool ok = true;
             for (Walk r(t0, t1, a.n_steps); r.more() && ok; r.next()) {
-                const int m0 = (r.tile % a.m_tiles) * a.mp;
+                const int m0 = ((r.tile + base_tile) % a.m_tiles) * a.mp;
                 for (int step = r.step; step < r.end; ++step) {
                     ok = wait(kBarXEmpty + x.i, x.phase ^ 1u);
                     if (!ok) break;
@@ -348,7 +349,7 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
         const size_t n_pad = (size_t)a.g.n_rb * kTileRows;
         const int M = a.g.M, N = a.g.N;
         const uint32_t acc = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(blk * a.mp);
-        auto row_of = [&](int tile) { return (tile / a.m_tiles) * kTileRowsN + blk * kBlockRows + quad * 32 + lane; };
+        auto row_of = [&](int tile) { return ((tile + base_tile) / a.m_tiles) * kTileRowsN + blk * kBlockRows + quad * 32 + lane; };
         auto put16 = [&](int m, int n, int count, const uint32_t (&v)[16]) {
             if (!(a.g.flags & (ELUTQ_FLAG_OUT_F32 | ELUTQ_FLAG_ACCUMULATE))) {
                 __half* y = reinterpret_cast<__half*>(a.g.Y) + (size_t)m * N + n;
@@ -495,7 +496,7 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
                     tail = r.tile;
                     break;
                 }
-                const int m0 = (r.tile % a.m_tiles) * a.mp, m_count = min(a.mp, M - m0), n = row_of(r.tile);
+                const int m0 = ((r.tile + base_tile) % a.m_tiles) * a.mp, m_count = min(a.mp, M - m0), n = row_of(r.tile);
                 float* part = a.g.partials + ((size_t)(b - r.tile * a.n_steps / a.per_cta) * M + m0) * n_pad + n;
                 for (int c0 = 16 * turn; c0 < m_count; c0 += 16 * kTurns) {
                     uint32_t v[16];
@@ -523,7 +524,7 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
             // Shared tiles: the warp that finds all other parts in the workspace adds them to its own in ascending k order (no
             // warp waits for another; a tile's other parts are mostly those that their CTAs began with, long written).
             if (live && tail >= 0) {
-                const int mine = b - tail * a.n_steps / a.per_cta, m0 = (tail % a.m_tiles) * a.mp, m_count = min(a.mp, M - m0), n = row_of(tail);
+                const int mine = b - tail * a.n_steps / a.per_cta, m0 = ((tail + base_tile) % a.m_tiles) * a.mp, m_count = min(a.mp, M - m0), n = row_of(tail);
                 if (ticket_seen(ticket_of(tail), lane, false) != (unsigned)(parts_of(tail) - 1)) {
                     float* part = a.g.partials + ((size_t)mine * M + m0) * n_pad + n;
                     for (int c0 = 16 * turn; c0 < m_count; c0 += 16 * kTurns) {
@@ -541,7 +542,7 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
                 const int tile = e ? head : tail;
                 if (tile < 0) continue;
                 const int parts = parts_of(tile), mine = e ? -1 : b - tile * a.n_steps / a.per_cta;
-                const int m0 = (tile % a.m_tiles) * a.mp, m_count = min(a.mp, M - m0), n = row_of(tile);
+                const int m0 = ((tile + base_tile) % a.m_tiles) * a.mp, m_count = min(a.mp, M - m0), n = row_of(tile);
                 for (int c0 = 16 * turn; c0 < m_count; c0 += 16 * kTurns) {
                     uint32_t v[16];
                     float y[16];
@@ -587,8 +588,8 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
         }
         __syncwarp();
         cluster_barrier();                                     // the parts are there
-        const int m0 = (tile % a.m_tiles) * a.mp + rank * share, count = min(min(share, a.mp - rank * share), a.g.M - m0);
-        const int row = (tid & 63) * 4, n = (tile / a.m_tiles) * kTileRowsN + row;
+        const int m0 = ((tile + base_tile) % a.m_tiles) * a.mp + rank * share, count = min(min(share, a.mp - rank * share), a.g.M - m0);
+        const int row = (tid & 63) * 4, n = ((tile + base_tile) / a.m_tiles) * kTileRowsN + row;
         if (warp >= kCtrlWarps && t1 > t0 && n < a.g.N) {
             grid_dependency_wait();
             const bool plain = !(a.g.flags & (ELUTQ_FLAG_OUT_F32 | ELUTQ_FLAG_ACCUMULATE)) && a.g.N % 4 == 0;
@@ -677,21 +678,21 @@ EncodeFn encode_fn() {
 // 224 tiles, M = 64: 127 and 157; 4096 x 14336, q = 3, M = 768, 96 tiles: 99 and 117, M = 1024, 128 tiles: 127 and 120.  Equal
 // shares against clusters: 4096 x 4096, q = 2, M = 16 / 64 / 384 11.0 / 14.4 / 31 and 9.3 / 11.3 / 21; 6144 x 4096, q = 4, M = 128 28.5 and
 // 19.8; 4096 x 14336, q = 3, M = 64 28.2 and 24.3.)
-struct Plan { int per_cta, split; };
-Plan plan_of(int q, int mp, int steps, int n_steps, int num_sms, const int (&max_clusters)[kMaxSplit + 1]) {
-    const double c = 0.25 + 0.2 * q + 0.0016 * mp;
-    const int tiles = steps / n_steps, whole = (tiles + num_sms - 1) / num_sms * n_steps;
+double step_us(int q, int mp) { return 0.25 + 0.2 * q + 0.0016 * mp; }
+struct Plan { int per_cta, split; double cost; };
+Plan plan_of(int q, int mp, int tiles, int n_steps, int num_sms, const int (&max_clusters)[kMaxSplit + 1]) {
+    const double c = step_us(q, mp);
+    const int steps = tiles * n_steps, whole = (tiles + num_sms - 1) / num_sms * n_steps;
     int share = (steps + num_sms - 1) / num_sms;
     if (share < 2) share = 2;                                 // the partial buffer holds 2 * n_kc slices
     const double ctas = (double)steps / share;
-    Plan best = {whole, 1};
-    double cost = c * whole;
+    Plan best = {whole, 1, c * whole};
     const double shared = 1.1 * c * share + (2 * share >= n_steps ? 5.0 : 8.0) + ctas * kTileRowsN * mp * 4.0 / 2.2e6;
-    if (shared < cost) { best = {share, 1}; cost = shared; }
+    if (shared < best.cost) best = {share, 1, shared};
     for (int s = 2; s <= kMaxSplit && s <= n_steps; ++s) {
         if (max_clusters[s] < tiles) continue;
         const double t = 1.1 * c * ((n_steps + s - 1) / s) + 1.0 + 0.035 * mp;
-        if (t < cost) { best = {n_steps, s}; cost = t; }
+        if (t < best.cost) best = {n_steps, s, t};
     }
     return best;
 }
@@ -732,14 +733,9 @@ int launch_tmem_q(const GemmArgs& g, int num_sms, cudaStream_t stream) {
     a.m_tiles = (g.M + kMaxTokens - 1) / kMaxTokens;
     a.mp = ((g.M + a.m_tiles - 1) / a.m_tiles + 15) / 16 * 16;
     a.n_steps = g.K / 128;
-    const long long steps = (long long)((g.N + kTileRowsN - 1) / kTileRowsN) * a.m_tiles * a.n_steps;
-    if (steps >= (1LL << 30)) return (int)cudaErrorNotSupported;
-    a.steps = (int)steps;
-    const Plan plan = plan_of(Q, a.mp, a.steps, a.n_steps, num_sms, max_clusters[dev]);
-    a.per_cta = plan.per_cta;
-    a.split = plan.split;
-    const int grid = (a.steps + a.per_cta - 1) / a.per_cta * a.split;
-    a.reduce = a.per_cta % a.n_steps != 0 && 2 * a.per_cta >= a.n_steps && grid <= kTmemTickets / (4 * kBlocks * kTurns);      // up to three parts
+    const long long all = (long long)((g.N + kTileRowsN - 1) / kTileRowsN) * a.m_tiles;
+    if (all * a.n_steps >= (1LL << 30)) return (int)cudaErrorNotSupported;
+    const int tiles = (int)all;
     a.ss = (kTmemCols - kBlocks * a.mp) / (kBlocks * kSlotCols);
     if (a.ss > kMaxSlots) a.ss = kMaxSlots;
     const int x_bytes = a.mp * 256, w_bytes = kBlocks * C::UNIT_BYTES;
@@ -761,29 +757,49 @@ int launch_tmem_q(const GemmArgs& g, int num_sms, cudaStream_t stream) {
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return (int)cudaErrorInvalidValue;
 
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(kTmThreads);
-    cfg.dynamicSmemBytes = a.xs * x_bytes + a.ws * w_bytes + kFixed;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = (unsigned)a.split;
-    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = a.split > 1 ? 2 : 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, a.split > 1 ? hlq_tmem_kernel<Q, true> : hlq_tmem_kernel<Q, false>, map, a);
-    count_launch(1);
-    if (e != cudaSuccess || a.reduce || a.per_cta % a.n_steps == 0 || grid == 1) return (int)e;
-    cfg.gridDim = dim3((unsigned)(grid - 1), (unsigned)((a.mp + 7) / 8));
-    cfg.blockDim = dim3(256);
-    cfg.dynamicSmemBytes = 0;
-    cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, hlq_tmem_finalize_kernel, a);
-    count_launch(1);
-    return (int)e;
+    auto launch = [&](int tile0, int n_tiles, const Plan& plan) -> int {
+        a.tile0 = tile0;
+        a.steps = n_tiles * a.n_steps;
+        a.per_cta = plan.per_cta;
+        a.split = plan.split;
+        const int grid = (a.steps + a.per_cta - 1) / a.per_cta * a.split;
+        a.reduce = a.per_cta % a.n_steps != 0 && 2 * a.per_cta >= a.n_steps && grid <= kTmemTickets / (4 * kBlocks * kTurns);      // up to three parts
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)grid);
+        cfg.blockDim = dim3(kTmThreads);
+        cfg.dynamicSmemBytes = a.xs * x_bytes + a.ws * w_bytes + kFixed;
+        cfg.stream = stream;
+        cudaLaunchAttribute attr[2];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        attr[1].id = cudaLaunchAttributeClusterDimension;
+        attr[1].val.clusterDim.x = (unsigned)a.split;
+        attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = a.split > 1 ? 2 : 1;
+        cudaError_t e = cudaLaunchKernelEx(&cfg, a.split > 1 ? hlq_tmem_kernel<Q, true> : hlq_tmem_kernel<Q, false>, map, a);
+        count_launch(1);
+        if (e != cudaSuccess || a.reduce || a.per_cta % a.n_steps == 0 || grid == 1) return (int)e;
+        cfg.gridDim = dim3((unsigned)(grid - 1), (unsigned)((a.mp + 7) / 8));
+        cfg.blockDim = dim3(256);
+        cfg.dynamicSmemBytes = 0;
+        cfg.numAttrs = 1;
+        e = cudaLaunchKernelEx(&cfg, hlq_tmem_finalize_kernel, a);
+        count_launch(1);
+        return (int)e;
+    };
+    // Whole rounds of whole tiles and a second launch for the rest of them, where that leaves less idle (28672 x 4096, q = 2, M = 384,
+    // 336 tiles = two rounds and 40 tiles by clusters of three: 93 -> 85 us; M = 320 83 -> 78).
+    const Plan plan = plan_of(Q, a.mp, tiles, a.n_steps, num_sms, max_clusters[dev]);
+    const int full = tiles / num_sms * num_sms;
+    if (full > 0 && full < tiles) {
+        const Plan rounds = {full / num_sms * a.n_steps, 1, 0.0}, rest = plan_of(Q, a.mp, tiles - full, a.n_steps, num_sms, max_clusters[dev]);
+        if (rest.split > 1 && step_us(Q, a.mp) * rounds.per_cta + 6.0 + rest.cost < plan.cost) {
+            const int ce = launch(0, full, rounds);
+            return ce != 0 ? ce : launch(full, tiles - full, rest);
+        }
+    }
+    return launch(0, tiles, plan);
 }
 
 }  // namespace

@@ -23,9 +23,9 @@ G, TOL = 128, 1e-3
 
 # (q, N, K, M): one step of K, a K that ends inside a 512-k chunk, ragged rows and tokens, one and several token tiles (9 -> 16 tokens,
 # 200 -> 2 x 112); whole tiles per CTA, shared tiles of two or three parts, of many parts, clusters of two CTAs and more (with K steps and
-# tokens that they do not divide evenly, and N no multiple of the stores' four)
+# tokens that they do not divide evenly, and N no multiple of the stores' four), whole rounds with the rest by clusters
 CASES = [(2, 4621, 128, 9), (1, 4480, 1152, 128), (3, 4600, 640, 200), (4, 5000, 2944, 100), (4, 12800, 2048, 384), (2, 38000, 256, 33),
-         (3, 10240, 1024, 130), (2, 11776, 7680, 16), (2, 16000, 1024, 100), (2, 3001, 4096, 20), (3, 1100, 1152, 90), (1, 300, 256, 33)]
+         (3, 10240, 1024, 130), (2, 11776, 7680, 16), (2, 16000, 1024, 100), (2, 3001, 4096, 20), (3, 1100, 1152, 90), (1, 300, 256, 33), (2, 13000, 2048, 384)]
 
 
 @pytest.mark.parametrize("q,N,K,M", CASES)
