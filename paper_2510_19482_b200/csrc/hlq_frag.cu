@@ -125,7 +125,6 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
     uint64_t* bars = reinterpret_cast<uint64_t*>(sSum + 4 * MP * kSumStride);
     volatile uint32_t* give_up = reinterpret_cast<uint32_t*>(bars + kNumBars);
     volatile uint32_t* ticket_box = give_up + 1;
-    volatile uint32_t* stop = give_up + 2;                    // a compute warp gave up (read behind their barrier)
     const uint32_t bar0 = smem_addr(bars);
     auto bar = [&](int i) { return bar0 + 8u * (uint32_t)i; };
 
@@ -143,7 +142,6 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         *give_up = 0;
-        *stop = 0;
     }
     __syncthreads();
 
@@ -335,6 +333,12 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
         else store_out(a.g, (size_t)m * N + n, y);
     };
     auto compute_sync = []() { asm volatile("bar.sync 1, 512;" ::: "memory"); };
+    auto compute_any = [](bool mine) {                        // the same barrier; one answer for all compute threads
+        int any;
+        asm volatile("{\n\t.reg .pred p, r;\n\tsetp.ne.s32 p, %1, 0;\n\tbar.red.or.pred r, 1, 512, p;\n\tselp.s32 %0, 1, 0, r;\n\t}"
+                     : "=r"(any) : "r"((int)mine) : "memory");
+        return any != 0;
+    };
     // The CTA that came last to a shared row tile adds the parts in ascending k order (all compute threads call this).
     auto finish_tile = [&](int tile) {
         if (tile < 0 || *ticket_box == 0u) return;
@@ -490,12 +494,12 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
             x.next();
         }
 
-        // The four steps' sums meet in shared memory and are added and written out row by row.  (A warp that gave up still joins
-        // the barriers, and all leave together.)
-        if (!live) *stop = 1;
-        compute_sync();                                       // the buffer has been read; the ticket of the run before is there
+        // The four steps' sums meet in shared memory and are added and written out row by row.  (Where a warp gave up all leave
+        // together: the barrier itself tells them, as a flag could be raised for the next run before every warp has read it for this one.)
+        const bool stop = compute_any(!live);                 // the buffer has been read; the ticket of the run before is there
         finish_tile(pending);
         pending = -1;
+        if (stop) break;
         {
             float* p = sSum + (step * MP + 2 * c) * kSumStride + 32 * rp + gq;
 #pragma unroll
@@ -506,7 +510,6 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
                     for (int i = 0; i < 4; ++i) p[(8 * nb + (i & 1)) * kSumStride + 16 * t + 8 * (i >> 1)] = acc[t][nb][i];
         }
         compute_sync();
-        if (*stop) break;
         const int row = tid & (kUnitRows - 1), n = tile * kUnitRows + row;
         const bool whole = n_units == C_;
         const int first = tile * C_ / a.per_cta;
@@ -536,7 +539,7 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
         }
     }
     compute_sync();
-    if (!*stop) finish_tile(pending);
+    finish_tile(pending);
     __syncthreads();                                          // nobody leaves while copies are in flight
 }
 

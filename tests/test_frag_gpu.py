@@ -59,3 +59,20 @@ def test_fragment_kernel_reports_a_wait_that_runs_out():
     y = gemm_f32(X, packed, N, K)
     assert elutq.elutq_device_status() == 0
     assert hlq.rel_fro_error(y, hlq.matmul(X, layer.planes, layer.scales, layer.offsets, G)) <= 5e-6
+
+
+def test_warps_that_give_up_leave_together():
+    # K in one chunk and four row tiles per CTA: no barrier but the compute warps' own lies between two runs of units
+    q, G, N, K, M = 2, 64, 128 * 148 * 4 - 5, 448, 9
+    layer = workloads.hlq_layer(63, "frag/expiry/runs", q, G, N, K)
+    X = synth.activations(63, "frag/expiry/runs/x", M, K)
+    packed = pack_layer(layer)
+    Y = torch.zeros((M, N), dtype=torch.float32, device="cuda")
+    for limit in (64, 1000, 4096):
+        elutq.elutq_release_scratch()
+        elutq.elutq_test_wait_expiry(x_dev(X), packed, Y, M, N, K, limit)
+        assert elutq.elutq_device_status() == 0x7C05
+    elutq.elutq_release_scratch()
+    y = gemm_f32(X, packed, N, K)
+    assert elutq.elutq_device_status() == 0
+    assert hlq.rel_fro_error(y, hlq.matmul(X, layer.planes, layer.scales, layer.offsets, G)) <= 5e-6
