@@ -241,7 +241,8 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
         return false;
     };
     auto wait_warp = [&](int i, uint32_t parity) { return __all_sync(0xffffffffu, wait(i, parity)) != 0; };
-    // the copies in flight of a loader that gave up land before the CTA may leave
+    // A loader's copies land before its CTA may leave (or a peer write into its shared memory), whoever gave up: a loader that has
+    // issued everything does not notice that the others did.
     auto drain = [&](int bar_full, int len, int issued) {
         for (int n = max(0, issued - len); n < issued; ++n)
             for (uint32_t t = 0; t < kTmWaitLimit && !mbar_try(bar(bar_full + n % len), (uint32_t)(n / len) & 1u); ++t) {}
@@ -268,7 +269,7 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
                 ++issued;
                 w.next();
             }
-            if (!ok) drain(kBarWFull + blk * kMaxW, a.ws, issued);
+            drain(kBarWFull + blk * kMaxW, a.ws, issued);
         }
     } else if (warp == 2) {
         // ---- activation loader: a step is two boxes of 64 k ------------------------------------------------------------------
@@ -291,7 +292,7 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
                     x.next();
                 }
             }
-            if (!ok) drain(kBarXFull, a.xs, issued);
+            drain(kBarXFull, a.xs, issued);
         }
     } else if (warp == 1) {
         // ---- MMA issuer: one elected lane ------------------------------------------------------------------------------------

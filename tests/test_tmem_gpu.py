@@ -79,3 +79,25 @@ def test_a_wait_that_runs_out_is_reported():
     y = gemm_f32(X, packed, N, K)
     assert elutq.elutq_device_status() == 0
     assert hlq.rel_fro_error(y, hlq.matmul(X, layer.planes, layer.scales, layer.offsets, G)) <= TOL
+
+
+@pytest.mark.parametrize("q,N,K,M", [(2, 512, 2048, 64), (1, 4096, 512, 9), (4, 40000, 384, 128)])
+def test_waits_that_run_out_behind_loaders_that_are_done(q, N, K, M):
+    # Clusters and whole tiles with so few steps of K that the loaders have requested everything when the other warps give up: they
+    # still wait for their copies.  The calls that follow at once get the shared memory.
+    layer = workloads.hlq_layer(73, f"tmem/drain/{N}", q, G, N, K)
+    X = synth.activations(73, f"tmem/drain/x/{M}/{K}", M, K)
+    packed = pack_layer(layer)
+    Y = torch.zeros((M, N), dtype=torch.float32, device="cuda")
+    ref = hlq.matmul(X, layer.planes, layer.scales, layer.offsets, G)
+    ws = torch.empty(elutq.elutq_workspace_bytes(M, N, K), dtype=torch.uint8, device="cuda")
+    elutq.elutq_workspace_init(ws)
+    y = torch.empty((M, N), dtype=torch.float32, device="cuda")
+    x = x_dev(X)
+    elutq.elutq_release_scratch()
+    elutq.elutq_test_wait_expiry(x, packed, Y, M, N, K, 64)
+    elutq.elutq_lut_gemm_ws(x, packed, y, M, N, K, elutq.FLAG_OUT_F32, ws)
+    assert elutq.elutq_device_status() == 0x7C05
+    assert int(ws.view(torch.int32)[0]) == 0
+    assert hlq.rel_fro_error(y.cpu().numpy(), ref) <= TOL
+    elutq.elutq_release_scratch()
