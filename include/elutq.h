@@ -376,9 +376,7 @@ int elutq_hlq_fit(const void* W, int q, int G, int N, int K, int t_max, uint8_t*
 /*
  * Device-side status of the library-owned scratch of `stream` (synchronises the stream).
  * *status is 0 unless a kernel gave up on a bounded wait (then a non-zero code that stays set
- * until elutq_release_scratch, or elutq_workspace_init of a caller-owned workspace).  Kernels never spin without a limit.
- * While it is ELUTQ_DEVICE_WAIT_EXPIRED, a call whose K is split over CTAs may leave parts of Y as they are: the
- * tickets by which the CTAs find out who adds up may be half counted.
+ * until elutq_release_scratch).  Kernels never spin without a limit.
  */
 int elutq_device_status(void* stream, int* status);
 

@@ -176,19 +176,10 @@ __device__ __forceinline__ float ld_cluster_f32(const float* local_smem_ptr, uns
 }
 // Device status codes (word 0 of the control area; read back by elutq_device_status / elutq_chain_status).
 constexpr unsigned kStatusWaitExpired = 0x7C05u;    // a bounded wait ran out
-constexpr unsigned kStatusBlobMismatch = 0x7C0Bu;   // the blob header does not describe what the kernel was launched for
-// A mismatch is found before any ticket is taken, an expiry leaves tickets half counted: it is not to be overwritten.
-__device__ __forceinline__ void raise_blob_mismatch(unsigned* status) {
-    if (status != nullptr) atomicCAS(status, 0u, kStatusBlobMismatch);
-}
-// Whether a wait has run out on this control area: its tickets may be half counted from then on, and whoever they name as the
-// last must not write (until the area is zeroed).  Behind the grid dependency wait.
-__device__ __forceinline__ bool tickets_void(const unsigned* status) {
-    return __ldcg(status) == kStatusWaitExpired;
-}
+constexpr unsigned kStatusBlobMismatch = 0x7C0Bu;
 // Internal flag (never accepted from callers; set by elutq_test_wait_expiry only): the tensor-core kernel's issuing
 // thread issues no MMA and no commit, so that the other threads' bounded waits for MMA completion run out.
-constexpr unsigned kFlagTestNoMma = 0x20000000u;
+constexpr unsigned kFlagTestNoMma = 0x20000000u;   // the blob header does not describe what the kernel was launched for
 
 // Every GEMM kernel compares the header of the blob it was handed with the geometry it was launched for before it
 // reads any tile: a stale description of an address that now holds another blob must never turn into reads
@@ -208,7 +199,7 @@ __device__ __forceinline__ bool blob_header_matches(const uint8_t* tiles, int q,
     uint2 h1;
     blob_header_load(tiles, h0, h1);
     const bool ok = blob_header_ok(h0, h1, q, G, N, K);
-    if (!ok && threadIdx.x == 0) raise_blob_mismatch(status);
+    if (!ok && status != nullptr && threadIdx.x == 0) atomicExch(status, kStatusBlobMismatch);
     return ok;
 }
 

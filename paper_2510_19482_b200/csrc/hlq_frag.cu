@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
     int u1 = min(a.units, u0 + a.per_cta);
     if (!blob_header_ok(h0, h1, Q, G, a.g.N, a.g.K)) {         // before any tile is read; the same answer in every thread: no work
         u1 = u0;
-        if (tid == 0) raise_blob_mismatch(a.g.counters);
+        if (tid == 0 && a.g.counters != nullptr) atomicExch(a.g.counters, kStatusBlobMismatch);
     }
     const uint32_t limit = a.g.wait_limit ? a.g.wait_limit : kFragWaitLimit;
     // Bounded wait; false once this CTA has given up.
@@ -533,7 +533,7 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
                 const bool last = t == (unsigned)(parts - 1);
                 if (last) a.tickets[tile] = 0;                // zero again for the next call
                 __threadfence();
-                *ticket_box = last && !tickets_void(a.g.counters) ? 1u : 0u;
+                *ticket_box = last ? 1u : 0u;
             }
             pending = tile;
         }

@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
     }
     if (!blob_header_ok(h0, h1, Q, 128, a.g.N, a.g.K)) {      // before any tile is read; the same answer in every thread: no work
         t1 = t0;
-        if (tid == 0) raise_blob_mismatch(a.g.counters);
+        if (tid == 0 && a.g.counters != nullptr) atomicExch(a.g.counters, kStatusBlobMismatch);
     }
     [[maybe_unused]] bool have_part = false;                 // CLUSTER: this warp's sums are in tensor memory
     const uint32_t limit = a.g.wait_limit ? a.g.wait_limit : kTmWaitLimit;
@@ -542,7 +542,6 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
             for (int e = 0; e < 2 && live; ++e) {
                 const int tile = e ? head : tail;
                 if (tile < 0) continue;
-                const bool is_void = tickets_void(a.g.counters);
                 const int parts = parts_of(tile), mine = e ? -1 : b - tile * a.n_steps / a.per_cta;
                 const int m0 = ((tile + base_tile) % a.m_tiles) * a.mp, m_count = min(a.mp, M - m0), n = row_of(tile);
                 for (int c0 = 16 * turn; c0 < m_count; c0 += 16 * kTurns) {
@@ -560,7 +559,7 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
                     }
 #pragma unroll
                     for (int i = 0; i < 16; ++i) v[i] = __float_as_uint(y[i]);
-                    if (n < N && !is_void) put16(m0 + c0, n, m_count - c0, v);
+                    if (n < N) put16(m0 + c0, n, m_count - c0, v);
                 }
                 if (lane == 0) *ticket_of(tile) = 0;               // zero again for the next call
             }

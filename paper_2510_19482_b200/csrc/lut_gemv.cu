@@ -186,10 +186,9 @@ __global__ void __launch_bounds__(kThreads, 1) lut_gemv_kernel(const GemmArgs a)
         uint32_t* last_box = reinterpret_cast<uint32_t*>(smem + kTableBytes + 64);
         __syncthreads();
         if (tid == 0) {
-            const bool is_void = tickets_void(a.counters);
             unsigned t;
             asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(t) : "l"(a.tickets + range) : "memory");
-            *last_box = t == (unsigned)(a.n_kc - 1) && !is_void;
+            *last_box = t == (unsigned)(a.n_kc - 1);
         }
         __syncthreads();
         if (*last_box) {
