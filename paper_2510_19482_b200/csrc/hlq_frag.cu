@@ -496,10 +496,9 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
 
         // The four steps' sums meet in shared memory and are added and written out row by row.  (Where a warp gave up all leave
         // together: the barrier itself tells them, as a flag could be raised for the next run before every warp has read it for this one.)
-        const bool stop = compute_any(!live);                 // the buffer has been read; the ticket of the run before is there
+        compute_sync();                                       // the buffer has been read; the ticket of the run before is there
         finish_tile(pending);
         pending = -1;
-        if (stop) break;
         {
             float* p = sSum + (step * MP + 2 * c) * kSumStride + 32 * rp + gq;
 #pragma unroll
@@ -509,7 +508,7 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
 #pragma unroll
                     for (int i = 0; i < 4; ++i) p[(8 * nb + (i & 1)) * kSumStride + 16 * t + 8 * (i >> 1)] = acc[t][nb][i];
         }
-        compute_sync();
+        if (compute_any(!live)) break;
         const int row = tid & (kUnitRows - 1), n = tile * kUnitRows + row;
         const bool whole = n_units == C_;
         const int first = tile * C_ / a.per_cta;
