@@ -167,6 +167,7 @@ __device__ __forceinline__ unsigned ticket_seen(unsigned* ticket, int lane, bool
         if (take) asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(t) : "l"(ticket) : "memory");
         else asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(t) : "l"(ticket) : "memory");
     }
+    __syncwarp();                                              // lane 0 has acquired for the whole warp (a shuffle orders no memory)
     return __shfl_sync(0xffffffffu, t, 0);
 }
 
@@ -561,6 +562,7 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
                     for (int i = 0; i < 16; ++i) v[i] = __float_as_uint(y[i]);
                     if (n < N) put16(m0 + c0, n, m_count - c0, v);
                 }
+                __syncwarp();
                 if (lane == 0) *ticket_of(tile) = 0;               // zero again for the next call
             }
         }
