@@ -376,7 +376,8 @@ int elutq_hlq_fit(const void* W, int q, int G, int N, int K, int t_max, uint8_t*
 /*
  * Device-side status of the library-owned scratch of `stream` (synchronises the stream).
  * *status is 0 unless a kernel gave up on a bounded wait (then a non-zero code that stays set
- * until elutq_release_scratch).  Kernels never spin without a limit.
+ * until elutq_release_scratch).  Kernels never spin without a limit.  While it is set, the finalize kernels
+ * of calls with a K split write no Y.
  */
 int elutq_device_status(void* stream, int* status);
 
@@ -386,7 +387,8 @@ int elutq_device_status(void* stream, int* status);
  * device-side waits set to `wait_limit`, so that the waits for MMA completion run out: the kernel gives up
  * waiting, still joins every barrier, frees its tensor memory and returns; elutq_device_status then reads
  * ELUTQ_DEVICE_WAIT_EXPIRED.  Y (float [M][N]) receives undefined values.  Nothing faults and nothing waits
- * without a limit.  Call elutq_release_scratch afterwards to clear the status.
+ * without a limit.  Call elutq_release_scratch afterwards to clear the status.  With the top bit of wait_limit set only
+ * every other CTA is told so (G = 64 and the kernel that rebuilds weights in tensor memory).
  */
 int elutq_test_wait_expiry(const void* X, const void* packed, float* Y, int M, int N, int K,
                            unsigned wait_limit, void* stream);

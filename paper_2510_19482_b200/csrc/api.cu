@@ -408,10 +408,10 @@ int elutq_lut_gemm_host(const void* X_host, const void* packed, void* Y_host, in
 }
 
 int elutq_test_wait_expiry(const void* X, const void* packed, float* Y, int M, int N, int K, unsigned wait_limit, void* stream) {
-    if (M < 9 || M > 128 || wait_limit == 0) return ELUTQ_ERR_UNSUPPORTED;   // the one-token-tile schedule only
+    if (M < 9 || M > 128 || (wait_limit & 0x7fffffffu) == 0) return ELUTQ_ERR_UNSUPPORTED;   // the one-token-tile schedule only
     if (K < 3 * 128) return ELUTQ_ERR_UNSUPPORTED;                                           // a wait needs a third K step
-    g_test_flags = kFlagTestNoMma;
-    g_test_wait_limit = wait_limit;
+    g_test_flags = kFlagTestNoMma | (wait_limit >> 31 ? kFlagTestHalf : 0u);
+    g_test_wait_limit = wait_limit & 0x7fffffffu;
     const int st = run_gemm(X, packed, Y, M, N, K, ELUTQ_FLAG_OUT_F32, nullptr, 0, true, stream);
     g_test_flags = 0;
     g_test_wait_limit = 0;

@@ -176,10 +176,17 @@ __device__ __forceinline__ float ld_cluster_f32(const float* local_smem_ptr, uns
 }
 // Device status codes (word 0 of the control area; read back by elutq_device_status / elutq_chain_status).
 constexpr unsigned kStatusWaitExpired = 0x7C05u;    // a bounded wait ran out
-constexpr unsigned kStatusBlobMismatch = 0x7C0Bu;
+constexpr unsigned kStatusBlobMismatch = 0x7C0Bu;   // the blob header does not describe what the kernel was launched for
 // Internal flag (never accepted from callers; set by elutq_test_wait_expiry only): the tensor-core kernel's issuing
 // thread issues no MMA and no commit, so that the other threads' bounded waits for MMA completion run out.
-constexpr unsigned kFlagTestNoMma = 0x20000000u;   // the blob header does not describe what the kernel was launched for
+constexpr unsigned kFlagTestNoMma = 0x20000000u;
+constexpr unsigned kFlagTestHalf = 0x40000000u;     // ... in every other CTA
+__device__ __forceinline__ bool test_stalls(unsigned flags) {
+    return (flags & kFlagTestNoMma) && (!(flags & kFlagTestHalf) || (blockIdx.x & 1u));
+}
+// Tickets count the parts of an output tile that several CTAs share, and are zero between calls.  A CTA that gives up on a wait takes
+// its tickets too, with this mark: the last to come then clears the ticket and writes nothing.
+constexpr unsigned kTicketNoPart = 0x10000u;
 
 // Every GEMM kernel compares the header of the blob it was handed with the geometry it was launched for before it
 // reads any tile: a stale description of an address that now holds another blob must never turn into reads

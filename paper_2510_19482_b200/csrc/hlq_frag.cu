@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
     if (warp >= kComputeWarps) {
         // ---- activation warps ------------------------------------------------------------------------------------------------
         const int step = warp - kComputeWarps;
-        const bool loads = !(a.g.flags & kFlagTestNoMma);     // (test flag: nothing is loaded, the waits run out)
+        const bool loads = !test_stalls(a.g.flags);           // (test flag: nothing is loaded, the waits run out)
         int wu = u0;                                          // next unit whose weights are to be loaded
         auto load_weights = [&](int upto) {                   // by one elected lane; slot = unit number in the CTA mod ws
             for (; wu < upto; ++wu) {
@@ -508,7 +508,18 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
 #pragma unroll
                     for (int i = 0; i < 4; ++i) p[(8 * nb + (i & 1)) * kSumStride + 16 * t + 8 * (i >> 1)] = acc[t][nb][i];
         }
-        if (compute_any(!live)) break;
+        if (compute_any(!live)) {                             // the tickets of this run of units and the rest are taken all the same
+            for (int v = u - n_units; v < u1 && tid == 0;) {
+                const int t_ = v / C_, end = min((t_ + 1) * C_, u1);
+                if (end - v < C_) {
+                    const int parts = (t_ * C_ + C_ - 1) / a.per_cta - t_ * C_ / a.per_cta + 1;
+                    const unsigned t = atomicAdd(a.tickets + t_, 1u + kTicketNoPart);
+                    if ((t & (kTicketNoPart - 1)) == (unsigned)(parts - 1)) a.tickets[t_] = 0;
+                }
+                v = end;
+            }
+            break;
+        }
         const int row = tid & (kUnitRows - 1), n = tile * kUnitRows + row;
         const bool whole = n_units == C_;
         const int first = tile * C_ / a.per_cta;
@@ -529,10 +540,9 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
                 const int parts = (tile * C_ + C_ - 1) / a.per_cta - first + 1;
                 __threadfence();
                 const unsigned t = atomicAdd(a.tickets + tile, 1u);
-                const bool last = t == (unsigned)(parts - 1);
-                if (last) a.tickets[tile] = 0;                // zero again for the next call
+                if ((t & (kTicketNoPart - 1)) == (unsigned)(parts - 1)) a.tickets[tile] = 0;      // zero again for the next call
                 __threadfence();
-                *ticket_box = last ? 1u : 0u;
+                *ticket_box = t == (unsigned)(parts - 1) ? 1u : 0u;
             }
             pending = tile;
         }

@@ -159,12 +159,12 @@ __device__ __forceinline__ void st_cluster_u32(uint32_t addr, uint32_t rank, uin
     asm volatile("st.shared::cluster.u32 [%0], %1;" :: "r"(remote), "r"(v) : "memory");
 }
 
-// How many warps before this one took the ticket: read, or (take) announced behind the warp's own writes.
-__device__ __forceinline__ unsigned ticket_seen(unsigned* ticket, int lane, bool take) {
+// How many warps before this one took the ticket: read, or (add = 1 and a mark) announced behind the warp's own writes.
+__device__ __forceinline__ unsigned ticket_seen(unsigned* ticket, int lane, unsigned add) {
     unsigned t = 0;
     __syncwarp();
     if (lane == 0) {
-        if (take) asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(t) : "l"(ticket) : "memory");
+        if (add) asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(t) : "l"(ticket), "r"(add) : "memory");
         else asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(t) : "l"(ticket) : "memory");
     }
     __syncwarp();                                              // lane 0 has acquired for the whole warp (a shuffle orders no memory)
@@ -297,7 +297,7 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
         }
     } else if (warp == 1) {
         // ---- MMA issuer: one elected lane ------------------------------------------------------------------------------------
-        const int last = (a.g.flags & kFlagTestNoMma) ? t0 : t1;   // (test flag: nothing is issued or completes, the waits run out)
+        const int last = test_stalls(a.g.flags) ? t0 : t1;   // (test flag: nothing is issued or completes, the waits run out)
         if (elect_one()) {
             const uint32_t idesc = (1u << 4) | ((uint32_t)(a.mp >> 3) << 17) | ((uint32_t)(kBlockRows >> 4) << 24);
             const uint64_t x_desc0 = sw128_desc(smem_addr(sX));
@@ -368,9 +368,14 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
         // is there now and whether it is the last.
         auto parts_of = [&](int tile) { return (tile * a.n_steps + a.n_steps - 1) / a.per_cta - tile * a.n_steps / a.per_cta + 1; };
         auto ticket_of = [&](int tile) { return a.g.tickets + tile * a.n_steps / a.per_cta * (4 * kBlocks * kTurns) + (warp - kCtrlWarps); };
-        auto announce = [&](int tile) { return ticket_seen(ticket_of(tile), lane, true) == (unsigned)(parts_of(tile) - 1); };
+        auto announce = [&](int tile, unsigned mark) {
+            const unsigned t = ticket_seen(ticket_of(tile), lane, 1u + mark), last = (unsigned)(parts_of(tile) - 1);
+            if ((t & (kTicketNoPart - 1)) == last && t + mark != last && lane == 0) *ticket_of(tile) = 0;     // parts are missing: nobody adds up
+            return t + mark == last;
+        };
         int head = -1, tail = -1;                              // shared tiles to add up, to finish
-        for (Walk r(t0, t1, a.n_steps); r.more() && live; r.next()) {
+        Walk r(t0, t1, a.n_steps);
+        for (; r.more() && live; r.next()) {
             live = wait_warp(kBarWFull + blk * kMaxW + w.i, w.phase);
             if (!live) break;
             const uint8_t* rec = sW + (blk * a.ws + w.i) * C::UNIT_BYTES + item * C::TILE_BYTES + l * 16;      // this row's packed tile
@@ -484,8 +489,9 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
                 s.next();
                 s.next();
             }
+            if (!live) break;
             w.next();
-            if (live && r.ends()) {
+            if (r.ends()) {
                 grid_dependency_wait();
                 live = wait_warp(kBarDFull + blk, d_phase);
                 if (!live) break;
@@ -515,7 +521,7 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
                         put16(m0 + c0, n, mc, v);
                     }
                 }
-                if (a.reduce && !whole && announce(r.tile)) head = r.tile;
+                if (a.reduce && !whole && announce(r.tile, 0)) head = r.tile;
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar(kBarDEmpty + blk));
@@ -523,11 +529,17 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
         }
         if constexpr (CLUSTER) have_part = live && tail >= 0;
         else {
+            if (!live && a.reduce) {                           // the tickets not taken yet: of the run's first tile (once it ends), of its last
+                grid_dependency_wait();
+                const int first = t0 / a.n_steps, last = (t1 - 1) / a.n_steps;
+                if (r.tile == first && parts_of(first) > 1) announce(first, kTicketNoPart);
+                if (last != first && t1 < (last + 1) * a.n_steps) announce(last, kTicketNoPart);
+            }
             // Shared tiles: the warp that finds all other parts in the workspace adds them to its own in ascending k order (no
             // warp waits for another; a tile's other parts are mostly those that their CTAs began with, long written).
             if (live && tail >= 0) {
                 const int mine = b - tail * a.n_steps / a.per_cta, m0 = ((tail + base_tile) % a.m_tiles) * a.mp, m_count = min(a.mp, M - m0), n = row_of(tail);
-                if (ticket_seen(ticket_of(tail), lane, false) != (unsigned)(parts_of(tail) - 1)) {
+                if (ticket_seen(ticket_of(tail), lane, 0) != (unsigned)(parts_of(tail) - 1)) {
                     float* part = a.g.partials + ((size_t)mine * M + m0) * n_pad + n;
                     for (int c0 = 16 * turn; c0 < m_count; c0 += 16 * kTurns) {
                         uint32_t v[16];
@@ -537,7 +549,7 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
                         for (int i = 0; i < 16; ++i)
                             if (c0 + i < m_count && (size_t)n < n_pad) part[(size_t)(c0 + i) * n_pad] = __uint_as_float(v[i]);
                     }
-                    if (!announce(tail)) tail = -1;
+                    if (!announce(tail, 0)) tail = -1;
                 }
             }
             for (int e = 0; e < 2 && live; ++e) {
