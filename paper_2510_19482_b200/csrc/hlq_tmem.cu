@@ -229,9 +229,11 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
     const uint32_t limit = a.g.wait_limit ? a.g.wait_limit : kTmWaitLimit;
 
     // Bounded wait; false once this CTA has given up.  (Sleeping between polls: the waiting warps' instructions cost the
-    // producers 3 to 8 %, whatever the length.)
+    // producers 3 to 8 %, whatever the length.)  What has to be waited for may hang on the kernel before this one, which the limit
+    // is not to time.
     auto wait = [&](int i, uint32_t parity) {
         if (mbar_try(bar(i), parity)) return true;
+        grid_dependency_wait();
         for (uint32_t n = 0; n < limit; ++n) {
             __nanosleep(kPollNs);
             if (mbar_try(bar(i), parity)) return true;
