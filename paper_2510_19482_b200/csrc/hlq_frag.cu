@@ -108,13 +108,15 @@ struct Ring {
     }
 };
 
-// NB = blocks of 8 batch rows (MMA N).
-template <int Q, int G, int NB>
+// NB = blocks of 8 batch rows (MMA N).  FOLD: long runs of units, whose sums are put by every two units.
+template <int Q, int G, int NB, bool FOLD>
 __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArgs a) {
     using C = FragCfg<Q, G>;
     static_assert(G == 128 || G == 64, "");
     constexpr int NSG = C::NSG;                               // groups per step: 1 or 2
     constexpr int MP = 8 * NB;
+    constexpr bool kStepSum = NB == 1;
+    static_assert(!(kStepSum && FOLD), "");
     constexpr int XF_BYTES = MP * 1024;                       // B fragments of a unit: [step][block][4][lane] 16 bytes
     constexpr int XM_FLOATS = 4 * (1 + NSG) * MP;             // per step: factor 2^(14-c) and group sums of every batch row
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -366,6 +368,9 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
         }
     };
 
+    float* own_sum = sSum + (step * MP + 2 * c) * kSumStride + 32 * rp + gq;      // where the lane's sums go in the buffer
+    auto sum_at = [](int nb, int t, int i) { return (8 * nb + (i & 1)) * kSumStride + 16 * t + 8 * (i >> 1); };
+
     Ring w(a.ws), x(kXSlots);
     bool live = true;
     int pending = -1;                                         // row tile whose ticket has been taken and not looked at
@@ -373,6 +378,7 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
         const int tile = u / C_, chunk0 = u - tile * C_;
         const int n_units = min(C_ - chunk0, u1 - u);
         u += n_units;
+        if (FOLD) compute_sync();                             // the buffer has been read
         float acc[2][NB][4];
 #pragma unroll
         for (int t = 0; t < 2; ++t)
@@ -402,6 +408,31 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
                 float2 fac[NB];
 #pragma unroll
                 for (int nb = 0; nb < NB; ++nb) fac[nb] = *reinterpret_cast<const float2*>(meta + 8 * nb);
+                // The step's sum is formed by itself where the registers allow it: in one chain over all chunks and planes the fp32
+                // roundings add up (4096 x 14336, q = 4, G = 64, M = 8: 2.0e-7 of the result, 1.1e-7 so; the look-up kernel 1.2e-7).
+                float own[kStepSum ? 2 : 1][kStepSum ? NB : 1][4];
+                auto& sum = [&]() -> auto& {
+                    if constexpr (kStepSum) return own;
+                    else return acc;
+                }();
+                // offsets times the groups' activation sums
+#pragma unroll
+                for (int p = 0; p < NSG; ++p) {
+                    float z[4];
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) z[r] = half_bits(parameter(wb, r, p, Q) & offset_mask);
+#pragma unroll
+                    for (int nb = 0; nb < NB; ++nb) {
+                        const float2 s = *reinterpret_cast<const float2*>(meta + (1 + p) * MP + 8 * nb);
+#pragma unroll
+                        for (int t = 0; t < 2; ++t)
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                const float zi = z[2 * t + (i >> 1)], si = (i & 1) ? s.y : s.x;
+                                sum[t][nb][i] = kStepSum && p == 0 ? zi * si : fmaf(zi, si, sum[t][nb][i]);
+                            }
+                    }
+                }
                 if (use_planes) {
 #pragma unroll(NB <= 2 ? Q : 1)
                 for (int j = 0; j < Q; ++j) {
@@ -460,38 +491,39 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
                             for (int t = 0; t < 2; ++t)
 #pragma unroll
                                 for (int nb = 0; nb < NB; ++nb) {
-                                    acc[t][nb][0] = fmaf(sc[2 * t], d[t][nb][0] * fac[nb].x, acc[t][nb][0]);
-                                    acc[t][nb][1] = fmaf(sc[2 * t], d[t][nb][1] * fac[nb].y, acc[t][nb][1]);
-                                    acc[t][nb][2] = fmaf(sc[2 * t + 1], d[t][nb][2] * fac[nb].x, acc[t][nb][2]);
-                                    acc[t][nb][3] = fmaf(sc[2 * t + 1], d[t][nb][3] * fac[nb].y, acc[t][nb][3]);
+                                    sum[t][nb][0] = fmaf(sc[2 * t], d[t][nb][0] * fac[nb].x, sum[t][nb][0]);
+                                    sum[t][nb][1] = fmaf(sc[2 * t], d[t][nb][1] * fac[nb].y, sum[t][nb][1]);
+                                    sum[t][nb][2] = fmaf(sc[2 * t + 1], d[t][nb][2] * fac[nb].x, sum[t][nb][2]);
+                                    sum[t][nb][3] = fmaf(sc[2 * t + 1], d[t][nb][3] * fac[nb].y, sum[t][nb][3]);
                                 }
                         }
                     }
                 }
                 }
-                // offsets times the groups' activation sums
+                if constexpr (kStepSum) {
 #pragma unroll
-                for (int p = 0; p < NSG; ++p) {
-                    float z[4];
+                    for (int t = 0; t < 2; ++t)
 #pragma unroll
-                    for (int r = 0; r < 4; ++r) z[r] = half_bits(parameter(wb, r, p, Q) & offset_mask);
+                        for (int nb = 0; nb < NB; ++nb)
 #pragma unroll
-                    for (int nb = 0; nb < NB; ++nb) {
-                        const float2 s = *reinterpret_cast<const float2*>(meta + (1 + p) * MP + 8 * nb);
-#pragma unroll
-                        for (int t = 0; t < 2; ++t) {
-                            acc[t][nb][0] = fmaf(z[2 * t], s.x, acc[t][nb][0]);
-                            acc[t][nb][1] = fmaf(z[2 * t], s.y, acc[t][nb][1]);
-                            acc[t][nb][2] = fmaf(z[2 * t + 1], s.x, acc[t][nb][2]);
-                            acc[t][nb][3] = fmaf(z[2 * t + 1], s.y, acc[t][nb][3]);
-                        }
-                    }
+                            for (int i = 0; i < 4; ++i) acc[t][nb][i] += sum[t][nb][i];
                 }
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(kBarXEmpty + x.i));
             w.next();
             x.next();
+            if (FOLD && (cu & 1)) {
+#pragma unroll
+                for (int nb = 0; nb < NB; ++nb)
+#pragma unroll
+                    for (int t = 0; t < 2; ++t)
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            own_sum[sum_at(nb, t, i)] = cu == 1 ? acc[t][nb][i] : own_sum[sum_at(nb, t, i)] + acc[t][nb][i];
+                            acc[t][nb][i] = 0.f;
+                        }
+            }
         }
 
         // The four steps' sums meet in shared memory and are added and written out row by row.  (Where a warp gave up all leave
@@ -499,15 +531,13 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
         compute_sync();                                       // the buffer has been read; the ticket of the run before is there
         finish_tile(pending);
         pending = -1;
-        {
-            float* p = sSum + (step * MP + 2 * c) * kSumStride + 32 * rp + gq;
 #pragma unroll
-            for (int nb = 0; nb < NB; ++nb)
+        for (int nb = 0; nb < NB; ++nb)
 #pragma unroll
-                for (int t = 0; t < 2; ++t)
+            for (int t = 0; t < 2; ++t)
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) p[(8 * nb + (i & 1)) * kSumStride + 16 * t + 8 * (i >> 1)] = acc[t][nb][i];
-        }
+                for (int i = 0; i < 4; ++i)
+                    own_sum[sum_at(nb, t, i)] = FOLD && n_units > 1 ? own_sum[sum_at(nb, t, i)] + acc[t][nb][i] : acc[t][nb][i];
         if (compute_any(!live)) {                             // the tickets of this run of units and the rest are taken all the same
             for (int v = u - n_units; v < u1 && tid == 0;) {
                 const int t_ = v / C_, end = min((t_ + 1) * C_, u1);
@@ -552,7 +582,7 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
     __syncthreads();                                          // nobody leaves while copies are in flight
 }
 
-template <int Q, int G, int NB>
+template <int Q, int G, int NB, bool FOLD = false>
 int launch_frag_cfg(const GemmArgs& g, int num_sms, cudaStream_t stream) {
     using C = FragCfg<Q, G>;
     constexpr int kMaxSmem = 232448, MP = 8 * NB;
@@ -561,7 +591,7 @@ int launch_frag_cfg(const GemmArgs& g, int num_sms, cudaStream_t stream) {
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev >= 0 && dev < 64 && !configured[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(hlq_frag_kernel<Q, G, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+        cudaError_t e = cudaFuncSetAttribute(hlq_frag_kernel<Q, G, NB, FOLD>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
         if (e != cudaSuccess) return (int)e;
         configured[dev] = true;
     }
@@ -574,6 +604,12 @@ int launch_frag_cfg(const GemmArgs& g, int num_sms, cudaStream_t stream) {
     if (units >= (1LL << 30)) return (int)cudaErrorInvalidValue;
     a.units = (int)units;
     a.per_cta = (a.units + num_sms - 1) / num_sms;
+    // Runs of more than two units without a sum per step: the sums are put by in between, for the same reason as there (4096 x 14336, q = 4,
+    // G = 64, M = 32, error of the fp32 result 1.65e-7 -> 1.05e-7, the look-up kernel 1.0e-7 to 1.5e-7 by the number of rows; time
+    // 65.5 -> 67.0 us, at M = 16 36.3 -> 36.8).
+    if constexpr (NB > 1 && !FOLD) {
+        if (a.per_cta > 2) return launch_frag_cfg<Q, G, NB, true>(g, num_sms, stream);
+    }
     const int grid = (a.units + a.per_cta - 1) / a.per_cta;
     a.tickets = g.tickets;
     static_assert((kMaxSmem - kFixed) / C::UNIT_BYTES >= 2, "shared memory");
@@ -590,7 +626,7 @@ int launch_frag_cfg(const GemmArgs& g, int num_sms, cudaStream_t stream) {
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, hlq_frag_kernel<Q, G, NB>, a);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, hlq_frag_kernel<Q, G, NB, FOLD>, a);
     count_launch(1);
     return (int)e;
 }

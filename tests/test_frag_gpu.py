@@ -76,3 +76,16 @@ def test_warps_that_give_up_leave_together():
     y = gemm_f32(X, packed, N, K)
     assert elutq.elutq_device_status() == 0
     assert hlq.rel_fro_error(y, hlq.matmul(X, layer.planes, layer.scales, layer.offsets, G)) <= 5e-6
+
+
+@pytest.mark.parametrize("G,N,M", [(64, 1024, 8), (64, 2900, 16), (64, 2900, 32), (128, 1024, 4), (128, 12800, 8)])
+def test_long_sums_are_as_exact_as_the_look_up_kernels(G, N, M):
+    # Many chunks and planes: fp32 roundings of one long chain would show.  The error in norm over N * M >= 4096 results varies by
+    # about 1 / sqrt(2 N M) (1 %) from sample to sample: 5 % leaves room for that and for nothing else.
+    q, K = 4, 14336 if N < 10000 else 4096
+    layer = workloads.hlq_layer(65, f"frag/exact/{G}/{N}", q, G, N, K)
+    X = synth.activations(65, f"frag/exact/x/{M}", M, K)
+    packed = pack_layer(layer)
+    ref = hlq.matmul(X, layer.planes, layer.scales, layer.offsets, G)
+    lut = hlq.rel_fro_error(gemm_f32(X, packed, N, K, elutq.FLAG_LUT_ONLY), ref)
+    assert hlq.rel_fro_error(gemm_f32(X, packed, N, K), ref) <= 1.05 * lut
