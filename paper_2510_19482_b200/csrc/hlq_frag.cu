@@ -173,6 +173,7 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
     if (warp >= kComputeWarps) {
         // ---- activation warps ------------------------------------------------------------------------------------------------
         const int step = warp - kComputeWarps;
+        const bool use_offset = !(a.g.flags & ELUTQ_FLAG_SKIP_OFFSET);
         const bool loads = !test_stalls(a.g.flags);           // (test flag: nothing is loaded, the waits run out)
         int wu = u0;                                          // next unit whose weights are to be loaded
         auto load_weights = [&](int upto) {                   // by one elected lane; slot = unit number in the CTA mod ws
@@ -250,8 +251,9 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
                     top = max(top, __shfl_xor_sync(0xffffffffu, top, 1));
                     top = max(top, __shfl_xor_sync(0xffffffffu, top, 2));
                     const int ex = max(1, (int)(top >> 10)), cx = 29 - ex, c1 = min(cx, 14);      // x 2^cx < 2^15
+                    const bool infinite = top == 0x7c00u && use_offset;
                     if (c == 0) {
-                        meta[8 * nb + gq] = __uint_as_float((uint32_t)(127 + 14 - cx) << 23);
+                        meta[8 * nb + gq] = __uint_as_float(infinite ? 0x7f000000u : (uint32_t)(127 + 14 - cx) << 23);
                         if (NSG == 1) {
                             meta[MP + 8 * nb + gq] = sum[0][0] + sum[1][0];
                         } else {
@@ -280,6 +282,19 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
                         }
                         frag[(nb * 4 + 2 * q) * 32] = make_uint4(o[0], o[1], o[2], o[3]);
                         frag[(nb * 4 + 2 * q + 1) * 32] = make_uint4(o[4], o[5], o[6], o[7]);
+                    }
+                    // An infinity: with the offset term the row's results are not finite whatever its other activations are.  As an
+                    // operand it would make 0 * infinity = NaN of every bit that is not set.  2^15 in its place (less what the bit's mask
+                    // does), zeros elsewhere and a factor of 2^127 make an infinity of the set bits' sum, and 0 of none.
+                    if (infinite) {
+                        uint32_t* w = reinterpret_cast<uint32_t*>(frag + nb * 128);
+#pragma unroll 1
+                        for (int i = 0; i < 16; ++i) {
+                            const uint32_t r = w[(i >> 2) * 128 + (i & 3)], size = r & 0x7fff7fffu;
+                            const uint32_t inf = __vcmpeq2(size, 0x7c007c00u), nan = __vcmpgtu2(size, 0x7c007c00u);
+                            const uint32_t in_place = 0x78007800u - (0x7310u >> (4 * (i & 3)) & 15u) * 0x04000400u;
+                            w[(i >> 2) * 128 + (i & 3)] = (inf & ((r & 0x80008000u) | in_place)) | (nan & r);
+                        }
                     }
                 }
                 }

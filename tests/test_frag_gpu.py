@@ -89,3 +89,22 @@ def test_long_sums_are_as_exact_as_the_look_up_kernels(G, N, M):
     ref = hlq.matmul(X, layer.planes, layer.scales, layer.offsets, G)
     lut = hlq.rel_fro_error(gemm_f32(X, packed, N, K, elutq.FLAG_LUT_ONLY), ref)
     assert hlq.rel_fro_error(gemm_f32(X, packed, N, K), ref) <= 1.05 * lut
+
+
+@pytest.mark.parametrize("G,M", [(128, 3), (128, 8), (64, 5), (64, 20)])
+@pytest.mark.parametrize("values", [(np.inf,), (-np.inf,), (np.inf, np.inf), (np.inf, -np.inf), (np.nan,), (np.inf, np.nan)])
+def test_activations_that_are_not_finite(G, M, values):
+    # the same kind of result as from the decode kernel row by row, and no other row changes
+    q, N, K = 2, 300, 1024
+    layer = workloads.hlq_layer(66, f"frag/inf/{G}", q, G, N, K)
+    layer.offsets[::7] = 0
+    X = synth.activations(66, f"frag/inf/x/{M}", M, K)
+    packed = pack_layer(layer)
+    clean = gemm_f32(X, packed, N, K)
+    X[1, 200:200 + 3 * len(values):3] = values
+    y = gemm_f32(X, packed, N, K)
+    one = gemm_f32(X[1:2], packed, N, K)[0]
+    for kind in (np.isnan, np.isposinf, np.isneginf):
+        assert np.array_equal(kind(y[1]), kind(one))
+    keep = np.arange(M) != 1
+    assert np.array_equal(y[keep], clean[keep])
