@@ -73,7 +73,7 @@ typedef enum elutq_status {
                                      applied to fp32 sums, as exact as the look-up kernels); larger batches rebuild
                                      W_hat in fp16 tiles (8B gate_up / down at q = 2, us: M = 8 26.9 / 15.9 and
                                      24.9 / 18.9, M = 12 36.6 / 21.2 and 25.0 / 19.3).
-                                     At G = 64 every batch takes the former, 32 rows at a time
+                                     At G = 64 every batch takes the former, in blocks of 8 or 16 rows
                                      (elutq_takes_tensor_path is 1 for both)                                        */
 
 #define ELUTQ_FLAG_LUT_ONLY 0x80u /* M > 1: stay on the look-up-table kernels.  Without this flag batches of more than

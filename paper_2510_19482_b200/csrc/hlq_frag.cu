@@ -17,10 +17,10 @@
 //            of the row's 128 k (at G = 64: bytes 2c, 2c+1 of each group) as two sub-words with one byte in each half, twice: a
 //            left shift by 2 brings the upper copy's bits 0-3 to the four positions, one by 6 the lower copy's bits 4-7 (as
 //            multiplications: the logic pipe is the busy one).
-//   unit     128 weight rows x 512 k (eight packed tiles, contiguous in the blob: one bulk copy).  The units of a call, row tile
-//            by row tile, are dealt to the CTAs (one per SM) in equal contiguous runs, so no SM idles for a wave.  A row
-//            tile that several CTAs share is summed in ascending k order (bit-reproducible) by the CTA that finishes it last
-//            (a ticket per row tile, no CTA waits for another).
+//   unit     128 weight rows x 512 k (eight packed tiles, contiguous in the blob: one bulk copy) x 8 NB batch rows.  The units of
+//            a call, output tile by output tile (the batch blocks of a row tile next to each other: its weights come from the L2 again), are
+//            dealt to the CTAs (one per SM) in equal contiguous runs, so no SM idles for a wave.  An output tile that several CTAs share
+//            is summed in ascending k order (bit-reproducible) by the CTA that finishes it last (a ticket, no CTA waits for another).
 //   warps    16 compute warps: warp 4 s + r takes step s (128 k) of every unit and rows 32 r .. 32 r + 31 of the tile, so each
 //            activation fragment serves two MMAs.  Four activation warps, one per step: scale the unit's activations and
 //            lay them out as B fragments, form the group sums; the first of them also loads the weights.
@@ -40,13 +40,26 @@ constexpr uint32_t kFragWaitLimit = 1u << 22;
 constexpr int kMaxRing = 8, kXSlots = 2;        // weight units (at most), units of prepared activations
 constexpr int kSumStride = kUnitRows + 4;       // floats per batch row of the sum buffer (conflict-free for fragments)
 
+// n / d for 0 <= n < 2^31 by one multiplication: a runtime division costs 50 cycles and more, and a call of few units does a dozen in a row.
+struct Div {
+    int d;
+    unsigned long long m;       // m d = 2^64 + e with 0 <= e < d, so n m / 2^64 exceeds n / d by less than n / 2^64 (0 stands for d = 1)
+    __host__ void set(int d_) {
+        d = d_;
+        m = d_ == 1 ? 0ull : ~0ull / (unsigned)d_ + 1ull;
+    }
+    __device__ __forceinline__ int of(int n) const { return m == 0ull ? n : (int)__umul64hi((unsigned long long)n, m); }
+};
+
 struct FragArgs {
     GemmArgs g;
     int n_steps;                // 128-k steps of the whole K
-    int chunks;                 // units per row tile (512-k chunks)
+    int chunks;                 // units per output tile (512-k chunks)
+    int blocks;                 // output tiles per row tile (batch blocks of 8 NB rows; one at G = 128)
     int units, per_cta;         // all units; units of one CTA
+    Div by_chunks, by_blocks, by_cta;
     int ws;                     // weight units in flight
-    unsigned* tickets;          // one per row tile, zero between calls
+    unsigned* tickets;          // zero between calls: one per row tile, or (several blocks) per CTA, for the tile that it begins and does not end
 };
 
 enum { kBarWFull = 0, kBarXFull = kBarWFull + kMaxRing, kBarXEmpty = kBarXFull + kXSlots, kNumBars = kBarXEmpty + kXSlots };
@@ -108,7 +121,7 @@ struct Ring {
     }
 };
 
-// NB = blocks of 8 batch rows (MMA N).  FOLD: long runs of units, whose sums are put by every two units.
+// NB = blocks of 8 batch rows (MMA N): 1 or 2.  FOLD: long runs of units, whose sums are put by every two units.
 template <int Q, int G, int NB, bool FOLD>
 __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArgs a) {
     using C = FragCfg<Q, G>;
@@ -154,6 +167,8 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
         u1 = u0;
         if (tid == 0 && a.g.counters != nullptr) atomicExch(a.g.counters, kStatusBlobMismatch);
     }
+    auto row_tile = [&](int tile) { return G == 128 ? tile : a.by_blocks.of(tile); };
+    auto batch0 = [&](int tile) { return G == 128 ? 0 : (tile - a.by_blocks.of(tile) * a.blocks) * MP; };
     const uint32_t limit = a.g.wait_limit ? a.g.wait_limit : kFragWaitLimit;
     // Bounded wait; false once this CTA has given up.
     auto wait_many = [&](auto poll) {
@@ -175,10 +190,10 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
         const int step = warp - kComputeWarps;
         const bool use_offset = !(a.g.flags & ELUTQ_FLAG_SKIP_OFFSET);
         const bool loads = !test_stalls(a.g.flags);           // (test flag: nothing is loaded, the waits run out)
-        int wu = u0;                                          // next unit whose weights are to be loaded
+        int wu = u0, wslot = 0;                               // next unit whose weights are to be loaded, its slot
         auto load_weights = [&](int upto) {                   // by one elected lane; slot = unit number in the CTA mod ws
             for (; wu < upto; ++wu) {
-                const int tile = wu / C_, rb0 = tile * 8, slot = (wu - u0) % a.ws;
+                const int tile = a.by_chunks.of(wu), rb0 = row_tile(tile) * 8, slot = wslot;
                 const uint32_t bytes = (uint32_t)(min(8, a.g.n_rb - rb0) * C::TILE_BYTES);
                 if (elect_one()) {
                     mbar_expect(bar(kBarWFull + slot), bytes);
@@ -188,6 +203,7 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
                                  : "memory");
                 }
                 __syncwarp();
+                if (++wslot == a.ws) wslot = 0;
             }
         };
         // weights do not depend on the previous kernel: the first units are requested before the dependency wait
@@ -197,21 +213,20 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
         // The lane's four 16-byte pieces (8 k each) of a batch row and step: the low and the high bytes of the two sub-words.
         const int piece[2][2] = {{G == 128 ? 4 * c : 2 * c, G == 128 ? 4 * c + 2 : 2 * c + 1},
                                  {G == 128 ? 4 * c + 1 : 8 + 2 * c, G == 128 ? 4 * c + 3 : 8 + 2 * c + 1}};
-        constexpr int RB = NB <= 2 ? NB : 2;                  // blocks of 8 rows fetched at a time
-        uint4 raw[RB][2][2];
-        auto fetch = [&](int chunk, int nb0) {
+        uint4 raw[NB][2][2];
+        auto fetch = [&](int mb, int chunk) {
 #pragma unroll
-            for (int nb = 0; nb < RB; ++nb)
+            for (int nb = 0; nb < NB; ++nb)
 #pragma unroll
                 for (int q = 0; q < 2; ++q)
 #pragma unroll
                     for (int e = 0; e < 2; ++e) {
-                        const int m = 8 * (nb0 + nb) + gq, k = chunk * kChunkK + step * 128 + piece[q][e] * 8;
+                        const int m = mb + 8 * nb + gq, k = chunk * kChunkK + step * 128 + piece[q][e] * 8;
                         raw[nb][q][e] = (m < M && k < a.g.K) ? __ldg(reinterpret_cast<const uint4*>(a.g.X + (size_t)m * a.g.K + k)) : make_uint4(0, 0, 0, 0);
                     }
         };
-        int chunk = u0 % C_;
-        if (u0 < u1) fetch(chunk, 0);
+        int tile = a.by_chunks.of(u0), chunk = u0 - tile * C_, mb = batch0(tile);
+        if (u0 < u1) fetch(mb, chunk);
         for (int u = u0; u < u1; ++u) {
             const int t = u - u0, slot = t & 1;
             if (!__all_sync(0xffffffffu, wait_many([&]() { return mbar_try(bar(kBarXEmpty + slot), (uint32_t)((t >> 1) & 1) ^ 1u); }))) break;
@@ -219,18 +234,14 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
             if (step < steps_of(chunk)) {
                 uint4* frag = reinterpret_cast<uint4*>(sX + slot * XF_BYTES) + step * (NB * 128) + lane;
                 float* meta = sM + slot * XM_FLOATS + step * ((1 + NSG) * MP);
-#pragma unroll 1
-                for (int nb0 = 0; nb0 < NB; nb0 += RB) {
-                if (nb0 > 0) fetch(chunk, nb0);
 #pragma unroll
-                for (int r8 = 0; r8 < RB; ++r8) {
-                    const int nb = nb0 + r8;
+                for (int nb = 0; nb < NB; ++nb) {
                     __half2 v[2][2][4];
 #pragma unroll
                     for (int q = 0; q < 2; ++q)
 #pragma unroll
                         for (int e = 0; e < 2; ++e) {
-                            const uint32_t r[4] = {raw[r8][q][e].x, raw[r8][q][e].y, raw[r8][q][e].z, raw[r8][q][e].w};
+                            const uint32_t r[4] = {raw[nb][q][e].x, raw[nb][q][e].y, raw[nb][q][e].z, raw[nb][q][e].w};
 #pragma unroll
                             for (int i = 0; i < 4; ++i) v[q][e][i] = *reinterpret_cast<const __half2*>(&r[i]);
                         }
@@ -297,10 +308,12 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
                         }
                     }
                 }
-                }
             }
-            if (++chunk == C_) chunk = 0;
-            if (u + 1 < u1) fetch(chunk, 0);
+            if (++chunk == C_) {
+                chunk = 0;
+                mb = batch0(++tile);
+            }
+            if (u + 1 < u1) fetch(mb, chunk);
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(kBarXFull + slot));
         }
@@ -356,14 +369,16 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
                      : "=r"(any) : "r"((int)mine) : "memory");
         return any != 0;
     };
-    // The CTA that came last to a shared row tile adds the parts in ascending k order (all compute threads call this).
+    // The CTA that came last to a shared output tile adds the parts in ascending k order (all compute threads call this).
+    auto parts_of = [&](int tile) { return a.by_cta.of(tile * C_ + C_ - 1) - a.by_cta.of(tile * C_) + 1; };
+    auto ticket_of = [&](int tile) { return a.tickets + (G == 128 || a.blocks == 1 ? tile : a.by_cta.of(tile * C_)); };
     auto finish_tile = [&](int tile) {
         if (tile < 0 || *ticket_box == 0u) return;
-        const int n = tile * kUnitRows + (tid & (kUnitRows - 1));
-        const int parts = (tile * C_ + C_ - 1) / a.per_cta - tile * C_ / a.per_cta + 1;
+        const int n = row_tile(tile) * kUnitRows + (tid & (kUnitRows - 1)), mb = batch0(tile), me = min(M, mb + MP);
+        const int parts = parts_of(tile);
         if (n >= N) return;
         const float* p0 = a.g.partials + n;
-        for (int m0 = tid >> 7; m0 < M; m0 += 16) {
+        for (int m0 = mb + (tid >> 7); m0 < me; m0 += 16) {
             float y[4] = {0.f, 0.f, 0.f, 0.f};
             for (int p = 0; p < parts; p += 4) {
                 float v[4][4];
@@ -371,7 +386,7 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
                 for (int e = 0; e < 4; ++e)
 #pragma unroll
                     for (int i = 0; i < 4; ++i)
-                        v[e][i] = (p + e < parts && m0 + 4 * i < M) ? __ldcg(p0 + ((size_t)(p + e) * M + m0 + 4 * i) * n_pad) : 0.f;
+                        v[e][i] = (p + e < parts && m0 + 4 * i < me) ? __ldcg(p0 + ((size_t)(p + e) * M + m0 + 4 * i) * n_pad) : 0.f;
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
 #pragma unroll
@@ -379,7 +394,7 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
             }
 #pragma unroll
             for (int i = 0; i < 4; ++i)
-                if (m0 + 4 * i < M) put(m0 + 4 * i, n, y[i]);
+                if (m0 + 4 * i < me) put(m0 + 4 * i, n, y[i]);
         }
     };
 
@@ -388,9 +403,9 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
 
     Ring w(a.ws), x(kXSlots);
     bool live = true;
-    int pending = -1;                                         // row tile whose ticket has been taken and not looked at
+    int pending = -1;                                         // output tile whose ticket has been taken and not looked at
     for (int u = u0; u < u1 && live;) {
-        const int tile = u / C_, chunk0 = u - tile * C_;
+        const int tile = a.by_chunks.of(u), chunk0 = u - tile * C_;
         const int n_units = min(C_ - chunk0, u1 - u);
         u += n_units;
         if (FOLD) compute_sync();                             // the buffer has been read
@@ -411,15 +426,11 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
                 const uint32_t wb = smem_addr(sW) + (uint32_t)(w.i * C::UNIT_BYTES);
                 const uint32_t xb = smem_addr(sX) + (uint32_t)(x.i * XF_BYTES + step * (NB * 2048) + lane * 16);
                 const float* meta = sM + x.i * XM_FLOATS + step * ((1 + NSG) * MP) + 2 * c;
-                // B fragments: held over the planes where they fit the registers
-                constexpr bool HOLD = NB <= 2;
-                uint4 xh[HOLD ? NB : 1][4];
-                if constexpr (HOLD) {
+                uint4 xh[NB][4];                              // B fragments, held over the planes
 #pragma unroll
-                    for (int nb = 0; nb < NB; ++nb)
+                for (int nb = 0; nb < NB; ++nb)
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) xh[nb][i] = lds128(xb + (uint32_t)((nb * 4 + i) * 512));
-                }
+                    for (int i = 0; i < 4; ++i) xh[nb][i] = lds128(xb + (uint32_t)((nb * 4 + i) * 512));
                 float2 fac[NB];
 #pragma unroll
                 for (int nb = 0; nb < NB; ++nb) fac[nb] = *reinterpret_cast<const float2*>(meta + 8 * nb);
@@ -449,7 +460,7 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
                     }
                 }
                 if (use_planes) {
-#pragma unroll(NB <= 2 ? Q : 1)
+#pragma unroll
                 for (int j = 0; j < Q; ++j) {
                     uint32_t sub[2][4];                       // sub-words of the four rows
 #pragma unroll
@@ -489,7 +500,7 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
                             }
 #pragma unroll
                             for (int nb = 0; nb < NB; ++nb) {
-                                const uint4 xv = HOLD ? xh[HOLD ? nb : 0][2 * q + i2] : lds128(xb + (uint32_t)((nb * 4 + 2 * q + i2) * 512));
+                                const uint4 xv = xh[nb][2 * q + i2];
 #pragma unroll
                                 for (int t = 0; t < 2; ++t) {
                                     mma_16816(d[t][nb], f[2 * t][0], f[2 * t + 1][0], f[2 * t][1], f[2 * t + 1][1], xv.x, xv.y);
@@ -555,26 +566,24 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
                     own_sum[sum_at(nb, t, i)] = FOLD && n_units > 1 ? own_sum[sum_at(nb, t, i)] + acc[t][nb][i] : acc[t][nb][i];
         if (compute_any(!live)) {                             // the tickets of this run of units and the rest are taken all the same
             for (int v = u - n_units; v < u1 && tid == 0;) {
-                const int t_ = v / C_, end = min((t_ + 1) * C_, u1);
+                const int t_ = a.by_chunks.of(v), end = min((t_ + 1) * C_, u1);
                 if (end - v < C_) {
-                    const int parts = (t_ * C_ + C_ - 1) / a.per_cta - t_ * C_ / a.per_cta + 1;
-                    const unsigned t = atomicAdd(a.tickets + t_, 1u + kTicketNoPart);
-                    if ((t & (kTicketNoPart - 1)) == (unsigned)(parts - 1)) a.tickets[t_] = 0;
+                    const unsigned t = atomicAdd(ticket_of(t_), 1u + kTicketNoPart);
+                    if ((t & (kTicketNoPart - 1)) == (unsigned)(parts_of(t_) - 1)) *ticket_of(t_) = 0;
                 }
                 v = end;
             }
             break;
         }
-        const int row = tid & (kUnitRows - 1), n = tile * kUnitRows + row;
+        const int row = tid & (kUnitRows - 1), n = row_tile(tile) * kUnitRows + row, mb = batch0(tile), m_end = min(MP, M - mb);
         const bool whole = n_units == C_;
-        const int first = tile * C_ / a.per_cta;
-        float* part = a.g.partials + (size_t)(b - first) * M * n_pad + n;
-        for (int m = tid >> 7; m < M; m += kComputeThreads / kUnitRows) {
+        float* part = a.g.partials + ((size_t)(b - a.by_cta.of(tile * C_)) * M + mb) * n_pad + n;
+        for (int m = tid >> 7; m < m_end; m += kComputeThreads / kUnitRows) {
             float y = sSum[m * kSumStride + row];
 #pragma unroll
             for (int s = 1; s < 4; ++s) y += sSum[(s * MP + m) * kSumStride + row];
             if (whole) {
-                if (n < N) put(m, n, y);
+                if (n < N) put(mb + m, n, y);
             } else if ((size_t)n < n_pad) {
                 part[(size_t)m * n_pad] = y;
             }
@@ -582,10 +591,10 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
         if (!whole) {                                         // a ticket; what it says is looked at after the next run of units
             compute_sync();
             if (tid == 0) {
-                const int parts = (tile * C_ + C_ - 1) / a.per_cta - first + 1;
+                const int parts = parts_of(tile);
                 __threadfence();
-                const unsigned t = atomicAdd(a.tickets + tile, 1u);
-                if ((t & (kTicketNoPart - 1)) == (unsigned)(parts - 1)) a.tickets[tile] = 0;      // zero again for the next call
+                const unsigned t = atomicAdd(ticket_of(tile), 1u);
+                if ((t & (kTicketNoPart - 1)) == (unsigned)(parts - 1)) *ticket_of(tile) = 0;      // zero again for the next call
                 __threadfence();
                 *ticket_box = t == (unsigned)(parts - 1) ? 1u : 0u;
             }
@@ -612,19 +621,22 @@ int launch_frag_cfg(const GemmArgs& g, int num_sms, cudaStream_t stream) {
     }
     FragArgs a;
     a.g = g;
-    const int n_tiles = (g.N + kUnitRows - 1) / kUnitRows;
     a.n_steps = (g.K + 127) / 128;
     a.chunks = g.n_kc;
-    const long long units = (long long)n_tiles * g.n_kc;
+    a.blocks = (g.M + MP - 1) / MP;
+    const long long units = (long long)((g.N + kUnitRows - 1) / kUnitRows) * a.blocks * g.n_kc;
     if (units >= (1LL << 30)) return (int)cudaErrorInvalidValue;
     a.units = (int)units;
     a.per_cta = (a.units + num_sms - 1) / num_sms;
     // Runs of more than two units without a sum per step: the sums are put by in between, for the same reason as there (4096 x 14336, q = 4,
-    // G = 64, M = 32, error of the fp32 result 1.65e-7 -> 1.05e-7, the look-up kernel 1.0e-7 to 1.5e-7 by the number of rows; time
-    // 65.5 -> 67.0 us, at M = 16 36.3 -> 36.8).
+    // G = 64, M = 16, error of the fp32 result 1.5e-7 -> 1.0e-7, the look-up kernel 1.0e-7 to 1.5e-7 by the number of rows; time
+    // 36.3 -> 36.8 us).
     if constexpr (NB > 1 && !FOLD) {
         if (a.per_cta > 2) return launch_frag_cfg<Q, G, NB, true>(g, num_sms, stream);
     }
+    a.by_chunks.set(a.chunks);
+    a.by_blocks.set(a.blocks);
+    a.by_cta.set(a.per_cta);
     const int grid = (a.units + a.per_cta - 1) / a.per_cta;
     a.tickets = g.tickets;
     static_assert((kMaxSmem - kFixed) / C::UNIT_BYTES >= 2, "shared memory");
@@ -648,9 +660,19 @@ int launch_frag_cfg(const GemmArgs& g, int num_sms, cudaStream_t stream) {
 
 template <int Q, int G>
 int launch_frag_qg(const GemmArgs& g, int num_sms, cudaStream_t stream) {
-    if (g.M <= 8) return launch_frag_cfg<Q, G, 1>(g, num_sms, stream);
-    if constexpr (G == 64) return g.M <= 16 ? launch_frag_cfg<Q, G, 2>(g, num_sms, stream) : launch_frag_cfg<Q, G, 4>(g, num_sms, stream);
-    return (int)cudaErrorInvalidValue;
+    if constexpr (G == 64) {
+        // The height of a batch block, by the longest run of units: a unit takes u us, the first one of a taller block u0 more.  (Fitted
+        // to 1100 calls, 256 to 28672 rows.  Blocks of 32 rows, whose sums do not fit the registers, are nowhere ahead: 4096 x 4096,
+        // q = 4, M = 32 23.3 us in blocks of 16, 28.3 of 32; 28672 x 8192 218 and 232.)
+        const long long tiles = (long long)((g.N + kUnitRows - 1) / kUnitRows) * g.n_kc;
+        auto us = [&](int rows, double u0, double u) {
+            const long long units = tiles * ((g.M + rows - 1) / rows);
+            return u0 + u * (double)((units + num_sms - 1) / num_sms);
+        };
+        if (g.M > 8 && us(16, 1.0, 1.0 + 0.86 * Q) < us(8, 0.0, 0.5 + 0.6 * Q)) return launch_frag_cfg<Q, G, 2>(g, num_sms, stream);
+        return launch_frag_cfg<Q, G, 1>(g, num_sms, stream);
+    }
+    return g.M <= 8 ? launch_frag_cfg<Q, G, 1>(g, num_sms, stream) : (int)cudaErrorInvalidValue;
 }
 
 template <int Q>
@@ -664,25 +686,15 @@ int launch_frag_q(const GemmArgs& g, int G, int num_sms, cudaStream_t stream) {
 
 }  // namespace
 
-// Up to ELUTQ_FRAGMENT_MAX_M rows at G = 128, any number at G = 64 (32 rows to a launch; the launches follow one another on
-// the stream and share the partial sums).
+// Up to ELUTQ_FRAGMENT_MAX_M rows at G = 128, any number at G = 64.
 int launch_hlq_frag(const GemmArgs& g, int q, int G, int num_sms, cudaStream_t stream) {
-    const size_t out = (g.flags & ELUTQ_FLAG_OUT_F32) ? sizeof(float) : sizeof(__half);
-    int ce = 0;
-    for (int m0 = 0; m0 < g.M && ce == 0; m0 += 32) {
-        GemmArgs p = g;
-        p.X = g.X + (size_t)m0 * g.K;
-        p.Y = reinterpret_cast<uint8_t*>(g.Y) + (size_t)m0 * g.N * out;
-        p.M = g.M - m0 < 32 ? g.M - m0 : 32;
-        switch (q) {
-            case 1: ce = launch_frag_q<1>(p, G, num_sms, stream); break;
-            case 2: ce = launch_frag_q<2>(p, G, num_sms, stream); break;
-            case 3: ce = launch_frag_q<3>(p, G, num_sms, stream); break;
-            case 4: ce = launch_frag_q<4>(p, G, num_sms, stream); break;
-            default: ce = (int)cudaErrorInvalidValue;
-        }
+    switch (q) {
+        case 1: return launch_frag_q<1>(g, G, num_sms, stream);
+        case 2: return launch_frag_q<2>(g, G, num_sms, stream);
+        case 3: return launch_frag_q<3>(g, G, num_sms, stream);
+        case 4: return launch_frag_q<4>(g, G, num_sms, stream);
+        default: return (int)cudaErrorInvalidValue;
     }
-    return ce;
 }
 
 }  // namespace elutq

@@ -19,7 +19,7 @@ pytestmark = pytest.mark.gpu
 
 from gpu_util import gemm_f32, pack_layer, x_dev  # noqa: E402
 
-# (q, G, N, K, M): edges of the 8- and 16-row fragments, the 32-row launch and the 128-row tile, K ending inside a 512-k chunk and
+# (q, G, N, K, M): edges of the 8- and 16-row blocks and of the 128-row tile, K ending inside a 512-k chunk and
 # a 64-k half step, one tile and one chunk, row tiles shared by several CTAs, every q
 CASES = [(2, 128, 128, 512, 3), (1, 128, 17, 128, 8), (3, 128, 129, 640, 7), (4, 128, 1000, 1408, 8), (2, 128, 4096, 4096, 5),
          (4, 128, 300, 4224, 8), (2, 64, 129, 640, 9), (3, 64, 127, 64, 3), (2, 64, 256, 1088, 16), (4, 64, 333, 2880, 17), (3, 64, 1000, 1984, 33),
@@ -108,3 +108,19 @@ def test_activations_that_are_not_finite(G, M, values):
         assert np.array_equal(kind(y[1]), kind(one))
     keep = np.arange(M) != 1
     assert np.array_equal(y[keep], clean[keep])
+
+
+@pytest.mark.parametrize("q,N,K,M", [(1, 129, 64, 257), (2, 1000, 1024, 33), (2, 2048, 4096, 130), (3, 4000, 2880, 57), (4, 300, 4160, 100)])
+def test_batch_blocks_of_one_launch(q, N, K, M):
+    # blocks of 8, 16 and 32 rows with a remainder, several to a row tile, output tiles shared by CTAs; one launch, no call slower for its rows
+    layer = workloads.hlq_layer(67, f"frag/blocks/{q}/{N}/{K}", q, 64, N, K)
+    X = synth.activations(67, f"frag/blocks/x/{M}/{K}", M, K, outliers=True)
+    packed = pack_layer(layer)
+    ref = hlq.matmul(X, layer.planes, layer.scales, layer.offsets, 64)
+    y = gemm_f32(X, packed, N, K)
+    before = elutq.elutq_launch_count()
+    again = gemm_f32(X, packed, N, K)
+    assert elutq.elutq_launch_count() == before + 1
+    assert max(hlq.rel_fro_error(y[m], ref[m]) for m in range(M)) <= 5e-6
+    assert np.array_equal(y, again)
+    assert elutq.elutq_device_status() == 0
