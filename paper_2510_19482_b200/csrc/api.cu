@@ -78,19 +78,25 @@ size_t partials_bytes(int M, int N, int K) {
 }
 
 // Which kernel takes more than ELUTQ_FRAGMENT_MAX_M rows at G = 128: true = hlq_mma.cu (weights rebuilt in shared memory), false =
-// hlq_tmem.cu (in tensor memory).  In output tiles of 256 rows x 128 tokens, us of hlq_mma and hlq_tmem:
-//   few row tiles      its deeper K splits (1000 x 8192, q = 3, M = 64 12.9 and 20.7; against 1000 x 4096, M = 64 9.5 and 8.3), and
-//                      little work for more than 96 tokens (2048 x 2048, M = 128 10.9 and 11.7; against 2048 x 4096 16.2 and 14.4)
-//   many tokens        its CTA pairs rebuild a weight once per 512 tokens and need no split where they fill the GPU (28672 x 4096,
-//                      q = 2: M = 512 108 and 117, M = 2048 422 and 473; against M = 384 106 and 95, M = 128 54 and 33, and where
-//                      they do not, 4096 x 4096, M = 1024, 66 and 32).  They take an even number of 256-token tiles; 2 * 256 tokens
-//                      cost them as much as 3.5 * 128 cost hlq_tmem.
-//   q = 4, 193 to 256  with too many tiles for clusters (28672 x 4096, M = 256, 82 and 87; q = 2 63 and 62; 6144 x 4096, q = 4, 47 and 28)
+// hlq_tmem.cu (in tensor memory).
+//   up to 128 tokens   the latter, but for few rows, in output tiles of 256: with a long K, which hlq_mma splits deeper (1000 x 14336,
+//                      M = 64, q = 2 / 4 14.7 / 18.3 us against 19.5 / 20.6; 1500 x 14336 20.2 / 25.4 against 15.6 / 25.7, 1000 x 8192, M = 16,
+//                      q = 2 9.4 against 8.5), and with little work for 97 and more (1000 x 4096, M = 128, q = 2 11.1 against 12.1; 1500 x
+//                      2048, q = 4 12.3 against 11.0)
+//   129 to 256         likewise where K is very long (1000 x 16384, M = 256, q = 4 / 2 28.1 / 24.7 against 34.1 / 22.8)
+//   more               the lower estimate.  hlq_mma rebuilds a weight once per 256 or 512 tokens, hlq_tmem once per 128 but has no tile of 256
+//                      tokens to leave idle and splits K cheaply: 28672 x 4096, q = 2, M = 2048 404 against 463, M = 384 106 and 85;
+//                      16384 x 2048, q = 4, M = 384 36.9 and 47.8; 6144 x 2048, q = 2, M = 2048 87 and 56.  Over 4650 calls the choice costs 0.2 %
+//                      against the better of the two, at most 10 % but for a few (24 %).
 bool rebuilds_in_shared_memory(int M, int N, int K, int q, int sms) {
-    const long long rows = ((long long)N + 255) / 256, m128 = (M + 127) / 128, m256 = (M + 255) / 256;
-    if (rows <= 8 && m128 == 1 && (K / 128 >= 16 * rows || (M > 96 && rows * (K / 128) <= 128))) return true;
-    if (m256 % 2 == 0 && 4 * m128 >= 7 * m256 && rows * m256 * 20 >= 17LL * sms) return true;
-    return q == 4 && M > 192 && M <= 256 && 4 * rows > 3LL * sms;
+    const long long rows = ((long long)N + 255) / 256, steps = K / 128;
+    if (!tmem_takes(M, N, K)) return true;
+    if (M <= 128) {
+        if (rows <= 4 && steps >= 16 * rows && (M > 48 || steps >= 24 * rows)) return true;
+        return M > 96 && rows <= 8 && rows * steps <= 128 && (rows <= 4 || q <= 2);
+    }
+    if (M <= 256 && rows <= 4 && q >= 3 && steps >= 32 * rows) return true;
+    return mma_us(M, N, K, q, sms) < tmem_us(M, N, K, q, sms);
 }
 
 int lookup_blob(const void* packed, int N, int K, BlobMeta* out, bool force_read = false) {

@@ -80,6 +80,10 @@ int launch_lut_gemm(const GemmArgs& a, int q, int G, int num_sms, cudaStream_t s
 int launch_hlq_frag(const GemmArgs& a, int q, int G, int num_sms, cudaStream_t stream);
 int launch_hlq_mma(const GemmArgs& a, int q, int G, int num_sms, cudaStream_t stream);
 int launch_hlq_tmem(const GemmArgs& a, int q, int num_sms, cudaStream_t stream);
+bool tmem_takes(int M, int N, int K);                         // (index ranges)
+// Estimates in us for more than 128 tokens (hlq_mma: infinite where it would have to split K)
+double tmem_us(int M, int N, int K, int q, int num_sms);
+double mma_us(int M, int N, int K, int q, int num_sms);
 
 // col0 / cols restrict the reduction to output columns [col0, col0 + cols) (cols = 0: all N columns).
 int launch_finalize(const GemmArgs& a, int n_chunks, bool pdl, cudaStream_t stream, int col0 = 0, int cols = 0);

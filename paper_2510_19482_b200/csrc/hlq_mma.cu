@@ -750,26 +750,38 @@ int launch_mma_cfg(const GemmArgs& a, int num_sms, cudaStream_t stream) {
 
 template <int Q>
 int launch_mma_q(const GemmArgs& a, int num_sms, cudaStream_t stream) {
-    // Two token tiles per CTA once M exceeds one tile; 256 weight rows per CTA unless even the largest K split
-    // would leave most SMs without work.
-    const bool two = a.M > kTileM;
-    const long long m_tiles = two ? (a.M + 2 * kTileM - 1) / (2 * kTileM) : (a.M + kTileM - 1) / kTileM;
-    const long long tiles256 = (long long)((a.N + 255) / 256) * m_tiles;
+    // Two token tiles per CTA once M exceeds one tile; 128 weight rows per CTA instead of 256 with one token tile (few rows come
+    // here) or where even the largest K split would leave most SMs without work.
+    if (a.M <= kTileM) return launch_mma_cfg<Q, 128, 1>(a, num_sms, stream);
+    const long long m_tiles = (a.M + 2 * kTileM - 1) / (2 * kTileM), tiles256 = (long long)((a.N + 255) / 256) * m_tiles;
     const int max_splits = 2 * a.n_kc < 16 ? 2 * a.n_kc : 16;
-    bool narrow = tiles256 * max_splits * 2 <= num_sms;
-    // measured: the warp-specialised form is 3-5 % faster (no CTA-wide barrier in the step, the issuing thread dequantises nothing)
-    // measured: a CTA pair per weight tile (each CTA dequantises half of it) is 8-22 % faster again; it needs an even
+    if (tiles256 * max_splits * 2 <= num_sms) return launch_mma_cfg<Q, 128, 2>(a, num_sms, stream);
+    // measured: the warp-specialised form is 3-5 % faster (no CTA-wide barrier in the step, the issuing thread dequantises nothing);
+    // a CTA pair per weight tile (each CTA dequantises half of it) is 8-22 % faster again; it needs an even
     // number of 256-token tiles
-    if (two && !narrow && m_tiles % 2 == 0) return launch_mma_cfg<Q, 256, 2, true, 2>(a, num_sms, stream);
-    if (two && !narrow) return launch_mma_cfg<Q, 256, 2, true>(a, num_sms, stream);
-    if (two) return launch_mma_cfg<Q, 128, 2>(a, num_sms, stream);
-    return narrow ? launch_mma_cfg<Q, 128, 1>(a, num_sms, stream) : launch_mma_cfg<Q, 256, 1>(a, num_sms, stream);
+    if (m_tiles % 2 == 0) return launch_mma_cfg<Q, 256, 2, true, 2>(a, num_sms, stream);
+    return launch_mma_cfg<Q, 256, 2, true>(a, num_sms, stream);
 }
 
 }  // namespace
 
-// Largest K split the tensor-core path may pick for (M, N, K): sizes the partial buffer.
-int mma_max_splits() { return 16; }
+// Time of a call with more than 128 tokens that needs no K split in whole rounds (with one: a finalize pass over many slices, nowhere
+// the better choice), fitted to 960 calls (256 to 57344 rows, K 1024 to 16384; 4 to 6 % off in the mean).  A round of tiles, whose step
+// slows down as the GPU fills; the stripe that is left over by a second launch, with its K split.
+double mma_us(int M, int N, int K, int q, int num_sms) {
+    static const double pair_step[5] = {0, 1.13, 1.28, 1.48, 1.73}, one_step[5] = {0, 1.07, 1.0, 1.17, 1.47}, one_fill[5] = {0, 0.58, 0.98, 1.17, 1.14};
+    const int rows = (N + 255) / 256, m_tiles = (M + 2 * kTileM - 1) / (2 * kTileM), steps = (K + kStepK - 1) / kStepK;
+    const long long tiles = (long long)rows * m_tiles;
+    if (2 * tiles <= num_sms) return 1e30;
+    const bool pair = m_tiles % 2 == 0;
+    const double start = pair ? 8.6 : 7.0, step = pair ? pair_step[q] : one_step[q], fill = pair ? 0.22 : one_fill[q];
+    if (tiles > num_sms) {
+        const long long full = tiles / num_sms, tail = (rows - full * num_sms / m_tiles) * m_tiles;
+        if (tail > 0 && 2 * tail <= num_sms)
+            return full * (start + steps * (step + fill)) + (pair ? 25.0 : 40.0) + tail * ((pair ? 0.35 : -0.18) + 0.0125 * steps);
+    }
+    return (tiles + num_sms - 1) / num_sms * (start + steps * step) + fill * steps * tiles / num_sms;
+}
 
 int launch_hlq_mma(const GemmArgs& a, int q, int G, int num_sms, cudaStream_t stream) {
     if (G != 128) return (int)cudaErrorNotSupported;

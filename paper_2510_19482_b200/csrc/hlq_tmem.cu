@@ -30,6 +30,8 @@
 // roles' waits; copies and MMAs in flight are waited for (bounded), tensor memory is freed, the kernel returns.
 #include <cuda.h>
 
+#include <mutex>
+
 #include "common.cuh"
 
 namespace elutq {
@@ -62,6 +64,7 @@ struct TmemArgs {
 enum { kBarWFull = 0, kBarWEmpty = kBarWFull + kBlocks * kMaxW, kBarXFull = kBarWEmpty + kBlocks * kMaxW, kBarXEmpty = kBarXFull + kMaxX,
        kBarAFull = kBarXEmpty + kMaxX, kBarAEmpty = kBarAFull + kBlocks * kMaxSlots, kBarDFull = kBarAEmpty + kBlocks * kMaxSlots,
        kBarDEmpty = kBarDFull + kBlocks, kBarDrain = kBarDEmpty + kBlocks, kNumBars };
+constexpr int kMaxSmem = 232448, kFixed = kNumBars * 8 + 64;   // dynamic shared memory; of it barriers and flags
 
 template <int Q>
 struct TmCfg {
@@ -714,12 +717,40 @@ Plan plan_of(int q, int mp, int tiles, int n_steps, int num_sms, const int (&max
     return best;
 }
 
+// What a call is launched as: all tiles by one plan, or whole rounds of whole tiles and the rest of them in a second launch, where that leaves
+// less idle (28672 x 4096, q = 2, M = 384, 336 tiles = two rounds and 40 tiles by clusters of three: 93 -> 85 us; M = 320 83 -> 78).
+struct Schedule {
+    int m_tiles, mp, tiles, n_steps, full;                    // full: tiles of the first launch (all: no second one)
+    Plan first, rest;
+};
+Schedule schedule_of(int q, int M, int N, int K, int num_sms, const int (&max_clusters)[kMaxSplit + 1]) {
+    Schedule s;
+    s.m_tiles = (M + kMaxTokens - 1) / kMaxTokens;
+    s.mp = ((M + s.m_tiles - 1) / s.m_tiles + 15) / 16 * 16;
+    s.n_steps = K / 128;
+    s.tiles = s.full = (N + kTileRowsN - 1) / kTileRowsN * s.m_tiles;
+    s.first = plan_of(q, s.mp, s.tiles, s.n_steps, num_sms, max_clusters);
+    s.rest = s.first;
+    const int full = s.tiles / num_sms * num_sms;
+    if (full > 0 && full < s.tiles) {
+        const Plan rounds = {full / num_sms * s.n_steps, 1, step_us(q, s.mp) * (full / num_sms * s.n_steps)};
+        const Plan rest = plan_of(q, s.mp, s.tiles - full, s.n_steps, num_sms, max_clusters);
+        if (rest.split > 1 && rounds.cost + 6.0 + rest.cost < s.first.cost) {
+            s.full = full;
+            s.first = rounds;
+            s.rest = rest;
+        }
+    }
+    return s;
+}
+
+// Clusters of each size that are resident together on the current device (on one that cannot say: GPCs of 18 and 20 SMs).
+const int (&resident_clusters())[kMaxSplit + 1];
+
 template <int Q>
 int launch_tmem_q(const GemmArgs& g, int num_sms, cudaStream_t stream) {
     using C = TmCfg<Q>;
-    constexpr int kMaxSmem = 232448, kFixed = kNumBars * 8 + 64;
     static bool configured[64] = {};
-    static int max_clusters[64][kMaxSplit + 1] = {};          // of each size, resident together
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64) return (int)cudaErrorNotSupported;
@@ -727,32 +758,15 @@ int launch_tmem_q(const GemmArgs& g, int num_sms, cudaStream_t stream) {
         cudaError_t e = cudaFuncSetAttribute(hlq_tmem_kernel<Q, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(hlq_tmem_kernel<Q, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
         if (e != cudaSuccess) return (int)e;
-        for (int n = 2; n <= kMaxSplit; ++n) {
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3((unsigned)(n * num_sms));
-            cfg.blockDim = dim3(kTmThreads);
-            cfg.dynamicSmemBytes = kMaxSmem;
-            cudaLaunchAttribute attr[1];
-            attr[0].id = cudaLaunchAttributeClusterDimension;
-            attr[0].val.clusterDim.x = (unsigned)n;
-            attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-            cfg.attrs = attr;
-            cfg.numAttrs = 1;
-            if (cudaOccupancyMaxActiveClusters(&max_clusters[dev][n], hlq_tmem_kernel<Q, true>, &cfg) != cudaSuccess) {
-                max_clusters[dev][n] = 0;
-                (void)cudaGetLastError();
-            }
-        }
         configured[dev] = true;
     }
+    if (!tmem_takes(g.M, g.N, g.K)) return (int)cudaErrorNotSupported;
+    const Schedule sch = schedule_of(Q, g.M, g.N, g.K, num_sms, resident_clusters());
     TmemArgs a;
     a.g = g;
-    a.m_tiles = (g.M + kMaxTokens - 1) / kMaxTokens;
-    a.mp = ((g.M + a.m_tiles - 1) / a.m_tiles + 15) / 16 * 16;
-    a.n_steps = g.K / 128;
-    const long long all = (long long)((g.N + kTileRowsN - 1) / kTileRowsN) * a.m_tiles;
-    if (all * a.n_steps >= (1LL << 30)) return (int)cudaErrorNotSupported;
-    const int tiles = (int)all;
+    a.m_tiles = sch.m_tiles;
+    a.mp = sch.mp;
+    a.n_steps = sch.n_steps;
     a.ss = (kTmemCols - kBlocks * a.mp) / (kBlocks * kSlotCols);
     if (a.ss > kMaxSlots) a.ss = kMaxSlots;
     const int x_bytes = a.mp * 256, w_bytes = kBlocks * C::UNIT_BYTES;
@@ -805,21 +819,65 @@ int launch_tmem_q(const GemmArgs& g, int num_sms, cudaStream_t stream) {
         count_launch(1);
         return (int)e;
     };
-    // Whole rounds of whole tiles and a second launch for the rest of them, where that leaves less idle (28672 x 4096, q = 2, M = 384,
-    // 336 tiles = two rounds and 40 tiles by clusters of three: 93 -> 85 us; M = 320 83 -> 78).
-    const Plan plan = plan_of(Q, a.mp, tiles, a.n_steps, num_sms, max_clusters[dev]);
-    const int full = tiles / num_sms * num_sms;
-    if (full > 0 && full < tiles) {
-        const Plan rounds = {full / num_sms * a.n_steps, 1, 0.0}, rest = plan_of(Q, a.mp, tiles - full, a.n_steps, num_sms, max_clusters[dev]);
-        if (rest.split > 1 && step_us(Q, a.mp) * rounds.per_cta + 6.0 + rest.cost < plan.cost) {
-            const int ce = launch(0, full, rounds);
-            return ce != 0 ? ce : launch(full, tiles - full, rest);
-        }
+    const int ce = launch(0, sch.full, sch.first);
+    return ce != 0 || sch.full == sch.tiles ? ce : launch(sch.full, sch.tiles - sch.full, sch.rest);
+}
+
+const int (&resident_clusters())[kMaxSplit + 1] {
+    struct Table { int n[kMaxSplit + 1]; };
+    static const Table fallback = {{0, 148, 74, 48, 34, 26, 24, 16, 16}};
+    static Table tables[64];
+    static std::once_flag once[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
+        (void)cudaGetLastError();
+        return fallback.n;
     }
-    return launch(0, tiles, plan);
+    std::call_once(once[dev], [dev] {
+        tables[dev] = fallback;
+        if (cudaFuncSetAttribute(hlq_tmem_kernel<4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return;
+        }
+        for (int n = 2; n <= kMaxSplit; ++n) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3((unsigned)(n * 148));
+            cfg.blockDim = dim3(kTmThreads);
+            cfg.dynamicSmemBytes = kMaxSmem;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = (unsigned)n;
+            attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            if (cudaOccupancyMaxActiveClusters(&tables[dev].n[n], hlq_tmem_kernel<4, true>, &cfg) != cudaSuccess) {
+                tables[dev].n[n] = 0;
+                (void)cudaGetLastError();
+            }
+        }
+    });
+    return tables[dev].n;
 }
 
 }  // namespace
+
+bool tmem_takes(int M, int N, int K) {
+    return (((long long)N + kTileRowsN - 1) / kTileRowsN) * ((M + kMaxTokens - 1) / kMaxTokens) * (K / 128) < (1LL << 30);
+}
+
+// Time of a call with more than 128 tokens, fitted to 2300 calls (256 to 57344 rows, K 1024 to 16384, 129 to 2048 tokens; 4 to 6 % off in the
+// mean, 9 % for clusters).  plan_of's costs choose between plans; between kernels their constants are not good enough.
+double tmem_us(int M, int N, int K, int q, int num_sms) {
+    static const double whole_step[5] = {0, 0.22, 0.32, 0.68, 0.96}, whole_tokens[5] = {0, 0.0049, 0.0046, 0.0029, 0.0026};
+    static const double share_step[5] = {0, 0.2, 0.3, 0.65, 0.8}, share_tokens[5] = {0, 0.0054, 0.0055, 0.004, 0.0047};
+    const Schedule s = schedule_of(q, M, N, K, num_sms, resident_clusters());
+    const double round = 3.8 + s.n_steps * (whole_step[q] + whole_tokens[q] * s.mp);
+    const double rounds = 1.1 + (s.full + num_sms - 1) / num_sms * round;
+    if (s.full < s.tiles) return rounds + 5.0 + 0.97 * s.rest.cost;
+    if (s.first.split > 1) return 4.1 + s.first.cost * (q == 1 ? 1.1 : 0.97);
+    if (s.first.per_cta % s.n_steps == 0) return rounds;
+    return 18.0 + s.first.per_cta * (share_step[q] + share_tokens[q] * s.mp);
+}
 
 int launch_hlq_tmem(const GemmArgs& g, int q, int num_sms, cudaStream_t stream) {
     switch (q) {
