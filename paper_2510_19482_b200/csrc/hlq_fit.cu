@@ -35,9 +35,15 @@ namespace elutq {
 namespace {
 
 constexpr int kFitWarps = 8;      // warps (groups) per CTA
-// Fewer groups than this (q <= 2; 16384 above) leave the sorted form waiting on its own latencies: 8192 groups of 128, q = 2, ten rounds:
-// 45 us sorted, 46 direct; q = 4: 142 / 127, at 16384 of 64 121 / 122, at 32768 of 128 199 / 423.
-constexpr long long kSortedMinGroups = 8192;
+// From how many groups on the sorted form is ahead: with fewer it waits on its own latencies, and its sort has to pay off over the rounds.
+// Rounds: 1, 2 to 4, 5 and more; in 1024 groups, measured at 2048 to 262144.  (us, direct and sorted: 8192 groups of 128, q = 2, ten rounds
+// 45 and 45, one 9.9 and 26.5; 32768 of 128, q = 1, one round 18 and 27, ten 49 and 34; 16384 of 32, q = 4, ten rounds 75 and 108.)
+constexpr int kSortedMinK[3][4][3] = {{{12, 12, 16}, {12, 8, 8}, {12, 8, 12}, {12, 12, 24}},               // G = 32: q = 1 to 4
+                                      {{32, 24, 16}, {24, 12, 12}, {12, 8, 8}, {12, 12, 16}},              // G = 64
+                                      {{128, 64, 24}, {32, 24, 12}, {24, 12, 8}, {24, 12, 12}}};           // G = 128
+inline long long sorted_min_groups(int q, int G, int t_max) {
+    return 1024LL * kSortedMinK[G == 128 ? 2 : G == 64 ? 1 : 0][q - 1][t_max == 1 ? 0 : t_max < 5 ? 1 : 2];
+}
 
 __device__ __forceinline__ long long warp_sum_ll(long long v) {
 #pragma unroll
@@ -621,7 +627,7 @@ template <int Q, int G>
 int launch_fit_qg(const __half* W, int N, int K, int t_max, uint8_t* planes, __half* scales, __half* offsets, double* trace,
                   cudaStream_t stream) {
     const long long n_groups = (long long)N * (K / G);
-    if (trace == nullptr && n_groups >= (Q <= 2 ? 1 : 2) * kSortedMinGroups) {
+    if (trace == nullptr && n_groups >= sorted_min_groups(Q, G, t_max)) {
         constexpr int kSmem = kSortWarps * 32 * sorted_record(G);
         static bool configured[64] = {};
         int dev = 0;

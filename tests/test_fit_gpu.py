@@ -11,7 +11,7 @@ from tests.gpu_util import gemm_f32, to_dev
 
 pytestmark = pytest.mark.gpu
 
-SORTED_MIN_GROUPS = 16384        # from this many groups on elutq_hlq_fit sorts the groups for every q (without a trace)
+SORTED_MIN_GROUPS = 24576        # from this many groups on elutq_hlq_fit sorts the groups for every q and G at ten rounds (without a trace)
 
 
 def _fit_gpu(W, q, G, t_max=10, trace=False):
@@ -116,3 +116,16 @@ def test_fit_of_sorted_groups_matches_oracle_bit_for_bit(q, G, N, K, shift):
         rows = slice(c * N, (c + 1) * N)
         assert np.array_equal(p[:, rows], p_ref)
         assert _same_bits(s[rows], s_ref) and _same_bits(z[rows], z_ref)
+
+
+# N rows of 1024 weights: the first number of groups that is sorted
+@pytest.mark.parametrize("q,G,N,t_max", [(1, 64, 2048, 1), (2, 64, 768, 2), (3, 128, 1536, 2), (4, 32, 384, 1), (2, 128, 4096, 1), (2, 128, 1536, 7)])
+def test_fit_on_both_sides_of_the_sorted_form_s_lower_end(q, G, N, t_max):
+    """The same bits as with a trace, which takes the direct form at any size."""
+    W = workloads.dense_weights(42, f"fit-ends{q}{G}", N, 1024)
+    Wd = to_dev(W.view(np.int16)).view(torch.float16)
+    for rows in (N - 1, N):
+        a = elutq.elutq_hlq_fit(Wd[:rows], q, G, t_max)
+        b = elutq.elutq_hlq_fit(Wd[:rows], q, G, t_max, trace=True)
+        for x, y in zip(a[:3], b[:3]):
+            assert torch.equal(x.view(torch.uint8), y.view(torch.uint8))
