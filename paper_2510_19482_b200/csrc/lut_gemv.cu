@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(kThreads, 1) lut_gemv_kernel(const GemmArgs a)
     }
     if constexpr (TICKETS) {
         // One launch instead of two: 2 us less of host time per call (of 6.8), and on the GPU, in a graph of calls, 4096 x 4096
-        // at q = 2/3/4 4.5 -> 4.7, 5.1 -> 4.9, 5.8 -> 5.5 us.
+        // at q = 2/3/4 4.6 -> 4.7, 5.1 -> 4.9, 5.8 -> 5.5 us.
         uint32_t* last_box = reinterpret_cast<uint32_t*>(smem + kTableBytes + 64);
         __syncthreads();
         if (tid == 0) {
@@ -405,6 +405,14 @@ int launch_one(const GemmArgs& a, int num_sms, cudaStream_t stream) {
         // kernel, in which every SM takes part (28672 x 4096, q = 2, two rows a thread: 12.8 us, finalize kernel 11.3).
         tickets = fast && a.tickets != nullptr && a.n_kc <= 32 && b.ranges <= kGemvTickets &&
                   (a.n_rb + b.ranges - 1) / b.ranges * kTileRows <= kThreads;
+        // In a graph the second launch costs no host time, and the finalize kernel, waiting beside the main one, is ahead where a range is done
+        // quickly or long (us in a graph, tickets and finalize kernel: 2048 x 2048, q = 2 / 4 4.3 / 4.8 and 3.9 / 4.4; 6144 x 4096, q = 1
+        // 5.0 and 4.6; 14336 x 4096, q = 3 10.3 and 9.8; but 4096 x 3072, q = 4 5.2 and 5.5, 1000 x 14336 5.5 and 6.4).  The bits are the same.
+        if (tickets && (a.n_kc == 4 || (Q == 1 && G == 128 && a.n_kc <= 16) || (a.n_kc <= 8 && (long long)a.n_rb * kTileRows > 768LL * b.ranges))) {
+            cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+            if (cudaStreamIsCapturing(stream, &capture) != cudaSuccess) (void)cudaGetLastError();
+            tickets = capture != cudaStreamCaptureStatusActive;
+        }
         if (tickets) kernel = lut_gemv_kernel<Q, G, MODE, true, true>;
         else if (fast) kernel = lut_gemv_kernel<Q, G, MODE, true, false>;
     }

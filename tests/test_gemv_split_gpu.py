@@ -37,3 +37,26 @@ def test_both_reductions_agree(q, G, N, K):
     y = gemm_f32(X, packed, N, K)
     ref = hlq.matmul(X, layer.planes, layer.scales, layer.offsets, G)
     assert np.all(np.abs(y - ref) <= K * 2.0 ** -24 * hlq.magnitude_bound(X, layer.scales, layer.offsets, G))
+
+
+@pytest.mark.parametrize("q,G,N,K", [(2, 128, 2048, 2048), (1, 128, 1000, 8192), (3, 64, 14336, 4096), (2, 128, 4096, 4096)])
+def test_calls_in_a_graph_give_the_same_bits(q, G, N, K):
+    layer = workloads.hlq_layer(63, f"split/graph/{q}/{G}/{N}/{K}", q, G, N, K)
+    X = synth.activations(63, f"split/graph/x/{K}", 1, K)
+    packed, x = pack_layer(layer), x_dev(X)
+    plain, replayed = (torch.empty((1, N), dtype=torch.float16, device="cuda") for _ in range(2))
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        elutq.elutq_lut_gemm(x, packed, plain, 1, N, K)
+        stream.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            for _ in range(3):
+                elutq.elutq_lut_gemm(x, packed, replayed, 1, N, K)
+        for _ in range(2):
+            graph.replay()
+        elutq.elutq_lut_gemm(x, packed, plain, 1, N, K)
+        stream.synchronize()
+    assert torch.equal(plain.view(torch.int16), replayed.view(torch.int16))
+    ref = hlq.matmul(X, layer.planes, layer.scales, layer.offsets, G)
+    assert hlq.rel_fro_error(plain.cpu().numpy(), ref) <= 1e-3
