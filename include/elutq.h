@@ -69,6 +69,9 @@ typedef enum elutq_status {
                                      variant flag).  Two rows stay on the batched look-up kernel: one pass, 17.3 us
                                      on 8B gate_up 28672 x 4096 at q = 2 against 25.6; from three rows on it needs a
                                      wider pass (M = 4: 26.2 / 25.9, 4096 x 4096 9.5 / 7.6, M = 8: 43.9 / 26.8)        */
+#define ELUTQ_TENSOR_MIN_M_NARROW ELUTQ_TENSOR_MIN_M   /* (kept for callers that ask for the smallest batch on the tensor cores at
+                                                          N <= ELUTQ_TENSOR_NARROW_N: the same for every N now)     */
+#define ELUTQ_TENSOR_NARROW_N 8192
 #define ELUTQ_FRAGMENT_MAX_M 8    /* G = 128: up to this many rows the bit-planes are contracted as they are (scales
                                      applied to fp32 sums, as exact as the look-up kernels); larger batches rebuild
                                      W_hat in fp16 tiles (8B gate_up / down at q = 2, us: M = 8 26.9 / 15.9 and
@@ -262,6 +265,15 @@ int elutq_lut_gemm_host(const void* X_host, const void* packed, void* Y_host,
  * look-up kernels; host-only, launches nothing.  (Above ELUTQ_FRAGMENT_MAX_M rows at G = 128 its results carry the fp16
  * rounding of W_hat.) */
 int elutq_takes_tensor_path(int M, int N, int K, int G, unsigned flags);
+
+/* The kernel that elutq_lut_gemm (and _f32, _ws, _host, _bias) runs a call of this shape on, on the current device: one of the
+ * ELUTQ_KERNEL_ values, or an ELUTQ_ERR_ code (negative).  Host-only, launches nothing. */
+#define ELUTQ_KERNEL_DECODE 0          /* M = 1: look-up tables                                                       */
+#define ELUTQ_KERNEL_LOOK_UP 1         /* batches on look-up tables                                                   */
+#define ELUTQ_KERNEL_FRAGMENT 2        /* bit-planes contracted as they are, scales on fp32 sums                      */
+#define ELUTQ_KERNEL_TENSOR_MEMORY 3   /* W_hat rebuilt in fp16, in tensor memory                                     */
+#define ELUTQ_KERNEL_SHARED_MEMORY 4   /* W_hat rebuilt in fp16, in shared memory                                     */
+int elutq_gemm_kernel(int M, int N, int K, int q, int G, unsigned flags);
 
 int elutq_lut_gemm_static(const void* X, const void* packed, void* Y, int M, int N, int K, void* stream);
 

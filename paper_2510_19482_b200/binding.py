@@ -20,6 +20,9 @@ FLAG_LUT_ONLY = 0x80
 FLAG_TABLE_F16 = 0x100
 FLAG_TABLE_I8 = 0x200
 
+# elutq_gemm_kernel
+KERNEL_DECODE, KERNEL_LOOK_UP, KERNEL_FRAGMENT, KERNEL_TENSOR_MEMORY, KERNEL_SHARED_MEMORY = range(5)
+
 
 class GemvCall(ctypes.Structure):
     """elutq_gemv_call: one M = 1 call of a chain."""
@@ -55,6 +58,7 @@ _SIGNATURES = {
     "elutq_lut_gemm_host": (c_int, [c_void_p, c_void_p, c_void_p, c_int, c_int, c_int, c_void_p]),
     "elutq_lut_gemm_static": (c_int, [c_void_p, c_void_p, c_void_p, c_int, c_int, c_int, c_void_p]),
     "elutq_takes_tensor_path": (c_int, [c_int, c_int, c_int, c_int, c_uint]),
+    "elutq_gemm_kernel": (c_int, [c_int, c_int, c_int, c_int, c_int, c_uint]),
     "elutq_hlq_fit": (c_int, [c_void_p, c_int, c_int, c_int, c_int, c_int, c_void_p, c_void_p, c_void_p, c_void_p, c_void_p]),
     "elutq_chain_plan_bytes": (c_int, [ctypes.POINTER(GemvCall), c_int, ctypes.POINTER(c_size_t)]),
     "elutq_chain_plan": (c_int, [ctypes.POINTER(GemvCall), c_int, c_void_p, c_size_t, c_void_p]),
@@ -201,6 +205,14 @@ def elutq_lut_gemm_host(X_host, packed, Y_host, M: int, N: int, K: int, stream=N
 def elutq_takes_tensor_path(M: int, N: int, K: int, G: int = 128, flags: int = 0) -> bool:
     """True when elutq_lut_gemm runs this shape on the tensor-core path (host-only)."""
     return bool(lib().elutq_takes_tensor_path(M, N, K, G, flags))
+
+
+def elutq_gemm_kernel(M: int, N: int, K: int, q: int, G: int = 128, flags: int = 0) -> int:
+    """The kernel a call of this shape runs on (KERNEL_...); host-only."""
+    kernel = lib().elutq_gemm_kernel(M, N, K, q, G, flags)
+    if kernel < 0:
+        _check(kernel, "elutq_gemm_kernel")
+    return kernel
 
 
 def elutq_lut_gemm_static(X, packed, Y, M: int, N: int, K: int, stream=None) -> None:

@@ -198,6 +198,14 @@ bool takes_tensor_path(int M, int G, unsigned flags) {
     return M >= ELUTQ_TENSOR_MIN_M && G != 32 && !(flags & lut_variants);
 }
 
+// The kernel of a call (ELUTQ_KERNEL_...).
+int kernel_of(int M, int N, int K, int q, int G, unsigned flags, int sms) {
+    if (M == 1) return ELUTQ_KERNEL_DECODE;
+    if (!takes_tensor_path(M, G, flags)) return ELUTQ_KERNEL_LOOK_UP;
+    if (G != 128 || M <= ELUTQ_FRAGMENT_MAX_M) return ELUTQ_KERNEL_FRAGMENT;
+    return rebuilds_in_shared_memory(M, N, K, q, sms) ? ELUTQ_KERNEL_SHARED_MEMORY : ELUTQ_KERNEL_TENSOR_MEMORY;
+}
+
 int run_gemm(const void* X, const void* packed, void* Y, int M, int N, int K, unsigned flags,
              void* workspace, size_t workspace_bytes, bool own_workspace, void* stream) {
     if (!X || !packed || !Y) return ELUTQ_ERR_INVALID_ARG;
@@ -243,13 +251,16 @@ int run_gemm(const void* X, const void* packed, void* Y, int M, int N, int K, un
     a.tickets = a.counters + 64;
     a.items_q = 0; a.items_r = 0; a.active_warps = 0; a.ranges = 0; a.rb_q = 0; a.rb_r = 0; a.cpc = 1; a.cluster_reduce = 0;
     const int sms = num_sms();
-    int ce;
-    if (M == 1) ce = launch_lut_gemv(a, m.q, m.G, sms, (cudaStream_t)stream);
-    else if (!takes_tensor_path(M, m.G, flags)) ce = launch_lut_gemm(a, m.q, m.G, sms, (cudaStream_t)stream);
-    else if (m.G == 128 && M > ELUTQ_FRAGMENT_MAX_M) {
-        ce = rebuilds_in_shared_memory(M, N, K, m.q, sms) ? (int)cudaErrorNotSupported : launch_hlq_tmem(a, m.q, sms, (cudaStream_t)stream);
-        if (ce == (int)cudaErrorNotSupported) ce = launch_hlq_mma(a, m.q, m.G, sms, (cudaStream_t)stream);
-    } else ce = launch_hlq_frag(a, m.q, m.G, sms, (cudaStream_t)stream);
+    int ce = (int)cudaErrorNotSupported;
+    switch (kernel_of(M, N, K, m.q, m.G, flags, sms)) {
+        case ELUTQ_KERNEL_DECODE: ce = launch_lut_gemv(a, m.q, m.G, sms, (cudaStream_t)stream); break;
+        case ELUTQ_KERNEL_LOOK_UP: ce = launch_lut_gemm(a, m.q, m.G, sms, (cudaStream_t)stream); break;
+        case ELUTQ_KERNEL_FRAGMENT: ce = launch_hlq_frag(a, m.q, m.G, sms, (cudaStream_t)stream); break;
+        case ELUTQ_KERNEL_TENSOR_MEMORY: ce = launch_hlq_tmem(a, m.q, sms, (cudaStream_t)stream);
+            if (ce != (int)cudaErrorNotSupported) break;
+            [[fallthrough]];
+        default: ce = launch_hlq_mma(a, m.q, m.G, sms, (cudaStream_t)stream);
+    }
     if (ce == (int)cudaErrorNotSupported) return ELUTQ_ERR_UNSUPPORTED;
     if (ce != 0) return cuda_fail((cudaError_t)ce);
     return ELUTQ_OK;
@@ -469,6 +480,12 @@ int elutq_takes_tensor_path(int M, int N, int K, int G, unsigned flags) {
     (void)N;
     (void)K;
     return takes_tensor_path(M, G, flags) ? 1 : 0;
+}
+
+int elutq_gemm_kernel(int M, int N, int K, int q, int G, unsigned flags) {
+    if (M <= 0 || N <= 0 || K <= 0) return ELUTQ_ERR_INVALID_ARG;
+    const int st = check_shape(q, G, N, K);
+    return st != ELUTQ_OK ? st : kernel_of(M, N, K, q, G, flags, num_sms());
 }
 
 int elutq_reserve(int M, int N, int K, void* stream) {

@@ -42,13 +42,19 @@ def gemm_f16(X: np.ndarray, packed, N: int, K: int) -> np.ndarray:
     return Y.cpu().numpy()
 
 
+def rebuilds_weights(M: int, N: int, K: int, q: int, G: int) -> bool:
+    """Whether the default path of a call rounds W_hat to fp16 (the other kernels, also those on the tensor cores, do not)."""
+    return elutq.elutq_gemm_kernel(M, N, K, q, G) in (elutq.KERNEL_TENSOR_MEMORY, elutq.KERNEL_SHARED_MEMORY)
+
+
 def assert_elementwise(y, ref, A, q: int, K: int, tensor_path: bool, out_f16: bool, where="") -> None:
     """Element-wise bound over ALL outputs (a norm can hide one wrong element in a large result).
 
     A = oracle.hlq.magnitude_bound(X, scales, offsets, G) bounds |X| |W_hat|^T and every intermediate of the +-1
     form.  Roundings of the paths, each at most its unit roundoff times A (worst case, all errors aligned):
       look-up kernels   fp32 table entries and fp32 accumulation over K terms      K * 2^-24 * A
-      tensor-core path  W_hat rebuilt in fp16: z^ rounded once, one rounding per plane add   (q + 1) * 2^-11 * A
+      fragment kernel   exact products, one truncation by 2^-23 per 16 terms and the fp32 sums: less than that
+      rebuilt weights   W_hat rebuilt in fp16: z^ rounded once, one rounding per plane add   (q + 1) * 2^-11 * A
                         then fp32 accumulation in tensor memory                    K * 2^-23 * A
       fp16 output       one more rounding of the result                            2^-11 * |y|
     """

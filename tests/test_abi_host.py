@@ -71,6 +71,10 @@ def test_pointer_validation_happens_before_any_launch():
     assert L.elutq_hlq_fit(17, 2, 128, 16, 512, 10, 16, 16, 16, None, None) == -3         # W not 2-byte aligned
     assert L.elutq_hlq_fit(16, 2, 128, 16, 512, 10, 16, 16, 16, 4, None) == -3            # trace not 8-byte aligned
     assert L.elutq_workspace_init(None, 16, None) == -1
+    assert L.elutq_gemm_kernel(0, 16, 512, 2, 128, 0) == -1 and L.elutq_gemm_kernel(4, 16, 512, 5, 128, 0) == -2
+    assert [elutq.elutq_gemm_kernel(M, 4096, 4096, 2) for M in (1, 2, 3, 8, 9, 4096)] == [0, 1, 2, 2, 3, 4]
+    assert elutq.elutq_gemm_kernel(64, 4096, 4096, 2, 64) == 2 and elutq.elutq_gemm_kernel(64, 4096, 4096, 2, 32) == 1
+    assert elutq.elutq_gemm_kernel(64, 4096, 4096, 2, 128, elutq.FLAG_LUT_ONLY) == 1
     assert L.elutq_forget(None) == -1
     assert elutq.elutq_launch_count() == before
     assert elutq.elutq_status_string(-4) == "buffer too small"

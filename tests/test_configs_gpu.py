@@ -16,7 +16,7 @@ from workloads import synth
 
 pytestmark = pytest.mark.gpu
 
-from gpu_util import assert_elementwise, gemm_f16, pack_layer, x_dev  # noqa: E402
+from gpu_util import assert_elementwise, gemm_f16, pack_layer, rebuilds_weights, x_dev  # noqa: E402
 
 TOL_F16 = 1e-3
 
@@ -79,7 +79,7 @@ def test_config2_every_call_of_the_small_batch_sweep(name, q):
         assert np.all(np.isfinite(y))
         assert hlq.rel_fro_error(y[:, rows], ref) <= TOL_F16, call
         A = hlq.magnitude_bound(X, layer.scales[rows], layer.offsets[rows], call.G)
-        assert_elementwise(y[:, rows], ref, A, call.q, call.K, elutq.elutq_takes_tensor_path(call.M, call.N, call.K, call.G), True,
+        assert_elementwise(y[:, rows], ref, A, call.q, call.K, rebuilds_weights(call.M, call.N, call.K, call.q, call.G), True,
                            f"config 2 {name} q{q} M{call.M}")
     assert elutq.elutq_device_status() == 0
 

@@ -28,6 +28,7 @@ CASES = [(2, 128, 128, 512, 3), (1, 128, 17, 128, 8), (3, 128, 129, 640, 7), (4,
 
 @pytest.mark.parametrize("q,G,N,K,M", CASES)
 def test_fragment_kernel_matches_oracle(q, G, N, K, M):
+    assert elutq.elutq_gemm_kernel(M, N, K, q, G) == elutq.KERNEL_FRAGMENT
     layer = workloads.hlq_layer(60, f"frag/{q}/{G}/{N}/{K}", q, G, N, K, signed_scales=(q % 2 == 1))
     X = synth.activations(60, f"frag/x/{M}/{K}", M, K, outliers=True)
     X[0] *= np.float16(2.0 ** -12)                       # rows of very different size: each has its own exponent
@@ -112,7 +113,7 @@ def test_activations_that_are_not_finite(G, M, values):
 
 @pytest.mark.parametrize("q,N,K,M", [(1, 129, 64, 257), (2, 1000, 1024, 33), (2, 2048, 4096, 130), (3, 4000, 2880, 57), (4, 300, 4160, 100)])
 def test_batch_blocks_of_one_launch(q, N, K, M):
-    # blocks of 8, 16 and 32 rows with a remainder, several to a row tile, output tiles shared by CTAs; one launch, no call slower for its rows
+    # blocks of 8 and 16 rows with a remainder, several to a row tile, output tiles shared by CTAs; one launch, no call slower for its rows
     layer = workloads.hlq_layer(67, f"frag/blocks/{q}/{N}/{K}", q, 64, N, K)
     X = synth.activations(67, f"frag/blocks/x/{M}/{K}", M, K, outliers=True)
     packed = pack_layer(layer)

@@ -11,7 +11,7 @@ from workloads import synth
 
 pytestmark = pytest.mark.gpu
 
-from gpu_util import assert_elementwise, gemm_f16, gemm_f32, pack_layer, x_dev  # noqa: E402
+from gpu_util import assert_elementwise, gemm_f16, gemm_f32, pack_layer, rebuilds_weights, x_dev  # noqa: E402
 
 TOL_F32 = 5e-6
 TOL_F16 = 1e-3
@@ -37,9 +37,8 @@ def test_batched_gemm_matches_oracle(q, G, N, K, M):
     assert_elementwise(y32, ref, A, q, K, False, False, "batched look-up kernel, fp32 out")
     y16 = gemm_f16(X, packed, N, K)                                # default path
     assert hlq.rel_fro_error(y16, ref) <= TOL_F16
-    tensor_path = elutq.elutq_takes_tensor_path(M, N, K, G)
-    assert_elementwise(y16, ref, A, q, K, tensor_path, True, "default path, fp16 out")
-    if not tensor_path:                                  # on the look-up kernels by default: the same kernels
+    assert_elementwise(y16, ref, A, q, K, rebuilds_weights(M, N, K, q, G), True, "default path, fp16 out")
+    if elutq.elutq_gemm_kernel(M, N, K, q, G) == elutq.KERNEL_LOOK_UP:                                  # on the look-up kernels by default: the same kernels
         assert np.array_equal(y16.view(np.uint16), y32.astype(np.float16).view(np.uint16))
 
 
@@ -48,7 +47,7 @@ def test_batched_rows_equal_single_row_calls_up_to_rounding():
     layer = workloads.hlq_layer(21, "gemm/rows", q, G, N, K)
     X = synth.activations(21, "gemm/rows/x", M, K)
     packed = pack_layer(layer)
-    yb = gemm_f32(X, packed, N, K, elutq.FLAG_LUT_ONLY)            # (a narrow layer at M = 6 would take the tensor cores by default)
+    yb = gemm_f32(X, packed, N, K, elutq.FLAG_LUT_ONLY)            # (the tensor cores by default)
     for m in range(M):
         y1 = gemm_f32(X[m:m + 1], packed, N, K)
         np.testing.assert_allclose(yb[m], y1[0], rtol=0, atol=4e-6 * np.abs(y1).max())
@@ -83,7 +82,7 @@ def test_prefill_sized_batch_on_a_layer_sized_matrix():
     packed = pack_layer(layer)
     ref = hlq.matmul(X, layer.planes, layer.scales, layer.offsets, G)
     A = hlq.magnitude_bound(X, layer.scales, layer.offsets, G)
-    y16 = gemm_f16(X, packed, N, K)                                  # default path for M >= 9: tensor cores
+    y16 = gemm_f16(X, packed, N, K)                                  # default path: weights rebuilt in fp16
     assert hlq.rel_fro_error(y16, ref) <= TOL_F16
     assert_elementwise(y16, ref, A, q, K, True, True, "tensor-core path, fp16 out")
     y32 = gemm_f32(X, packed, N, K, elutq.FLAG_LUT_ONLY)           # look-up-table kernels

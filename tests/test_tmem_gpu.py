@@ -25,11 +25,12 @@ G, TOL = 128, 1e-3
 # 200 -> 2 x 112); whole tiles per CTA, shared tiles of two or three parts, of many parts, clusters of two CTAs and more (with K steps and
 # tokens that they do not divide evenly, and N no multiple of the stores' four), whole rounds with the rest by clusters
 CASES = [(2, 4621, 128, 9), (1, 4480, 1152, 128), (3, 4600, 640, 200), (4, 5000, 2944, 100), (4, 12800, 2048, 384), (2, 38000, 256, 33),
-         (3, 10240, 1024, 130), (2, 11776, 7680, 16), (2, 16000, 1024, 100), (2, 3001, 4096, 20), (3, 1100, 1152, 90), (1, 300, 256, 33), (2, 13000, 2048, 384)]
+         (3, 10240, 1024, 130), (2, 11776, 7680, 16), (2, 16000, 1024, 100), (2, 3001, 4096, 20), (3, 1100, 1152, 90), (1, 300, 256, 33), (2, 13000, 2560, 384)]
 
 
 @pytest.mark.parametrize("q,N,K,M", CASES)
 def test_tensor_memory_kernel_matches_oracle(q, N, K, M):
+    assert elutq.elutq_gemm_kernel(M, N, K, q, G) == elutq.KERNEL_TENSOR_MEMORY
     layer = workloads.hlq_layer(70, f"tmem/{q}/{N}/{K}", q, G, N, K, signed_scales=(q == 3))
     X = synth.activations(70, f"tmem/x/{M}/{K}", M, K, outliers=True)
     packed = pack_layer(layer)
@@ -51,6 +52,7 @@ def test_tensor_memory_kernel_matches_oracle(q, N, K, M):
 @pytest.mark.parametrize("q", [1, 2, 4])
 def test_scales_of_one_and_more(q):
     N, K, M = 4700, 256, 40
+    assert elutq.elutq_gemm_kernel(M, N, K, q, G) == elutq.KERNEL_TENSOR_MEMORY
     layer = workloads.hlq_layer(71, f"tmem/scales/{q}", q, G, N, K)
     s = layer.scales.astype(np.float32)
     s[1::4] *= 64.0                                      # around 1: only some groups of a row
@@ -68,6 +70,7 @@ def test_scales_of_one_and_more(q):
 
 def test_a_wait_that_runs_out_is_reported():
     q, N, K, M = 2, 8192, 2048, 64
+    assert elutq.elutq_gemm_kernel(M, N, K, q, G) == elutq.KERNEL_TENSOR_MEMORY
     layer = workloads.hlq_layer(72, "tmem/expiry", q, G, N, K)
     X = synth.activations(72, "tmem/expiry/x", M, K)
     packed = pack_layer(layer)
@@ -85,6 +88,7 @@ def test_a_wait_that_runs_out_is_reported():
 def test_waits_that_run_out_behind_loaders_that_are_done(q, N, K, M):
     # Clusters and whole tiles with so few steps of K that the loaders have requested everything when the other warps give up: they
     # still wait for their copies.  The calls that follow at once get the shared memory.
+    assert elutq.elutq_gemm_kernel(M, N, K, q, G) == elutq.KERNEL_TENSOR_MEMORY
     layer = workloads.hlq_layer(73, f"tmem/drain/{N}", q, G, N, K)
     X = synth.activations(73, f"tmem/drain/x/{M}/{K}", M, K)
     packed = pack_layer(layer)
