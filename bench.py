@@ -399,7 +399,7 @@ def _secondary(torch, elutq, name, stream, l2_bytes, hbm_peak, tensor_peak, devi
         layers.append(dict(call=c, packed=cache[key], X=X, Y=torch.empty((c.M, c.N), dtype=torch.float16, device="cuda")))
     step_bytes = _bytes_of(calls)
     all_m1 = all(c.M == 1 for c in calls)
-    tensor = all(c.M >= 9 and c.G == 128 for c in calls)           # (every call a tensor-core contraction at any N)
+    tensor = all(c.M >= 9 and c.G == 128 for c in calls)           # (above ELUTQ_FRAGMENT_MAX_M: every call a dense contraction)
     # distinct blobs are shared between the calls of a step here, so rotate whole copies only while they are small
     distinct = sum(t.numel() for t in cache.values())
     out = {"workload": WORKLOAD_NAMES[name], "calls_per_step": len(calls), "algorithmic_bytes_per_step": step_bytes,
@@ -761,7 +761,7 @@ def run_cuda(args) -> None:
                 "peak_source": peak_src,
                 "traffic": traffic.get("dram_bytes_per_step") if traffic else None,
                 "traffic_note": traffic.get("note") if traffic else None}
-    tensor_path = all(c.M >= 9 and c.G == 128 for c in calls) and not (args.flags & 0x3F0)   # ELUTQ_TENSOR_MIN_M
+    tensor_path = all(c.M >= 9 and c.G == 128 for c in calls) and not (args.flags & 0x3F0)   # > ELUTQ_FRAGMENT_MAX_M
     if tensor_path:
         # every call of the step is a dense contraction on the tensor cores: report FLOP/s against the measured
         # GEMM peak (the sustained figure, since the kernels are timed inside a long step)

@@ -1,5 +1,5 @@
-// Batches of more than ELUTQ_FRAGMENT_MAX_M rows at G = 128: dequantise-and-contract on the 5th-generation tensor cores, the
-// rebuilt weights as the A operand in TENSOR MEMORY.
+// Batches of more than ELUTQ_FRAGMENT_MAX_M rows at G = 128, but for those that hlq_mma.cu takes (rebuilds_in_shared_memory in
+// api.cu): dequantise-and-contract on the 5th-generation tensor cores, the rebuilt weights as the A operand in TENSOR MEMORY.
 //
 // A rebuilt fp16 weight never passes through shared memory: a producer lane owns one weight row (= one TMEM lane), rebuilds
 // 128 k of it in registers and stores them to its lane; the activations are the B operand, so the MMA's N is the batch and a
@@ -23,7 +23,7 @@
 //
 //   bound      the producers' integer logic pipe (q = 4: 320 of a slot's 470 operations are the dequantisation itself, 65 to 75 % of
 //              the pipe's cycles); from 96 tokens also the activations' way from the L2.  Against weights rebuilt in shared memory with one
-//              barrier per step, us: 57344 x 8192, q = 4, M = 64 277 -> 127; 28672 x 4096, q = 2, M = 32 / 128 / 384
+//              barrier per step, us: 57344 x 8192, q = 4, M = 64 277 -> 145; 28672 x 4096, q = 2, M = 32 / 128 / 384
 //              49 / 51 / 110 -> 25 / 33 / 95; 4096 x 14336, q = 3, M = 64 34 -> 24; 4096 x 4096, q = 2, M = 256 30 -> 18.
 //
 // Every wait is bounded; a thread whose wait runs out raises the status word and a CTA-wide flag that ends the other
@@ -695,7 +695,7 @@ EncodeFn encode_fn() {
 // c when the other SMs do not fight for the L2, 10 % more when all do, the parts 5 (a second kernel 8) and their fp32 bytes at 2.2 TB/s, a cluster's
 // sums 1 and 0.035 a token.
 // (Measured, equal shares against whole tiles: 28672 x 4096, q = 2, 112 tiles, M = 32: 27 and 25, M = 128: 45 and 32; 57344 x 8192, q = 4,
-// 224 tiles, M = 64: 127 and 157; 4096 x 14336, q = 3, M = 768, 96 tiles: 99 and 117, M = 1024, 128 tiles: 127 and 120.  Equal
+// 224 tiles, M = 64, the same layer again and again: 127 and 157; 4096 x 14336, q = 3, M = 768, 96 tiles: 99 and 117, M = 1024, 128 tiles: 127 and 120.  Equal
 // shares against clusters: 4096 x 4096, q = 2, M = 16 / 64 / 384 11.0 / 14.4 / 31 and 9.3 / 11.3 / 21; 6144 x 4096, q = 4, M = 128 28.5 and
 // 19.8; 4096 x 14336, q = 3, M = 64 28.2 and 24.3.)
 double step_us(int q, int mp) { return 0.25 + 0.2 * q + 0.0016 * mp; }
