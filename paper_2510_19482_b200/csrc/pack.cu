@@ -1,7 +1,6 @@
 // Offline packing of HLQ bit-planes, scales and offsets into the device layout, and its inverse.
 //
-// Packing runs in gather form: every thread owns one 16-byte plane vector (or one 32-bit
-// parameter word) of the output and collects the logical elements that belong there.
+// Packing: a warp owns 32 plane vectors of 16 bytes of the output, a thread a 32-bit parameter word.
 // Unpacking runs per logical element.  Neither is on the per-token path.
 #include "common.cuh"
 
@@ -31,75 +30,100 @@ __device__ __forceinline__ uint32_t nonzero_bytes(uint32_t x) {
     return (m * 0x10204080u) >> 28;
 }
 
-// One thread per plane vector: (tile, vec = u*q + j, lane) -> 16 bytes, byte i = column tau(l,i).  The lanes' 128 input bytes each
-// are whole lines, so sixteen 8-byte loads in flight per thread read every byte from memory once.
-__device__ __forceinline__ void pack_plane_vector(const uint8_t* __restrict__ planes, uint8_t* __restrict__ tiles, const Geo& g, long long idx) {
-    const int lane = (int)(idx & 31);
-    const int vec = (int)((idx >> 5) % (2 * g.q));
-    const long long tile = idx / (64LL * g.q);
-    const int kc = (int)(tile / g.n_rb), rb = (int)(tile % g.n_rb);
-    const int u = vec / g.q, j = vec % g.q;
-    const int h = lane >> 4, l = lane & 15;
-    const int n = rb * kTileRows + l;
-    const int sigma = h + 2 * u;
-    uint32_t out[4] = {0u, 0u, 0u, 0u};
-    if (n < g.N) {
-        const uint8_t* row = planes + ((size_t)j * g.N + n) * g.K;
-        uint2 x[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const int k0 = kc * kChunkK + (16 * sigma + tau_of(l, i, g.w, g.nsg)) * 8;
-            x[i] = k0 < g.K ? __ldg(reinterpret_cast<const uint2*>(row + k0)) : make_uint2(0u, 0u);
-        }
-#pragma unroll
-        for (int i = 0; i < 16; ++i) out[i >> 2] |= (nonzero_bytes(x[i].x) | nonzero_bytes(x[i].y) << 4) << (8 * (i & 3));
+// n / d for 0 <= n < 2^31 by one multiplication (a division by a runtime value costs some 20 instructions, a 64-bit one 100).
+struct Div {
+    int d;
+    unsigned long long m;       // m d = 2^64 + e with 0 <= e < d, so n m / 2^64 exceeds n / d by less than n / 2^64 (0 stands for d = 1)
+    __host__ void set(int d_) {
+        d = d_;
+        m = d_ == 1 ? 0ull : ~0ull / (unsigned)d_ + 1ull;
     }
-    uint4* dst = reinterpret_cast<uint4*>(tiles + (size_t)tile * g.tile_bytes) + vec * 32 + lane;
-    *dst = make_uint4(out[0], out[1], out[2], out[3]);
+    __device__ __forceinline__ int of(int n) const { return m == 0ull ? n : (int)__umul64hi((unsigned long long)n, m); }
+};
+
+constexpr int kPackWarps = 8;
+
+// One warp per 32 plane vectors of a tile: (tile, vec = u*q + j), 16 rows x 2 super-groups of 128 input bytes.  A load covers whole
+// lines (four rows' 128 bytes), the bits go through shared memory to their places in the rows' rotated order, and the lanes store
+// 16 bytes each.  (A thread per vector with sixteen loads of 8 bytes 128 bytes apart, and the order's divisions at run time: 4096 x 4096,
+// q = 2 22 us.)
+template <int Q, int G>
+__device__ __forceinline__ void pack_plane_vectors(const uint8_t* __restrict__ planes, uint8_t* __restrict__ tiles, const Geo& g, int tile, int kc, int vec,
+                                                   int lane, bool wide, uint8_t* place) {
+    constexpr int W = G / 8, NSG = 128 / G;
+    const int rb = tile - kc * g.n_rb, u = vec / Q, j = vec - u * Q;
+    const int col = 2 * (lane & 7);                               // the lane's 16 input bytes: byte columns col, col + 1 of a super-group
+    uint4 x[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int seg = 4 * i + (lane >> 3), n = rb * kTileRows + (seg & 15), k0 = kc * kChunkK + ((seg >> 4) + 2 * u) * 128 + col * 8;
+        const uint8_t* src = planes + ((size_t)j * g.N + n) * g.K + k0;
+        x[i] = make_uint4(0u, 0u, 0u, 0u);
+        if (n < g.N && k0 < g.K) {
+            if (wide) {
+                x[i] = __ldg(reinterpret_cast<const uint4*>(src));
+            } else {
+                const uint2 lo = __ldg(reinterpret_cast<const uint2*>(src)), hi = __ldg(reinterpret_cast<const uint2*>(src) + 1);
+                x[i] = make_uint4(lo.x, lo.y, hi.x, hi.y);
+            }
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int seg = 4 * i + (lane >> 3), l = seg & 15;
+        const uint32_t bits[2] = {nonzero_bytes(x[i].x) | nonzero_bytes(x[i].y) << 4, nonzero_bytes(x[i].z) | nonzero_bytes(x[i].w) << 4};
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {                             // the inverse of tau(l, i)
+            const int c = col + e, at = ((c / W - l / W) & (NSG - 1)) * W + ((c - l) & (W - 1));
+            place[seg * 16 + at] = (uint8_t)bits[e];
+        }
+    }
+    __syncwarp();
+    reinterpret_cast<uint4*>(tiles + (size_t)tile * g.tile_bytes)[vec * 32 + lane] = reinterpret_cast<const uint4*>(place)[lane];
 }
 
 // One thread per parameter word: (tile, word, lane) -> two fp16 values of the lane's record.
+template <int Q, int G>
 __device__ __forceinline__ void pack_param_word(const uint16_t* __restrict__ scales, const uint16_t* __restrict__ offsets,
-                                                uint8_t* __restrict__ tiles, const Geo& g, long long idx) {
-    const int words = g.gl * (g.q + 1) / 2;
-    const int lane = (int)(idx & 31);
-    const int word = (int)((idx >> 5) % words);
-    const long long tile = idx / (32LL * words);
-    const int kc = (int)(tile / g.n_rb), rb = (int)(tile % g.n_rb);
+                                                uint8_t* __restrict__ tiles, const Geo& g, int tile, int kc, int word, int lane) {
+    constexpr int W = G / 8, NSG = 128 / G;
+    const int rb = tile - kc * g.n_rb;
     const int h = lane >> 4, l = lane & 15;
     const int n = rb * kTileRows + l;
-    const int Gn = g.K / g.G;
-    const int a = l / g.w;
+    const int Gn = g.K / G;
+    const int a = l / W;
     uint32_t packed = 0;
+#pragma unroll
     for (int half = 0; half < 2; ++half) {
         const int e = 2 * word + half;
-        const int comp = e % (g.q + 1);
-        const int uv = e / (g.q + 1);
-        const int u = uv / g.nsg, v = uv % g.nsg;
-        const int gamma = g.nsg * (h + 2 * u) + (a + v) % g.nsg;    // group inside the chunk
-        const int gi = kc * (kChunkK / g.G) + gamma;
+        const int uv = e / (Q + 1), comp = e - uv * (Q + 1);
+        const int u = uv / NSG, v = uv % NSG;
+        const int gamma = NSG * (h + 2 * u) + (a + v) % NSG;      // group inside the chunk
+        const int gi = kc * (kChunkK / G) + gamma;
         uint32_t bits = 0;
-        if (n < g.N && gi < Gn)
-            bits = comp < g.q ? scales[((size_t)n * Gn + gi) * g.q + comp] : offsets[(size_t)n * Gn + gi];
+        if (n < g.N && gi < Gn) bits = comp < Q ? scales[((size_t)n * Gn + gi) * Q + comp] : offsets[(size_t)n * Gn + gi];
         packed |= bits << (16 * half);
     }
-    uint32_t* dst = reinterpret_cast<uint32_t*>(tiles + (size_t)tile * g.tile_bytes + g.plane_bytes) + word * 32 + lane;
-    *dst = packed;
+    reinterpret_cast<uint32_t*>(tiles + (size_t)tile * g.tile_bytes + g.plane_bytes)[word * 32 + lane] = packed;
 }
 
 // The whole blob in one launch: plane vectors, parameter words (blocks from plane_blocks on), the header.
-__global__ void __launch_bounds__(256) pack_kernel(const uint8_t* __restrict__ planes, const uint16_t* __restrict__ scales,
-                                                   const uint16_t* __restrict__ offsets, uint8_t* __restrict__ packed, const Geo g,
-                                                   const unsigned plane_blocks) {
+template <int Q, int G>
+__global__ void __launch_bounds__(32 * kPackWarps) pack_kernel(const uint8_t* __restrict__ planes, const uint16_t* __restrict__ scales,
+                                                               const uint16_t* __restrict__ offsets, uint8_t* __restrict__ packed, const Geo g,
+                                                               const int plane_blocks, const Div by_rows, const bool wide) {
+    constexpr int kVectors = 2 * Q, kWords = 2 * (128 / G) * (Q + 1) / 2;        // warps' works of a tile
+    __shared__ __align__(16) uint8_t place[kPackWarps][512];
     uint8_t* tiles = packed + ELUTQ_HEADER_BYTES;
-    if (blockIdx.x < plane_blocks) {
-        const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-        if (idx < (long long)g.n_kc * g.n_rb * 2 * g.q * 32) pack_plane_vector(planes, tiles, g, idx);
-    } else {
-        const long long idx = (long long)(blockIdx.x - plane_blocks) * blockDim.x + threadIdx.x;
-        if (idx < (long long)g.n_kc * g.n_rb * (g.gl * (g.q + 1) / 2) * 32) pack_param_word(scales, offsets, tiles, g, idx);
-        if (idx < ELUTQ_HEADER_BYTES / 4) reinterpret_cast<uint32_t*>(packed)[idx] = header_word(g, (int)idx);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const bool params = (int)blockIdx.x >= plane_blocks;
+    const int i = ((int)blockIdx.x - (params ? plane_blocks : 0)) * kPackWarps + warp, per = params ? kWords : kVectors;
+    const int tile = i / per, kc = by_rows.of(tile);
+    if (tile < g.n_kc * g.n_rb) {
+        if (params) pack_param_word<Q, G>(scales, offsets, tiles, g, tile, kc, i - tile * per, lane);
+        else pack_plane_vectors<Q, G>(planes, tiles, g, tile, kc, i - tile * per, lane, wide, place[warp]);
     }
+    if (params && i == 0 && lane < ELUTQ_HEADER_BYTES / 4) reinterpret_cast<uint32_t*>(packed)[lane] = header_word(g, lane);
 }
 
 // One thread per (plane j, row n, byte-column cg): expands a packed byte to 8 uint8 {0,1}.
@@ -158,15 +182,42 @@ inline unsigned blocks_for(long long total, int threads) { return (unsigned)((to
 
 }  // namespace
 
-int launch_pack(const uint8_t* planes, const __half* scales, const __half* offsets, const Geo& g,
-                uint8_t* packed, cudaStream_t stream) {
-    const long long nvec = (long long)g.n_kc * g.n_rb * 2 * g.q * 32;
-    const long long nwords = (long long)g.n_kc * g.n_rb * (g.gl * (g.q + 1) / 2) * 32;
-    const unsigned plane_blocks = blocks_for(nvec, 256);
-    pack_kernel<<<plane_blocks + blocks_for(nwords, 256), 256, 0, stream>>>(
-        planes, reinterpret_cast<const uint16_t*>(scales), reinterpret_cast<const uint16_t*>(offsets), packed, g, plane_blocks);
+namespace {
+
+template <int Q, int G>
+int launch_pack_qg(const uint8_t* planes, const uint16_t* scales, const uint16_t* offsets, const Geo& g, uint8_t* packed, cudaStream_t stream) {
+    const long long tiles = (long long)g.n_kc * g.n_rb, vectors = tiles * 2 * Q, words = tiles * g.gl * (Q + 1) / 2;
+    if (vectors >= (1LL << 31) - 64 || words >= (1LL << 31) - 64) return (int)cudaErrorInvalidValue;
+    Div by_rows;
+    by_rows.set(g.n_rb);
+    const unsigned plane_blocks = blocks_for(vectors, kPackWarps);
+    pack_kernel<Q, G><<<plane_blocks + blocks_for(words, kPackWarps), 32 * kPackWarps, 0, stream>>>(
+        planes, scales, offsets, packed, g, (int)plane_blocks, by_rows, (reinterpret_cast<uintptr_t>(planes) & 15) == 0);
     count_launch(1);
     return (int)cudaGetLastError();
+}
+
+template <int Q>
+int launch_pack_q(const uint8_t* planes, const uint16_t* scales, const uint16_t* offsets, const Geo& g, uint8_t* packed, cudaStream_t stream) {
+    switch (g.G) {
+        case 32: return launch_pack_qg<Q, 32>(planes, scales, offsets, g, packed, stream);
+        case 64: return launch_pack_qg<Q, 64>(planes, scales, offsets, g, packed, stream);
+        default: return launch_pack_qg<Q, 128>(planes, scales, offsets, g, packed, stream);
+    }
+}
+
+}  // namespace
+
+int launch_pack(const uint8_t* planes, const __half* scales, const __half* offsets, const Geo& g,
+                uint8_t* packed, cudaStream_t stream) {
+    const uint16_t* s = reinterpret_cast<const uint16_t*>(scales);
+    const uint16_t* z = reinterpret_cast<const uint16_t*>(offsets);
+    switch (g.q) {
+        case 1: return launch_pack_q<1>(planes, s, z, g, packed, stream);
+        case 2: return launch_pack_q<2>(planes, s, z, g, packed, stream);
+        case 3: return launch_pack_q<3>(planes, s, z, g, packed, stream);
+        default: return launch_pack_q<4>(planes, s, z, g, packed, stream);
+    }
 }
 
 int launch_unpack(const uint8_t* packed, const Geo& g, uint8_t* planes, __half* scales, __half* offsets,
