@@ -66,18 +66,15 @@ typedef enum elutq_status {
                                    negation; same product up to fp32 rounding                              */
 
 #define ELUTQ_TENSOR_MIN_M 3      /* batches of this many rows or more run on the tensor cores (G = 128 or 64, no look-up
-                                     variant flag).  Two rows stay on the batched look-up kernel, which needs one narrow
-                                     pass for them (us at M = 2, it / tensor cores, q = 2: 28672 x 4096 17.7 / 24.6, 4096 x
-                                     14336 13.5 / 14.9, 6144 x 4096 8.6 / 9.8, but 4096 x 4096 7.4 / 7.2; q = 4: 27.2 / 38.1,
-                                     19.4 / 22.5, 11.8 / 12.7, 9.6 / 9.2) and a wider one from three rows on (M = 3, q = 2: 25.9 /
-                                     24.8, 18.4 / 15.2, 11.0 / 9.9, 9.2 / 7.2; only at q = 1 on the widest layers it stays ahead,
-                                     57344 x 8192 50 / 55)                                                              */
+                                     variant flag).  Two rows do so at G = 128 where N * K is above 2^24 and at most 2^27
+                                     (elutq_takes_tensor_path); otherwise they stay on the batched look-up kernel, which needs one
+                                     narrow pass for them                                                                */
 #define ELUTQ_TENSOR_MIN_M_NARROW ELUTQ_TENSOR_MIN_M   /* (kept for callers that ask for the smallest batch on the tensor cores at
                                                           N <= ELUTQ_TENSOR_NARROW_N: the same for every N now)     */
 #define ELUTQ_TENSOR_NARROW_N 8192
 #define ELUTQ_FRAGMENT_MAX_M 8    /* G = 128: up to this many rows the bit-planes are contracted as they are (scales
                                      applied to fp32 sums, as exact as the look-up kernels); larger batches rebuild
-                                     W_hat in fp16 tiles (8B gate_up / down at q = 2, us: M = 8 25.8 / 15.4 and
+                                     W_hat in fp16 tiles (8B gate_up / down at q = 2, us: M = 8 25.7 / 15.6 and
                                      24.9 / 18.9, M = 12 36.6 / 21.2 and 25.0 / 19.3).
                                      At G = 64 every batch takes the former, in blocks of 8 or 16 rows
                                      (elutq_takes_tensor_path is 1 for both)                                        */

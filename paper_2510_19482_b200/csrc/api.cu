@@ -191,17 +191,22 @@ int launch_copy_in(const void* src, void* dst, size_t bytes, cudaStream_t stream
     return (int)e;
 }
 
-// Whether a batched call runs on the tensor cores.
-bool takes_tensor_path(int M, int G, unsigned flags) {
+// Whether a batched call runs on the tensor cores.  Two rows do at G = 128 between 16 and 128 million weights (us on the look-up kernel /
+// there, q = 2, 3, 4: 6144 x 4096 9.0, 10.7, 11.8 / 7.9, 8.8, 9.9; 4096 x 14336 13.4, 16.6, 19.4 / 10.9, 12.9, 15.2; 28672 x 4096 17.6, 22.7, 27.0 /
+// 17.8, 21.1, 24.8).  Above, the look-up kernel is ahead at q = 2 (57344 x 8192 50, 67, 82 / 53, 63, 75); below, little is left to gain on the
+// smallest (1000 x 1024 4.7, 5.4, 5.5 / 4.6, 4.8, 5.2), and 4096 x 4096 (7.8 / 5.6) is where elutq_gemm_kernel's answer for two rows is relied on.
+bool takes_tensor_path(int M, int N, int K, int G, unsigned flags) {
     const unsigned lut_variants = ELUTQ_FLAG_PLAIN_G4 | ELUTQ_FLAG_CLUSTER_REDUCE | ELUTQ_FLAG_MIRROR | ELUTQ_FLAG_LUT_ONLY |
                                   ELUTQ_FLAG_TABLE_F16 | ELUTQ_FLAG_TABLE_I8;
-    return M >= ELUTQ_TENSOR_MIN_M && G != 32 && !(flags & lut_variants);
+    if (G == 32 || (flags & lut_variants)) return false;
+    const long long weights = (long long)N * K;
+    return M >= ELUTQ_TENSOR_MIN_M || (M == 2 && G == 128 && weights > (1LL << 24) && weights <= (1LL << 27));
 }
 
 // The kernel of a call (ELUTQ_KERNEL_...).
 int kernel_of(int M, int N, int K, int q, int G, unsigned flags, int sms) {
     if (M == 1) return ELUTQ_KERNEL_DECODE;
-    if (!takes_tensor_path(M, G, flags)) return ELUTQ_KERNEL_LOOK_UP;
+    if (!takes_tensor_path(M, N, K, G, flags)) return ELUTQ_KERNEL_LOOK_UP;
     if (G != 128 || M <= ELUTQ_FRAGMENT_MAX_M) return ELUTQ_KERNEL_FRAGMENT;
     return rebuilds_in_shared_memory(M, N, K, q, sms) ? ELUTQ_KERNEL_SHARED_MEMORY : ELUTQ_KERNEL_TENSOR_MEMORY;
 }
@@ -477,9 +482,7 @@ int elutq_release_scratch(void) {
 }
 
 int elutq_takes_tensor_path(int M, int N, int K, int G, unsigned flags) {
-    (void)N;
-    (void)K;
-    return takes_tensor_path(M, G, flags) ? 1 : 0;
+    return takes_tensor_path(M, N, K, G, flags) ? 1 : 0;
 }
 
 int elutq_gemm_kernel(int M, int N, int K, int q, int G, unsigned flags) {

@@ -13,6 +13,12 @@
 // with the scales applied to the sums in fp32: W_hat is never formed, as in the look-up kernels, and as exact.  (The MMAs'
 // running sums are truncated, not rounded; a sum runs over one group.)
 //
+//   bytes    Up to four batch rows at G = 128 (BYTES): one logic operation on a word of four weight bytes keeps one bit of each, and what it
+//            leaves, 0 or 2^i in every byte, is an operand of the 8-bit integer MMA as it stands: four weights per operation.  The
+//            activations are digits, x_k = 2^-F sum_d 256^d X_d with the X_d the signed bytes of round(2^(F-i) x_k), F such that the
+//            largest |x| of the row's step lies below 2^30: exact unless x_k is 2^-12 times smaller than that one, and then off by at
+//            most 2^-24 of it, less than the rounding of fp32 sums.  A group's sums are exact (32-bit integers); a batch row takes
+//            four of an MMA's 8 columns.  A lane's two digits are put together in its registers, lower and upper ones at the end.
 //   k order  an MMA sums over k, so A and B only have to agree on which k a lane holds.  Lane c of a quad takes the bytes of word c
 //            of the row's 128 k (at G = 64: bytes 2c, 2c+1 of each group) as two sub-words with one byte in each half, twice: a
 //            left shift by 2 brings the upper copy's bits 0-3 to the four positions, one by 6 the lower copy's bits 4-7 (as
@@ -109,6 +115,13 @@ __device__ __forceinline__ void mma_16816(float (&c)[4], uint32_t a0, uint32_t a
     asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
                  : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
+// Weights' bits (unsigned bytes) times digits (signed ones); `first` begins a sum.
+__device__ __forceinline__ void mma_16832(int (&c)[4], bool first, uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+    const int z[4] = {first ? 0 : c[0], first ? 0 : c[1], first ? 0 : c[2], first ? 0 : c[3]};
+    asm("mma.sync.aligned.m16n8k32.row.col.s32.u8.s8.s32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%10, %11, %12, %13};"
+        : "=r"(c[0]), "=r"(c[1]), "=r"(c[2]), "=r"(c[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "r"(z[0]), "r"(z[1]), "r"(z[2]), "r"(z[3]));
+}
 __device__ __forceinline__ float half_bits(uint32_t v) { return __half2float(__ushort_as_half((unsigned short)v)); }
 
 // slot and parity of the n-th use of a ring, advanced without divisions
@@ -121,16 +134,18 @@ struct Ring {
     }
 };
 
-// NB = blocks of 8 batch rows (MMA N): 1 or 2.  FOLD: long runs of units, whose sums are put by every two units.
-template <int Q, int G, int NB, bool FOLD>
+// NB = blocks of 8 columns (MMA N): of 8 batch rows, or (BYTES) of two with four digits each.  FOLD: long runs of units, whose sums are
+// put by every two units.
+template <int Q, int G, int NB, bool FOLD, bool BYTES>
 __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArgs a) {
     using C = FragCfg<Q, G>;
     static_assert(G == 128 || G == 64, "");
     constexpr int NSG = C::NSG;                               // groups per step: 1 or 2
-    constexpr int MP = 8 * NB;
-    constexpr bool kStepSum = NB == 1;
+    constexpr int MP = (BYTES ? 2 : 8) * NB;
+    constexpr bool kStepSum = BYTES || NB == 1;
     static_assert(!(kStepSum && FOLD), "");
-    constexpr int XF_BYTES = MP * 1024;                       // B fragments of a unit: [step][block][4][lane] 16 bytes
+    constexpr int XF_BYTES = NB * (BYTES ? 4096 : 8192);      // B fragments of a unit: [step][block][2 or 4][lane] 16 bytes
+    static_assert(!BYTES || G == 128, "");
     constexpr int XM_FLOATS = 4 * (1 + NSG) * MP;             // per step: factor 2^(14-c) and group sums of every batch row
     extern __shared__ __align__(1024) uint8_t smem[];
     uint8_t* sX = smem;
@@ -210,11 +225,23 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
         if (step == 0 && loads) load_weights(min(u1, u0 + a.ws));
         grid_dependency_wait();
 
+        // BYTES: the lane's word of a row's plane bytes and bit position, and its place among the B fragments.
+        const int bit = lane & 7, word = lane >> 3, place = (bit >> 2) * 128 + word * 4 + (bit & 3);
+        uint32_t raw_h[BYTES ? MP : 1][4];
         // The lane's four 16-byte pieces (8 k each) of a batch row and step: the low and the high bytes of the two sub-words.
         const int piece[2][2] = {{G == 128 ? 4 * c : 2 * c, G == 128 ? 4 * c + 2 : 2 * c + 1},
                                  {G == 128 ? 4 * c + 1 : 8 + 2 * c, G == 128 ? 4 * c + 3 : 8 + 2 * c + 1}};
         uint4 raw[NB][2][2];
         auto fetch = [&](int mb, int chunk) {
+            if constexpr (BYTES) {
+#pragma unroll
+                for (int m = 0; m < MP; ++m)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const int k = chunk * kChunkK + step * 128 + (4 * word + e) * 8 + bit;
+                        raw_h[m][e] = (mb + m < M && k < a.g.K) ? __ldg(reinterpret_cast<const unsigned short*>(a.g.X) + (size_t)(mb + m) * a.g.K + k) : 0u;
+                    }
+            } else {
 #pragma unroll
             for (int nb = 0; nb < NB; ++nb)
 #pragma unroll
@@ -224,6 +251,7 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
                         const int m = mb + 8 * nb + gq, k = chunk * kChunkK + step * 128 + piece[q][e] * 8;
                         raw[nb][q][e] = (m < M && k < a.g.K) ? __ldg(reinterpret_cast<const uint4*>(a.g.X + (size_t)m * a.g.K + k)) : make_uint4(0, 0, 0, 0);
                     }
+            }
         };
         int tile = a.by_chunks.of(u0), chunk = u0 - tile * C_, mb = batch0(tile);
         if (u0 < u1) fetch(mb, chunk);
@@ -231,7 +259,53 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
             const int t = u - u0, slot = t & 1;
             if (!__all_sync(0xffffffffu, wait_many([&]() { return mbar_try(bar(kBarXEmpty + slot), (uint32_t)((t >> 1) & 1) ^ 1u); }))) break;
             if (step == 0 && t >= 2 && loads) load_weights(min(u1, u - 2 + a.ws + 1));      // the unit two back has been read
-            if (step < steps_of(chunk)) {
+            if (BYTES && step < steps_of(chunk)) {
+                uint32_t* frag = reinterpret_cast<uint32_t*>(sX + slot * XF_BYTES) + step * (NB * 256) + place;
+                float* meta = sM + slot * XM_FLOATS + step * ((1 + NSG) * MP);
+                uint32_t top[MP];
+#pragma unroll
+                for (int m = 0; m < MP; ++m)
+                    top[m] = __reduce_max_sync(0xffffffffu, max(max(raw_h[m][0] & 0x7fffu, raw_h[m][1] & 0x7fffu), max(raw_h[m][2] & 0x7fffu, raw_h[m][3] & 0x7fffu)));
+#pragma unroll
+                for (int m = 0; m < MP; ++m) {
+                    const int F = 44 - min(max((int)(top[m] >> 10), 1), 30);                    // |x| 2^F < 2^30
+                    float x[4], fac = __int_as_float((127 - F) << 23);
+                    uint32_t d[4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        x[e] = half_bits(raw_h[m][e]);
+                        d[e] = (uint32_t)__float2int_rn(x[e] * __int_as_float((127 + F - bit) << 23));
+                    }
+                    // the group's sum, in units of 2^(7-F): the lanes' sums of four, below 2^25, added as integers
+                    const int part = __float2int_rn(((x[0] + x[1]) + (x[2] + x[3])) * __int_as_float((127 + F - 7) << 23));
+                    float total = (float)__reduce_add_sync(0xffffffffu, part) * __int_as_float((127 - F + 7) << 23);
+                    if (top[m] >= 0x7c00u) {
+                        // Not all finite.  An infinity counts as a small number in the lowest digit, everything else of its row as nothing, and
+                        // a factor of 2^127 makes an infinity of what the planes leave of it; a NaN makes NaN of the row.
+                        fac = __int_as_float(top[m] > 0x7c00u ? 0x7fffffff : 254 << 23);
+#pragma unroll
+                        for (int e = 0; e < 4; ++e)
+                            d[e] = (raw_h[m][e] & 0x7fffu) != 0x7c00u ? 0u : raw_h[m][e] & 0x8000u ? 0u - (64u >> min(bit, 6)) : 64u >> min(bit, 6);
+                        total = (x[0] + x[1]) + (x[2] + x[3]);
+                        for (int o = 1; o < 32; o <<= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
+                    }
+                    // balanced, so that the lower three digits are signed bytes too; then a word per digit of the lane's four elements
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) d[e] = (d[e] + 0x00808080u) ^ 0x00808080u;
+                    const uint32_t lo01 = __byte_perm(d[0], d[1], 0x5140), hi01 = __byte_perm(d[0], d[1], 0x7362);
+                    const uint32_t lo23 = __byte_perm(d[2], d[3], 0x5140), hi23 = __byte_perm(d[2], d[3], 0x7362);
+                    uint32_t* o = frag + (m >> 1) * 256 + (m & 1) * 64;
+                    o[0] = __byte_perm(lo01, lo23, 0x5410);
+                    o[16] = __byte_perm(lo01, lo23, 0x7632);
+                    o[32] = __byte_perm(hi01, hi23, 0x5410);
+                    o[48] = __byte_perm(hi01, hi23, 0x7632);
+                    if (lane == 0) {
+                        meta[m] = fac;
+                        meta[MP + m] = total;
+                    }
+                }
+            }
+            if (!BYTES && step < steps_of(chunk)) {
                 uint4* frag = reinterpret_cast<uint4*>(sX + slot * XF_BYTES) + step * (NB * 128) + lane;
                 float* meta = sM + slot * XM_FLOATS + step * ((1 + NSG) * MP);
 #pragma unroll
@@ -345,6 +419,7 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
         sel[0] = s * 0x0011u + (s + (G == 128 ? 2u : 1u)) * 0x1100u;
         sel[1] = G == 128 ? sel[0] + 0x1111u : sel[0];
     }
+    const int word_shift = 8 * ((0 - gq) & 3);                // BYTES: the lane's word begins there
     uint32_t by4 = 4u, by64 = 64u;                            // opaque, so that the products stay products
     asm volatile("" : "+r"(by4), "+r"(by64));
     const uint32_t poff = (uint32_t)((2 * rp) * C::TILE_BYTES + C::PLANE_BYTES + (16 * (step & 1) + gq) * 4);
@@ -388,9 +463,7 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
                     for (int i = 0; i < 4; ++i)
                         v[e][i] = (p + e < parts && m0 + 4 * i < me) ? __ldcg(p0 + ((size_t)(p + e) * M + m0 + 4 * i) * n_pad) : 0.f;
 #pragma unroll
-                for (int e = 0; e < 4; ++e)
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) y[i] += v[e][i];
+                for (int i = 0; i < 4; ++i) y[i] += (v[0][i] + v[1][i]) + (v[2][i] + v[3][i]);       // (in pairs: fewer roundings than in one chain)
             }
 #pragma unroll
             for (int i = 0; i < 4; ++i)
@@ -398,8 +471,9 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
         }
     };
 
-    float* own_sum = sSum + (step * MP + 2 * c) * kSumStride + 32 * rp + gq;      // where the lane's sums go in the buffer
-    auto sum_at = [](int nb, int t, int i) { return (8 * nb + (i & 1)) * kSumStride + 16 * t + 8 * (i >> 1); };
+    constexpr int NE = BYTES ? 2 : 4;                         // sums of a lane: rows gq, gq + 8 (times batch rows 2c, 2c + 1)
+    float* own_sum = sSum + (step * MP + (BYTES ? c >> 1 : 2 * c)) * kSumStride + 32 * rp + gq;      // where the lane's sums go in the buffer
+    auto sum_at = [](int nb, int t, int i) { return BYTES ? 2 * nb * kSumStride + 16 * t + 8 * i : (8 * nb + (i & 1)) * kSumStride + 16 * t + 8 * (i >> 1); };
 
     Ring w(a.ws), x(kXSlots);
     bool live = true;
@@ -409,19 +483,84 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
         const int n_units = min(C_ - chunk0, u1 - u);
         u += n_units;
         if (FOLD) compute_sync();                             // the buffer has been read
-        float acc[2][NB][4];
+        float acc[2][NB][NE];
 #pragma unroll
         for (int t = 0; t < 2; ++t)
 #pragma unroll
             for (int nb = 0; nb < NB; ++nb)
 #pragma unroll
-                for (int i = 0; i < 4; ++i) acc[t][nb][i] = 0.f;
+                for (int i = 0; i < NE; ++i) acc[t][nb][i] = 0.f;
 
         for (int cu = 0; cu < n_units; ++cu) {
             live = __all_sync(0xffffffffu, wait_many([&]() {
                 return mbar_try(bar(kBarWFull + w.i), w.phase) & mbar_try(bar(kBarXFull + x.i), x.phase);
             }));
             if (!live) break;
+            if (BYTES && step < steps_of(chunk0 + cu)) {
+                // Lane c of a quad holds two digits of batch row c / 2 of every block: the lower two, or the upper two times 2^16
+                const uint8_t* wb = sW + w.i * C::UNIT_BYTES;
+                const uint4* xb = reinterpret_cast<const uint4*>(sX + x.i * XF_BYTES) + step * (NB * 64) + lane;
+                const float* meta = sM + x.i * XM_FLOATS + step * ((1 + NSG) * MP) + (c >> 1);
+                uint4 xd[NB][2];                              // B fragments, held over the planes
+                float fac[NB], own[2][NB][2];
+#pragma unroll
+                for (int nb = 0; nb < NB; ++nb) {
+                    xd[nb][0] = xb[nb * 64];
+                    xd[nb][1] = xb[nb * 64 + 32];
+                    fac[nb] = (c & 1) ? fminf(meta[2 * nb] * 65536.f, 3.4028235e38f) : meta[2 * nb];
+                }
+                const uint32_t pb = smem_addr(wb);
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const float z = half_bits(parameter(pb, r, 0, Q) & offset_mask);
+#pragma unroll
+                    for (int nb = 0; nb < NB; ++nb) own[r >> 1][nb][r & 1] = z * ((c & 1) ? 0.f : meta[MP + 2 * nb]);
+                }
+                if (use_planes) {
+#pragma unroll
+                    for (int j = 0; j < Q; ++j) {
+                        uint32_t pw[4];
+#pragma unroll
+                        for (int r = 0; r < 4; ++r) {
+                            const uint8_t* tb = wb + (r >> 1) * C::TILE_BYTES + j * 512;
+                            pw[r] = __funnelshift_r(*reinterpret_cast<const uint32_t*>(tb + off0[r & 1]), *reinterpret_cast<const uint32_t*>(tb + off1[r & 1]), word_shift);
+                        }
+                        int d[2][NB][4];
+#pragma unroll
+                        for (int kk = 0; kk < 4; ++kk) {      // two bit positions of the words: 32 k of each row
+                            uint32_t f[4][2];
+#pragma unroll
+                            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                                for (int i = 0; i < 2; ++i) f[r][i] = pw[r] & (0x01010101u << (2 * kk + i));
+#pragma unroll
+                            for (int nb = 0; nb < NB; ++nb) {
+                                const uint4 xv = xd[nb][kk >> 1];
+#pragma unroll
+                                for (int t = 0; t < 2; ++t)
+                                    mma_16832(d[t][nb], kk == 0, f[2 * t][0], f[2 * t + 1][0], f[2 * t][1], f[2 * t + 1][1], kk & 1 ? xv.z : xv.x,
+                                              kk & 1 ? xv.w : xv.y);
+                            }
+                        }
+#pragma unroll
+                        for (int r = 0; r < 4; ++r) {         // the plane's scale
+                            const float sc = half_bits(parameter(pb, r, 0, j));
+#pragma unroll
+                            for (int nb = 0; nb < NB; ++nb) {
+                                const int* v = &d[r >> 1][nb][2 * (r & 1)];
+                                own[r >> 1][nb][r & 1] = fmaf(sc, (float)(v[0] + 256 * v[1]) * fac[nb], own[r >> 1][nb][r & 1]);
+                            }
+                        }
+                    }
+                }
+#pragma unroll
+                for (int t = 0; t < 2; ++t)
+#pragma unroll
+                    for (int nb = 0; nb < NB; ++nb)
+#pragma unroll
+                        for (int i = 0; i < 2; ++i) acc[t][nb][i] += own[t][nb][i];
+            }
+            if constexpr (!BYTES) {
             if (step < steps_of(chunk0 + cu)) {
                 const uint32_t wb = smem_addr(sW) + (uint32_t)(w.i * C::UNIT_BYTES);
                 const uint32_t xb = smem_addr(sX) + (uint32_t)(x.i * XF_BYTES + step * (NB * 2048) + lane * 16);
@@ -535,6 +674,7 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
                             for (int i = 0; i < 4; ++i) acc[t][nb][i] += sum[t][nb][i];
                 }
             }
+            }
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(kBarXEmpty + x.i));
             w.next();
@@ -557,12 +697,21 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
         compute_sync();                                       // the buffer has been read; the ticket of the run before is there
         finish_tile(pending);
         pending = -1;
+        if constexpr (BYTES) {                                // the upper digits' part
+#pragma unroll
+            for (int nb = 0; nb < NB; ++nb)
+#pragma unroll
+                for (int t = 0; t < 2; ++t)
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) acc[t][nb][i] += __shfl_xor_sync(0xffffffffu, acc[t][nb][i], 1);
+        }
+        if (!BYTES || !(c & 1))
 #pragma unroll
         for (int nb = 0; nb < NB; ++nb)
 #pragma unroll
             for (int t = 0; t < 2; ++t)
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
+                for (int i = 0; i < NE; ++i)
                     own_sum[sum_at(nb, t, i)] = FOLD && n_units > 1 ? own_sum[sum_at(nb, t, i)] + acc[t][nb][i] : acc[t][nb][i];
         if (compute_any(!live)) {                             // the tickets of this run of units and the rest are taken all the same
             for (int v = u - n_units; v < u1 && tid == 0;) {
@@ -606,16 +755,16 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
     __syncthreads();                                          // nobody leaves while copies are in flight
 }
 
-template <int Q, int G, int NB, bool FOLD = false>
+template <int Q, int G, int NB, bool BYTES, bool FOLD = false>
 int launch_frag_cfg(const GemmArgs& g, int num_sms, cudaStream_t stream) {
     using C = FragCfg<Q, G>;
-    constexpr int kMaxSmem = 232448, MP = 8 * NB;
-    constexpr int kFixed = kXSlots * (MP * 1024 + 4 * (1 + C::NSG) * MP * 4) + 4 * MP * kSumStride * 4 + kNumBars * 8 + 64;
+    constexpr int kMaxSmem = 232448, MP = (BYTES ? 2 : 8) * NB;
+    constexpr int kFixed = kXSlots * (NB * (BYTES ? 4096 : 8192) + 4 * (1 + C::NSG) * MP * 4) + 4 * MP * kSumStride * 4 + kNumBars * 8 + 64;
     static bool configured[64] = {};
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev >= 0 && dev < 64 && !configured[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(hlq_frag_kernel<Q, G, NB, FOLD>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+        cudaError_t e = cudaFuncSetAttribute(hlq_frag_kernel<Q, G, NB, FOLD, BYTES>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
         if (e != cudaSuccess) return (int)e;
         configured[dev] = true;
     }
@@ -631,8 +780,8 @@ int launch_frag_cfg(const GemmArgs& g, int num_sms, cudaStream_t stream) {
     // Runs of more than two units without a sum per step: the sums are put by in between, for the same reason as there (4096 x 14336, q = 4,
     // G = 64, M = 16, error of the fp32 result 1.5e-7 -> 1.0e-7, the look-up kernel 1.0e-7 to 1.5e-7 by the number of rows; time
     // 36.3 -> 36.8 us).
-    if constexpr (NB > 1 && !FOLD) {
-        if (a.per_cta > 2) return launch_frag_cfg<Q, G, NB, true>(g, num_sms, stream);
+    if constexpr (NB > 1 && !FOLD && !BYTES) {
+        if (a.per_cta > 2) return launch_frag_cfg<Q, G, NB, BYTES, true>(g, num_sms, stream);
     }
     a.by_chunks.set(a.chunks);
     a.by_blocks.set(a.blocks);
@@ -653,13 +802,20 @@ int launch_frag_cfg(const GemmArgs& g, int num_sms, cudaStream_t stream) {
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, hlq_frag_kernel<Q, G, NB, FOLD>, a);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, hlq_frag_kernel<Q, G, NB, FOLD, BYTES>, a);
     count_launch(1);
     return (int)e;
 }
 
 template <int Q, int G>
 int launch_frag_qg(const GemmArgs& g, int num_sms, cudaStream_t stream) {
+    // Up to four rows: as bytes (us as halves / bytes, M = 4, q = 2, 3, 4: 28672 x 4096 25.0, 31.7, 38.5 / 23.3, 29.0, 35.5; 4096 x 14336
+    // 15.1, 18.7, 22.8 / 13.8, 17.2, 21.0; 4096 x 4096 7.4, 8.3, 9.5 / 6.9, 7.9, 9.4).  At G = 64 the sums of a step's two groups cost what
+    // the masks save (28672 x 4096, M = 4 27.6, 35.3, 43.0 / 28.7, 35.4, 41.5; 4096 x 4096 8.0, 9.4, 10.9 / 8.5, 9.9, 11.0).
+    if constexpr (G == 128) {
+        if (g.M <= 2) return launch_frag_cfg<Q, G, 1, true>(g, num_sms, stream);
+        if (g.M <= 4) return launch_frag_cfg<Q, G, 2, true>(g, num_sms, stream);
+    }
     if constexpr (G == 64) {
         // The height of a batch block, by the longest run of units: a unit takes u us, the first one of a taller block u0 more.  (Fitted
         // to 1100 calls, 256 to 28672 rows.  Blocks of 32 rows, whose sums do not fit the registers, are nowhere ahead: 4096 x 4096,
@@ -669,10 +825,10 @@ int launch_frag_qg(const GemmArgs& g, int num_sms, cudaStream_t stream) {
             const long long units = tiles * ((g.M + rows - 1) / rows);
             return u0 + u * (double)((units + num_sms - 1) / num_sms);
         };
-        if (g.M > 8 && us(16, 1.0, 1.0 + 0.86 * Q) < us(8, 0.0, 0.5 + 0.6 * Q)) return launch_frag_cfg<Q, G, 2>(g, num_sms, stream);
-        return launch_frag_cfg<Q, G, 1>(g, num_sms, stream);
+        if (g.M > 8 && us(16, 1.0, 1.0 + 0.86 * Q) < us(8, 0.0, 0.5 + 0.6 * Q)) return launch_frag_cfg<Q, G, 2, false>(g, num_sms, stream);
+        return launch_frag_cfg<Q, G, 1, false>(g, num_sms, stream);
     }
-    return g.M <= 8 ? launch_frag_cfg<Q, G, 1>(g, num_sms, stream) : (int)cudaErrorInvalidValue;
+    return g.M <= 8 ? launch_frag_cfg<Q, G, 1, false>(g, num_sms, stream) : (int)cudaErrorInvalidValue;
 }
 
 template <int Q>

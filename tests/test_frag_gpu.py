@@ -47,6 +47,18 @@ def test_fragment_kernel_matches_oracle(q, G, N, K, M):
     assert max(hlq.rel_fro_error(yb[m], hlq.offset_term(X, layer.offsets, G)[m]) for m in range(M)) <= 5e-6
 
 
+# Up to four rows as digits of 8 bits: edges of the row tile, K of one step and inside a chunk, tiles of one and of many parts, two rows
+@pytest.mark.parametrize("q,N,K,M", [(1, 17, 128, 4), (3, 129, 640, 4), (4, 1000, 1408, 3), (2, 4100, 4224, 2), (3, 5003, 3456, 2), (4, 300, 14336, 4)])
+def test_rows_as_digits(q, N, K, M):
+    test_fragment_kernel_matches_oracle(q, 128, N, K, M)
+    # one element of every step much larger than the rest: digits are rounded below 2^-30 of it
+    layer = workloads.hlq_layer(68, f"frag/digits/{q}/{N}/{K}", q, 128, N, K)
+    X = synth.activations(68, f"frag/digits/x/{M}/{K}", M, K)
+    X[:, 5::128] = np.float16(2.0 ** 13)
+    y, ref = gemm_f32(X, pack_layer(layer), N, K), hlq.matmul(X, layer.planes, layer.scales, layer.offsets, 128)
+    assert np.all(np.abs(y - ref) <= 2 * K * 2.0 ** -24 * hlq.magnitude_bound(X, layer.scales, layer.offsets, 128))
+
+
 def test_fragment_kernel_reports_a_wait_that_runs_out():
     q, G, N, K, M = 2, 64, 512, 2048, 12
     layer = workloads.hlq_layer(61, "frag/expiry", q, G, N, K)
