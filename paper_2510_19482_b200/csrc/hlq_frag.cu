@@ -1,4 +1,4 @@
-// Batches of up to ELUTQ_FRAGMENT_MAX_M rows (any at G = 64): bit-planes as MMA fragments, without dequantising.
+// Batches of up to ELUTQ_FRAGMENT_MAX_M rows (any at G = 64): bit-planes as MMA fragments, without dequantising.  In two forms, halves and bytes.
 //
 // A warp forms the A fragments of mma.sync (16 weight rows x 16 k) in the registers that the MMA reads, with ONE logic
 // operation per two weights: of a register with two weight bytes, one in each half, a mask leaves one bit of each half, at
@@ -19,11 +19,13 @@
 //            largest |x| of the row's step lies below 2^30: exact unless x_k is 2^-12 times smaller than that one, and then off by at
 //            most 2^-24 of it, less than the rounding of fp32 sums.  A group's sums are exact (32-bit integers); a batch row takes
 //            four of an MMA's 8 columns.  A lane's two digits are put together in its registers, lower and upper ones at the end.
+//            Bound: latencies (issue 50 %, logic pipe 41 %, LSU 21 % of the cycles at M = 2, 28672 x 4096, q = 2; the halves 55, 47 and 17 at
+//            M = 4, q = 3).  us as halves / bytes, M = 4, q = 2 / 4: 28672 x 4096 25.0, 38.5 / 23.3, 35.5; 4096 x 14336 15.1, 22.8 / 13.8, 21.0.
 //   k order  an MMA sums over k, so A and B only have to agree on which k a lane holds.  Lane c of a quad takes the bytes of word c
 //            of the row's 128 k (at G = 64: bytes 2c, 2c+1 of each group) as two sub-words with one byte in each half, twice: a
 //            left shift by 2 brings the upper copy's bits 0-3 to the four positions, one by 6 the lower copy's bits 4-7 (as
 //            multiplications: the logic pipe is the busy one).
-//   unit     128 weight rows x 512 k (eight packed tiles, contiguous in the blob: one bulk copy) x 8 NB batch rows.  The units of
+//   unit     128 weight rows x 512 k (eight packed tiles, contiguous in the blob: one bulk copy) x 8 NB batch rows (bytes: 2 NB).  The units of
 //            a call, output tile by output tile (the batch blocks of a row tile next to each other: its weights come from the L2 again), are
 //            dealt to the CTAs (one per SM) in equal contiguous runs, so no SM idles for a wave.  An output tile that several CTAs share
 //            is summed in ascending k order (bit-reproducible) by the CTA that finishes it last (a ticket, no CTA waits for another).

@@ -1,4 +1,5 @@
-// 2 <= M < ELUTQ_TENSOR_MIN_M (any M > 1 at G = 32 or on request): batched look-up GEMM over the same packed layout.
+// Batches off the tensor cores (takes_tensor_path in api.cu: two rows of some sizes, any M > 1 at G = 32 or on request): batched look-up GEMM
+// over the same packed layout.
 //
 // MB activation rows are processed per pass: a table entry holds the partial sums of all MB rows for one
 // (byte value, column), so one weight byte costs one byte-permute, one shared-memory load and the adds of MB
