@@ -14,13 +14,16 @@
 // running sums are truncated, not rounded; a sum runs over one group.)
 //
 //   bytes    Up to four batch rows at G = 128 (BYTES): one logic operation on a word of four weight bytes keeps one bit of each, and what it
-//            leaves, 0 or 2^i in every byte, is an operand of the 8-bit integer MMA as it stands: four weights per operation.  The
-//            activations are digits, x_k = 2^-F sum_d 256^d X_d with the X_d the signed bytes of round(2^(F-i) x_k), F such that the
-//            largest |x| of the row's step lies below 2^30: exact unless x_k is 2^-12 times smaller than that one, and then off by at
-//            most 2^-24 of it, less than the rounding of fp32 sums.  A group's sums are exact (32-bit integers); a batch row takes
-//            four of an MMA's 8 columns.  A lane's two digits are put together in its registers, lower and upper ones at the end.
-//            Bound: latencies (issue 50 %, logic pipe 41 %, LSU 21 % of the cycles at M = 2, 28672 x 4096, q = 2; the halves 55, 47 and 17 at
-//            M = 4, q = 3).  us as halves / bytes, M = 4, q = 2 / 4: 28672 x 4096 25.0, 38.5 / 23.3, 35.5; 4096 x 14336 15.1, 22.8 / 13.8, 21.0.
+//            leaves, 0 or 2^i in every byte, is an operand of the 8-bit integer MMA as it stands: four weights per operation (bits 4-7 as
+//            bits 0-3 of the word shifted by 4).  The activations are digits, x_k = 2^(i-F) sum_d 256^d X_d with the X_d the signed bytes of
+//            the integer nearest to 2^(F-i) x_k, F such that the largest |x| of the row's step lies just below 2^31.  A value with a bit
+//            below the lowest unit, 2^-17 of that largest one, leaves a rest: the step is contracted a second time, with the rests' digits.
+//            So every activation enters exactly, also next to one that is 2^40 times larger and whose bits are clear.  (Without the second
+//            pass, and with i to 7, such sums were off by 2^-23 of the large one.)  A group's sums are exact (digits' below 2^16, two of
+//            them together below 2^24); a batch row takes four of an MMA's 8 columns.  A lane's two digits are put together in its
+//            registers, lower and upper ones at the end.
+//            How often there is a rest: no step in 10000 of N(0,1) activations, 5 in 1000 with 1 % of the channels times 20.  us at 28672 x
+//            4096, M = 4, q = 2, 3, 4: as halves 25.2, 31.8, 38.7, without the second pass and the shift 23.3, 29.1, 35.6, so 25.4, 30.3, 36.0.
 //   k order  an MMA sums over k, so A and B only have to agree on which k a lane holds.  Lane c of a quad takes the bytes of word c
 //            of the row's 128 k (at G = 64: bytes 2c, 2c+1 of each group) as two sub-words with one byte in each half, twice: a
 //            left shift by 2 brings the upper copy's bits 0-3 to the four positions, one by 6 the lower copy's bits 4-7 (as
@@ -136,6 +139,38 @@ struct Ring {
     }
 };
 
+// BYTES: a word per digit of a lane's four elements d (integers, |d| <= 2^31 - 2^23) to its places o, o + 16, ... in the B fragments.
+__device__ __forceinline__ void store_digits(uint32_t* o, uint32_t (&d)[4]) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) d[e] = (d[e] + 0x00808080u) ^ 0x00808080u;      // balanced, so that the lower three digits are signed bytes too
+    const uint32_t lo01 = __byte_perm(d[0], d[1], 0x5140), hi01 = __byte_perm(d[0], d[1], 0x7362);
+    const uint32_t lo23 = __byte_perm(d[2], d[3], 0x5140), hi23 = __byte_perm(d[2], d[3], 0x7362);
+    o[0] = __byte_perm(lo01, lo23, 0x5410);
+    o[16] = __byte_perm(lo01, lo23, 0x7632);
+    o[32] = __byte_perm(hi01, hi23, 0x5410);
+    o[48] = __byte_perm(hi01, hi23, 0x7632);
+}
+
+__device__ __forceinline__ float power_of_two(int e) { return __int_as_float((127 + e) << 23); }
+
+// BYTES: what the digits of a step leave of the batch rows' values: fractions of a unit, which are multiples of 2^-13 (of 2^-24 in the value, whose
+// unit is at most 2^(3-14)), times 2^15, in digits.  x: the lane's first element in row 0; meta: the rows' factors 2^-F.
+__device__ __noinline__ void store_rest(const unsigned short* x, int K, int M, int rows, int bit, const float* meta, uint32_t* frag) {
+#pragma unroll 1
+    for (int m = 0; m < rows; ++m) {
+        uint32_t d[4] = {};
+        if (m < M && meta[m] < 1.f) {                         // (2^127: not all finite)
+            const int F = 127 - (int)(__float_as_uint(meta[m]) >> 23);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float v = half_bits(__ldg(x + (size_t)m * K + 8 * e)) * power_of_two(F - (bit & 3));
+                d[e] = (uint32_t)__float2int_rn((v - rintf(v)) * 32768.f);
+            }
+        }
+        store_digits(frag + (m >> 1) * 256 + (m & 1) * 64, d);
+    }
+}
+
 // NB = blocks of 8 columns (MMA N): of 8 batch rows, or (BYTES) of two with four digits each.  FOLD: long runs of units, whose sums are
 // put by every two units.
 template <int Q, int G, int NB, bool FOLD, bool BYTES>
@@ -146,9 +181,10 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
     constexpr int MP = (BYTES ? 2 : 8) * NB;
     constexpr bool kStepSum = BYTES || NB == 1;
     static_assert(!(kStepSum && FOLD), "");
-    constexpr int XF_BYTES = NB * (BYTES ? 4096 : 8192);      // B fragments of a unit: [step][block][2 or 4][lane] 16 bytes
+    constexpr int XF_BYTES = 8192 * NB;                       // B fragments of a unit: [digits, rest (BYTES)][step][block][2 or 4][lane] 16 bytes
     static_assert(!BYTES || G == 128, "");
-    constexpr int XM_FLOATS = 4 * (1 + NSG) * MP;             // per step: factor 2^(14-c) and group sums of every batch row
+    constexpr int XM_STEP = (1 + NSG) * MP + (BYTES ? 1 : 0); // per step: factor and group sums of every batch row (BYTES: whether there is a rest)
+    constexpr int XM_FLOATS = 4 * XM_STEP;
     extern __shared__ __align__(1024) uint8_t smem[];
     uint8_t* sX = smem;
     uint8_t* sW = sX + kXSlots * XF_BYTES;
@@ -261,55 +297,66 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
             const int t = u - u0, slot = t & 1;
             if (!__all_sync(0xffffffffu, wait_many([&]() { return mbar_try(bar(kBarXEmpty + slot), (uint32_t)((t >> 1) & 1) ^ 1u); }))) break;
             if (step == 0 && t >= 2 && loads) load_weights(min(u1, u - 2 + a.ws + 1));      // the unit two back has been read
-            if (BYTES && step < steps_of(chunk)) {
-                uint32_t* frag = reinterpret_cast<uint32_t*>(sX + slot * XF_BYTES) + step * (NB * 256) + place;
-                float* meta = sM + slot * XM_FLOATS + step * ((1 + NSG) * MP);
+            if constexpr (BYTES) {
+                const int k0 = chunk * kChunkK + step * 128;
+                float x[MP][4];
                 uint32_t top[MP];
 #pragma unroll
-                for (int m = 0; m < MP; ++m)
+                for (int m = 0; m < MP; ++m) {
                     top[m] = __reduce_max_sync(0xffffffffu, max(max(raw_h[m][0] & 0x7fffu, raw_h[m][1] & 0x7fffu), max(raw_h[m][2] & 0x7fffu, raw_h[m][3] & 0x7fffu)));
 #pragma unroll
-                for (int m = 0; m < MP; ++m) {
-                    const int F = 44 - min(max((int)(top[m] >> 10), 1), 30);                    // |x| 2^F < 2^30
-                    float x[4], fac = __int_as_float((127 - F) << 23);
-                    uint32_t d[4];
+                    for (int e = 0; e < 4; ++e) x[m][e] = half_bits(raw_h[m][e]);
+                }
+                const bool there = step < steps_of(chunk);
+                if (++chunk == C_) {
+                    chunk = 0;
+                    mb = batch0(++tile);
+                }
+                if (u + 1 < u1) fetch(mb, chunk);             // (in flight while this unit's are worked on)
+                if (there) {
+                    uint32_t* frag = reinterpret_cast<uint32_t*>(sX + slot * XF_BYTES) + step * (NB * 256) + place;
+                    float* meta = sM + slot * XM_FLOATS + step * XM_STEP;
+                    bool rest = false;
+                    float four[MP];
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        x[e] = half_bits(raw_h[m][e]);
-                        d[e] = (uint32_t)__float2int_rn(x[e] * __int_as_float((127 + F - bit) << 23));
+                    for (int m = 0; m < MP; ++m) {
+                        const int F = 45 - min(max((int)((top[m] + 8u) >> 10), 1), 31);         // |x| 2^F <= 2^31 - 9 2^20
+                        const float scale = power_of_two(F - (bit & 3));
+                        uint32_t d[4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const int n = __float2int_rn(x[m][e] * scale);
+                            rest |= (float)n != x[m][e] * scale && top[m] < 0x7c00u;
+                            d[e] = (uint32_t)n;
+                            // Not all finite: an infinity counts as a small number in the lowest digit, everything else of its row as nothing, and
+                            // a factor of 2^127 makes an infinity of what the planes leave of it; a NaN makes NaN of the row.
+                            if (top[m] >= 0x7c00u) d[e] = fabsf(x[m][e]) <= 65504.f ? 0u : x[m][e] < 0.f ? 0u - (64u >> (bit & 3)) : 64u >> (bit & 3);
+                        }
+                        store_digits(frag + (m >> 1) * 256 + (m & 1) * 64, d);
+                        four[m] = (x[m][0] + x[m][1]) + (x[m][2] + x[m][3]);
+                        if (lane == 0) meta[m] = top[m] < 0x7c00u ? power_of_two(-F) : __int_as_float(top[m] > 0x7c00u ? 0x7fffffff : 254 << 23);
                     }
-                    // the group's sum, in units of 2^(7-F): the lanes' sums of four, below 2^25, added as integers
-                    const int part = __float2int_rn(((x[0] + x[1]) + (x[2] + x[3])) * __int_as_float((127 + F - 7) << 23));
-                    float total = (float)__reduce_add_sync(0xffffffffu, part) * __int_as_float((127 - F + 7) << 23);
-                    if (top[m] >= 0x7c00u) {
-                        // Not all finite.  An infinity counts as a small number in the lowest digit, everything else of its row as nothing, and
-                        // a factor of 2^127 makes an infinity of what the planes leave of it; a NaN makes NaN of the row.
-                        fac = __int_as_float(top[m] > 0x7c00u ? 0x7fffffff : 254 << 23);
+                    // the rows' sums over the lanes, row m in lanes m, m + MP, ...
+                    auto fold = [&](float even, float odd, int b) {
+                        const bool up = (lane & b) != 0;
+                        return (up ? odd : even) + __shfl_xor_sync(0xffffffffu, up ? even : odd, b);
+                    };
+                    float total = fold(four[0], four[1], 1);
+                    if constexpr (MP == 4) total = fold(total, fold(four[2], four[3], 1), 2);
 #pragma unroll
-                        for (int e = 0; e < 4; ++e)
-                            d[e] = (raw_h[m][e] & 0x7fffu) != 0x7c00u ? 0u : raw_h[m][e] & 0x8000u ? 0u - (64u >> min(bit, 6)) : 64u >> min(bit, 6);
-                        total = (x[0] + x[1]) + (x[2] + x[3]);
-                        for (int o = 1; o < 32; o <<= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
-                    }
-                    // balanced, so that the lower three digits are signed bytes too; then a word per digit of the lane's four elements
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) d[e] = (d[e] + 0x00808080u) ^ 0x00808080u;
-                    const uint32_t lo01 = __byte_perm(d[0], d[1], 0x5140), hi01 = __byte_perm(d[0], d[1], 0x7362);
-                    const uint32_t lo23 = __byte_perm(d[2], d[3], 0x5140), hi23 = __byte_perm(d[2], d[3], 0x7362);
-                    uint32_t* o = frag + (m >> 1) * 256 + (m & 1) * 64;
-                    o[0] = __byte_perm(lo01, lo23, 0x5410);
-                    o[16] = __byte_perm(lo01, lo23, 0x7632);
-                    o[32] = __byte_perm(hi01, hi23, 0x5410);
-                    o[48] = __byte_perm(hi01, hi23, 0x7632);
-                    if (lane == 0) {
-                        meta[m] = fac;
-                        meta[MP + m] = total;
+                    for (int o = MP; o < 32; o <<= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
+                    if (lane < MP) meta[MP + lane] = total;
+                    rest = __any_sync(0xffffffffu, rest);
+                    if (lane == 0) reinterpret_cast<uint32_t*>(meta)[2 * MP] = rest ? 1u : 0u;
+                    if (__builtin_expect(rest, 0)) {
+                        __syncwarp();
+                        store_rest(reinterpret_cast<const unsigned short*>(a.g.X) + k0 + 32 * word + bit, a.g.K, M, MP, bit, meta, frag + NB * 1024);
                     }
                 }
             }
             if (!BYTES && step < steps_of(chunk)) {
                 uint4* frag = reinterpret_cast<uint4*>(sX + slot * XF_BYTES) + step * (NB * 128) + lane;
-                float* meta = sM + slot * XM_FLOATS + step * ((1 + NSG) * MP);
+                float* meta = sM + slot * XM_FLOATS + step * XM_STEP;
 #pragma unroll
                 for (int nb = 0; nb < NB; ++nb) {
                     __half2 v[2][2][4];
@@ -385,11 +432,13 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
                     }
                 }
             }
-            if (++chunk == C_) {
-                chunk = 0;
-                mb = batch0(++tile);
+            if constexpr (!BYTES) {
+                if (++chunk == C_) {
+                    chunk = 0;
+                    mb = batch0(++tile);
+                }
+                if (u + 1 < u1) fetch(mb, chunk);
             }
-            if (u + 1 < u1) fetch(mb, chunk);
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(kBarXFull + slot));
         }
@@ -502,25 +551,27 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
                 // Lane c of a quad holds two digits of batch row c / 2 of every block: the lower two, or the upper two times 2^16
                 const uint8_t* wb = sW + w.i * C::UNIT_BYTES;
                 const uint4* xb = reinterpret_cast<const uint4*>(sX + x.i * XF_BYTES) + step * (NB * 64) + lane;
-                const float* meta = sM + x.i * XM_FLOATS + step * ((1 + NSG) * MP) + (c >> 1);
-                uint4 xd[NB][2];                              // B fragments, held over the planes
-                float fac[NB], own[2][NB][2];
-#pragma unroll
-                for (int nb = 0; nb < NB; ++nb) {
-                    xd[nb][0] = xb[nb * 64];
-                    xd[nb][1] = xb[nb * 64 + 32];
-                    fac[nb] = (c & 1) ? fminf(meta[2 * nb] * 65536.f, 3.4028235e38f) : meta[2 * nb];
-                }
+                const float* meta = sM + x.i * XM_FLOATS + step * XM_STEP;
+                float own[2][NB][2];
                 const uint32_t pb = smem_addr(wb);
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {
                     const float z = half_bits(parameter(pb, r, 0, Q) & offset_mask);
 #pragma unroll
-                    for (int nb = 0; nb < NB; ++nb) own[r >> 1][nb][r & 1] = z * ((c & 1) ? 0.f : meta[MP + 2 * nb]);
+                    for (int nb = 0; nb < NB; ++nb) own[r >> 1][nb][r & 1] = z * ((c & 1) ? 0.f : meta[MP + 2 * nb + (c >> 1)]);
                 }
                 if (use_planes) {
+                    uint4 xd[NB][2];                          // B fragments, held over the planes
+                    float fac[NB];
+                    auto load_digits = [&](int pass, float unit) {
 #pragma unroll
-                    for (int j = 0; j < Q; ++j) {
+                        for (int nb = 0; nb < NB; ++nb) {
+                            xd[nb][0] = xb[pass * (NB * 256) + nb * 64];
+                            xd[nb][1] = xb[pass * (NB * 256) + nb * 64 + 32];
+                            fac[nb] = (c & 1) ? fminf(meta[2 * nb + (c >> 1)] * 65536.f, 3.4028235e38f) * unit : meta[2 * nb + (c >> 1)] * unit;
+                        }
+                    };
+                    auto plane = [&](int j) {
                         uint32_t pw[4];
 #pragma unroll
                         for (int r = 0; r < 4; ++r) {
@@ -534,7 +585,7 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
 #pragma unroll
                             for (int r = 0; r < 4; ++r)
 #pragma unroll
-                                for (int i = 0; i < 2; ++i) f[r][i] = pw[r] & (0x01010101u << (2 * kk + i));
+                                for (int i = 0; i < 2; ++i) f[r][i] = (kk < 2 ? pw[r] : pw[r] >> 4) & (0x01010101u << (2 * (kk & 1) + i));
 #pragma unroll
                             for (int nb = 0; nb < NB; ++nb) {
                                 const uint4 xv = xd[nb][kk >> 1];
@@ -553,6 +604,14 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
                                 own[r >> 1][nb][r & 1] = fmaf(sc, (float)(v[0] + 256 * v[1]) * fac[nb], own[r >> 1][nb][r & 1]);
                             }
                         }
+                    };
+                    load_digits(0, 1.f);
+#pragma unroll
+                    for (int j = 0; j < Q; ++j) plane(j);
+                    if (__builtin_expect(reinterpret_cast<const uint32_t*>(meta)[2 * MP] != 0u, 0)) {        // what the digits leave, in units 2^15 times smaller
+                        load_digits(1, 0x1p-15f);
+#pragma unroll 1
+                        for (int j = 0; j < Q; ++j) plane(j);
                     }
                 }
 #pragma unroll
@@ -566,7 +625,7 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
             if (step < steps_of(chunk0 + cu)) {
                 const uint32_t wb = smem_addr(sW) + (uint32_t)(w.i * C::UNIT_BYTES);
                 const uint32_t xb = smem_addr(sX) + (uint32_t)(x.i * XF_BYTES + step * (NB * 2048) + lane * 16);
-                const float* meta = sM + x.i * XM_FLOATS + step * ((1 + NSG) * MP) + 2 * c;
+                const float* meta = sM + x.i * XM_FLOATS + step * XM_STEP + 2 * c;
                 uint4 xh[NB][4];                              // B fragments, held over the planes
 #pragma unroll
                 for (int nb = 0; nb < NB; ++nb)
@@ -761,7 +820,7 @@ template <int Q, int G, int NB, bool BYTES, bool FOLD = false>
 int launch_frag_cfg(const GemmArgs& g, int num_sms, cudaStream_t stream) {
     using C = FragCfg<Q, G>;
     constexpr int kMaxSmem = 232448, MP = (BYTES ? 2 : 8) * NB;
-    constexpr int kFixed = kXSlots * (NB * (BYTES ? 4096 : 8192) + 4 * (1 + C::NSG) * MP * 4) + 4 * MP * kSumStride * 4 + kNumBars * 8 + 64;
+    constexpr int kFixed = kXSlots * (NB * 8192 + 4 * ((1 + C::NSG) * MP + (BYTES ? 1 : 0)) * 4) + 4 * MP * kSumStride * 4 + kNumBars * 8 + 64;
     static bool configured[64] = {};
     int dev = 0;
     cudaGetDevice(&dev);

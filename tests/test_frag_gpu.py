@@ -59,6 +59,49 @@ def test_rows_as_digits(q, N, K, M):
     assert np.all(np.abs(y - ref) <= 2 * K * 2.0 ** -24 * hlq.magnitude_bound(X, layer.scales, layer.offsets, 128))
 
 
+def clear_of_large_values(seed, q, N, K, M, large, size):
+    """A layer and activations of the given size with one large value in every 128 k, whose bits are clear and whose group has no offset:
+    no result depends on it.  Returns also the activations without it."""
+    layer = workloads.hlq_layer(seed, f"frag/large/{q}/{N}/{K}", q, 128, N, K)
+    at = 128 * np.arange(K // 128) + 37 * np.arange(K // 128) % 128
+    layer.planes[:, :, at] = 0
+    layer.offsets[:] = 0
+    X = (synth.activations(seed, f"frag/large/x/{M}/{K}", M, K).astype(np.float32) * size).astype(np.float16)
+    X[:, at] = 0
+    with_large = X.copy()
+    with_large[:, at] = np.float16(large)
+    return layer, with_large, X
+
+
+# Digits hold every value exactly, also next to one of another size.  Bound: a result is a sum of K / 128 groups of q products, each exact up to
+# one rounding in its lower and one in its upper digits' part (together at most 3 |x|), added over a step, the chunks, the four steps of a chunk and
+# the parts of a tile: at most q + K / 512 + 11 roundings.  Without its lowest digit a value would be off by 2^-21 of the large one.
+@pytest.mark.parametrize("q,N,K,M", [(1, 4100, 4224, 2), (2, 4100, 4224, 2), (4, 4100, 4224, 2), (2, 300, 1408, 4), (3, 129, 640, 3), (4, 300, 4224, 4)])
+@pytest.mark.parametrize("large,size", [(2.0 ** 10, 0.02), (2.0 ** 13, 1.0), (-65504.0, 1.0), (65504.0, 2.0 ** -18)])
+def test_values_next_to_a_large_one_keep_every_bit(q, N, K, M, large, size):
+    assert elutq.elutq_gemm_kernel(M, N, K, q, 128) == elutq.KERNEL_FRAGMENT
+    layer, X, small = clear_of_large_values(69, q, N, K, M, large, size)
+    packed = pack_layer(layer)
+    ref = hlq.matmul(small, layer.planes, layer.scales, layer.offsets, 128)
+    A = hlq.magnitude_bound(small, layer.scales, layer.offsets, 128)
+    for flags in (0, elutq.FLAG_SKIP_OFFSET):
+        y = gemm_f32(X, packed, N, K, flags)
+        assert np.all(np.abs(y - ref) <= 3 * (q + K / 512 + 11) * 2.0 ** -24 * A)
+        assert hlq.rel_fro_error(y, ref) <= 4e-7           # (about 1e-7)
+
+
+@pytest.mark.parametrize("q,N,K,M", [(2, 4100, 4224, 2), (3, 300, 1408, 4)])
+def test_group_sums_are_fp32_sums(q, N, K, M):
+    # many values of one sign that are small next to one: a sum of 128 in pairs has 7 roundings, and the groups' products and sums as above
+    layer = workloads.hlq_layer(70, f"frag/sums/{q}/{N}/{K}", q, 128, N, K)
+    X = np.full((M, K), np.float16(0.49 * 2.0 ** -11))
+    X[:, 77::128] = np.float16(2.0 ** 13)
+    y, ref = gemm_f32(X, pack_layer(layer), N, K, elutq.FLAG_OFFSET_ONLY), hlq.offset_term(X, layer.offsets, 128)
+    A = hlq.offset_term(np.abs(X), np.abs(layer.offsets), 128)
+    assert np.all(np.abs(y - ref) <= (7 + K / 512 + 11) * 2.0 ** -24 * A)
+    assert hlq.rel_fro_error(y, ref) <= 7 * 2.0 ** -24
+
+
 def test_fragment_kernel_reports_a_wait_that_runs_out():
     q, G, N, K, M = 2, 64, 512, 2048, 12
     layer = workloads.hlq_layer(61, "frag/expiry", q, G, N, K)
