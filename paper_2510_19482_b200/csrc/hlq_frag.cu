@@ -23,7 +23,7 @@
 //            them together below 2^24); a batch row takes four of an MMA's 8 columns.  A lane's two digits are put together in its
 //            registers, lower and upper ones at the end.
 //            How often there is a rest: no step in 10000 of N(0,1) activations, 5 in 1000 with 1 % of the channels times 20.  us at 28672 x
-//            4096, M = 4, q = 2, 3, 4: as halves 25.2, 31.8, 38.7, without the second pass and the shift 23.3, 29.1, 35.6, so 25.4, 30.3, 36.0.
+//            4096, M = 4, q = 2, 3, 4: as halves 25.2, 31.8, 38.7, without the second pass and the shift 23.3, 29.1, 35.6, so 24.1, 29.5, 35.4.
 //   k order  an MMA sums over k, so A and B only have to agree on which k a lane holds.  Lane c of a quad takes the bytes of word c
 //            of the row's 128 k (at G = 64: bytes 2c, 2c+1 of each group) as two sub-words with one byte in each half, twice: a
 //            left shift by 2 brings the upper copy's bits 0-3 to the four positions, one by 6 the lower copy's bits 4-7 (as
@@ -159,7 +159,7 @@ __device__ __noinline__ void store_rest(const unsigned short* x, int K, int M, i
 #pragma unroll 1
     for (int m = 0; m < rows; ++m) {
         uint32_t d[4] = {};
-        if (m < M && meta[m] < 1.f) {                         // (2^127: not all finite)
+        if (m < M) {
             const int F = 127 - (int)(__float_as_uint(meta[m]) >> 23);
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
@@ -169,6 +169,45 @@ __device__ __noinline__ void store_rest(const unsigned short* x, int K, int M, i
         }
         store_digits(frag + (m >> 1) * 256 + (m & 1) * 64, d);
     }
+}
+
+// What chunks [chunk, end) add to Y[m][n], element by element (G = 128).  For infinities and NaN, of which digits cannot say what a bit
+// leaves: an infinite activation is none where its bit is 0, an infinite scale or offset times sums of both signs is an infinity.  Some 500
+// instructions a step; no call with finite values comes here.
+template <int Q>
+__device__ __noinline__ float plain_sum(const __half* __restrict__ x, const uint8_t* __restrict__ tiles, size_t chunk_bytes, int l, int chunk, int end, int n_steps,
+                                        unsigned flags) {
+    using C = FragCfg<Q, 128>;
+    const int last = min(4 * end, n_steps);
+    float y = 0.f;
+#pragma unroll 1
+    for (int s = 4 * chunk; s < last; ++s) {                  // (x: row m; tiles: the row block's of chunk 0; l: the row in it)
+        const int u = (s >> 1) & 1, h = s & 1;
+        const uint8_t* tb = tiles + (size_t)(s >> 2) * chunk_bytes;
+        const uint8_t* planes = tb + (u * Q * 32 + 16 * h + l) * 16;
+        const uint8_t* params = tb + C::PLANE_BYTES + (16 * h + l) * 4;
+        const unsigned short* xs = reinterpret_cast<const unsigned short*>(x) + s * 128;
+        float sum[Q + 1] = {};                                // of the planes; of the group
+#pragma unroll 1
+        for (int b = 0; b < 16; ++b) {
+#pragma unroll 1
+            for (int i = 0; i < 8; ++i) {
+                const float v = half_bits(__ldg(xs + 8 * b + i));
+#pragma unroll
+                for (int j = 0; j < Q; ++j) sum[j] += planes[j * 512 + ((b - l) & 15)] >> i & 1 ? v : 0.f;
+                sum[Q] += v;
+            }
+        }
+        float own = 0.f;
+#pragma unroll
+        for (int j = 0; j <= Q; ++j) {                        // scales, offset
+            const int rec = u * (Q + 1) + j;
+            const float p = half_bits(*reinterpret_cast<const unsigned short*>(params + (rec >> 1) * 128 + (rec & 1) * 2));
+            if (!(flags & (j < Q ? ELUTQ_FLAG_OFFSET_ONLY : ELUTQ_FLAG_SKIP_OFFSET))) own = fmaf(p, sum[j], own);
+        }
+        y += own;
+    }
+    return y;
 }
 
 // NB = blocks of 8 columns (MMA N): of 8 batch rows, or (BYTES) of two with four digits each.  FOLD: long runs of units, whose sums are
@@ -326,15 +365,13 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
 #pragma unroll
                         for (int e = 0; e < 4; ++e) {
                             const int n = __float2int_rn(x[m][e] * scale);
-                            rest |= (float)n != x[m][e] * scale && top[m] < 0x7c00u;
+                            rest |= (float)n != x[m][e] * scale;
                             d[e] = (uint32_t)n;
-                            // Not all finite: an infinity counts as a small number in the lowest digit, everything else of its row as nothing, and
-                            // a factor of 2^127 makes an infinity of what the planes leave of it; a NaN makes NaN of the row.
-                            if (top[m] >= 0x7c00u) d[e] = fabsf(x[m][e]) <= 65504.f ? 0u : x[m][e] < 0.f ? 0u - (64u >> (bit & 3)) : 64u >> (bit & 3);
                         }
                         store_digits(frag + (m >> 1) * 256 + (m & 1) * 64, d);
                         four[m] = (x[m][0] + x[m][1]) + (x[m][2] + x[m][3]);
-                        if (lane == 0) meta[m] = top[m] < 0x7c00u ? power_of_two(-F) : __int_as_float(top[m] > 0x7c00u ? 0x7fffffff : 254 << 23);
+                        // (a row that is not all finite: the write-out sums it anew)
+                        if (lane == 0) meta[m] = top[m] < 0x7c00u ? power_of_two(-F) : __int_as_float(0x7fffffff);
                     }
                     // the rows' sums over the lanes, row m in lanes m, m + MP, ...
                     auto fold = [&](float even, float odd, int b) {
@@ -453,6 +490,7 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
     const int step = warp >> 2, rp = warp & 3;                // the warp's 128 k of every chunk, its 32 rows of the tile
     const bool use_planes = !(a.g.flags & ELUTQ_FLAG_OFFSET_ONLY), use_offset = !(a.g.flags & ELUTQ_FLAG_SKIP_OFFSET);
     const uint32_t offset_mask = use_offset ? 0xffffffffu : 0u;
+    const bool add_offset = use_offset && !(lane & 1);        // BYTES: by the lanes of the lower digits
 
     // Where the lane finds its bytes of rows gq and gq + 8 of a packed tile (the layout rotates groups and bytes by the row):
     // two 32-bit words at off0 / off1 (G = 64: per group), of which the selectors pick the bytes of a sub-word.
@@ -556,9 +594,9 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
                 const uint32_t pb = smem_addr(wb);
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {
-                    const float z = half_bits(parameter(pb, r, 0, Q) & offset_mask);
+                    const float z = half_bits(parameter(pb, r, 0, Q));
 #pragma unroll
-                    for (int nb = 0; nb < NB; ++nb) own[r >> 1][nb][r & 1] = z * ((c & 1) ? 0.f : meta[MP + 2 * nb + (c >> 1)]);
+                    for (int nb = 0; nb < NB; ++nb) own[r >> 1][nb][r & 1] = add_offset ? z * meta[MP + 2 * nb + (c >> 1)] : 0.f;
                 }
                 if (use_planes) {
                     uint4 xd[NB][2];                          // B fragments, held over the planes
@@ -568,7 +606,7 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
                         for (int nb = 0; nb < NB; ++nb) {
                             xd[nb][0] = xb[pass * (NB * 256) + nb * 64];
                             xd[nb][1] = xb[pass * (NB * 256) + nb * 64 + 32];
-                            fac[nb] = (c & 1) ? fminf(meta[2 * nb + (c >> 1)] * 65536.f, 3.4028235e38f) * unit : meta[2 * nb + (c >> 1)] * unit;
+                            fac[nb] = meta[2 * nb + (c >> 1)] * ((c & 1) ? 65536.f * unit : unit);
                         }
                     };
                     auto plane = [&](int j) {
@@ -792,6 +830,11 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
             float y = sSum[m * kSumStride + row];
 #pragma unroll
             for (int s = 1; s < 4; ++s) y += sSum[(s * MP + m) * kSumStride + row];
+            if constexpr (BYTES) {
+                if (__builtin_expect((__float_as_uint(y) & 0x7f800000u) == 0x7f800000u, 0) && n < N)
+                    y = plain_sum<Q>(a.g.X + (size_t)m * a.g.K, a.g.tiles + (size_t)(n >> 4) * C::TILE_BYTES, (size_t)a.g.n_rb * C::TILE_BYTES, n & 15, chunk0,
+                                     chunk0 + n_units, a.n_steps, a.g.flags);
+            }
             if (whole) {
                 if (n < N) put(mb + m, n, y);
             } else if ((size_t)n < n_pad) {

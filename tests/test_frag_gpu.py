@@ -166,6 +166,49 @@ def test_activations_that_are_not_finite(G, M, values):
     assert np.array_equal(y[keep], clean[keep])
 
 
+def plain_row(x, layer, G, flags):
+    """One row of the product in 64 bits, element by element: what is not selected is not there (0 * infinity does not come up)."""
+    x, groups = x.astype(np.float64), (layer.N, layer.K // G, G)
+    with np.errstate(invalid="ignore", over="ignore"):
+        y = np.zeros(layer.N)
+        if flags != elutq.FLAG_OFFSET_ONLY:
+            for j in range(layer.q):
+                y += (layer.scales[:, :, j].astype(np.float64) * np.where(layer.planes[j] != 0, x, 0.0).reshape(groups).sum(-1)).sum(-1)
+        if flags != elutq.FLAG_SKIP_OFFSET:
+            y += (layer.offsets.astype(np.float64) * x.reshape(groups[1:]).sum(-1)).sum(-1)
+    return y
+
+
+@pytest.mark.parametrize("q,N,K,M", [(1, 4100, 4224, 2), (2, 4100, 4224, 2), (3, 300, 1024, 4), (4, 300, 1408, 3), (2, 300, 14336, 4)])
+@pytest.mark.parametrize("where", ["activation", "activations", "nan", "scale", "offset"])
+def test_infinities_up_to_four_rows(q, N, K, M, where):
+    # every result is of the kind that the sum of its terms has, finite ones have their value, and no other row or output changes
+    layer = workloads.hlq_layer(71, f"frag/inf/{q}/{N}/{K}", q, 128, N, K)
+    layer.offsets[::7] = 0
+    X = synth.activations(71, f"frag/inf/x/{M}/{K}", M, K)
+    clean, rows = gemm_f32(X, pack_layer(layer), N, K), np.arange(M)
+    if where in ("activation", "activations", "nan"):
+        X[1, 200] = np.nan if where == "nan" else np.inf
+        if where == "activations":
+            X[1, K - 3] = -np.inf
+        touched = np.broadcast_to((rows == 1)[:, None], (M, N))
+    else:
+        (layer.scales[:, :, 0] if where == "scale" else layer.offsets)[5:40, 1] = np.inf
+        touched = np.broadcast_to((np.arange(N) >= 5) & (np.arange(N) < 40), (M, N))
+    packed = pack_layer(layer)
+    for flags in (0, elutq.FLAG_SKIP_OFFSET, elutq.FLAG_OFFSET_ONLY):
+        y = gemm_f32(X, packed, N, K, flags)
+        ref = np.stack([plain_row(x, layer, 128, flags) for x in X])
+        for kind in (np.isnan, np.isposinf, np.isneginf):
+            assert np.array_equal(kind(y), kind(ref))
+        finite = np.isfinite(ref)
+        A = hlq.magnitude_bound(np.nan_to_num(X, posinf=0.0, neginf=0.0), np.nan_to_num(layer.scales, posinf=0.0), np.nan_to_num(layer.offsets, posinf=0.0), 128)
+        assert np.all(np.abs(np.where(finite, y, 0) - np.where(finite, ref, 0)) <= 2 * K * 2.0 ** -24 * A)
+        if flags == 0:
+            assert np.array_equal(y[~touched], clean[~touched])
+    assert elutq.elutq_device_status() == 0
+
+
 @pytest.mark.parametrize("q,N,K,M", [(1, 129, 64, 257), (2, 1000, 1024, 33), (2, 2048, 4096, 130), (3, 4000, 2880, 57), (4, 300, 4160, 100)])
 def test_batch_blocks_of_one_launch(q, N, K, M):
     # blocks of 8 and 16 rows with a remainder, several to a row tile, output tiles shared by CTAs; one launch, no call slower for its rows
