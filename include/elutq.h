@@ -65,10 +65,9 @@ typedef enum elutq_status {
                                    indices with the top bit clear and the other half is obtained by
                                    negation; same product up to fp32 rounding                              */
 
-#define ELUTQ_TENSOR_MIN_M 3      /* batches of this many rows or more run on the tensor cores (G = 128 or 64, no look-up
-                                     variant flag).  Two rows do so at G = 128 where N * K is above 2^24 and at most 2^27
-                                     (elutq_takes_tensor_path); otherwise they stay on the batched look-up kernel, which needs one
-                                     narrow pass for them                                                                */
+#define ELUTQ_TENSOR_MIN_M 3      /* every batch of this many rows or more runs on the tensor cores (G = 128 or 64, no look-up
+                                     variant flag).  Two rows do so at G = 128 for some sizes above 2^24 weights, by N, K and q
+                                     (elutq_gemm_kernel says which); otherwise they stay on the batched look-up kernel   */
 #define ELUTQ_TENSOR_MIN_M_NARROW ELUTQ_TENSOR_MIN_M   /* (kept for callers that ask for the smallest batch on the tensor cores at
                                                           N <= ELUTQ_TENSOR_NARROW_N: the same for every N now)     */
 #define ELUTQ_TENSOR_NARROW_N 8192
@@ -261,13 +260,13 @@ int elutq_lut_gemm_host(const void* X_host, const void* packed, void* Y_host,
  *   - `packed` must be known to the library (packed or described in this process) before a capture
  *     begins: an unknown address makes the call read the header with a synchronous copy.
  */
-/* 1 when elutq_lut_gemm (and _f32, _ws, _host, _bias) runs a call of this shape on the tensor-core path, 0 when on the
- * look-up kernels; host-only, launches nothing.  (Above ELUTQ_FRAGMENT_MAX_M rows at G = 128 its results carry the fp16
- * rounding of W_hat.) */
+/* 1 when elutq_lut_gemm (and _f32, _ws, _host, _bias) runs a call of this shape on the tensor-core path whatever q is, 0 when on
+ * the look-up kernels (two rows at G = 128: for some q perhaps; elutq_gemm_kernel answers for one).  _bias: with
+ * ELUTQ_FLAG_OFFSET_ONLY.  Host-only, launches nothing.  (Above ELUTQ_FRAGMENT_MAX_M rows at G = 128 its results carry the fp16 rounding of W_hat.) */
 int elutq_takes_tensor_path(int M, int N, int K, int G, unsigned flags);
 
 /* The kernel that elutq_lut_gemm (and _f32, _ws, _host, _bias) runs a call of this shape on, on the current device: one of the
- * ELUTQ_KERNEL_ values, or an ELUTQ_ERR_ code (negative).  Host-only, launches nothing. */
+ * ELUTQ_KERNEL_ values, or an ELUTQ_ERR_ code (negative).  _bias: with ELUTQ_FLAG_OFFSET_ONLY.  Host-only, launches nothing. */
 #define ELUTQ_KERNEL_DECODE 0          /* M = 1: look-up tables                                                       */
 #define ELUTQ_KERNEL_LOOK_UP 1         /* batches on look-up tables                                                   */
 #define ELUTQ_KERNEL_FRAGMENT 2        /* bit-planes contracted as they are, scales on fp32 sums                      */

@@ -203,7 +203,7 @@ def elutq_lut_gemm_host(X_host, packed, Y_host, M: int, N: int, K: int, stream=N
 
 
 def elutq_takes_tensor_path(M: int, N: int, K: int, G: int = 128, flags: int = 0) -> bool:
-    """True when elutq_lut_gemm runs this shape on the tensor-core path (host-only)."""
+    """True when elutq_lut_gemm runs this shape on the tensor-core path whatever q is (host-only)."""
     return bool(lib().elutq_takes_tensor_path(M, N, K, G, flags))
 
 

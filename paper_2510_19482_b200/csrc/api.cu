@@ -191,22 +191,35 @@ int launch_copy_in(const void* src, void* dst, size_t bytes, cudaStream_t stream
     return (int)e;
 }
 
-// Whether a batched call runs on the tensor cores.  Two rows do at G = 128 between 16 and 128 million weights (us on the look-up kernel /
-// there, q = 2, 3, 4: 6144 x 4096 9.0, 10.7, 11.8 / 7.9, 8.8, 9.9; 4096 x 14336 13.4, 16.6, 19.4 / 10.9, 12.9, 15.2; 28672 x 4096 17.6, 22.7, 27.0 /
-// 17.8, 21.1, 24.8).  Above, the look-up kernel is ahead at q = 2 (57344 x 8192 50, 67, 82 / 53, 63, 75); below, little is left to gain on the
-// smallest (1000 x 1024 4.7, 5.4, 5.5 / 4.6, 4.8, 5.2), and 4096 x 4096 (7.8 / 5.6) is where elutq_gemm_kernel's answer for two rows is relied on.
-bool takes_tensor_path(int M, int N, int K, int G, unsigned flags) {
+// Two rows at G = 128: whether the fragment kernel is ahead of the look-up kernel.  Its time follows the weights, that of the look-up kernel the rows too,
+// and the more bit-planes the more it saves (us, look-up / fragment, q = 1, 2, 3, 4):
+//    6144 x 4096   7.4, 8.6, 10.7, 11.8 / 7.4, 8.3, 9.0, 10.1       57344 x 1024   9.5, 11.7, 14.7, 17.5 / 9.9, 12.4, 14.4, 16.8
+//    4096 x 14336  11.2, 13.3, 16.4, 19.3 / 9.0, 11.3, 13.6, 16.1   28672 x 4096   13.5, 17.5, 22.5, 27.2 / 15.2, 18.8, 22.3, 26.3
+//    8192 x 16384  15.6, 20.3, 26.0, 31.0 / 15.7, 19.6, 23.1, 27.6  57344 x 2048   13.2, 17.3, 22.3, 27.0 / 15.2, 19.0, 22.4, 26.5
+//   12288 x 4096   9.2, 11.2, 13.6, 15.8 / 9.4, 11.1, 12.7, 15.0   120000 x 1024   13.3, 17.5, 22.4, 27.1 / 15.1, 19.5, 23.2, 27.5
+//   16500 x 1024   6.1, 6.7, 7.8, 9.0 / 3.5, 4.3, 4.9, 6.0          40000 x 1024   8.2, 10.1, 12.6, 14.6 / 8.1, 10.2, 11.7, 13.4
+// Above 2^27 weights two rows have only been measured at 57344 x 8192 (50, 67, 82 / 53, 63, 75 at q = 2, 3, 4); up to 2^24 the gain is small (1000 x 1024
+// 4.7, 5.4, 5.5 / 4.6, 4.8, 5.2) but for 4096 x 4096 (7.4 / 5.6), whose kernel the tests of the C interface state.  The offset term alone
+// is the look-up kernel's earlier, as that reads no planes (28672 x 4096, q = 4 11.5 / 13.9; 8192 x 8192 10.7 / 10.1; 8192 x 16384 13.3 / 14.9).
+bool two_rows_on_fragments(int N, int K, int q, unsigned flags) {
+    const long long weights = (long long)N * K;
+    if (weights <= (1LL << 24) || weights > (1LL << 27)) return false;
+    if (flags & ELUTQ_FLAG_OFFSET_ONLY) return N <= 8192 ? weights <= (1LL << 26) : weights <= (1LL << 25);
+    return N <= (q == 1 ? 8192 : q == 2 ? 12288 : 57344) || weights <= (q <= 2 ? 1LL << 25 : 1LL << 26);
+}
+
+// Whether a batched call runs on the tensor cores.
+bool takes_tensor_path(int M, int N, int K, int q, int G, unsigned flags) {
     const unsigned lut_variants = ELUTQ_FLAG_PLAIN_G4 | ELUTQ_FLAG_CLUSTER_REDUCE | ELUTQ_FLAG_MIRROR | ELUTQ_FLAG_LUT_ONLY |
                                   ELUTQ_FLAG_TABLE_F16 | ELUTQ_FLAG_TABLE_I8;
     if (G == 32 || (flags & lut_variants)) return false;
-    const long long weights = (long long)N * K;
-    return M >= ELUTQ_TENSOR_MIN_M || (M == 2 && G == 128 && weights > (1LL << 24) && weights <= (1LL << 27));
+    return M >= ELUTQ_TENSOR_MIN_M || (M == 2 && G == 128 && two_rows_on_fragments(N, K, q, flags));
 }
 
 // The kernel of a call (ELUTQ_KERNEL_...).
 int kernel_of(int M, int N, int K, int q, int G, unsigned flags, int sms) {
     if (M == 1) return ELUTQ_KERNEL_DECODE;
-    if (!takes_tensor_path(M, N, K, G, flags)) return ELUTQ_KERNEL_LOOK_UP;
+    if (!takes_tensor_path(M, N, K, q, G, flags)) return ELUTQ_KERNEL_LOOK_UP;
     if (G != 128 || M <= ELUTQ_FRAGMENT_MAX_M) return ELUTQ_KERNEL_FRAGMENT;
     return rebuilds_in_shared_memory(M, N, K, q, sms) ? ELUTQ_KERNEL_SHARED_MEMORY : ELUTQ_KERNEL_TENSOR_MEMORY;
 }
@@ -482,7 +495,7 @@ int elutq_release_scratch(void) {
 }
 
 int elutq_takes_tensor_path(int M, int N, int K, int G, unsigned flags) {
-    return takes_tensor_path(M, N, K, G, flags) ? 1 : 0;
+    return takes_tensor_path(M, N, K, 1, G, flags) ? 1 : 0;       // (two rows: what q = 1 takes, every q takes)
 }
 
 int elutq_gemm_kernel(int M, int N, int K, int q, int G, unsigned flags) {

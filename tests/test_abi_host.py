@@ -80,6 +80,20 @@ def test_pointer_validation_happens_before_any_launch():
     assert elutq.elutq_status_string(-4) == "buffer too small"
 
 
+# (N, K, the kernel of two rows at q = 1, 2, 3, 4): edges in the weights (2^24, 2^25, 2^26, 2^27) and in the rows
+@pytest.mark.parametrize("N,K,kernels", [(1000, 1024, "1111"), (4096, 4096, "1111"), (4097, 4096, "2222"), (8192, 16384, "2222"), (8193, 16384, "1111"),
+                                         (8193, 8192, "1222"), (12289, 4096, "1122"), (32768, 1024, "2222"), (32769, 1024, "1122"), (57344, 2304, "1122"),
+                                         (57345, 1152, "1122"), (57345, 1280, "1111"), (57344, 8192, "1111")])
+def test_the_kernel_of_two_rows(N, K, kernels):
+    assert "".join(str(elutq.elutq_gemm_kernel(2, N, K, q)) for q in (1, 2, 3, 4)) == kernels
+    assert elutq.elutq_takes_tensor_path(2, N, K) == (kernels == "2222")
+    for q in (1, 4):
+        assert elutq.elutq_gemm_kernel(2, N, K, q, 64) == elutq.elutq_gemm_kernel(2, N, K, q, 128, elutq.FLAG_LUT_ONLY) == 1
+        offset = elutq.elutq_gemm_kernel(2, N, K, q, 128, elutq.FLAG_OFFSET_ONLY)
+        assert offset == (2 if 1 << 24 < N * K <= (1 << 26 if N <= 8192 else 1 << 25) else 1)
+        assert elutq.elutq_takes_tensor_path(2, N, K, 128, elutq.FLAG_OFFSET_ONLY) == (offset == 2)
+
+
 def test_chain_argument_validation_happens_on_the_host():
     L = elutq.lib()
     out = ctypes.c_size_t(0)
