@@ -913,12 +913,15 @@ int launch_frag_cfg(const GemmArgs& g, int num_sms, cudaStream_t stream) {
 
 template <int Q, int G>
 int launch_frag_qg(const GemmArgs& g, int num_sms, cudaStream_t stream) {
-    // Up to four rows: as bytes (us as halves / bytes, M = 4, q = 2, 3, 4: 28672 x 4096 25.0, 31.7, 38.5 / 23.3, 29.0, 35.5; 4096 x 14336
-    // 15.1, 18.7, 22.8 / 13.8, 17.2, 21.0; 4096 x 4096 7.4, 8.3, 9.5 / 6.9, 7.9, 9.4).  At G = 64 the sums of a step's two groups cost what
-    // the masks save (28672 x 4096, M = 4 27.6, 35.3, 43.0 / 28.7, 35.4, 41.5; 4096 x 4096 8.0, 9.4, 10.9 / 8.5, 9.9, 11.0).
+    // Up to four rows: as bytes (us as halves / bytes, M = 4, q = 2, 3, 4: 28672 x 4096 25.1, 31.6, 38.2 / 24.0, 29.4, 35.1; 4096 x 14336
+    // 15.0, 18.5, 22.8 / 14.1, 17.3, 20.9; 4096 x 4096 7.4, 8.3, 9.5 / 7.2, 8.1, 9.1), but for three and four at q = 1, where preparing the
+    // digits takes as long as the one plane (18.7, 11.1, 6.1 / 19.5, 11.5, 6.2; two rows at 4096 x 14336 9.0, on the look-up kernel 11.1).  At G = 64 the sums of a
+    // step's two groups cost what the masks save (28672 x 4096, M = 4 27.6, 35.3, 43.0 / 28.7, 35.4, 41.5; 4096 x 4096 8.0, 9.4, 10.9 / 8.5, 9.9, 11.0).
     if constexpr (G == 128) {
         if (g.M <= 2) return launch_frag_cfg<Q, G, 1, true>(g, num_sms, stream);
-        if (g.M <= 4) return launch_frag_cfg<Q, G, 2, true>(g, num_sms, stream);
+        if constexpr (Q > 1) {
+            if (g.M <= 4) return launch_frag_cfg<Q, G, 2, true>(g, num_sms, stream);
+        }
     }
     if constexpr (G == 64) {
         // The height of a batch block, by the longest run of units: a unit takes u us, the first one of a taller block u0 more.  (Fitted
