@@ -70,6 +70,17 @@ struct GemmArgs {
     unsigned wait_limit;     // poll limit of the tensor-core kernel's bounded waits (0: the default)
 };
 
+// n / d for 0 <= n < 2^31 by one multiplication: a division by a runtime value costs some 20 instructions, a 64-bit one 100.
+struct Div {
+    int d;
+    unsigned long long m;       // m d = 2^64 + e with 0 <= e < d, so n m / 2^64 exceeds n / d by less than n / 2^64 (0 stands for d = 1)
+    __host__ void set(int d_) {
+        d = d_;
+        m = d_ == 1 ? 0ull : ~0ull / (unsigned)d_ + 1ull;
+    }
+    __device__ __forceinline__ int of(int n) const { return m == 0ull ? n : (int)__umul64hi((unsigned long long)n, m); }
+};
+
 // Kernel launchers (defined in the .cu files); return a cudaError_t value.
 int launch_pack(const uint8_t* planes, const __half* scales, const __half* offsets,
                 const Geo& g, uint8_t* packed, cudaStream_t stream);

@@ -51,17 +51,6 @@ constexpr uint32_t kFragWaitLimit = 1u << 22;
 constexpr int kMaxRing = 8, kXSlots = 2;        // weight units (at most), units of prepared activations
 constexpr int kSumStride = kUnitRows + 4;       // floats per batch row of the sum buffer (conflict-free for fragments)
 
-// n / d for 0 <= n < 2^31 by one multiplication: a runtime division costs 50 cycles and more, and a call of few units does a dozen in a row.
-struct Div {
-    int d;
-    unsigned long long m;       // m d = 2^64 + e with 0 <= e < d, so n m / 2^64 exceeds n / d by less than n / 2^64 (0 stands for d = 1)
-    __host__ void set(int d_) {
-        d = d_;
-        m = d_ == 1 ? 0ull : ~0ull / (unsigned)d_ + 1ull;
-    }
-    __device__ __forceinline__ int of(int n) const { return m == 0ull ? n : (int)__umul64hi((unsigned long long)n, m); }
-};
-
 struct FragArgs {
     GemmArgs g;
     int n_steps;                // 128-k steps of the whole K

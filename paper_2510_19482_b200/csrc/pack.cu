@@ -30,17 +30,6 @@ __device__ __forceinline__ uint32_t nonzero_bytes(uint32_t x) {
     return (m * 0x10204080u) >> 28;
 }
 
-// n / d for 0 <= n < 2^31 by one multiplication (a division by a runtime value costs some 20 instructions, a 64-bit one 100).
-struct Div {
-    int d;
-    unsigned long long m;       // m d = 2^64 + e with 0 <= e < d, so n m / 2^64 exceeds n / d by less than n / 2^64 (0 stands for d = 1)
-    __host__ void set(int d_) {
-        d = d_;
-        m = d_ == 1 ? 0ull : ~0ull / (unsigned)d_ + 1ull;
-    }
-    __device__ __forceinline__ int of(int n) const { return m == 0ull ? n : (int)__umul64hi((unsigned long long)n, m); }
-};
-
 constexpr int kPackWarps = 8;
 
 // One warp per 32 plane vectors of a tile: (tile, vec = u*q + j), 16 rows x 2 super-groups of 128 input bytes.  A load covers whole

@@ -35,6 +35,22 @@ def test_pack_is_byte_exact_and_round_trips(q, G, N, K):
     assert np.array_equal(offsets.cpu().numpy().view(np.uint16), layer.offsets.view(np.uint16))
 
 
+# Every (q, G) with ragged N and K, and planes that begin 8 bytes after a multiple of 16 (loads of 8 bytes instead of 16)
+@pytest.mark.parametrize("q", [1, 2, 3, 4])
+@pytest.mark.parametrize("G", [32, 64, 128])
+def test_every_form_and_planes_on_8_bytes(q, G):
+    N, K = 16 * 9 + q, 512 + G * (1 if G == 128 else 3)
+    layer = workloads.hlq_layer(8, f"pack/form/{q}/{G}", q, G, N, K, signed_scales=True)
+    ref = layout.pack_reference(layer.planes, layer.scales, layer.offsets, G)
+    assert np.array_equal(pack_layer(layer).cpu().numpy(), ref)
+    room = torch.empty(q * N * K + 8, dtype=torch.uint8, device="cuda")
+    planes = room[8:].view(q, N, K)
+    planes.copy_(to_dev(layer.planes))
+    assert planes.data_ptr() % 16 == 8
+    packed = elutq.elutq_pack(planes, to_dev(layer.scales.view(np.int16)).view(torch.float16), to_dev(layer.offsets.view(np.int16)).view(torch.float16), q, G, N, K)
+    assert np.array_equal(packed.cpu().numpy(), ref)
+
+
 def test_nonzero_plane_bytes_count_as_one():
     # a weight bit is (value != 0): any non-zero byte is a set bit
     q, G, N, K = 2, 128, 16, 512
