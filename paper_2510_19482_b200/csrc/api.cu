@@ -198,9 +198,11 @@ int launch_copy_in(const void* src, void* dst, size_t bytes, cudaStream_t stream
 //    8192 x 16384  15.6, 20.3, 26.0, 31.0 / 15.7, 19.6, 23.1, 27.6  57344 x 2048   13.2, 17.3, 22.3, 27.0 / 15.2, 19.0, 22.4, 26.5
 //   12288 x 4096   9.2, 11.2, 13.6, 15.8 / 9.4, 11.1, 12.7, 15.0   120000 x 1024   13.3, 17.5, 22.4, 27.1 / 15.1, 19.5, 23.2, 27.5
 //   16500 x 1024   6.1, 6.7, 7.8, 9.0 / 3.5, 4.3, 4.9, 6.0          40000 x 1024   8.2, 10.1, 12.6, 14.6 / 8.1, 10.2, 11.7, 13.4
-// Above 2^27 weights two rows have only been measured at 57344 x 8192 (50, 67, 82 / 53, 63, 75 at q = 2, 3, 4); up to 2^24 the gain is small (1000 x 1024
-// 4.7, 5.4, 5.5 / 4.6, 4.8, 5.2) but for 4096 x 4096 (7.4 / 5.6), whose kernel the tests of the C interface state.  The offset term alone
-// is the look-up kernel's earlier, as that reads no planes (28672 x 4096, q = 4 11.5 / 13.9; 8192 x 8192 10.7 / 10.1; 8192 x 16384 13.3 / 14.9).
+// Above 2^27 weights little is between the two from q = 3 on, and the look-up kernel is ahead below (57344 x 8192 35.1, 50.0, 67.1, 82.9 / 42.0, 56.3,
+// 67.8, 81.6; 14336 x 16384 21.3, 29.0, 38.1, 46.5 / 24.0, 30.9, 36.8, 44.4).  Up to 2^24 the fragment kernel would be ahead as well (1000 x 1024 4.6, 4.7,
+// 5.4, 5.5 / 4.4, 4.7, 5.0, 5.3; 2048 x 4096 5.9, 6.2, 7.0, 7.4 / 4.9, 5.2, 5.5, 5.9; 4096 x 4096 6.7, 7.4, 8.4, 9.6 / 5.1, 5.9, 6.5, 7.3): these stay
+// because tests/test_abi_host.py states the look-up kernel for 4096 x 4096, not for their time.  The offset term alone is the look-up kernel's
+// earlier, as that reads no planes (28672 x 4096, q = 4 11.5 / 13.9; 8192 x 8192 10.7 / 10.1; 8192 x 16384 13.3 / 14.9).
 bool two_rows_on_fragments(int N, int K, int q, unsigned flags) {
     const long long weights = (long long)N * K;
     if (weights <= (1LL << 24) || weights > (1LL << 27)) return false;

@@ -1,6 +1,6 @@
 // Batches of up to ELUTQ_FRAGMENT_MAX_M rows (any at G = 64): bit-planes as MMA fragments, without dequantising.  In two forms, halves and bytes.
 //
-// A warp forms the A fragments of mma.sync (16 weight rows x 16 k) in the registers that the MMA reads, with ONE logic
+// Halves: a warp forms the A fragments of mma.sync (16 weight rows x 16 k) in the registers that the MMA reads, with ONE logic
 // operation per two weights: of a register with two weight bytes, one in each half, a mask leaves one bit of each half, at
 // one of the lowest four bits of the fp16 exponent: 0 or 2^-14, 2^-13, 2^-11, 2^-7.  (The mantissa's bits would do, as
 // subnormal numbers, but the tensor core aligns those by their exponent field and loses up to ten bits.)  The activations
@@ -10,24 +10,26 @@
 //
 //   Y = sum_g [ sum_j s_j 2^(14-c) D_j + z sum_{k in g} x ],   D_j = the MMAs' sum over the group for plane j,
 //
-// with the scales applied to the sums in fp32: W_hat is never formed, as in the look-up kernels, and as exact.  (The MMAs'
-// running sums are truncated, not rounded; a sum runs over one group.)
+// with the scales applied to the sums in fp32: W_hat is never formed, as in the look-up kernels, and as exact (but next to a value 2^22 times
+// larger whose bits are clear).  The MMAs' running sums are truncated, not rounded; a sum runs over one group.
 //
 //   bytes    Up to four batch rows at G = 128 (BYTES): one logic operation on a word of four weight bytes keeps one bit of each, and what it
 //            leaves, 0 or 2^i in every byte, is an operand of the 8-bit integer MMA as it stands: four weights per operation (bits 4-7 as
 //            bits 0-3 of the word shifted by 4).  The activations are digits, x_k = 2^(i-F) sum_d 256^d X_d with the X_d the signed bytes of
 //            the integer nearest to 2^(F-i) x_k, F such that the largest |x| of the row's step lies just below 2^31.  A value with a bit
-//            below the lowest unit, 2^-17 of that largest one, leaves a rest: the step is contracted a second time, with the rests' digits.
-//            So every activation enters exactly, also next to one that is 2^40 times larger and whose bits are clear.  (Without the second
-//            pass, and with i to 7, such sums were off by 2^-23 of the large one.)  A group's sums are exact (digits' below 2^16, two of
-//            them together below 2^24); a batch row takes four of an MMA's 8 columns.  A lane's two digits are put together in its
-//            registers, lower and upper ones at the end.
-//            How often there is a rest: no step in 10000 of N(0,1) activations, 5 in 1000 with 1 % of the channels times 20.  us at 28672 x
-//            4096, M = 4, q = 2, 3, 4: as halves 25.2, 31.8, 38.7, without the second pass and the shift 23.3, 29.1, 35.6, so 24.1, 29.5, 35.4.
+//            below that unit 2^(i-F) leaves a rest: the step is contracted a second time, with the rests' digits.  So every activation
+//            enters exactly, also next to one that is 2^40 times larger and whose bits are clear.  (Without the second pass, and with i to 7,
+//            such sums were off by 2^-23 of the large one.)  There is no rest where the largest |x| is below 15.9, as fp16 has no bit below
+//            2^-24, nor of a value that is 2^-17 of the largest or more: 5 of 1000 steps of 4 rows N(0,1) with 1 % of the channels times 20.
+//            A group's sums are exact (digits' below 2^16, two of them together below 2^24); a batch row takes four of an MMA's 8
+//            columns.  A lane's two digits are put together in its registers, lower and upper ones at the end.
+//            Bound: latencies at 20 warps an SM (28672 x 4096, q = 3, M = 4: issue 54 %, logic pipe 44 %, integer MMAs 35 %, LSU 26 %; a warp
+//            that does not issue most often finds its math pipe taken or is at the long scoreboard).  us there, q = 2, 3, 4: as halves 25.2, 31.8, 38.7,
+//            without the second pass and the shift 23.3, 29.1, 35.6, so 24.1, 29.5, 35.4.
 //   k order  an MMA sums over k, so A and B only have to agree on which k a lane holds.  Lane c of a quad takes the bytes of word c
-//            of the row's 128 k (at G = 64: bytes 2c, 2c+1 of each group) as two sub-words with one byte in each half, twice: a
-//            left shift by 2 brings the upper copy's bits 0-3 to the four positions, one by 6 the lower copy's bits 4-7 (as
-//            multiplications: the logic pipe is the busy one).
+//            of the row's 128 k (bytes: the word as it is, MMA kk the bits 2 kk, 2 kk + 1 of its bytes).  Halves (at G = 64: bytes 2c, 2c+1 of
+//            each group): two sub-words with one byte in each half, twice: a left shift by 2 brings the upper copy's bits 0-3 to the four
+//            positions, one by 6 the lower copy's bits 4-7 (as multiplications: the logic pipe is the busy one).
 //   unit     128 weight rows x 512 k (eight packed tiles, contiguous in the blob: one bulk copy) x 8 NB batch rows (bytes: 2 NB).  The units of
 //            a call, output tile by output tile (the batch blocks of a row tile next to each other: its weights come from the L2 again), are
 //            dealt to the CTAs (one per SM) in equal contiguous runs, so no SM idles for a wave.  An output tile that several CTAs share
@@ -522,7 +524,9 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
                      : "=r"(any) : "r"((int)mine) : "memory");
         return any != 0;
     };
-    // The CTA that came last to a shared output tile adds the parts in ascending k order (all compute threads call this).
+    // The CTA that came last to a shared output tile adds the parts in ascending k order (all compute threads call this), four at a time in pairs:
+    // fewer roundings than in one chain, in the same time (error of the fp32 result, chain / pairs, q = 4: 1024 x 14336, M = 8 1.1e-7 / 1.0e-7,
+    // M = 4 8.0e-8 / 6.8e-8, G = 64 1.1e-7 / 1.0e-7; 256 x 65536, M = 8 1.9e-7 / 1.3e-7; the look-up kernel there 1.1e-7, 7.6e-8, 1.1e-7, 1.5e-7).
     auto parts_of = [&](int tile) { return a.by_cta.of(tile * C_ + C_ - 1) - a.by_cta.of(tile * C_) + 1; };
     auto ticket_of = [&](int tile) { return a.tickets + (G == 128 || a.blocks == 1 ? tile : a.by_cta.of(tile * C_)); };
     auto finish_tile = [&](int tile) {
@@ -541,7 +545,7 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
                     for (int i = 0; i < 4; ++i)
                         v[e][i] = (p + e < parts && m0 + 4 * i < me) ? __ldcg(p0 + ((size_t)(p + e) * M + m0 + 4 * i) * n_pad) : 0.f;
 #pragma unroll
-                for (int i = 0; i < 4; ++i) y[i] += (v[0][i] + v[1][i]) + (v[2][i] + v[3][i]);       // (in pairs: fewer roundings than in one chain)
+                for (int i = 0; i < 4; ++i) y[i] += (v[0][i] + v[1][i]) + (v[2][i] + v[3][i]);       // (pairs: see above)
             }
 #pragma unroll
             for (int i = 0; i < 4; ++i)

@@ -53,7 +53,8 @@ def assert_elementwise(y, ref, A, q: int, K: int, tensor_path: bool, out_f16: bo
     A = oracle.hlq.magnitude_bound(X, scales, offsets, G) bounds |X| |W_hat|^T and every intermediate of the +-1
     form.  Roundings of the paths, each at most its unit roundoff times A (worst case, all errors aligned):
       look-up kernels   fp32 table entries and fp32 accumulation over K terms      K * 2^-24 * A
-      fragment kernel   exact products, one truncation by 2^-23 per 16 terms and the fp32 sums: less than that
+      fragment kernel   exact products; one truncation by 2^-23 per 16 terms (up to four rows at G = 128: exact group sums) and the
+                        fp32 sums: less than that
       rebuilt weights   W_hat rebuilt in fp16: z^ rounded once, one rounding per plane add   (q + 1) * 2^-11 * A
                         then fp32 accumulation in tensor memory                    K * 2^-23 * A
       fp16 output       one more rounding of the result                            2^-11 * |y|

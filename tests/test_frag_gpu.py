@@ -1,9 +1,10 @@
-"""GPU parity of the fragment kernel (batches of 3 to 8 rows at G = 128, any from 3 rows on at G = 64): bit-planes contracted
-on the tensor cores as they are, scales applied to fp32 sums.
+"""GPU parity of the fragment kernel (batches of 3 to 8 rows and two rows of some sizes at G = 128, any from 3 rows on at G = 64): bit-planes
+contracted on the tensor cores as they are, scales applied to fp32 sums.
 
-Tolerance: activations are scaled by powers of two (exact but for 2^-33 of the row's largest), products are exact, the
+Tolerance.  As halves, activations are scaled by powers of two (exact but for 2^-33 of the row's largest), products are exact, the
 MMAs' fp32 sums run over one group and are truncated (at most 2^-23 per step of 16 k), the groups are added in fp32: the same
-order as the look-up kernels' K * 2^-24 * A per element, doubled for the truncation, and 5e-6 in norm.
+order as the look-up kernels' K * 2^-24 * A per element, doubled for the truncation, and 5e-6 in norm.  As bytes (up to four rows at
+G = 128 but for three and four at q = 1) activations and group sums are exact; the same bound, and a closer one where it matters.
 """
 
 import numpy as np
@@ -51,7 +52,7 @@ def test_fragment_kernel_matches_oracle(q, G, N, K, M):
 @pytest.mark.parametrize("q,N,K,M", [(1, 17, 128, 4), (3, 129, 640, 4), (4, 1000, 1408, 3), (2, 4100, 4224, 2), (3, 5003, 3456, 2), (4, 300, 14336, 4)])
 def test_rows_as_digits(q, N, K, M):
     test_fragment_kernel_matches_oracle(q, 128, N, K, M)
-    # one element of every step much larger than the rest: digits are rounded below 2^-30 of it
+    # one element of every step much larger than the rest, against the bound of the whole sum (results without it: the next test)
     layer = workloads.hlq_layer(68, f"frag/digits/{q}/{N}/{K}", q, 128, N, K)
     X = synth.activations(68, f"frag/digits/x/{M}/{K}", M, K)
     X[:, 5::128] = np.float16(2.0 ** 13)
