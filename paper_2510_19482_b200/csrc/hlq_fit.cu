@@ -6,10 +6,10 @@
 //   sorted   a lane per group.  The nearest candidate of a weight only depends on between which candidates it lies, so once
 //            a group's weights are sorted a round needs the 2^q - 1 places where the choice changes, not a look at every
 //            weight: a binary search on an estimate of each place, settled by the exact comparison of the two candidates at the
-//            neighbouring weights; bit counts and right-hand sides follow from the places and prefix sums.  A warp sorts its 32
-//            groups (two at a time in the halves of a register), then every lane runs its group's rounds, then
-//            the warp writes the bits.  A round's instructions are shared by 32 groups.  4096 x 4096, G = 128, ten rounds:
-//            q = 2 688 us direct (561 with the stop at unchanged bits), 113 sorted; q = 4 2293 (1616), 605.
+//            neighbouring weights; bit counts and right-hand sides follow from the places and prefix sums.  A lane sorts its group in its
+//            registers, two weights in each (no shuffles: 1600 instructions for a warp's 32 groups of 128; a warp that sorts them two at a time
+//            takes over 5000), runs its rounds, then the warp writes the bits.  A round's instructions are shared by 32 groups.  4096 x 4096, G = 128,
+//            ten rounds, us: q = 2 688 direct (561 with the stop at unchanged bits), 112 sorted by the warp, 91 by lanes; q = 4 2293 (1616), 611, 541.
 //   direct   a warp per group (G / 32 weights per lane) that evaluates every candidate for every weight: for few groups, for the error
 //            trace, and for groups with two candidates so close that rounding decides between them.
 //
@@ -279,8 +279,9 @@ __global__ void __launch_bounds__(kFitWarps * 32) hlq_fit_kernel(const __half* _
 }
 
 constexpr int kSortWarps = 4;     // warps (of 32 groups) per CTA of the sorted form
-// Bytes of a group's record.  It bounds the warps on an SM, and with them the latencies hidden: prefix sums of every 8 weights instead
-// of 4 took G = 128 from 146 to 113 us (q = 2, 4096 x 4096); at G = 32 the longer remainders cost more (1027 / 1083 us, q = 4).
+// Bytes of a group's record: weight i of a warp's lanes lies at 64 i, so that each lane has half a bank of its own whatever it looks at.  The record
+// bounds the warps on an SM, and with them the latencies hidden: prefix sums of every 8 weights instead of 4 took G = 128 from 146 to 113 us (q = 2,
+// 4096 x 4096, sorted by the warp); at G = 32 the longer remainders cost more (1027 / 1083 us, q = 4).
 __host__ __device__ constexpr int sorted_step(int G) { return G == 32 ? 4 : 8; }
 __host__ __device__ constexpr int sorted_record(int G) { return 2 * G + 8 * (G / sorted_step(G) + 1); }
 
@@ -311,17 +312,22 @@ __device__ __forceinline__ bool gram_singular(const int (&m)[NV][NV]) {
     }
 }
 
+__host__ __device__ constexpr int log2_of(int n) { return n > 1 ? 1 + log2_of(n / 2) : 0; }
+
 template <int Q, int G>
 __global__ void __launch_bounds__(kSortWarps * 32) hlq_fit_sorted_kernel(const __half* __restrict__ W, long long n_groups, int t_max,
                                                                          uint8_t* __restrict__ planes, __half* __restrict__ scales,
-                                                                         __half* __restrict__ offsets, const bool aligned) {
-    constexpr int NC = 1 << Q, NV = Q + 1, NB = 32 * G / 128;     // NB: blocks of 128 weights of a warp's 32 groups
-    constexpr int PS = sorted_step(G), REC = sorted_record(G);    // a group's sorted weights, and prefix sums of every PS of them
+                                                                         __half* __restrict__ offsets, const bool aligned, const bool wide) {
+    constexpr int NC = 1 << Q, NV = Q + 1, NB = 32 * G / 128, H = G / 2;     // NB: blocks of 128 weights of a warp's 32 groups
+    constexpr int PS = sorted_step(G), REC = sorted_record(G), RES = 40;    // a group's sorted weights, and prefix sums of every PS of them; its result
+    static_assert(8 + 2 * (NC - 1) <= RES && RES <= REC, "");
     extern __shared__ __align__(16) uint8_t smem[];
     const int lane = threadIdx.x & 31;
     uint8_t* recs = smem + (threadIdx.x >> 5) * (32 * REC);
     const long long grp0 = ((long long)blockIdx.x * kSortWarps + (threadIdx.x >> 5)) * 32;
     if (grp0 >= n_groups) return;
+    __half* sorted = reinterpret_cast<__half*>(recs) + lane;      // weight i of the lane's group at 32 i: every lane has its bank (half a bank)
+    double* pre = reinterpret_cast<double*>(recs + 64 * G) + lane;
     const long long total = n_groups * G, w0 = grp0 * G;          // weights in all; the warp's first
     const size_t plane_stride = (size_t)total;
 
@@ -336,85 +342,66 @@ __global__ void __launch_bounds__(kSortWarps * 32) hlq_fit_sorted_kernel(const _
         }
     };
 
-    // ---- sort: bitonic over runs of G, two blocks at a time in the halves of a register.  Every merge begins against the mirrored
-    // half, so that all exchanges are ascending. -----------------------------------------------------------------------------
-    auto exchange = [&](__half2 mine, __half2 other, bool low) {  // the smaller for the lower index, the larger for the higher
-        const __half2 mn = __hmin2(mine, other), mx = __hmax2(mine, other);
-        return low ? mn : mx;
-    };
-    for (int blk = 0; blk < NB; blk += 2) {
-        __half ha[4], hb[4];
-        load4(blk, ha);
-        load4(blk + 1, hb);
-        __half2 v[4];
+    // ---- sort: a lane its group, in registers.  Both halves of the registers are runs of their own, sorted by one network (Batcher's
+    // odd-even merges) and then merged. ------------------------------------------------------------------------------------------
+    const long long grp = grp0 + lane;
+    const bool valid = grp < n_groups;
+    {
+        __half2 v[H];
+        const __half* src = W + grp * G;
+        if (wide) {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) v[e] = __halves2half2(ha[e], hb[e]);
-        auto in_lane = [&](int a, int b) {
+            for (int i = 0; i < H; i += 4) {
+                const uint4 r = valid ? __ldg(reinterpret_cast<const uint4*>(src + 2 * i)) : make_uint4(0, 0, 0, 0);
+                *reinterpret_cast<uint4*>(&v[i]) = r;
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < H; ++i) v[i] = valid ? __halves2half2(src[2 * i], src[2 * i + 1]) : __float2half2_rn(0.f);
+        }
+        auto exchange = [&](int a, int b) {
             const __half2 mn = __hmin2(v[a], v[b]), mx = __hmax2(v[a], v[b]);
             v[a] = mn;
             v[b] = mx;
         };
+        static_for<0, log2_of(H)>([&](auto p_c) {
+            constexpr int p = 1 << decltype(p_c)::value;
+            static_for<0, decltype(p_c)::value + 1>([&](auto k_c) {
+                constexpr int k = p >> decltype(k_c)::value;
 #pragma unroll
-        for (int size = 2; size <= G; size <<= 1) {
-            if (size == 2) {
-                in_lane(0, 1);
-                in_lane(2, 3);
-                continue;
-            }
-            if (size == 4) {
-                in_lane(0, 3);
-                in_lane(1, 2);
-            } else {                                              // against index ^ (size - 1)
-                const bool low = (lane & (size / 8)) == 0;
-                __half2 o[4];
+                for (int j = k % p; j <= H - 1 - k; j += 2 * k)
 #pragma unroll
-                for (int e = 0; e < 4; ++e) o[e] = __shfl_xor_sync(0xffffffffu, v[3 - e], size / 4 - 1);
+                    for (int i = 0; i < k; ++i)
+                        if (i + j + k < H && (i + j) / (2 * p) == (i + j + k) / (2 * p)) exchange(i + j, i + j + k);
+            });
+        });
+        // the lower halves against the upper ones in reverse: the smaller ones are the lower half of the result, and bitonic
 #pragma unroll
-                for (int e = 0; e < 4; ++e) v[e] = exchange(v[e], o[e], low);
-            }
-#pragma unroll
-            for (int stride = size / 4; stride >= 4; stride >>= 1) {
-                const bool low = (lane & (stride / 4)) == 0;
-#pragma unroll
-                for (int e = 0; e < 4; ++e) v[e] = exchange(v[e], __shfl_xor_sync(0xffffffffu, v[e], stride / 4), low);
-            }
-            if (size >= 8) {
-                in_lane(0, 2);
-                in_lane(1, 3);
-            }
-            in_lane(0, 1);
-            in_lane(2, 3);
+        for (int i = 0; i < H / 2; ++i) {
+            const int j = H - 1 - i;
+            const __half2 o = __lowhigh2highlow(v[j]), mn = __hmin2(v[i], o), mx = __hmax2(v[i], o);
+            v[i] = __lows2half2(mn, mx);
+            v[j] = __highs2half2(mn, mx);
         }
 #pragma unroll
-        for (int half = 0; half < 2; ++half) {
-            __half h[4];
+        for (int k = H / 2; k >= 1; k >>= 1)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) h[e] = half ? __high2half(v[e]) : __low2half(v[e]);
-            // sums of fp16 values are exact in fp64
-            const double own = (double)__half2float(h[0]) + (double)__half2float(h[1]) + (double)__half2float(h[2]) + (double)__half2float(h[3]);
-            double incl = own;
+            for (int i = 0; i < H; ++i)
+                if (!(i & k)) exchange(i, i + k);
+        // sums of fp16 values are exact in fp64
+        double run = 0.0;
 #pragma unroll
-            for (int o = 1; o < G / 4; o <<= 1) {
-                const double below = __shfl_up_sync(0xffffffffu, incl, o, G / 4);
-                if ((lane & (G / 4 - 1)) >= o) incl += below;
-            }
-            const int i = (blk + half) * 128 + 4 * lane, g = i / G, pos = i % G;
-            uint8_t* rec = recs + g * REC;
-            *reinterpret_cast<uint2*>(rec + 2 * pos) = *reinterpret_cast<const uint2*>(h);
-            double* pre = reinterpret_cast<double*>(rec + 2 * G);
-            if (pos % PS == 0) pre[pos / PS] = incl - own;
-            if (pos == G - 4) pre[G / PS] = incl;
+        for (int i = 0; i < G; ++i) {
+            const __half w = i < H ? __low2half(v[i % H]) : __high2half(v[i % H]);
+            if (i % PS == 0) pre[i / PS * 32] = run;
+            run += (double)__half2float(w);
+            sorted[i * 32] = w;
         }
+        pre[G / PS * 32] = run;
     }
-    __syncwarp();
 
     // ---- rounds: lane = group --------------------------------------------------------------------------------------------------
-    uint8_t* rec = recs + lane * REC;
-    const __half* sorted = reinterpret_cast<const __half*>(rec);
-    double* pre = reinterpret_cast<double*>(rec + 2 * G);
-    const long long grp = grp0 + lane;
-    const bool valid = grp < n_groups;
-    auto weight = [&](int i) { return __half2float(sorted[i]); };
+    auto weight = [&](int i) { return __half2float(sorted[i * 32]); };
     const double wmin = (double)weight(0), wmax = (double)weight(G - 1);
     double s[Q], z = wmin;
     const double delta = __ddiv_rn(__dsub_rn(wmax, wmin), (double)(NC - 1));
@@ -506,14 +493,14 @@ __global__ void __launch_bounds__(kSortWarps * 32) hlq_fit_sorted_kernel(const _
             for (int j = 0; j < NV; ++j) A[i][j] = 0;
         }
         A[Q][Q] = G;
-        b[Q] = 0.0 + pre[G / PS];                                // (never a negative zero)
+        b[Q] = 0.0 + pre[G / PS * 32];                                // (never a negative zero)
         {
             int from = 0;
             double below = 0.0;
 #pragma unroll
             for (int r = 0; r < NC; ++r) {
                 const int to = r < NC - 1 ? cut[r < NC - 1 ? r : 0] : G;
-                double upto = pre[to / PS];
+                double upto = pre[to / PS * 32];
 #pragma unroll
                 for (int e = 0; e < PS - 1; ++e)
                     if (e < to % PS) upto += (double)weight(to / PS * PS + e);
@@ -570,8 +557,9 @@ __global__ void __launch_bounds__(kSortWarps * 32) hlq_fit_sorted_kernel(const _
     // ---- results: parameters by lane; per group the weights at the places and the codes, then the bits by the warp -----------
     __half place[NC - 1];
 #pragma unroll
-    for (int r = 0; r < NC - 1; ++r) place[r] = cut[r] < G ? sorted[max(cut[r], 0)] : __ushort_as_half(0x7c00);      // (infinity: none)
+    for (int r = 0; r < NC - 1; ++r) place[r] = cut[r] < G ? sorted[max(cut[r], 0) * 32] : __ushort_as_half(0x7c00);      // (infinity: none)
     __syncwarp();
+    uint8_t* rec = recs + lane * RES;
     __half* places = reinterpret_cast<__half*>(rec + 8);
     *reinterpret_cast<unsigned long long*>(rec) = map;
 #pragma unroll
@@ -588,7 +576,7 @@ __global__ void __launch_bounds__(kSortWarps * 32) hlq_fit_sorted_kernel(const _
         load4(blk, h);
         const int g = (blk * 128 + 4 * lane) / G;
         const long long i = w0 + blk * 128 + 4 * lane;
-        const uint8_t* gr = recs + g * REC;
+        const uint8_t* gr = recs + g * RES;
         const __half* pl = reinterpret_cast<const __half*>(gr + 8);
         const unsigned long long codes = *reinterpret_cast<const unsigned long long*>(gr);
         __half2 rank[2] = {__float2half2_rn(1024.f), __float2half2_rn(1024.f)};      // (1024 + rank: the rank in the low bits)
@@ -639,7 +627,7 @@ int launch_fit_qg(const __half* W, int N, int K, int t_max, uint8_t* planes, __h
         }
         const bool aligned = ((reinterpret_cast<uintptr_t>(W) & 7) | (reinterpret_cast<uintptr_t>(planes) & 3)) == 0;
         const unsigned grid = (unsigned)((n_groups + 32 * kSortWarps - 1) / (32 * kSortWarps));
-        hlq_fit_sorted_kernel<Q, G><<<grid, kSortWarps * 32, kSmem, stream>>>(W, n_groups, t_max, planes, scales, offsets, aligned);
+        hlq_fit_sorted_kernel<Q, G><<<grid, kSortWarps * 32, kSmem, stream>>>(W, n_groups, t_max, planes, scales, offsets, aligned, (reinterpret_cast<uintptr_t>(W) & 15) == 0);
     } else {
         const unsigned grid = (unsigned)((n_groups + kFitWarps - 1) / kFitWarps);
         hlq_fit_kernel<Q, G / 32><<<grid, kFitWarps * 32, 0, stream>>>(W, n_groups, t_max, planes, scales, offsets, trace);
