@@ -9,7 +9,8 @@
 //            neighbouring weights; bit counts and right-hand sides follow from the places and prefix sums.  A lane sorts its group in its
 //            registers, two weights in each (no shuffles: 1600 instructions for a warp's 32 groups of 128; a warp that sorts them two at a time
 //            takes over 5000), runs its rounds, then the warp writes the bits.  A round's instructions are shared by 32 groups.  4096 x 4096, G = 128,
-//            ten rounds, us: q = 2 688 direct (561 with the stop at unchanged bits), 112 sorted by the warp, 91 by lanes; q = 4 2293 (1616), 611, 541.
+//            ten rounds, us: q = 2 688 direct (561 with the stop at unchanged bits), 112 sorted by the warp, 91 by lanes, 79 with a round's searches
+//            side by side; q = 4 2293 (1616), 611, 541, 517.
 //   direct   a warp per group (G / 32 weights per lane) that evaluates every candidate for every weight: for few groups, for the error
 //            trace, and for groups with two candidates so close that rounding decides between them.
 //
@@ -461,23 +462,45 @@ __global__ void __launch_bounds__(kSortWarps * 32) hlq_fit_sorted_kernel(const _
         for (int r = 0; r < NC; ++r) new_map |= (unsigned long long)code[r] << (4 * r);
         bool changed = new_map != map;
         map = new_map;
+        // The places: a search on estimates of them, all side by side, and where a neighbouring weight is not clearly on its side, by the exact choice.
+        // (An estimate is off by its rounding to fp32, the choice's own roundings are far below `gap`.)
+        float guess[NC - 1];
+        int pos[NC - 1];
 #pragma unroll
         for (int r = 0; r < NC - 1; ++r) {
-            const float guess = (float)(z + 0.5 * (V[r] + V[r + 1]));
-            int pos = 0;
+            guess[r] = (float)(z + 0.5 * (V[r] + V[r + 1]));
+            pos[r] = 0;
+        }
 #pragma unroll
-            for (int st = G / 2; st >= 1; st >>= 1)
-                if (weight(pos + st - 1) < guess) pos += st;
-            if (weight(pos) < guess) ++pos;
-            auto above = [&](int i) {                             // the exact choice between candidates r and r + 1
-                const double shifted = __dsub_rn((double)weight(i), z);
-                const double da = fabs(__dsub_rn(shifted, V[r])), db = fabs(__dsub_rn(shifted, V[r + 1]));
-                return db < da || (db == da && code[r + 1] < code[r]);
-            };
-            while (pos > 0 && above(pos - 1)) --pos;
-            while (pos < G && !above(pos)) ++pos;
-            changed |= pos != cut[r];
-            cut[r] = pos;
+        for (int st = G / 2; st >= 1; st >>= 1)
+#pragma unroll
+            for (int r = 0; r < NC - 1; ++r)
+                if (weight(pos[r] + st - 1) < guess[r]) pos[r] += st;
+        const float gap_up = __double2float_ru(gap);
+        bool clear = true;
+#pragma unroll
+        for (int r = 0; r < NC - 1; ++r) {
+            if (weight(pos[r]) < guess[r]) ++pos[r];
+            const float near = fabsf(guess[r]) * 0x1p-22f + gap_up;
+            clear &= pos[r] == 0 || guess[r] - weight(max(pos[r] - 1, 0)) > near;
+            clear &= pos[r] == G || weight(min(pos[r], G - 1)) - guess[r] > near;
+        }
+        if (!clear) {
+#pragma unroll
+            for (int r = 0; r < NC - 1; ++r) {
+                auto above = [&](int i) {                         // the exact choice between candidates r and r + 1
+                    const double shifted = __dsub_rn((double)weight(i), z);
+                    const double da = fabs(__dsub_rn(shifted, V[r])), db = fabs(__dsub_rn(shifted, V[r + 1]));
+                    return db < da || (db == da && code[r + 1] < code[r]);
+                };
+                while (pos[r] > 0 && above(pos[r] - 1)) --pos[r];
+                while (pos[r] < G && !above(pos[r])) ++pos[r];
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < NC - 1; ++r) {
+            changed |= pos[r] != cut[r];
+            cut[r] = pos[r];
         }
         // the same bits as in the round before: the parameters are theirs already, and so on in every later round
         if (!changed) {
@@ -501,9 +524,17 @@ __global__ void __launch_bounds__(kSortWarps * 32) hlq_fit_sorted_kernel(const _
             for (int r = 0; r < NC; ++r) {
                 const int to = r < NC - 1 ? cut[r < NC - 1 ? r : 0] : G;
                 double upto = pre[to / PS * 32];
+                if (r < NC - 1) {                                 // (exact in any order; what lies behind the place is read and left out)
+                    double w[PS];
 #pragma unroll
-                for (int e = 0; e < PS - 1; ++e)
-                    if (e < to % PS) upto += (double)weight(to / PS * PS + e);
+                    for (int e = 0; e < PS - 1; ++e) w[e] = e < to % PS ? (double)weight(to / PS * PS + e) : 0.0;
+                    w[PS - 1] = upto;
+#pragma unroll
+                    for (int o = PS / 2; o > 0; o >>= 1)
+#pragma unroll
+                        for (int e = 0; e < o; ++e) w[e] += w[e + o];
+                    upto = w[0];
+                }
                 const int cnt = to - from;
                 const double part = upto - below;                 // exact
                 from = to;
