@@ -313,6 +313,13 @@ __device__ __forceinline__ bool gram_singular(const int (&m)[NV][NV]) {
     }
 }
 
+template <int IMM>
+__device__ __forceinline__ __half lds_half(uint32_t addr) {
+    unsigned short v;
+    asm volatile("ld.shared.u16 %0, [%1+%2];" : "=h"(v) : "r"(addr), "n"(IMM));
+    return __ushort_as_half(v);
+}
+
 __host__ __device__ constexpr int log2_of(int n) { return n > 1 ? 1 + log2_of(n / 2) : 0; }
 
 template <int Q, int G>
@@ -320,8 +327,8 @@ __global__ void __launch_bounds__(kSortWarps * 32) hlq_fit_sorted_kernel(const _
                                                                          uint8_t* __restrict__ planes, __half* __restrict__ scales,
                                                                          __half* __restrict__ offsets, const bool aligned, const bool wide) {
     constexpr int NC = 1 << Q, NV = Q + 1, NB = 32 * G / 128, H = G / 2;     // NB: blocks of 128 weights of a warp's 32 groups
-    constexpr int PS = sorted_step(G), REC = sorted_record(G), RES = 40;    // a group's sorted weights, and prefix sums of every PS of them; its result
-    static_assert(8 + 2 * (NC - 1) <= RES && RES <= REC, "");
+    constexpr int PS = sorted_step(G), REC = sorted_record(G), RES = 48;    // a group's sorted weights, and prefix sums of every PS of them; its result
+    static_assert(16 + 2 * (NC - 1) <= RES && RES <= REC, "");
     extern __shared__ __align__(16) uint8_t smem[];
     const int lane = threadIdx.x & 31;
     uint8_t* recs = smem + (threadIdx.x >> 5) * (32 * REC);
@@ -403,6 +410,7 @@ __global__ void __launch_bounds__(kSortWarps * 32) hlq_fit_sorted_kernel(const _
 
     // ---- rounds: lane = group --------------------------------------------------------------------------------------------------
     auto weight = [&](int i) { return __half2float(sorted[i * 32]); };
+    const uint32_t sorted_at = (uint32_t)__cvta_generic_to_shared(sorted);
     const double wmin = (double)weight(0), wmax = (double)weight(G - 1);
     double s[Q], z = wmin;
     const double delta = __ddiv_rn(__dsub_rn(wmax, wmin), (double)(NC - 1));
@@ -465,25 +473,31 @@ __global__ void __launch_bounds__(kSortWarps * 32) hlq_fit_sorted_kernel(const _
         // The places: a search on estimates of them, all side by side, and where a neighbouring weight is not clearly on its side, by the exact choice.
         // (An estimate is off by its rounding to fp32, the choice's own roundings are far below `gap`.)
         float guess[NC - 1];
+        __half guess_up[NC - 1];                                  // (a weight is below the one where it is below the other)
+        uint32_t at[NC - 1];                                      // where the place's weight lies: 64 bytes a weight
         int pos[NC - 1];
 #pragma unroll
         for (int r = 0; r < NC - 1; ++r) {
             guess[r] = (float)(z + 0.5 * (V[r] + V[r + 1]));
-            pos[r] = 0;
+            guess_up[r] = __float2half_ru(guess[r]);
+            at[r] = sorted_at;
         }
-#pragma unroll
-        for (int st = G / 2; st >= 1; st >>= 1)
+        static_for<0, log2_of(G)>([&](auto i_c) {
+            constexpr int st = G >> (decltype(i_c)::value + 1);
 #pragma unroll
             for (int r = 0; r < NC - 1; ++r)
-                if (weight(pos[r] + st - 1) < guess[r]) pos[r] += st;
+                if (__hlt(lds_half<64 * (st - 1)>(at[r]), guess_up[r])) at[r] += 64 * st;
+        });
         const float gap_up = __double2float_ru(gap);
         bool clear = true;
 #pragma unroll
         for (int r = 0; r < NC - 1; ++r) {
-            if (weight(pos[r]) < guess[r]) ++pos[r];
+            if (__hlt(lds_half<0>(at[r]), guess_up[r])) at[r] += 64;
             const float near = fabsf(guess[r]) * 0x1p-22f + gap_up;
-            clear &= pos[r] == 0 || guess[r] - weight(max(pos[r] - 1, 0)) > near;
-            clear &= pos[r] == G || weight(min(pos[r], G - 1)) - guess[r] > near;
+            const float below = __half2float(lds_half<0>(max(at[r] - 64, sorted_at))), above = __half2float(lds_half<0>(min(at[r], sorted_at + 64 * (G - 1))));
+            clear &= at[r] == sorted_at || guess[r] - below > near;
+            clear &= at[r] == sorted_at + 64 * G || above - guess[r] > near;
+            pos[r] = (int)(at[r] - sorted_at) / 64;
         }
         if (!clear) {
 #pragma unroll
@@ -527,7 +541,10 @@ __global__ void __launch_bounds__(kSortWarps * 32) hlq_fit_sorted_kernel(const _
                 if (r < NC - 1) {                                 // (exact in any order; what lies behind the place is read and left out)
                     double w[PS];
 #pragma unroll
-                    for (int e = 0; e < PS - 1; ++e) w[e] = e < to % PS ? (double)weight(to / PS * PS + e) : 0.0;
+                    for (int e = 0; e < PS - 1; ++e) {
+                        const double v = (double)weight(to / PS * PS + e);
+                        w[e] = e < to % PS ? v : 0.0;
+                    }
                     w[PS - 1] = upto;
 #pragma unroll
                     for (int o = PS / 2; o > 0; o >>= 1)
@@ -591,8 +608,9 @@ __global__ void __launch_bounds__(kSortWarps * 32) hlq_fit_sorted_kernel(const _
     for (int r = 0; r < NC - 1; ++r) place[r] = cut[r] < G ? sorted[max(cut[r], 0) * 32] : __ushort_as_half(0x7c00);      // (infinity: none)
     __syncwarp();
     uint8_t* rec = recs + lane * RES;
-    __half* places = reinterpret_cast<__half*>(rec + 8);
-    *reinterpret_cast<unsigned long long*>(rec) = map;
+    __half* places = reinterpret_cast<__half*>(rec + 16);
+#pragma unroll
+    for (int r = 0; r < NC; ++r) rec[r] = (uint8_t)(map >> (4 * r) & 15u);
 #pragma unroll
     for (int r = 0; r < NC - 1; ++r) places[r] = place[r];
     if (valid && !direct) {
@@ -608,8 +626,9 @@ __global__ void __launch_bounds__(kSortWarps * 32) hlq_fit_sorted_kernel(const _
         const int g = (blk * 128 + 4 * lane) / G;
         const long long i = w0 + blk * 128 + 4 * lane;
         const uint8_t* gr = recs + g * RES;
-        const __half* pl = reinterpret_cast<const __half*>(gr + 8);
-        const unsigned long long codes = *reinterpret_cast<const unsigned long long*>(gr);
+        const __half* pl = reinterpret_cast<const __half*>(gr + 16);
+        const uint4 cw = *reinterpret_cast<const uint4*>(gr);     // code of every rank, a byte each
+        const uint32_t codes[4] = {cw.x, cw.y, cw.z, cw.w};
         __half2 rank[2] = {__float2half2_rn(1024.f), __float2half2_rn(1024.f)};      // (1024 + rank: the rank in the low bits)
         const __half2 w2[2] = {__halves2half2(h[0], h[1]), __halves2half2(h[2], h[3])};
 #pragma unroll
@@ -618,11 +637,17 @@ __global__ void __launch_bounds__(kSortWarps * 32) hlq_fit_sorted_kernel(const _
             rank[0] = __hadd2(rank[0], __hge2(w2[0], p2));
             rank[1] = __hadd2(rank[1], __hge2(w2[1], p2));
         }
-        uint32_t four = 0;                                        // the codes of four weights, a byte each
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const __half rk = (e & 1) ? __high2half(rank[e >> 1]) : __low2half(rank[e >> 1]);
-            four |= (uint32_t)((codes >> (4 * (__half_as_ushort(rk) & 15))) & 15u) << (8 * e);
+        // the ranks as the nibbles of a selector, the codes of the four weights as bytes
+        const uint32_t r0 = *reinterpret_cast<const uint32_t*>(&rank[0]), r1 = *reinterpret_cast<const uint32_t*>(&rank[1]);
+        const uint32_t lows = __byte_perm(r0, r1, 0x6420) & 0x0f0f0f0fu, sel = lows | lows >> 4;       // bytes: ranks; nibbles 0, 1, 4, 5 of sel
+        const uint32_t pick = __byte_perm(sel, 0u, 0x4420);
+        uint32_t four;
+        if constexpr (Q <= 3) {
+            four = __byte_perm(codes[0], codes[1], pick);
+        } else {                                                  // ranks of 8 and more in the upper half
+            const uint32_t lo = __byte_perm(codes[0], codes[1], pick & 0x7777u), hi = __byte_perm(codes[2], codes[3], pick & 0x7777u);
+            const uint32_t upper = (lows >> 3 & 0x01010101u) * 0xffu;
+            four = (lo & ~upper) | (hi & upper);
         }
         if (i < total && !((directs >> g) & 1u)) {
 #pragma unroll
