@@ -10,7 +10,7 @@
 //            registers, two weights in each (no shuffles: 1600 instructions for a warp's 32 groups of 128; a warp that sorts them two at a time
 //            takes over 5000), runs its rounds, then the warp writes the bits.  A round's instructions are shared by 32 groups.  4096 x 4096, G = 128,
 //            ten rounds, us: q = 2 688 direct (561 with the stop at unchanged bits), 112 sorted by the warp, 91 by lanes, 79 with a round's searches
-//            side by side; q = 4 2293 (1616), 611, 541, 517.
+//            side by side; q = 4 2293 (1616), 611, 541, 517, and 349 with its candidates in registers.
 //   direct   a warp per group (G / 32 weights per lane) that evaluates every candidate for every weight: for few groups, for the error
 //            trace, and for groups with two candidates so close that rounding decides between them.
 //
@@ -436,25 +436,24 @@ __global__ void __launch_bounds__(kSortWarps * 32) hlq_fit_sorted_kernel(const _
             code[k] = k;
         }
         // candidates in ascending order (odd-even merge exchanges)
-#pragma unroll
-        for (int p = 1; p < NC; p <<= 1)
-#pragma unroll
-            for (int k = p; k >= 1; k >>= 1)
-#pragma unroll
-                for (int j = k % p; j <= NC - 1 - k; j += 2 * k)
-#pragma unroll
-                    for (int i = 0; i < k; ++i) {
-                        const int x = i + j, y = i + j + k;
-                        if (y < NC && x / (2 * p) == y / (2 * p)) {
-                            const bool swap = V[y] < V[x];
-                            const double lo = swap ? V[y] : V[x], hi = swap ? V[x] : V[y];
-                            const int cl = swap ? code[y] : code[x], ch = swap ? code[x] : code[y];
-                            V[x] = lo;
-                            V[y] = hi;
-                            code[x] = cl;
-                            code[y] = ch;
-                        }
+        static_for<0, Q>([&](auto p_c) {                          // (unrolled for certain: the indices are constants)
+            constexpr int p = 1 << decltype(p_c)::value;
+            static_for<0, decltype(p_c)::value + 1>([&](auto k_c) {
+                constexpr int k = p >> decltype(k_c)::value;
+                static_for<0, NC - k>([&](auto x_c) {
+                    constexpr int x = decltype(x_c)::value, y = x + k;
+                    if constexpr ((x - k % p + 2 * k) % (2 * k) < k && x >= k % p && x / (2 * p) == y / (2 * p)) {
+                        const bool swap = V[y] < V[x];
+                        const double lo = swap ? V[y] : V[x], hi = swap ? V[x] : V[y];
+                        const int cl = swap ? code[y] : code[x], ch = swap ? code[x] : code[y];
+                        V[x] = lo;
+                        V[y] = hi;
+                        code[x] = cl;
+                        code[y] = ch;
                     }
+                });
+            });
+        });
         // Only the two candidates around a weight are in question as long as no two are within rounding of each other.
         const double gap = 9.094947017729282e-13 /* 2^-40 */ * (fmax(fabs(wmin), fabs(wmax)) + fabs(z) + fmax(fabs(V[0]), fabs(V[NC - 1])));
         bool apart = true;
