@@ -10,7 +10,7 @@
 //            registers, two weights in each (no shuffles: 1600 instructions for a warp's 32 groups of 128; a warp that sorts them two at a time
 //            takes over 5000), runs its rounds, then the warp writes the bits.  A round's instructions are shared by 32 groups.  4096 x 4096, G = 128,
 //            ten rounds, us: q = 2 688 direct (561 with the stop at unchanged bits), 112 sorted by the warp, 91 by lanes, 79 with a round's searches
-//            side by side; q = 4 2293 (1616), 611, 541, 517, and 349 with its candidates in registers.
+//            side by side, 70 with the output's loads in flight; q = 4 2293 (1616), 611, 541, 517, 349 with its candidates in registers, 340.
 //   direct   a warp per group (G / 32 weights per lane) that evaluates every candidate for every weight: for few groups, for the error
 //            trace, and for groups with two candidates so close that rounding decides between them.
 //
@@ -619,9 +619,7 @@ __global__ void __launch_bounds__(kSortWarps * 32) hlq_fit_sorted_kernel(const _
     }
     const unsigned directs = __ballot_sync(0xffffffffu, direct);
     __syncwarp();
-    for (int blk = 0; blk < NB; ++blk) {
-        __half h[4];
-        load4(blk, h);
+    auto put_bits = [&](int blk, const __half (&h)[4]) {
         const int g = (blk * 128 + 4 * lane) / G;
         const long long i = w0 + blk * 128 + 4 * lane;
         const uint8_t* gr = recs + g * RES;
@@ -660,6 +658,28 @@ __global__ void __launch_bounds__(kSortWarps * 32) hlq_fit_sorted_kernel(const _
                     for (int e = 0; e < 4; ++e) dst[e] = (uint8_t)(bits >> (8 * e));
                 }
             }
+        }
+    };
+    if (aligned) {                                                // a few blocks' weights on their way at a time
+        constexpr int kAhead = Q <= 2 ? 8 : Q == 3 ? 4 : G == 128 ? 2 : 1;      // (more of the longer code costs instruction fetches)
+        static_assert(NB % kAhead == 0, "");
+#pragma unroll 1
+        for (int blk = 0; blk < NB; blk += kAhead) {
+            uint2 raw[kAhead];
+#pragma unroll
+            for (int a = 0; a < kAhead; ++a) {
+                const long long i = w0 + (blk + a) * 128 + 4 * lane;
+                raw[a] = i < total ? __ldg(reinterpret_cast<const uint2*>(W + i)) : make_uint2(0, 0);
+            }
+#pragma unroll
+            for (int a = 0; a < kAhead; ++a) put_bits(blk + a, reinterpret_cast<const __half (&)[4]>(raw[a]));
+        }
+    } else {
+#pragma unroll 1
+        for (int blk = 0; blk < NB; ++blk) {
+            __half h[4];
+            load4(blk, h);
+            put_bits(blk, h);
         }
     }
     for (unsigned left = directs; left != 0; left &= left - 1)
