@@ -37,11 +37,12 @@ namespace {
 
 constexpr int kFitWarps = 8;      // warps (groups) per CTA
 // From how many groups on the sorted form is ahead: with fewer it waits on its own latencies, and its sort has to pay off over the rounds.
-// Rounds: 1, 2 to 4, 5 and more; in 1024 groups, measured at 2048 to 262144.  (us, direct and sorted: 8192 groups of 128, q = 2, ten rounds
-// 45 and 45, one 9.9 and 26.5; 32768 of 128, q = 1, one round 18 and 27, ten 49 and 34; 16384 of 32, q = 4, ten rounds 75 and 108.)
-constexpr int kSortedMinK[3][4][3] = {{{12, 12, 16}, {12, 8, 8}, {12, 8, 12}, {12, 12, 24}},               // G = 32: q = 1 to 4
-                                      {{32, 24, 16}, {24, 12, 12}, {12, 8, 8}, {12, 12, 16}},              // G = 64
-                                      {{128, 64, 24}, {32, 24, 12}, {24, 12, 8}, {24, 12, 12}}};           // G = 128
+// Rounds: 1, 2 to 4, 5 and more; in 1024 groups, measured at 256 to 131072 with 1, 3, 5 and 10 rounds.  (us, direct and sorted: 4096 groups of 128, q = 2,
+// ten rounds 29 and 20, three 11 and 12, one 6 and 9; 3072 of 128, q = 4, ten rounds 67 and 67; 16384 of 128, q = 1, one round 9 and 9, ten 27 and 15;
+// 6144 of 32, q = 4, five rounds 32 and 31, ten 34 and 53, 12288 60 and 53.)
+constexpr int kSortedMinK[3][4][3] = {{{6, 4, 8}, {4, 3, 4}, {4, 4, 6}, {6, 6, 10}},                       // G = 32: q = 1 to 4
+                                      {{10, 6, 6}, {6, 4, 4}, {6, 4, 4}, {6, 5, 7}},                       // G = 64
+                                      {{20, 12, 8}, {10, 5, 4}, {7, 4, 3}, {8, 5, 3}}};                    // G = 128
 inline long long sorted_min_groups(int q, int G, int t_max) {
     return 1024LL * kSortedMinK[G == 128 ? 2 : G == 64 ? 1 : 0][q - 1][t_max == 1 ? 0 : t_max < 5 ? 1 : 2];
 }
