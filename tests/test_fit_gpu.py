@@ -129,3 +129,35 @@ def test_fit_on_both_sides_of_the_sorted_form_s_lower_end(q, G, N, t_max):
         b = elutq.elutq_hlq_fit(Wd[:rows], q, G, t_max, trace=True)
         for x, y in zip(a[:3], b[:3]):
             assert torch.equal(x.view(torch.uint8), y.view(torch.uint8))
+
+
+# the same at the lower ends where a lane sorts its group itself, and weights that begin 8 bytes after a 16-byte boundary (loads of 2 bytes instead of 16)
+@pytest.mark.parametrize("q,G,N,t_max", [(1, 64, 640, 1), (2, 64, 256, 2), (3, 128, 512, 2), (4, 32, 192, 1), (2, 128, 1280, 1), (2, 128, 512, 7), (4, 128, 384, 10)])
+@pytest.mark.parametrize("shift", [0, 4])
+def test_fit_on_both_sides_of_the_lane_sort_s_lower_end(q, G, N, t_max, shift):
+    W = workloads.dense_weights(43, f"fit-lanes{q}{G}", N, 1024)
+    buf = torch.zeros(W.size + 8, dtype=torch.int16, device="cuda")
+    Wd = buf[shift: shift + W.size].view(W.shape)
+    Wd.copy_(to_dev(W.view(np.int16)))
+    Wd = Wd.view(torch.float16)
+    for rows in (N - 1, N):
+        a = elutq.elutq_hlq_fit(Wd[:rows], q, G, t_max)
+        b = elutq.elutq_hlq_fit(Wd[:rows], q, G, t_max, trace=True)
+        for x, y in zip(a[:3], b[:3]):
+            assert torch.equal(x.view(torch.uint8), y.view(torch.uint8))
+
+
+def test_fit_of_weights_next_to_a_place():
+    """Weights at, and an ulp or two beside, the middle of two candidates: the exact choice decides, with the lower code where both are equally far."""
+    rng = np.random.default_rng(44)
+    q, G, n = 2, 128, 4096 + 32
+    mid = np.array([0.5, 1.5, 2.5], dtype=np.float16)
+    near = np.concatenate([mid, np.nextafter(mid, np.float16(9)), np.nextafter(mid, np.float16(-9)), np.nextafter(np.nextafter(mid, np.float16(9)), np.float16(9))])
+    W = rng.choice(np.concatenate([near, np.arange(4, dtype=np.float16)]), (n, G)).astype(np.float16)
+    W[:, 0], W[:, 1] = 0.0, 3.0                          # the first round's candidates are 0, 1, 2, 3
+    W *= np.float16(2.0) ** rng.integers(-12, 8, (n, 1)).astype(np.float16)
+    Wd = to_dev(W.view(np.int16)).view(torch.float16)
+    for t_max in (2, 5):
+        a, b = elutq.elutq_hlq_fit(Wd, q, G, t_max), elutq.elutq_hlq_fit(Wd, q, G, t_max, trace=True)
+        for x, y in zip(a[:3], b[:3]):
+            assert torch.equal(x.view(torch.uint8), y.view(torch.uint8))
