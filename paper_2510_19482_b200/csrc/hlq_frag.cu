@@ -838,10 +838,9 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
             compute_sync();
             if (tid == 0) {
                 const int parts = parts_of(tile);
-                __threadfence();
-                const unsigned t = atomicAdd(ticket_of(tile), 1u);
+                unsigned t;                                   // (one operation that releases and acquires: between two fences it takes twice as long)
+                asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(t) : "l"(ticket_of(tile)) : "memory");
                 if ((t & (kTicketNoPart - 1)) == (unsigned)(parts - 1)) *ticket_of(tile) = 0;      // zero again for the next call
-                __threadfence();
                 *ticket_box = t == (unsigned)(parts - 1) ? 1u : 0u;
             }
             pending = tile;
