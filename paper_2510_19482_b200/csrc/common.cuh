@@ -91,6 +91,8 @@ int launch_lut_gemm(const GemmArgs& a, int q, int G, int num_sms, cudaStream_t s
 int launch_hlq_frag(const GemmArgs& a, int q, int G, int num_sms, cudaStream_t stream);
 int launch_hlq_mma(const GemmArgs& a, int q, int G, int num_sms, cudaStream_t stream);
 int launch_hlq_tmem(const GemmArgs& a, int q, int num_sms, cudaStream_t stream);
+// Clusters of `size` CTAs (2 to 8, one per SM) that are resident together on the current device.
+int resident_clusters(int size);
 bool tmem_takes(int M, int N, int K);                         // (index ranges)
 // Estimates in us for more than 128 tokens (hlq_mma: infinite where it would have to split K)
 double tmem_us(int M, int N, int K, int q, int num_sms);
@@ -177,9 +179,16 @@ __device__ __forceinline__ void store_out(const GemmArgs& a, size_t idx, float y
     }
 }
 // Thread-block cluster helpers (distributed shared memory).
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_barrier() {
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    cluster_arrive();
+    cluster_wait();
+}
+__device__ __forceinline__ void st_cluster_u32(uint32_t addr, uint32_t rank, uint32_t v) {
+    uint32_t remote;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr), "r"(rank));
+    asm volatile("st.shared::cluster.u32 [%0], %1;" :: "r"(remote), "r"(v) : "memory");
 }
 __device__ __forceinline__ float ld_cluster_f32(const float* local_smem_ptr, unsigned cta_rank) {
     const uint32_t local = (uint32_t)__cvta_generic_to_shared(local_smem_ptr);

@@ -33,7 +33,8 @@
 //   unit     128 weight rows x 512 k (eight packed tiles, contiguous in the blob: one bulk copy) x 8 NB batch rows (bytes: 2 NB).  The units of
 //            a call, output tile by output tile (the batch blocks of a row tile next to each other: its weights come from the L2 again), are
 //            dealt to the CTAs (one per SM) in equal contiguous runs, so no SM idles for a wave.  An output tile that several CTAs share
-//            is summed in ascending k order (bit-reproducible) by the CTA that finishes it last (a ticket, no CTA waits for another).
+//            is summed in ascending k order (bit-reproducible) by the CTA that finishes it last (a ticket, no CTA waits for another).  Few output
+//              tiles are shared by clusters of CTAs instead, whose first CTA adds up.
 //   warps    16 compute warps: warp 4 s + r takes step s (128 k) of every unit and rows 32 r .. 32 r + 31 of the tile, so each
 //            activation fragment serves two MMAs.  Four activation warps, one per step: scale the unit's activations and
 //            lay them out as B fragments, form the group sums; the first of them also loads the weights.
@@ -61,6 +62,7 @@ struct FragArgs {
     int units, per_cta;         // all units; units of one CTA
     Div by_chunks, by_blocks, by_cta;
     int ws;                     // weight units in flight
+    int split;                  // CTAs of a cluster, which share an output tile's chunks (1: no cluster)
     unsigned* tickets;          // zero between calls: one per row tile, or (several blocks) per CTA, for the tile that it begins and does not end
 };
 
@@ -202,8 +204,8 @@ __device__ __noinline__ float plain_sum(const __half* __restrict__ x, const uint
 }
 
 // NB = blocks of 8 columns (MMA N): of 8 batch rows, or (BYTES) of two with four digits each.  FOLD: long runs of units, whose sums are
-// put by every two units.
-template <int Q, int G, int NB, bool FOLD, bool BYTES>
+// put by every two units.  SPLIT: the chunks of an output tile are shared by the CTAs of a cluster.
+template <int Q, int G, int NB, bool FOLD, bool BYTES, bool SPLIT>
 __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArgs a) {
     using C = FragCfg<Q, G>;
     static_assert(G == 128 || G == 64, "");
@@ -223,6 +225,8 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
     uint64_t* bars = reinterpret_cast<uint64_t*>(sSum + 4 * MP * kSumStride);
     volatile uint32_t* give_up = reinterpret_cast<uint32_t*>(bars + kNumBars);
     volatile uint32_t* ticket_box = give_up + 1;
+    volatile uint32_t* lost_box = ticket_box + 1;             // split: another CTA of the cluster gave up
+    float* sParts = reinterpret_cast<float*>(bars + kNumBars + 2);        // split: the other CTAs' sums, [rank - 1][MP][kUnitRows]
     const uint32_t bar0 = smem_addr(bars);
     auto bar = [&](int i) { return bar0 + 8u * (uint32_t)i; };
 
@@ -240,13 +244,21 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         *give_up = 0;
+        *lost_box = 0;
     }
     __syncthreads();
+    if constexpr (SPLIT) cluster_arrive();                        // (the box is clear, the CTA is there: awaited before a peer writes)
 
     const int b = blockIdx.x, C_ = a.chunks;
-    const int u0 = b * a.per_cta;
-    int u1 = min(a.units, u0 + a.per_cta);
-    if (!blob_header_ok(h0, h1, Q, G, a.g.N, a.g.K)) {         // before any tile is read; the same answer in every thread: no work
+    int u0 = b * a.per_cta, u1 = min(a.units, u0 + a.per_cta), rank = 0;
+    if constexpr (SPLIT) {                                    // a tile's chunks in ascending shares
+        const int tile = b / a.split;
+        rank = b - tile * a.split;
+        u0 = tile * C_ + C_ * rank / a.split;
+        u1 = tile * C_ + C_ * (rank + 1) / a.split;
+    }
+    const bool refused = !blob_header_ok(h0, h1, Q, G, a.g.N, a.g.K);
+    if (refused) {                                            // before any tile is read; the same answer in every thread: no work
         u1 = u0;
         if (tid == 0 && a.g.counters != nullptr) atomicExch(a.g.counters, kStatusBlobMismatch);
     }
@@ -473,6 +485,12 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
         if (step == 0)                                        // copies in flight land before the CTA may leave (given up or not)
             for (int n = max(u0, wu - a.ws); n < wu; ++n)
                 for (uint32_t t = 0; t < kFragWaitLimit && !mbar_try(bar(kBarWFull + (n - u0) % a.ws), (uint32_t)((n - u0) / a.ws) & 1u); ++t) {}
+        if constexpr (SPLIT) {
+            __syncwarp();
+            cluster_wait();
+            cluster_arrive();
+            cluster_wait();
+        }
         __syncthreads();
         return;
     }
@@ -557,8 +575,20 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
     float* own_sum = sSum + (step * MP + (BYTES ? c >> 1 : 2 * c)) * kSumStride + 32 * rp + gq;      // where the lane's sums go in the buffer
     auto sum_at = [](int nb, int t, int i) { return BYTES ? 2 * nb * kSumStride + 16 * t + 8 * i : (8 * nb + (i & 1)) * kSumStride + 16 * t + 8 * (i >> 1); };
 
+    auto sum_of = [&](int m, int row, int n, int chunk, int end) {         // this CTA's part of Y[mb + m][n]
+        float y = sSum[m * kSumStride + row];
+#pragma unroll
+        for (int s = 1; s < 4; ++s) y += sSum[(s * MP + m) * kSumStride + row];
+        if constexpr (BYTES) {
+            if (__builtin_expect((__float_as_uint(y) & 0x7f800000u) == 0x7f800000u, 0) && n < N)
+                y = plain_sum<Q>(a.g.X + (size_t)m * a.g.K, a.g.tiles + (size_t)(n >> 4) * C::TILE_BYTES, (size_t)a.g.n_rb * C::TILE_BYTES, n & 15, chunk, end,
+                                 a.n_steps, a.g.flags);
+        }
+        return y;
+    };
+
     Ring w(a.ws), x(kXSlots);
-    bool live = true;
+    bool live = true, gone = refused;                         // gone: the compute warps gave up together
     int pending = -1;                                         // output tile whose ticket has been taken and not looked at
     for (int u = u0; u < u1 && live;) {
         const int tile = a.by_chunks.of(u), chunk0 = u - tile * C_;
@@ -806,7 +836,8 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
                 for (int i = 0; i < NE; ++i)
                     own_sum[sum_at(nb, t, i)] = FOLD && n_units > 1 ? own_sum[sum_at(nb, t, i)] + acc[t][nb][i] : acc[t][nb][i];
         if (compute_any(!live)) {                             // the tickets of this run of units and the rest are taken all the same
-            for (int v = u - n_units; v < u1 && tid == 0;) {
+            gone = true;
+            for (int v = u - n_units; v < u1 && tid == 0 && !SPLIT;) {
                 const int t_ = a.by_chunks.of(v), end = min((t_ + 1) * C_, u1);
                 if (end - v < C_) {
                     const unsigned t = atomicAdd(ticket_of(t_), 1u + kTicketNoPart);
@@ -816,18 +847,12 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
             }
             break;
         }
+        if constexpr (SPLIT) break;                           // (its only run: the cluster adds up)
         const int row = tid & (kUnitRows - 1), n = row_tile(tile) * kUnitRows + row, mb = batch0(tile), m_end = min(MP, M - mb);
         const bool whole = n_units == C_;
         float* part = a.g.partials + ((size_t)(b - a.by_cta.of(tile * C_)) * M + mb) * n_pad + n;
         for (int m = tid >> 7; m < m_end; m += kComputeThreads / kUnitRows) {
-            float y = sSum[m * kSumStride + row];
-#pragma unroll
-            for (int s = 1; s < 4; ++s) y += sSum[(s * MP + m) * kSumStride + row];
-            if constexpr (BYTES) {
-                if (__builtin_expect((__float_as_uint(y) & 0x7f800000u) == 0x7f800000u, 0) && n < N)
-                    y = plain_sum<Q>(a.g.X + (size_t)m * a.g.K, a.g.tiles + (size_t)(n >> 4) * C::TILE_BYTES, (size_t)a.g.n_rb * C::TILE_BYTES, n & 15, chunk0,
-                                     chunk0 + n_units, a.n_steps, a.g.flags);
-            }
+            const float y = sum_of(m, row, n, chunk0, chunk0 + n_units);
             if (whole) {
                 if (n < N) put(mb + m, n, y);
             } else if ((size_t)n < n_pad) {
@@ -848,6 +873,38 @@ __global__ void __launch_bounds__(kFragThreads, 1) hlq_frag_kernel(const FragArg
     }
     compute_sync();
     finish_tile(pending);
+    if constexpr (SPLIT) {
+        // The first CTA of the cluster adds the others' sums to its own, in ascending k order (and in pairs, as above), and writes them out.
+        const int tile = b / a.split, row = tid & (kUnitRows - 1), n = row_tile(tile) * kUnitRows + row, mb = batch0(tile), m_end = min(MP, M - mb);
+        __syncwarp();
+        cluster_wait();                                       // the first CTA is there
+        float y[MP / 4 + 1];
+        if (gone) {
+            if (tid == 0) st_cluster_u32((uint32_t)__cvta_generic_to_shared((const void*)lost_box), 0u, 1u);
+        } else {
+#pragma unroll
+            for (int i = 0; i < (MP + 3) / 4; ++i) {
+                const int m = (tid >> 7) + 4 * i;
+                if (m >= m_end) continue;
+                y[i] = sum_of(m, row, n, u0 - tile * C_, u1 - tile * C_);
+                if (rank > 0) st_cluster_u32(smem_addr(sParts + ((rank - 1) * MP + m) * kUnitRows + row), 0u, __float_as_uint(y[i]));
+            }
+        }
+        __syncwarp();
+        cluster_arrive();
+        cluster_wait();                                       // the parts are there
+        if (rank == 0 && !gone && *lost_box == 0u && n < N) {
+#pragma unroll
+            for (int i = 0; i < (MP + 3) / 4; ++i) {
+                const int m = (tid >> 7) + 4 * i;
+                if (m >= m_end) continue;
+                auto part = [&](int r) { return r == 0 ? y[i] : r < a.split ? sParts[((r - 1) * MP + m) * kUnitRows + row] : 0.f; };
+                float sum = 0.f;
+                for (int r = 0; r < a.split; r += 4) sum += (part(r) + part(r + 1)) + (part(r + 2) + part(r + 3));
+                put(mb + m, n, sum);
+            }
+        }
+    }
     __syncthreads();                                          // nobody leaves while copies are in flight
 }
 
@@ -860,7 +917,8 @@ int launch_frag_cfg(const GemmArgs& g, int num_sms, cudaStream_t stream) {
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev >= 0 && dev < 64 && !configured[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(hlq_frag_kernel<Q, G, NB, FOLD, BYTES>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+        cudaError_t e = cudaFuncSetAttribute(hlq_frag_kernel<Q, G, NB, FOLD, BYTES, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(hlq_frag_kernel<Q, G, NB, FOLD, BYTES, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
         if (e != cudaSuccess) return (int)e;
         configured[dev] = true;
     }
@@ -873,32 +931,52 @@ int launch_frag_cfg(const GemmArgs& g, int num_sms, cudaStream_t stream) {
     if (units >= (1LL << 30)) return (int)cudaErrorInvalidValue;
     a.units = (int)units;
     a.per_cta = (a.units + num_sms - 1) / num_sms;
+    // Few output tiles: each to a cluster of CTAs, where its longest share is no longer than equal runs of all units would be.  A ticket's round trip
+    // through the L2, behind its fence, costs 1800 cycles and the parts as much again; the cluster's barriers and its writes to the first CTA's shared
+    // memory about 1000.  (us, tickets / clusters: 4096 x 4096, M = 4, q = 2, 3, 4 6.8, 7.7, 8.8 / 6.1, 7.4, 8.7, M = 8 7.3, 8.3, 9.6 / 6.3, 7.4, 8.7; 4096 x 14336,
+    // M = 8, q = 3 18.9 / 17.7; 5003 x 2880, G = 64, q = 3, M = 16 13.1 / 11.3.  A longer share loses: a unit more takes 0.5 + 0.6 q us.)
+    a.split = 1;
+    int longest = a.per_cta;
+    if (a.per_cta < a.chunks) {
+        const int tiles = a.units / a.chunks;
+        for (int n = 2; n <= 8 && n <= a.chunks; ++n) {
+            const int share = (a.chunks + n - 1) / n;
+            if (tiles <= resident_clusters(n) && (share < longest || (share == longest && a.split == 1))) {
+                a.split = n;
+                longest = share;
+            }
+        }
+    }
     // Runs of more than two units without a sum per step: the sums are put by in between, for the same reason as there (4096 x 14336, q = 4,
     // G = 64, M = 16, error of the fp32 result 1.5e-7 -> 1.0e-7, the look-up kernel 1.0e-7 to 1.5e-7 by the number of rows; time
     // 36.3 -> 36.8 us).
     if constexpr (NB > 1 && !FOLD && !BYTES) {
-        if (a.per_cta > 2) return launch_frag_cfg<Q, G, NB, BYTES, true>(g, num_sms, stream);
+        if (longest > 2) return launch_frag_cfg<Q, G, NB, BYTES, true>(g, num_sms, stream);
     }
     a.by_chunks.set(a.chunks);
     a.by_blocks.set(a.blocks);
     a.by_cta.set(a.per_cta);
-    const int grid = (a.units + a.per_cta - 1) / a.per_cta;
+    const int grid = a.split > 1 ? a.units / a.chunks * a.split : (a.units + a.per_cta - 1) / a.per_cta;
+    const int parts_bytes = (a.split - 1) * MP * kUnitRows * 4;
     a.tickets = g.tickets;
-    static_assert((kMaxSmem - kFixed) / C::UNIT_BYTES >= 2, "shared memory");
-    a.ws = (kMaxSmem - kFixed) / C::UNIT_BYTES;
+    static_assert((kMaxSmem - kFixed - 7 * MP * kUnitRows * 4) / C::UNIT_BYTES >= 2, "shared memory");
+    a.ws = (kMaxSmem - kFixed - parts_bytes) / C::UNIT_BYTES;
     if (a.ws > 5) a.ws = 5;
 
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3(kFragThreads);
-    cfg.dynamicSmemBytes = a.ws * C::UNIT_BYTES + kFixed;
+    cfg.dynamicSmemBytes = a.ws * C::UNIT_BYTES + kFixed + parts_bytes;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)a.split;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, hlq_frag_kernel<Q, G, NB, FOLD, BYTES>, a);
+    cfg.numAttrs = a.split > 1 ? 2 : 1;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, a.split > 1 ? hlq_frag_kernel<Q, G, NB, FOLD, BYTES, true> : hlq_frag_kernel<Q, G, NB, FOLD, BYTES, false>, a);
     count_launch(1);
     return (int)e;
 }

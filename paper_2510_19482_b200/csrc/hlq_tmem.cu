@@ -156,12 +156,6 @@ __device__ __forceinline__ uint32_t opaque(uint32_t v) {
     return v;
 }
 
-__device__ __forceinline__ void st_cluster_u32(uint32_t addr, uint32_t rank, uint32_t v) {
-    uint32_t remote;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr), "r"(rank));
-    asm volatile("st.shared::cluster.u32 [%0], %1;" :: "r"(remote), "r"(v) : "memory");
-}
-
 // How many warps before this one took the ticket: read, or (add = 1 and a mark) announced behind the warp's own writes.
 __device__ __forceinline__ unsigned ticket_seen(unsigned* ticket, int lane, unsigned add) {
     unsigned t = 0;
@@ -745,7 +739,7 @@ Schedule schedule_of(int q, int M, int N, int K, int num_sms, const int (&max_cl
 }
 
 // Clusters of each size that are resident together on the current device (on one that cannot say: GPCs of 18 and 20 SMs).
-const int (&resident_clusters())[kMaxSplit + 1];
+const int (&cluster_table())[kMaxSplit + 1];
 
 template <int Q>
 int launch_tmem_q(const GemmArgs& g, int num_sms, cudaStream_t stream) {
@@ -761,7 +755,7 @@ int launch_tmem_q(const GemmArgs& g, int num_sms, cudaStream_t stream) {
         configured[dev] = true;
     }
     if (!tmem_takes(g.M, g.N, g.K)) return (int)cudaErrorNotSupported;
-    const Schedule sch = schedule_of(Q, g.M, g.N, g.K, num_sms, resident_clusters());
+    const Schedule sch = schedule_of(Q, g.M, g.N, g.K, num_sms, cluster_table());
     TmemArgs a;
     a.g = g;
     a.m_tiles = sch.m_tiles;
@@ -823,7 +817,7 @@ int launch_tmem_q(const GemmArgs& g, int num_sms, cudaStream_t stream) {
     return ce != 0 || sch.full == sch.tiles ? ce : launch(sch.full, sch.tiles - sch.full, sch.rest);
 }
 
-const int (&resident_clusters())[kMaxSplit + 1] {
+const int (&cluster_table())[kMaxSplit + 1] {
     struct Table { int n[kMaxSplit + 1]; };
     static const Table fallback = {{0, 148, 74, 48, 34, 26, 24, 16, 16}};
     static Table tables[64];
@@ -861,6 +855,8 @@ const int (&resident_clusters())[kMaxSplit + 1] {
 
 }  // namespace
 
+int resident_clusters(int size) { return cluster_table()[size]; }
+
 bool tmem_takes(int M, int N, int K) {
     return (((long long)N + kTileRowsN - 1) / kTileRowsN) * ((M + kMaxTokens - 1) / kMaxTokens) * (K / 128) < (1LL << 30);
 }
@@ -870,7 +866,7 @@ bool tmem_takes(int M, int N, int K) {
 double tmem_us(int M, int N, int K, int q, int num_sms) {
     static const double whole_step[5] = {0, 0.22, 0.32, 0.68, 0.96}, whole_tokens[5] = {0, 0.0049, 0.0046, 0.0029, 0.0026};
     static const double share_step[5] = {0, 0.2, 0.3, 0.65, 0.8}, share_tokens[5] = {0, 0.0054, 0.0055, 0.004, 0.0047};
-    const Schedule s = schedule_of(q, M, N, K, num_sms, resident_clusters());
+    const Schedule s = schedule_of(q, M, N, K, num_sms, cluster_table());
     const double round = 3.8 + s.n_steps * (whole_step[q] + whole_tokens[q] * s.mp);
     const double rounds = 1.1 + (s.full + num_sms - 1) / num_sms * round;
     if (s.full < s.tiles) return rounds + 5.0 + 0.97 * s.rest.cost;

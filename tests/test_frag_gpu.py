@@ -224,3 +224,47 @@ def test_batch_blocks_of_one_launch(q, N, K, M):
     assert max(hlq.rel_fro_error(y[m], ref[m]) for m in range(M)) <= 5e-6
     assert np.array_equal(y, again)
     assert elutq.elutq_device_status() == 0
+
+
+# Few output tiles, each shared by a cluster of CTAs: more CTAs than fit (as many as its chunks), shares of unequal length, a last chunk of one step,
+# ragged rows, several batch blocks, every form; the widest call that clusters of two take, and one tile more
+@pytest.mark.parametrize("q,G,N,K,M", [(3, 128, 1500, 4736, 4), (1, 128, 130, 1024, 4), (2, 128, 4100, 4224, 2), (4, 128, 3000, 2688, 8), (1, 128, 200, 7680, 3),
+                                       (2, 64, 1300, 3648, 7), (3, 64, 257, 5184, 16), (4, 64, 1000, 2112, 40), (2, 128, 74 * 128, 1152, 6), (2, 128, 74 * 128 + 1, 1152, 6)])
+def test_output_tiles_of_clusters(q, G, N, K, M):
+    layer = workloads.hlq_layer(72, f"frag/clusters/{q}/{G}/{N}/{K}", q, G, N, K)
+    X = synth.activations(72, f"frag/clusters/x/{M}/{K}", M, K, outliers=True)
+    packed = pack_layer(layer)
+    assert elutq.elutq_gemm_kernel(M, N, K, q, G) == elutq.KERNEL_FRAGMENT
+    ref = hlq.matmul(X, layer.planes, layer.scales, layer.offsets, G)
+    y = gemm_f32(X, packed, N, K)
+    assert elutq.elutq_device_status() == 0
+    assert max(hlq.rel_fro_error(y[m], ref[m]) for m in range(M)) <= 5e-6
+    assert np.all(np.abs(y - ref) <= 2 * K * 2.0 ** -24 * hlq.magnitude_bound(X, layer.scales, layer.offsets, G))
+    assert np.array_equal(y, gemm_f32(X, packed, N, K))
+    Y = torch.full((M, N), 1.5, dtype=torch.float32, device="cuda")
+    elutq.elutq_lut_gemm_f32(x_dev(X), packed, Y, M, N, K, elutq.FLAG_ACCUMULATE)
+    np.testing.assert_allclose(Y.cpu().numpy(), y + 1.5, rtol=0, atol=1e-5 * np.abs(y).max())
+    # a value that is not finite in the share of a later CTA
+    X[1, K - 5] = np.inf
+    z = gemm_f32(X, packed, N, K)
+    keep = np.arange(M) != 1
+    assert np.array_equal(z[keep], y[keep]) and not np.isfinite(z[1]).any()
+
+
+@pytest.mark.parametrize("M,half", [(9, 0), (20, 0), (9, 0x80000000), (20, 0x80000000)])
+def test_clusters_report_a_wait_that_runs_out(M, half):
+    # in all CTAs, or in every other one: nothing is written where a part is missing, and the next call is whole
+    q, G, N, K = 3, 64, 1500, 4672
+    layer = workloads.hlq_layer(73, "frag/clusters/expiry", q, G, N, K)
+    X = synth.activations(73, f"frag/clusters/expiry/x/{M}", M, K)
+    packed = pack_layer(layer)
+    ref = hlq.matmul(X, layer.planes, layer.scales, layer.offsets, G)
+    for limit in (300, 20000):
+        elutq.elutq_release_scratch()
+        Y = torch.full((M, N), 7.5, dtype=torch.float32, device="cuda")
+        elutq.elutq_test_wait_expiry(x_dev(X), packed, Y, M, N, K, half | limit)
+        assert elutq.elutq_device_status() == 0x7C05
+        assert torch.all(Y == 7.5)
+    elutq.elutq_release_scratch()
+    assert hlq.rel_fro_error(gemm_f32(X, packed, N, K), ref) <= 5e-6
+    assert elutq.elutq_device_status() == 0

@@ -19,7 +19,8 @@ HALF = 0x80000000          # every other CTA gives up
 
 
 # the fragment kernel with one and with several chunks per CTA; the tensor-memory kernel with tiles of two parts
-@pytest.mark.parametrize("q,G,N,K,M", [(3, 64, 1000, 1984, 20), (2, 64, 9000, 2240, 9), (4, 128, 20480, 2048, 16)])
+# (and with more output tiles than clusters take, with one and with several batch blocks)
+@pytest.mark.parametrize("q,G,N,K,M", [(3, 64, 1000, 1984, 20), (2, 64, 9000, 2240, 9), (4, 128, 20480, 2048, 16), (3, 64, 20000, 2688, 9), (2, 64, 10000, 2240, 20)])
 def test_tickets_are_zero_after_some_ctas_gave_up(q, G, N, K, M):
     layer = workloads.hlq_layer(64, f"tickets/{q}/{G}/{N}/{K}", q, G, N, K)
     X = synth.activations(64, f"tickets/x/{M}/{K}", M, K)
