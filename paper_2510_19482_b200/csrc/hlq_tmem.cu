@@ -11,8 +11,8 @@
 //              parts of a tile that several CTAs share go to the workspace and are added in ascending k order (bit-reproducible)
 //              by the CTA that comes last or, where there are many, by a second kernel.  Or the CTAs of a cluster share the K of a
 //              tile and add up through their shared memory (a rule on costs: plan_of).
-//   warps      0 and 3 weight loaders (one bulk copy per row block and 512 k: eight packed tiles, contiguous in the blob), 1 MMA
-//              issuer, 2 activation loader (TMA, 128-byte swizzle), 4-19 producers: two warpgroups per row block, which take
+//   warps      0 weight loader (one bulk copy per row block and 512 k: eight packed tiles, contiguous in the blob), 1 MMA issuer, 2 activation loader
+//              (TMA, 128-byte swizzle; few tokens: 2 and 3, by loads and stores, in another order), 4-19 producers: two warpgroups per row block, which take
 //              the steps in turn, rebuild the weights, and at the end of a tile write out half of its tokens each.  (Four warps
 //              per scheduler: with two, the latencies of a step's parameters, waits and stores were half of the time.)
 //   slot       one 128-k step of one row block: 64 TMEM columns above the accumulators (2 x tokens columns).
@@ -20,6 +20,8 @@
 //              one logic operation leaves the bits of one weight pair, which read as fp16 are powers of two (at position 15 a
 //              sign), and one packed fma multiplies with the scale over that power and adds: 3.5 half-rate or full-rate issue
 //              slots per pair and plane.  (Moving the bits to the sign positions by a multiplication, an xor with s_j / 2 and an add: 5.5.)
+//              Few tokens (PERM): k and k + 16 of the activations side by side, as the two halves of a word of weight bits lie.  A word shifted (by a
+//              multiplication, but for one in four) has four bits of each half at positions 11 to 14; no byte permute, no sign.
 //
 //   bound      the producers' integer logic pipe (q = 4: 320 of a slot's 470 operations are the dequantisation itself, 65 to 75 % of
 //              the pipe's cycles); from 96 tokens also the activations' way from the L2.  Against weights rebuilt in shared memory with one
@@ -30,6 +32,7 @@
 // roles' waits; copies and MMAs in flight are waited for (bounded), tensor memory is freed, the kernel returns.
 #include <cuda.h>
 
+#include <initializer_list>
 #include <mutex>
 
 #include "common.cuh"
@@ -72,6 +75,7 @@ struct TmCfg {
     static constexpr int PLANE_BYTES = 1024 * Q;
     static constexpr int TILE_BYTES = PLANE_BYTES + 128 * (Q + 1);
     static constexpr int UNIT_BYTES = 8 * TILE_BYTES;         // 512 k of one row block
+    static constexpr int PERM_TOKENS = Q == 3 ? 32 : 16;      // tokens of a tile up to which PERM may be taken (launch_tmem_q)
 };
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -171,8 +175,8 @@ __device__ __forceinline__ unsigned ticket_seen(unsigned* ticket, int lane, unsi
 
 __device__ __forceinline__ __half2 as_half2(uint32_t v) { return *reinterpret_cast<const __half2*>(&v); }
 
-// CLUSTER: a tile's K is shared by the CTAs of a cluster.
-template <int Q, bool CLUSTER>
+// CLUSTER: a tile's K is shared by the CTAs of a cluster.  PERM: few tokens, whose activations are put in the order of a word's halves.
+template <int Q, bool CLUSTER, bool PERM>
 __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_constant__ CUtensorMap xmap, const TmemArgs a) {
     using C = TmCfg<Q>;
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -250,28 +254,69 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
             for (uint32_t t = 0; t < kTmWaitLimit && !mbar_try(bar(bar_full + n % len), (uint32_t)(n / len) & 1u); ++t) {}
     };
 
-    if (warp == 0 || warp == 3) {
-        // ---- weight loaders, one per row block (weights do not depend on the previous kernel) ---------------------------------
+    if (warp == 0) {
+        // ---- weight loader (weights do not depend on the previous kernel) ----------------------------------------------------------
         grid_launch_dependents();
-        const int blk = warp == 3;
         if (lane == 0) {
             Ring w(a.ws);
-            int issued = 0;
+            int issued[kBlocks] = {};
             bool ok = true;
-            for (Walk r(t0, t1, a.n_steps); r.more(); r.next()) {
-                ok = wait(kBarWEmpty + blk * kMaxW + w.i, w.phase ^ 1u);
-                if (!ok) break;
-                const int rb0 = ((r.tile + base_tile) / a.m_tiles) * (kBlocks * 8) + blk * 8, nrb = max(0, min(8, a.g.n_rb - rb0));
-                const uint32_t bytes = (uint32_t)(nrb * C::TILE_BYTES), mb = bar(kBarWFull + blk * kMaxW + w.i);
-                mbar_expect(mb, bytes);
-                if (nrb > 0)
-                    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                                 :: "r"(smem_addr(sW) + (uint32_t)((blk * a.ws + w.i) * C::UNIT_BYTES)),
-                                    "l"(a.g.tiles + ((size_t)(r.step >> 2) * a.g.n_rb + rb0) * C::TILE_BYTES), "r"(bytes), "r"(mb) : "memory");
-                ++issued;
+            for (Walk r(t0, t1, a.n_steps); r.more() && ok; r.next()) {
+                for (int blk = 0; blk < kBlocks; ++blk) {
+                    ok = wait(kBarWEmpty + blk * kMaxW + w.i, w.phase ^ 1u);
+                    if (!ok) break;
+                    const int rb0 = ((r.tile + base_tile) / a.m_tiles) * (kBlocks * 8) + blk * 8, nrb = max(0, min(8, a.g.n_rb - rb0));
+                    const uint32_t bytes = (uint32_t)(nrb * C::TILE_BYTES), mb = bar(kBarWFull + blk * kMaxW + w.i);
+                    mbar_expect(mb, bytes);
+                    if (nrb > 0)
+                        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                                     :: "r"(smem_addr(sW) + (uint32_t)((blk * a.ws + w.i) * C::UNIT_BYTES)),
+                                        "l"(a.g.tiles + ((size_t)(r.step >> 2) * a.g.n_rb + rb0) * C::TILE_BYTES), "r"(bytes), "r"(mb) : "memory");
+                    ++issued[blk];
+                }
                 w.next();
             }
-            drain(kBarWFull + blk * kMaxW, a.ws, issued);
+            for (int blk = 0; blk < kBlocks; ++blk) drain(kBarWFull + blk * kMaxW, a.ws, issued[blk]);
+        }
+    } else if (PERM && (warp == 2 || warp == 3)) {
+        // ---- activation loaders of few tokens, which take the steps in turn: a lane takes 32 k of a token and puts k and k + 16 side by side, as the
+        // two halves of a word of weight bits lie.  (16 tokens a turn and two turns' loads on their way: M = 16 0 to 1.5 % slower, M = 32, q = 3 5 to 14 %.)  ---
+        grid_dependency_wait();
+        const int total = t1 - t0, m_lane = lane >> 2, c = lane & 3;
+        uint4 v[C::PERM_TOKENS / 8][4];
+        auto fetch = [&](int xs) {
+            const int t = t0 + xs, tile = t / a.n_steps, step = t - tile * a.n_steps, m0 = ((tile + base_tile) % a.m_tiles) * a.mp + m_lane;
+#pragma unroll
+            for (int g = 0; g < C::PERM_TOKENS / 8; ++g)
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    v[g][e] = xs < total && 8 * g < a.mp && m0 + 8 * g < a.g.M
+                                  ? reinterpret_cast<const uint4*>(a.g.X + (size_t)(m0 + 8 * g) * a.g.K + step * 128 + c * 32)[e] : make_uint4(0, 0, 0, 0);
+        };
+        int xs = warp - 2;
+        fetch(xs);
+        for (; xs < total; xs += 2) {
+            const int slot = xs % a.xs;
+            if (!wait_warp(kBarXEmpty + slot, ((uint32_t)(xs / a.xs) & 1u) ^ 1u)) break;
+            uint8_t* dst = sX + slot * x_bytes + (c >> 1) * blk_bytes;
+#pragma unroll
+            for (int g = 0; g < C::PERM_TOKENS / 8; ++g) {
+                if (8 * g >= a.mp) break;
+                const int row = m_lane + 8 * g;
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {                 // bytes e and e + 2 of the words
+                    const uint4 lo = v[g][e], hi = v[g][e + 2];
+                    const uint4 o[2] = {make_uint4(__byte_perm(lo.x, hi.x, 0x5410), __byte_perm(lo.x, hi.x, 0x7632), __byte_perm(lo.y, hi.y, 0x5410), __byte_perm(lo.y, hi.y, 0x7632)),
+                                        make_uint4(__byte_perm(lo.z, hi.z, 0x5410), __byte_perm(lo.z, hi.z, 0x7632), __byte_perm(lo.w, hi.w, 0x5410), __byte_perm(lo.w, hi.w, 0x7632))};
+#pragma unroll
+                    for (int i = 0; i < 2; ++i)
+                        *reinterpret_cast<uint4*>(dst + row * 128 + (((4 * (c & 1) + 2 * e + i) ^ (row & 7)) << 4)) = o[i];
+                }
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(kBarXFull + slot));
+            fetch(xs + 2);
         }
     } else if (warp == 2) {
         // ---- activation loader: a step is two boxes of 64 k ------------------------------------------------------------------
@@ -400,6 +445,49 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
 #pragma unroll
                     for (int i = 0; i < 4; ++i) pw[j][i] = __funnelshift_l(t[(i + 3) & 3], t[i], byte_rot);
                 }
+                __half2 factor[Q][4], z2, start3;
+                int down;
+                bool any_up;
+                // Its parameters s_0 .. s_{Q-1}, z, two to a word.  Plane j's bit at position 11 .. 14 of a half is 2^-13, 2^-11, 2^-7, 2 as an fp16
+                // number, so that with factor[j][position] it contributes s_j (exact products).  Scales of 1 and more would not fit the factors:
+                // such a row is built 2^-down times its size (down = exponent of its largest scale, plus one) and scaled up at the end.
+                if constexpr (PERM) {
+                    uint32_t sc[Q / 2 + 1];
+#pragma unroll
+                    for (int i = 0; i <= Q / 2; ++i)
+                        sc[i] = *reinterpret_cast<const uint32_t*>(rec + C::PLANE_BYTES - l * 12 + h * 64 + (uu * ((Q + 1) / 2) + i) * 128);
+                    if (Q % 2 == 0) {                         // (an odd number of them: the second step's begin in the middle of a word)
+#pragma unroll
+                        for (int i = 0; i <= Q / 2; ++i) sc[i] = __funnelshift_r(sc[i], i < Q / 2 ? sc[i + 1] : 0u, uu * 16);
+                    }
+                    if (a.g.flags & (ELUTQ_FLAG_OFFSET_ONLY | ELUTQ_FLAG_SKIP_OFFSET)) {
+#pragma unroll
+                        for (int j = 0; j <= Q; ++j)
+                            if (a.g.flags & (j < Q ? ELUTQ_FLAG_OFFSET_ONLY : ELUTQ_FLAG_SKIP_OFFSET)) sc[j / 2] &= j & 1 ? 0x0000ffffu : 0xffff0000u;
+                    }
+                    if (step + 2 >= r.end) release();
+                    auto param = [&](int j) { return j & 1 ? __high2half2(as_half2(sc[j / 2])) : __low2half2(as_half2(sc[j / 2])); };
+                    __half2 most = __habs2(param(0));
+#pragma unroll
+                    for (int j = 1; j < Q; ++j) most = __hmax2(most, __habs2(param(j)));
+                    any_up = __any_sync(0xffffffffu, __low2float(most) >= 1.f);
+                    __half2 down2 = __float2half2_rn(1.f);
+                    z2 = param(Q);
+                    down = 0;
+                    if (any_up) {
+                        down = max((int)(__half_as_ushort(__low2half(most)) >> 10) - 14, 0);
+                        down2 = __float2half2_rn(__int_as_float((127 - down) << 23));          // exact, 2^-16 as a subnormal
+                        z2 = __hmul2(z2, down2);
+                    }
+#pragma unroll
+                    for (int j = 0; j < Q; ++j) {
+                        const __half2 s2 = any_up ? __hmul2(param(j), down2) : param(j);
+                        factor[j][0] = __hmul2(s2, __float2half2_rn(8192.f));
+                        factor[j][1] = __hmul2(s2, __float2half2_rn(2048.f));
+                        factor[j][2] = __hmul2(s2, __float2half2_rn(128.f));
+                        factor[j][3] = __hmul2(s2, __float2half2_rn(0.5f));
+                    }
+                } else {
                 // Its parameters s_0 .. s_{Q-1}, z.  Plane j's bit at position 8..14 of a half is 2^-16, 2^-15, 2^-14, 2^-13, 2^-11, 2^-7,
                 // 2 as an fp16 number and at position 15 a sign, so that with factor[j][p] it contributes s_j (exact products),
                 // as a sign +-s_j/2.  Scales of 1 and more would not fit the factors: such a row is built 2^-down times its
@@ -421,9 +509,9 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
                     if (c < Q) top = max(top, sc[c] & 0x7c00u);
                 }
                 if (step + 2 >= r.end) release();
-                const int down = max((int)(top >> 10) - 14, 0);
-                const bool any_up = __any_sync(0xffffffffu, down != 0);
-                __half2 factor[Q][4], z2 = as_half2(sc[Q]);
+                down = max((int)(top >> 10) - 14, 0);
+                any_up = __any_sync(0xffffffffu, down != 0);
+                z2 = as_half2(sc[Q]);
                 float zhat = __low2float(z2);
 #pragma unroll
                 for (int j = 0; j < Q; ++j) zhat += 0.5f * __low2float(as_half2(sc[j]));
@@ -446,7 +534,8 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
                     factor[j][2] = __hmul2(s2, __floats2half2_rn(2048.f, 128.f));
                     factor[j][3] = __hmul2(s2, __float2half2_rn(0.5f));
                 }
-                const __half2 start3 = __lows2half2(z2, zh2);  // weight 7 of a byte has its bit at the sign
+                start3 = __lows2half2(z2, zh2);  // weight 7 of a byte has its bit at the sign
+                }
 
                 live = wait_warp(kBarAEmpty + blk * kMaxSlots + s.i, s.phase ^ 1u);
                 if (!live) break;
@@ -455,6 +544,21 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
 #pragma unroll
                 for (int i4 = 0; i4 < 4; ++i4) {
                     uint32_t o[16];
+                    if constexpr (PERM) {
+                        // 32 weights: register 8 e + i holds bit i of bytes e and e + 2
+#pragma unroll
+                        for (int v = 0; v < 4; ++v) {         // bits 0-3 and 4-7 of bytes 0 and 2, of bytes 1 and 3
+                            __half2 acc[4] = {z2, z2, z2, z2};
+#pragma unroll
+                            for (int j = 0; j < Q; ++j) {
+                                const uint32_t w = pw[j][i4], x = v == 0 ? w * 2048u : v == 1 ? w * 128u : v == 2 ? w * 8u : w >> 1;
+#pragma unroll
+                                for (int p = 0; p < 4; ++p) acc[p] = __hfma2(as_half2(x & (0x08000800u << p)), factor[j][p], acc[p]);
+                            }
+#pragma unroll
+                            for (int p = 0; p < 4; ++p) o[4 * v + p] = *reinterpret_cast<const uint32_t*>(&acc[p]);
+                        }
+                    } else {
 #pragma unroll
                     for (int by = 0; by < 4; ++by) {
                         __half2 acc[4] = {z2, z2, z2, start3};
@@ -471,6 +575,7 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
                         }
 #pragma unroll
                         for (int p = 0; p < 4; ++p) o[4 * by + p] = *reinterpret_cast<const uint32_t*>(&acc[p]);
+                    }
                     }
                     if (any_up) {
                         const __half2 up0 = __float2half2_rn(__int_as_float((127 + (down >> 1)) << 23));
@@ -753,8 +858,9 @@ int launch_tmem_q(const GemmArgs& g, int num_sms, cudaStream_t stream) {
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64) return (int)cudaErrorNotSupported;
     if (!configured[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(hlq_tmem_kernel<Q, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(hlq_tmem_kernel<Q, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+        cudaError_t e = cudaSuccess;
+        for (auto kernel : {hlq_tmem_kernel<Q, false, false>, hlq_tmem_kernel<Q, true, false>, hlq_tmem_kernel<Q, false, true>, hlq_tmem_kernel<Q, true, true>})
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
         if (e != cudaSuccess) return (int)e;
         configured[dev] = true;
     }
@@ -814,7 +920,14 @@ int launch_tmem_q(const GemmArgs& g, int num_sms, cudaStream_t stream) {
         attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = a.split > 1 ? 2 : 1;
-        cudaError_t e = cudaLaunchKernelEx(&cfg, a.split > 1 ? hlq_tmem_kernel<Q, true> : hlq_tmem_kernel<Q, false>, map, a);
+        // PERM is ahead where the rebuild is the bound and two warps put the activations in order in time.  us without and with it, q = 2, 3, 4: M = 16,
+        // 4096 x 4096 8.6, 9.9, 11.3 / 8.3, 9.6, 10.9; 4096 x 14336 18.0, 22.3, 26.6 / 16.9, 20.7, 24.6; 28672 x 4096 25.1, 33.2, 40.7 / 23.6, 30.6, 38.8;
+        // 57344 x 8192 75.1, 100, 123 / 69.6, 91.6, 116.7.  On less than half of the SMs the next kernel's CTAs rebuild meanwhile, the activations' way is
+        // what counts: 1000 x 4096 5.0, 5.2, 5.35 / 5.1, 5.4, 5.55.  M = 32: only q = 3 gains, with some steps per CTA (28672 x 4096 25.5, 33.6, 41.1 /
+        // 26.0, 32.0, 41.3; 6144 x 4096, q = 3 12.65 / 12.4; 2560 x 4096, four steps, 7.95 / 8.2).
+        const bool perm = 2 * grid > num_sms && (a.mp <= 16 || (a.mp <= C::PERM_TOKENS && (a.split > 1 ? a.n_steps / a.split : a.per_cta) >= 5));
+        cudaError_t e = cudaLaunchKernelEx(&cfg, a.split > 1 ? (perm ? hlq_tmem_kernel<Q, true, true> : hlq_tmem_kernel<Q, true, false>)
+                                                             : (perm ? hlq_tmem_kernel<Q, false, true> : hlq_tmem_kernel<Q, false, false>), map, a);
         count_launch(1);
         if (e != cudaSuccess || a.reduce || a.per_cta % a.n_steps == 0 || grid == 1) return (int)e;
         cfg.gridDim = dim3((unsigned)(grid - 1), (unsigned)((a.mp + 7) / 8));
@@ -841,7 +954,7 @@ const int (&cluster_table())[kMaxSplit + 1] {
     }
     std::call_once(once[dev], [dev] {
         tables[dev] = fallback;
-        if (cudaFuncSetAttribute(hlq_tmem_kernel<4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) != cudaSuccess) {
+        if (cudaFuncSetAttribute(hlq_tmem_kernel<4, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) != cudaSuccess) {
             (void)cudaGetLastError();
             return;
         }
@@ -856,7 +969,7 @@ const int (&cluster_table())[kMaxSplit + 1] {
             attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
             cfg.attrs = attr;
             cfg.numAttrs = 1;
-            if (cudaOccupancyMaxActiveClusters(&tables[dev].n[n], hlq_tmem_kernel<4, true>, &cfg) != cudaSuccess) {
+            if (cudaOccupancyMaxActiveClusters(&tables[dev].n[n], hlq_tmem_kernel<4, true, false>, &cfg) != cudaSuccess) {
                 tables[dev].n[n] = 0;
                 (void)cudaGetLastError();
             }

@@ -25,7 +25,11 @@ G, TOL = 128, 1e-3
 # 200 -> 2 x 112); whole tiles per CTA, shared tiles of two or three parts, of many parts, clusters of two CTAs and more (with K steps and
 # tokens that they do not divide evenly, and N no multiple of the stores' four), whole rounds with the rest by clusters
 CASES = [(2, 4621, 128, 9), (1, 4480, 1152, 128), (3, 4600, 640, 200), (4, 5000, 2944, 100), (4, 12800, 2048, 384), (2, 38000, 256, 33),
-         (3, 10240, 1024, 130), (2, 11776, 7680, 16), (2, 16000, 1024, 100), (2, 3001, 4096, 20), (3, 1100, 1152, 90), (1, 300, 256, 33), (2, 13000, 2560, 384)]
+         (3, 10240, 1024, 130), (2, 11776, 7680, 16), (2, 16000, 1024, 100), (2, 3001, 4096, 20), (3, 1100, 1152, 90), (1, 300, 256, 33), (2, 13000, 2560, 384),
+         # few tokens, whose activations the kernel puts in another order: the last sizes on that path and the first beyond it, loaders of one, two and
+         # three steps, clusters, shared tiles, whole rounds with a rest
+         (1, 4480, 128, 12), (2, 4621, 256, 10), (4, 1100, 384, 15), (3, 4600, 1152, 17), (3, 12800, 640, 32), (4, 38000, 512, 25), (4, 3001, 4096, 33),
+         (2, 16000, 1024, 17), (4, 10240, 1024, 32), (3, 38000, 256, 16)]
 
 
 @pytest.mark.parametrize("q,N,K,M", CASES)
@@ -50,8 +54,8 @@ def test_tensor_memory_kernel_matches_oracle(q, N, K, M):
 
 
 @pytest.mark.parametrize("q", [1, 2, 4])
-def test_scales_of_one_and_more(q):
-    N, K, M = 4700, 256, 40
+def test_scales_of_one_and_more(q, M=40):
+    N, K = 4700, 256
     assert elutq.elutq_gemm_kernel(M, N, K, q, G) == elutq.KERNEL_TENSOR_MEMORY
     layer = workloads.hlq_layer(71, f"tmem/scales/{q}", q, G, N, K)
     s = layer.scales.astype(np.float32)
@@ -66,6 +70,11 @@ def test_scales_of_one_and_more(q):
     assert elutq.elutq_device_status() == 0
     for first in range(4):
         assert hlq.rel_fro_error(y[:, first::4], ref[:, first::4]) <= TOL
+
+
+@pytest.mark.parametrize("q,M", [(1, 12), (2, 16), (3, 9), (4, 17)])
+def test_scales_of_one_and_more_with_few_tokens(q, M):
+    test_scales_of_one_and_more(q, M)
 
 
 def test_a_wait_that_runs_out_is_reported():
