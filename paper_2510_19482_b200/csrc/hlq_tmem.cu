@@ -75,7 +75,6 @@ struct TmCfg {
     static constexpr int PLANE_BYTES = 1024 * Q;
     static constexpr int TILE_BYTES = PLANE_BYTES + 128 * (Q + 1);
     static constexpr int UNIT_BYTES = 8 * TILE_BYTES;         // 512 k of one row block
-    static constexpr int PERM_TOKENS = Q == 3 ? 32 : 16;      // tokens of a tile up to which PERM may be taken (launch_tmem_q)
 };
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -175,8 +174,8 @@ __device__ __forceinline__ unsigned ticket_seen(unsigned* ticket, int lane, unsi
 
 __device__ __forceinline__ __half2 as_half2(uint32_t v) { return *reinterpret_cast<const __half2*>(&v); }
 
-// CLUSTER: a tile's K is shared by the CTAs of a cluster.  PERM: few tokens, whose activations are put in the order of a word's halves.
-template <int Q, bool CLUSTER, bool PERM>
+// CLUSTER: a tile's K is shared by the CTAs of a cluster.  PERM > 0: that many tokens, whose activations are put in the order of a word's halves.
+template <int Q, bool CLUSTER, int PERM>
 __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_constant__ CUtensorMap xmap, const TmemArgs a) {
     using C = TmCfg<Q>;
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -278,45 +277,59 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
             }
             for (int blk = 0; blk < kBlocks; ++blk) drain(kBarWFull + blk * kMaxW, a.ws, issued[blk]);
         }
-    } else if (PERM && (warp == 2 || warp == 3)) {
+    } else if (PERM > 0 && (warp == 2 || warp == 3)) {
         // ---- activation loaders of few tokens, which take the steps in turn: a lane takes 32 k of a token and puts k and k + 16 side by side, as the
-        // two halves of a word of weight bits lie.  (16 tokens a turn and two turns' loads on their way: M = 16 0 to 1.5 % slower, M = 32, q = 3 5 to 14 %.)  ---
+        // two halves of a word of weight bits lie.  (Walking instead of dividing: M = 32 3 to 5 % faster, since the divisions take the rebuild's pipes.) ---
         grid_dependency_wait();
-        const int total = t1 - t0, m_lane = lane >> 2, c = lane & 3;
-        uint4 v[C::PERM_TOKENS / 8][4];
-        auto fetch = [&](int xs) {
-            const int t = t0 + xs, tile = t / a.n_steps, step = t - tile * a.n_steps, m0 = ((tile + base_tile) % a.m_tiles) * a.mp + m_lane;
+        const int m_lane = lane >> 2, c = lane & 3;           // (one token tile: step t is step t mod n_steps of K)
+        const __half* x = a.g.X + (size_t)m_lane * a.g.K + c * 32;
+        const uint32_t at = (uint32_t)((c >> 1) * blk_bytes + m_lane * 128 + ((4 * (c & 1) ^ m_lane) << 4));
+        constexpr int kTokens = PERM > 0 ? PERM : 16;         // = a.mp
+        int step = t0 % a.n_steps;
+        uint4 v[kTokens / 8][4];
+        auto fetch = [&](bool more) {
+            const __half* xk = x + step * 128;
 #pragma unroll
-            for (int g = 0; g < C::PERM_TOKENS / 8; ++g)
+            for (int g = 0; g < kTokens / 8; ++g) {
+                const bool there = more && m_lane + 8 * g < a.g.M;
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
-                    v[g][e] = xs < total && 8 * g < a.mp && m0 + 8 * g < a.g.M
-                                  ? reinterpret_cast<const uint4*>(a.g.X + (size_t)(m0 + 8 * g) * a.g.K + step * 128 + c * 32)[e] : make_uint4(0, 0, 0, 0);
+                    v[g][e] = there ? reinterpret_cast<const uint4*>(xk + (size_t)(8 * g) * a.g.K)[e] : make_uint4(0, 0, 0, 0);
+            }
         };
-        int xs = warp - 2;
-        fetch(xs);
-        for (; xs < total; xs += 2) {
-            const int slot = xs % a.xs;
-            if (!wait_warp(kBarXEmpty + slot, ((uint32_t)(xs / a.xs) & 1u) ^ 1u)) break;
-            uint8_t* dst = sX + slot * x_bytes + (c >> 1) * blk_bytes;
+        auto on = [&](int by) {
+            step += by;
+            while (step >= a.n_steps) step -= a.n_steps;
+        };
+        int left = t1 - t0 - (warp - 2), slot = warp - 2;
+        uint32_t phase = 0;
+        on(slot);
+        fetch(left > 0);
+        while (left > 0) {
+            if (!wait_warp(kBarXEmpty + slot, phase ^ 1u)) break;
+            uint8_t* dst = sX + slot * x_bytes;
 #pragma unroll
-            for (int g = 0; g < C::PERM_TOKENS / 8; ++g) {
-                if (8 * g >= a.mp) break;
-                const int row = m_lane + 8 * g;
+            for (int g = 0; g < kTokens / 8; ++g) {
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {                 // bytes e and e + 2 of the words
                     const uint4 lo = v[g][e], hi = v[g][e + 2];
                     const uint4 o[2] = {make_uint4(__byte_perm(lo.x, hi.x, 0x5410), __byte_perm(lo.x, hi.x, 0x7632), __byte_perm(lo.y, hi.y, 0x5410), __byte_perm(lo.y, hi.y, 0x7632)),
                                         make_uint4(__byte_perm(lo.z, hi.z, 0x5410), __byte_perm(lo.z, hi.z, 0x7632), __byte_perm(lo.w, hi.w, 0x5410), __byte_perm(lo.w, hi.w, 0x7632))};
 #pragma unroll
-                    for (int i = 0; i < 2; ++i)
-                        *reinterpret_cast<uint4*>(dst + row * 128 + (((4 * (c & 1) + 2 * e + i) ^ (row & 7)) << 4)) = o[i];
+                    for (int i = 0; i < 2; ++i) *reinterpret_cast<uint4*>(dst + (at ^ ((2 * e + i) << 4)) + g * 1024) = o[i];
                 }
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(kBarXFull + slot));
-            fetch(xs + 2);
+            left -= 2;
+            on(2);
+            fetch(left > 0);
+            slot += 2;
+            if (slot >= a.xs) {
+                slot -= a.xs;
+                phase ^= 1u;
+            }
         }
     } else if (warp == 2) {
         // ---- activation loader: a step is two boxes of 64 k ------------------------------------------------------------------
@@ -451,7 +464,7 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
                 // Its parameters s_0 .. s_{Q-1}, z, two to a word.  Plane j's bit at position 11 .. 14 of a half is 2^-13, 2^-11, 2^-7, 2 as an fp16
                 // number, so that with factor[j][position] it contributes s_j (exact products).  Scales of 1 and more would not fit the factors:
                 // such a row is built 2^-down times its size (down = exponent of its largest scale, plus one) and scaled up at the end.
-                if constexpr (PERM) {
+                if constexpr (PERM > 0) {
                     uint32_t sc[Q / 2 + 1];
 #pragma unroll
                     for (int i = 0; i <= Q / 2; ++i)
@@ -544,7 +557,7 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
 #pragma unroll
                 for (int i4 = 0; i4 < 4; ++i4) {
                     uint32_t o[16];
-                    if constexpr (PERM) {
+                    if constexpr (PERM > 0) {
                         // 32 weights: register 8 e + i holds bit i of bytes e and e + 2
 #pragma unroll
                         for (int v = 0; v < 4; ++v) {         // bits 0-3 and 4-7 of bytes 0 and 2, of bytes 1 and 3
@@ -859,7 +872,8 @@ int launch_tmem_q(const GemmArgs& g, int num_sms, cudaStream_t stream) {
     if (dev < 0 || dev >= 64) return (int)cudaErrorNotSupported;
     if (!configured[dev]) {
         cudaError_t e = cudaSuccess;
-        for (auto kernel : {hlq_tmem_kernel<Q, false, false>, hlq_tmem_kernel<Q, true, false>, hlq_tmem_kernel<Q, false, true>, hlq_tmem_kernel<Q, true, true>})
+        for (auto kernel : {hlq_tmem_kernel<Q, false, 0>, hlq_tmem_kernel<Q, true, 0>, hlq_tmem_kernel<Q, false, 16>, hlq_tmem_kernel<Q, true, 16>,
+                            hlq_tmem_kernel<Q, false, 32>, hlq_tmem_kernel<Q, true, 32>})
             if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
         if (e != cudaSuccess) return (int)e;
         configured[dev] = true;
@@ -920,14 +934,15 @@ int launch_tmem_q(const GemmArgs& g, int num_sms, cudaStream_t stream) {
         attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = a.split > 1 ? 2 : 1;
-        // PERM is ahead where the rebuild is the bound and two warps put the activations in order in time.  us without and with it, q = 2, 3, 4: M = 16,
-        // 4096 x 4096 8.6, 9.9, 11.3 / 8.3, 9.6, 10.9; 4096 x 14336 18.0, 22.3, 26.6 / 16.9, 20.7, 24.6; 28672 x 4096 25.1, 33.2, 40.7 / 23.6, 30.6, 38.8;
-        // 57344 x 8192 75.1, 100, 123 / 69.6, 91.6, 116.7.  On less than half of the SMs the next kernel's CTAs rebuild meanwhile, the activations' way is
-        // what counts: 1000 x 4096 5.0, 5.2, 5.35 / 5.1, 5.4, 5.55.  M = 32: only q = 3 gains, with some steps per CTA (28672 x 4096 25.5, 33.6, 41.1 /
-        // 26.0, 32.0, 41.3; 6144 x 4096, q = 3 12.65 / 12.4; 2560 x 4096, four steps, 7.95 / 8.2).
-        const bool perm = 2 * grid > num_sms && (a.mp <= 16 || (a.mp <= C::PERM_TOKENS && (a.split > 1 ? a.n_steps / a.split : a.per_cta) >= 5));
-        cudaError_t e = cudaLaunchKernelEx(&cfg, a.split > 1 ? (perm ? hlq_tmem_kernel<Q, true, true> : hlq_tmem_kernel<Q, true, false>)
-                                                             : (perm ? hlq_tmem_kernel<Q, false, true> : hlq_tmem_kernel<Q, false, false>), map, a);
+        // PERM is ahead where the rebuild is the bound and two warps put the activations in order in time and beside the rebuild.  us without and with it,
+        // q = 2, 3, 4: M = 16, 4096 x 4096 8.5, 9.8, 11.3 / 8.1, 9.35, 10.8; 4096 x 14336 18.0, 22.1, 26.4 / 16.7, 20.3, 25.1; 28672 x 4096 25.0, 33.0, 40.6 /
+        // 23.3, 30.0, 38.2; 57344 x 8192 74.9, 99.7, 122.6 / 69.0, 91, 115.  M = 32 9.0, 10.3, 11.8 / 8.8, 10.2, 11.4; 18.5, 22.5, 27.0 / 17.3, 21.2, 25.3; 25.3, 33.5, 40.9 /
+        // 24.2, 30.5, 38.6; 76.5, 101.8, 124.5 / 72.3, 94.7, 116.6.  M = 48, two turns of loads a step, 28672 x 4096 25.7, 33.9, 41.4 / 30.0, 34.9, 42.3.  On less than
+        // half of the SMs the next kernel's CTAs rebuild meanwhile, the activations' way is what counts: 1000 x 4096, M = 16 5.0, 5.2, 5.35 / 5.1, 5.4, 5.55.
+        const int perm = 2 * grid <= num_sms || a.mp > 32 ? 0 : a.mp;
+        auto kernel = a.split > 1 ? (perm == 16 ? hlq_tmem_kernel<Q, true, 16> : perm == 32 ? hlq_tmem_kernel<Q, true, 32> : hlq_tmem_kernel<Q, true, 0>)
+                                  : (perm == 16 ? hlq_tmem_kernel<Q, false, 16> : perm == 32 ? hlq_tmem_kernel<Q, false, 32> : hlq_tmem_kernel<Q, false, 0>);
+        cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, map, a);
         count_launch(1);
         if (e != cudaSuccess || a.reduce || a.per_cta % a.n_steps == 0 || grid == 1) return (int)e;
         cfg.gridDim = dim3((unsigned)(grid - 1), (unsigned)((a.mp + 7) / 8));
@@ -954,7 +969,7 @@ const int (&cluster_table())[kMaxSplit + 1] {
     }
     std::call_once(once[dev], [dev] {
         tables[dev] = fallback;
-        if (cudaFuncSetAttribute(hlq_tmem_kernel<4, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) != cudaSuccess) {
+        if (cudaFuncSetAttribute(hlq_tmem_kernel<4, true, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) != cudaSuccess) {
             (void)cudaGetLastError();
             return;
         }
@@ -969,7 +984,7 @@ const int (&cluster_table())[kMaxSplit + 1] {
             attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
             cfg.attrs = attr;
             cfg.numAttrs = 1;
-            if (cudaOccupancyMaxActiveClusters(&tables[dev].n[n], hlq_tmem_kernel<4, true, false>, &cfg) != cudaSuccess) {
+            if (cudaOccupancyMaxActiveClusters(&tables[dev].n[n], hlq_tmem_kernel<4, true, 0>, &cfg) != cudaSuccess) {
                 tables[dev].n[n] = 0;
                 (void)cudaGetLastError();
             }
