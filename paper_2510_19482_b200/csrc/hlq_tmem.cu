@@ -830,6 +830,13 @@ Plan plan_of(int q, int mp, int tiles, int n_steps, int num_sms, const int (&max
         const double t = 1.1 * c * ((n_steps + s - 1) / s) + 1.0 + 0.035 * mp;
         if (t < best.cost) best = {n_steps, s, t};
     }
+    // Up to 32 tokens the SMs hardly fight for the L2: equal shares cost whole tiles' steps and 4.4 us with the parts' bytes (whole tiles / equal shares, q = 2, 3, 4: 28672 x
+    // 4096, M = 16 23.2, 29.9, 38.3 / 24.2, 29.4, 35.7, M = 32 24.6, 30.8, 40.0 / 26.4, 31.4, 38.6; 26624 x 4096, q = 3, M = 16 29.6 / 27.9; 33000 x 4096, q = 4
+    // 38.9 / 39.2; 28672 x 8192, q = 2, M = 32 46.4 / 41.8; 43008 x 1024, q = 4, M = 16 21.6 / 19.0).
+    if (mp <= 32 && best.split == 1 && best.per_cta == whole && 2 * share >= n_steps) {
+        const double few = 0.075 + 0.235 * q + 0.0016 * mp;
+        if (few * (whole - share) > 4.4 + ctas * kTileRowsN * mp * 4.0 / 2.2e6) best.per_cta = share;
+    }
     return best;
 }
 

@@ -29,7 +29,9 @@ CASES = [(2, 4621, 128, 9), (1, 4480, 1152, 128), (3, 4600, 640, 200), (4, 5000,
          # few tokens, whose activations the kernel puts in another order: the last sizes on that path and the first beyond it, loaders of one, two and
          # three steps, clusters, shared tiles, whole rounds with a rest
          (1, 4480, 128, 12), (2, 4621, 256, 10), (4, 1100, 384, 15), (3, 4600, 1152, 17), (3, 12800, 640, 32), (4, 38000, 512, 25), (4, 3001, 4096, 33),
-         (2, 16000, 1024, 17), (4, 10240, 1024, 32), (3, 38000, 256, 16)]
+         (2, 16000, 1024, 17), (4, 10240, 1024, 32), (3, 38000, 256, 16),
+         # few tokens in equal shares instead of whole tiles: in one round, in two
+         (4, 21500, 2048, 9), (4, 43001, 1024, 16)]
 
 
 @pytest.mark.parametrize("q,N,K,M", CASES)
