@@ -36,13 +36,14 @@ namespace elutq {
 namespace {
 
 constexpr int kFitWarps = 8;      // warps (groups) per CTA
-// From how many groups on the sorted form is ahead: with fewer it waits on its own latencies, and its sort has to pay off over the rounds.
-// Rounds: 1, 2 to 4, 5 and more; in 1024 groups, measured at 256 to 131072 with 1, 3, 5 and 10 rounds.  (us, direct and sorted: 4096 groups of 128, q = 2,
-// ten rounds 29 and 20, three 11 and 12, one 6 and 9; 3072 of 128, q = 4, ten rounds 67 and 67; 16384 of 128, q = 1, one round 9 and 9, ten 27 and 15;
-// 6144 of 32, q = 4, five rounds 32 and 31, ten 34 and 53, 12288 60 and 53.)
-constexpr int kSortedMinK[3][4][3] = {{{6, 4, 8}, {4, 3, 4}, {4, 4, 6}, {6, 6, 10}},                       // G = 32: q = 1 to 4
-                                      {{10, 6, 6}, {6, 4, 4}, {6, 4, 4}, {6, 5, 7}},                       // G = 64
-                                      {{20, 12, 8}, {10, 5, 4}, {7, 4, 3}, {8, 5, 3}}};                    // G = 128
+// From how many groups on the sorted form is taken, by the rounds asked for: 1, 2 to 4, 5 and more; in 1024 groups.  Its sort has to pay off over the rounds
+// that a group runs.  With weights as trained layers have them it is ahead from a third to a half of these numbers on, but groups whose bits settle at once
+// take the direct form two rounds, and those with candidates within rounding of each other are taken direct after all, the 32 of a warp in turn.  (us, direct /
+// sorted, 4096, 8192 and 12288 groups of 128, ten rounds: q = 2, ordinary 28 / 20, 44 / 21, 62 / 21, on a grid of four values 6.7 / 9.2, 10 / 10, 14 / 10, of one value
+// 6 / 44, 9 / 44, 13 / 44, of three 9.5 / 73, 14 / 73, 19 / 75; q = 4, ordinary 73 / 66, 125 / 74, 177 / 75, of sixteen values 29 / 43, 47 / 48, 66 / 49, of one 12 / 78, 20 / 79, 30 / 79.)
+constexpr int kSortedMinK[3][4][3] = {{{12, 12, 16}, {12, 8, 8}, {12, 8, 12}, {12, 12, 24}},               // G = 32: q = 1 to 4
+                                      {{32, 24, 16}, {24, 12, 12}, {12, 8, 8}, {12, 12, 16}},              // G = 64
+                                      {{128, 64, 24}, {32, 24, 12}, {24, 12, 8}, {24, 12, 12}}};           // G = 128
 inline long long sorted_min_groups(int q, int G, int t_max) {
     return 1024LL * kSortedMinK[G == 128 ? 2 : G == 64 ? 1 : 0][q - 1][t_max == 1 ? 0 : t_max < 5 ? 1 : 2];
 }

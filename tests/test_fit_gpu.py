@@ -161,3 +161,25 @@ def test_fit_of_weights_next_to_a_place():
         a, b = elutq.elutq_hlq_fit(Wd, q, G, t_max), elutq.elutq_hlq_fit(Wd, q, G, t_max, trace=True)
         for x, y in zip(a[:3], b[:3]):
             assert torch.equal(x.view(torch.uint8), y.view(torch.uint8))
+
+
+@pytest.mark.parametrize("q,G,groups", [(2, 128, 4096), (2, 128, 12000), (4, 128, 8192), (2, 64, 8192), (3, 32, 8192)])
+def test_groups_that_settle_at_once_take_no_longer_than_their_rounds(q, G, groups):
+    """Groups of one value are done after two rounds, whatever number is asked for: below the sorted form's lower end they cost what the direct form costs (the
+    call with a trace, which writes more), not a sort and a warp's groups in turn (three to seven times as much)."""
+    W = torch.full((groups, G), 0.25, dtype=torch.float16, device="cuda")
+
+    def us(trace):
+        times = []
+        for _ in range(7):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(10):
+                elutq.elutq_hlq_fit(W, q, G, 10, trace)
+            b.record()
+            b.synchronize()
+            times.append(a.elapsed_time(b) * 100)
+        return sorted(times)[3]
+
+    us(False), us(True)
+    assert us(False) <= 1.5 * us(True)
