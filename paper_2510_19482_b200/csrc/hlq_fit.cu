@@ -315,12 +315,9 @@ __device__ __forceinline__ bool gram_singular(const int (&m)[NV][NV]) {
     }
 }
 
+// (A plain load, so that the compiler keeps it behind the stores of what it reads.)
 template <int IMM>
-__device__ __forceinline__ __half lds_half(uint32_t addr) {
-    unsigned short v;
-    asm volatile("ld.shared.u16 %0, [%1+%2];" : "=h"(v) : "r"(addr), "n"(IMM));
-    return __ushort_as_half(v);
-}
+__device__ __forceinline__ __half lds_half(uint32_t addr) { return *reinterpret_cast<const __half*>(__cvta_shared_to_generic(addr + IMM)); }
 
 __host__ __device__ constexpr int log2_of(int n) { return n > 1 ? 1 + log2_of(n / 2) : 0; }
 
