@@ -815,6 +815,12 @@ EncodeFn encode_fn() {
 // shares against clusters: 4096 x 4096, q = 2, M = 16 / 64 / 384 11.0 / 14.4 / 31 and 9.3 / 11.3 / 21; 6144 x 4096, q = 4, M = 128 28.5 and
 // 19.8; 4096 x 14336, q = 3, M = 64 28.2 and 24.3.)
 double step_us(int q, int mp) { return 0.25 + 0.2 * q + 0.0016 * mp; }
+// Up to 32 tokens the SMs hardly fight for the L2: equal shares cost whole tiles' steps and 4.4 us with the parts' bytes.  (us, whole tiles / equal shares: 28672 x
+// 4096, q = 2, 3, 4, M = 16 23.2, 29.9, 38.3 / 24.2, 29.4, 35.7, M = 32 24.6, 30.8, 40.0 / 26.4, 31.4, 38.6; 28672 x 8192, q = 2, M = 32 46.4 / 41.8.  In two
+// rounds, with whole rounds and the rest by clusters third: 43008 x 4096, M = 16, q = 2, 3, 4 43.3, 56.7, 73.1 / 32.1, 39.7, 49.2 / 33.1, 41.2, 52.1; 49382 x 9344, q = 2,
+// M = 24 98.9 / 71.3 / 89.0; 45064 x 1024, q = 3, M = 32 18.7 / 18.0 / 19.2; 96638 x 4608, q = 4, M = 16 122.7 / 110.5 / 110.5; 65641 x 1664, q = 1, M = 24 18.3 / 21.9 / 18.3.
+// Over 230 calls of 75 to 390 tiles the choice is 0.3 % behind the best of the three, at most 11 % where K is short: 45985 x 1536, q = 2, M = 9 18.9 / 17.1.)
+double few_step_us(int q, int mp) { return (q == 1 ? 0.5 : 0.075 + 0.235 * q) + 0.0016 * mp; }
 struct Plan { int per_cta, split; double cost; };
 Plan plan_of(int q, int mp, int tiles, int n_steps, int num_sms, const int (&max_clusters)[kMaxSplit + 1]) {
     const double c = step_us(q, mp);
@@ -830,12 +836,9 @@ Plan plan_of(int q, int mp, int tiles, int n_steps, int num_sms, const int (&max
         const double t = 1.1 * c * ((n_steps + s - 1) / s) + 1.0 + 0.035 * mp;
         if (t < best.cost) best = {n_steps, s, t};
     }
-    // Up to 32 tokens the SMs hardly fight for the L2: equal shares cost whole tiles' steps and 4.4 us with the parts' bytes (whole tiles / equal shares, q = 2, 3, 4: 28672 x
-    // 4096, M = 16 23.2, 29.9, 38.3 / 24.2, 29.4, 35.7, M = 32 24.6, 30.8, 40.0 / 26.4, 31.4, 38.6; 26624 x 4096, q = 3, M = 16 29.6 / 27.9; 33000 x 4096, q = 4
-    // 38.9 / 39.2; 28672 x 8192, q = 2, M = 32 46.4 / 41.8; 43008 x 1024, q = 4, M = 16 21.6 / 19.0).
-    if (mp <= 32 && best.split == 1 && best.per_cta == whole && 2 * share >= n_steps) {
-        const double few = 0.075 + 0.235 * q + 0.0016 * mp;
-        if (few * (whole - share) > 4.4 + ctas * kTileRowsN * mp * 4.0 / 2.2e6) best.per_cta = share;
+    if (mp <= 32 && best.split == 1 && 2 * share >= n_steps) {
+        const double f = few_step_us(q, mp), equal = f * share + 4.4 + ctas * kTileRowsN * mp * 4.0 / 2.2e6;
+        best = equal < f * whole ? Plan{share, 1, equal} : Plan{whole, 1, f * whole};
     }
     return best;
 }
@@ -856,7 +859,7 @@ Schedule schedule_of(int q, int M, int N, int K, int num_sms, const int (&max_cl
     s.rest = s.first;
     const int full = s.tiles / num_sms * num_sms;
     if (full > 0 && full < s.tiles) {
-        const Plan rounds = {full / num_sms * s.n_steps, 1, step_us(q, s.mp) * (full / num_sms * s.n_steps)};
+        const Plan rounds = {full / num_sms * s.n_steps, 1, (s.mp <= 32 ? few_step_us(q, s.mp) : step_us(q, s.mp)) * (full / num_sms * s.n_steps)};
         const Plan rest = plan_of(q, s.mp, s.tiles - full, s.n_steps, num_sms, max_clusters);
         if (rest.split > 1 && rounds.cost + 6.0 + rest.cost < s.first.cost) {
             s.full = full;

@@ -55,6 +55,23 @@ def test_tensor_memory_kernel_matches_oracle(q, N, K, M):
     np.testing.assert_allclose(Y.cpu().numpy(), y + 1.5, rtol=0, atol=1e-5 * np.abs(y).max())
 
 
+# Two rounds of tiles less a part: the equal shares' own cost is below that of whole rounds and the rest by clusters, which are two launches
+@pytest.mark.parametrize("q,N,K,M", [(4, 42703, 1280, 24), (4, 43008, 2048, 16)])
+def test_equal_shares_of_few_tokens_are_one_launch(q, N, K, M):
+    assert elutq.elutq_gemm_kernel(M, N, K, q, G) == elutq.KERNEL_TENSOR_MEMORY
+    gen = torch.Generator(device="cuda").manual_seed(74)
+    planes = torch.randint(0, 2, (q, N, K), generator=gen, device="cuda", dtype=torch.uint8)
+    scales = (torch.randn((N, K // G, q), generator=gen, device="cuda") * 0.02).abs().half()
+    offsets = (torch.randn((N, K // G), generator=gen, device="cuda") * 0.01).half()
+    packed = elutq.elutq_pack(planes, scales, offsets, q, G, N, K)
+    X = synth.activations(74, f"tmem/shares/{M}/{K}", M, K)
+    gemm_f32(X, packed, N, K)
+    before = elutq.elutq_launch_count()
+    y = gemm_f32(X, packed, N, K)
+    assert elutq.elutq_launch_count() == before + 1
+    assert hlq.rel_fro_error(y, gemm_f32(X, packed, N, K, elutq.FLAG_LUT_ONLY)) <= TOL
+
+
 @pytest.mark.parametrize("q", [1, 2, 4])
 def test_scales_of_one_and_more(q, M=40):
     N, K = 4700, 256
