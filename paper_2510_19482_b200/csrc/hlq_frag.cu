@@ -935,13 +935,18 @@ int launch_frag_cfg(const GemmArgs& g, int num_sms, cudaStream_t stream) {
     // through the L2, behind its fence, costs 1800 cycles and the parts as much again; the cluster's barriers and its writes to the first CTA's shared
     // memory about 1000.  (us, tickets / clusters: 4096 x 4096, M = 4, q = 2, 3, 4 6.8, 7.7, 8.8 / 6.1, 7.4, 8.7, M = 8 7.3, 8.3, 9.6 / 6.3, 7.4, 8.7; 4096 x 14336,
     // M = 8, q = 3 18.9 / 17.7; 5003 x 2880, G = 64, q = 3, M = 16 13.1 / 11.3.  A longer share loses: a unit more takes 0.5 + 0.6 q us.)
+    // Of clusters of 3, 5 or 7 an eighth less than are resident together: behind a launch whose CTAs are still leaving, the last odd clusters
+    // find no place and make a second wave (of 45 and 26 resident clusters of 3 and 5, from 43 and, after an idle chip, 24 on; even sizes, up to all
+    // resident ones, never.  us, before there were clusters / with up to 45 / now: 1834 x 4416, G = 64, q = 4, M = 35 19.0 / 29.3 / 18.7; 3261 x 6784, q = 4,
+    // M = 4, with 26 of five 14.7 / 16.7 / 14.4.  Up to 40 and 23 they are 2 to 16 % ahead of tickets behind every kernel tried.)
     a.split = 1;
     int longest = a.per_cta;
     if (a.per_cta < a.chunks) {
         const int tiles = a.units / a.chunks;
         for (int n = 2; n <= 8 && n <= a.chunks; ++n) {
             const int share = (a.chunks + n - 1) / n;
-            if (tiles <= resident_clusters(n) && (share < longest || (share == longest && a.split == 1))) {
+            const int most = resident_clusters(n) - (n % 2 ? resident_clusters(n) / 8 : 0);
+            if (tiles <= most && (share < longest || (share == longest && a.split == 1))) {
                 a.split = n;
                 longest = share;
             }

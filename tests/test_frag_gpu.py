@@ -268,3 +268,29 @@ def test_clusters_report_a_wait_that_runs_out(M, half):
     elutq.elutq_release_scratch()
     assert hlq.rel_fro_error(gemm_f32(X, packed, N, K), ref) <= 5e-6
     assert elutq.elutq_device_status() == 0
+
+
+@pytest.mark.parametrize("chunks,tiles,more", [(27, 45, 48), (17, 45, 49), (29, 26, 30), (13, 26, 30)])
+def test_fewer_output_tiles_take_no_longer(chunks, tiles, more):
+    """As many clusters of three or five CTAs as the device counts as resident do not all find a place behind the call before (a third more time)."""
+    q, G, M, K = 4, 64, 4, 512 * chunks - 128
+    gen = torch.Generator(device="cuda").manual_seed(75)
+    X = torch.randn((M, K), generator=gen, device="cuda").half()
+
+    def us(N):
+        planes = torch.randint(0, 2, (q, N, K), generator=gen, device="cuda", dtype=torch.uint8)
+        scales = (torch.randn((N, K // G, q), generator=gen, device="cuda") * 0.02).abs().half()
+        packed = elutq.elutq_pack(planes, scales, torch.zeros((N, K // G), dtype=torch.float16, device="cuda"), q, G, N, K)
+        Y = torch.empty((M, N), dtype=torch.float16, device="cuda")
+        times = []
+        for _ in range(9):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(20):
+                elutq.elutq_lut_gemm(X, packed, Y, M, N, K)
+            b.record()
+            b.synchronize()
+            times.append(a.elapsed_time(b) * 50)
+        return sorted(times)[4]
+
+    assert us(128 * tiles) <= 1.1 * us(128 * more)
