@@ -226,8 +226,8 @@ def test_batch_blocks_of_one_launch(q, N, K, M):
     assert elutq.elutq_device_status() == 0
 
 
-# Few output tiles, each shared by a cluster of CTAs: more CTAs than fit (as many as its chunks), shares of unequal length, a last chunk of one step,
-# ragged rows, several batch blocks, every form; the widest call that clusters of two take, and one tile more
+# Few output tiles, most of them shared by a cluster of CTAs (1500 x 4736, 200 x 7680 and 257 x 5184 have more chunks than a cluster has CTAs: tickets), shares of
+# unequal length, a last chunk of one step, ragged rows, several batch blocks; the widest call that clusters of two take, and one tile more
 @pytest.mark.parametrize("q,G,N,K,M", [(3, 128, 1500, 4736, 4), (1, 128, 130, 1024, 4), (2, 128, 4100, 4224, 2), (4, 128, 3000, 2688, 8), (1, 128, 200, 7680, 3),
                                        (2, 64, 1300, 3648, 7), (3, 64, 257, 5184, 16), (4, 64, 1000, 2112, 40), (2, 128, 74 * 128, 1152, 6), (2, 128, 74 * 128 + 1, 1152, 6)])
 def test_output_tiles_of_clusters(q, G, N, K, M):
@@ -253,7 +253,7 @@ def test_output_tiles_of_clusters(q, G, N, K, M):
 
 @pytest.mark.parametrize("M,half", [(9, 0), (20, 0), (9, 0x80000000), (20, 0x80000000)])
 def test_clusters_report_a_wait_that_runs_out(M, half):
-    # in all CTAs, or in every other one: nothing is written where a part is missing, and the next call is whole
+    # in all CTAs, or in every other one: nothing is written where a part is missing, and the next call is whole (ten chunks: tickets, no clusters)
     q, G, N, K = 3, 64, 1500, 4672
     layer = workloads.hlq_layer(73, "frag/clusters/expiry", q, G, N, K)
     X = synth.activations(73, f"frag/clusters/expiry/x/{M}", M, K)
@@ -294,3 +294,44 @@ def test_fewer_output_tiles_take_no_longer(chunks, tiles, more):
         return sorted(times)[4]
 
     assert us(128 * tiles) <= 1.1 * us(128 * more)
+
+
+def parts_meet_in_the_workspace(X, packed, N, K):
+    """Whether the call leaves parts of its output tiles in the workspace (tickets).  With fewer output tiles than SMs every tile is shared: if not there, in a cluster."""
+    M = X.shape[0]
+    assert -(-N // 128) * -(-M // 8) < torch.cuda.get_device_properties(0).multi_processor_count
+    ws = torch.zeros(elutq.elutq_workspace_bytes(M, N, K), dtype=torch.uint8, device="cuda")
+    elutq.elutq_workspace_init(ws)
+    before = ws.clone()
+    Y = torch.empty((M, N), dtype=torch.float32, device="cuda")
+    elutq.elutq_lut_gemm_ws(x_dev(X), packed, Y, M, N, K, elutq.FLAG_OUT_F32, ws)
+    return not torch.equal(ws, before)
+
+
+# Digits of four rows in shares of two units; halves of three rows, of 16 and of 7 in clusters of eight; blocks of 16 rows in clusters of three
+@pytest.mark.parametrize("q,G,N,K,M", [(3, 128, 3700, 4096, 4), (1, 128, 200, 3712, 3), (3, 64, 257, 3904, 16), (4, 64, 1500, 3648, 7), (2, 64, 4400, 2880, 16)])
+def test_clusters_of_every_form(q, G, N, K, M):
+    X = synth.activations(72, f"frag/clusters/x/{M}/{K}", M, K, outliers=True)
+    packed = pack_layer(workloads.hlq_layer(72, f"frag/clusters/{q}/{G}/{N}/{K}", q, G, N, K))
+    assert not parts_meet_in_the_workspace(X, packed, N, K)
+    test_output_tiles_of_clusters(q, G, N, K, M)
+
+
+# clusters of 4, of 8, of 5 (whose first CTA is sometimes the one that gives up), and shares of several units
+@pytest.mark.parametrize("N,K,M", [(1000, 1984, 20), (1500, 3648, 9), (890, 2496, 9), (800, 4608, 40)])
+@pytest.mark.parametrize("half", [0, 0x80000000])
+def test_clusters_write_nothing_where_a_part_is_missing(N, K, M, half):
+    q, G = 3, 64
+    layer = workloads.hlq_layer(76, "frag/clusters/missing", q, G, N, K)
+    X = synth.activations(76, f"frag/clusters/missing/x/{M}", M, K)
+    packed = pack_layer(layer)
+    assert not parts_meet_in_the_workspace(X, packed, N, K)
+    for limit in (300, 20000):
+        elutq.elutq_release_scratch()
+        Y = torch.full((M, N), 7.5, dtype=torch.float32, device="cuda")
+        elutq.elutq_test_wait_expiry(x_dev(X), packed, Y, M, N, K, half | limit)
+        assert elutq.elutq_device_status() == 0x7C05
+        assert torch.all(Y == 7.5)
+    elutq.elutq_release_scratch()
+    assert hlq.rel_fro_error(gemm_f32(X, packed, N, K), hlq.matmul(X, layer.planes, layer.scales, layer.offsets, G)) <= 5e-6
+    assert elutq.elutq_device_status() == 0
