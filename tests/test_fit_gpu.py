@@ -131,7 +131,7 @@ def test_fit_on_both_sides_of_the_sorted_form_s_lower_end(q, G, N, t_max):
             assert torch.equal(x.view(torch.uint8), y.view(torch.uint8))
 
 
-# the same at the lower ends where a lane sorts its group itself, and weights that begin 8 bytes after a 16-byte boundary (loads of 2 bytes instead of 16)
+# the same with fewer groups, which are the direct form's with and without a trace, and weights that begin 8 bytes after a 16-byte boundary
 @pytest.mark.parametrize("q,G,N,t_max", [(1, 64, 640, 1), (2, 64, 256, 2), (3, 128, 512, 2), (4, 32, 192, 1), (2, 128, 1280, 1), (2, 128, 512, 7), (4, 128, 384, 10)])
 @pytest.mark.parametrize("shift", [0, 4])
 def test_fit_on_both_sides_of_the_lane_sort_s_lower_end(q, G, N, t_max, shift):
@@ -183,3 +183,30 @@ def test_groups_that_settle_at_once_take_no_longer_than_their_rounds(q, G, group
 
     us(False), us(True)
     assert us(False) <= 1.5 * us(True)
+
+
+# The sorted form's lower ends again, with weights that begin 8 and 2 bytes after a 16-byte boundary (loads of 2 bytes instead of 16; of the output's weights, too)
+@pytest.mark.parametrize("q,G,N,t_max", [(1, 64, 2048, 1), (2, 64, 768, 2), (3, 128, 1536, 2), (4, 32, 384, 1), (2, 128, 1536, 7), (4, 128, 768, 10)])
+@pytest.mark.parametrize("shift", [1, 4])
+def test_sorted_form_of_weights_off_the_boundary(q, G, N, t_max, shift):
+    test_fit_on_both_sides_of_the_lane_sort_s_lower_end(q, G, N, t_max, shift)
+
+
+@pytest.mark.parametrize("q,G", [(1, 128), (2, 128), (3, 64), (4, 32), (4, 128)])
+def test_first_choice_next_to_a_place(q, G):
+    """Weights at, and an ulp or two beside, the middle of two candidates, in so many groups that all q and G are sorted from one round on.  After one round the
+    planes are the first choice itself, so that a wrong one cannot have been mended by a later round."""
+    rng = np.random.default_rng(45)
+    top, n = 2 ** q - 1, 4128
+    grid = np.arange(top + 1).astype(np.float16)
+    mid = (grid[:-1].astype(np.float32) + 0.5).astype(np.float16)
+    up = np.nextafter(mid, np.float16(99))
+    near = np.concatenate([mid, up, np.nextafter(mid, np.float16(-9)), np.nextafter(up, np.float16(99))])
+    W = rng.choice(np.concatenate([near, grid]), (n, G)).astype(np.float16)
+    W[:, 0], W[:, 1] = 0.0, top                          # the first round's candidates are 0 .. top
+    W *= np.float16(2.0) ** rng.integers(-12, 8, (n, 1)).astype(np.float16)
+    Wd = to_dev(W.view(np.int16)).view(torch.float16).repeat(32, 1)
+    for t_max in (1, 2, 5):
+        a, b = elutq.elutq_hlq_fit(Wd, q, G, t_max), elutq.elutq_hlq_fit(Wd, q, G, t_max, trace=True)
+        for x, y in zip(a[:3], b[:3]):
+            assert torch.equal(x.view(torch.uint8), y.view(torch.uint8))
