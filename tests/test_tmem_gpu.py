@@ -1,7 +1,7 @@
 """GPU parity of the kernel that rebuilds weights in tensor memory (batches of more than 8 rows at G = 128 with enough weight rows).
 
-Tolerance: W_hat = z + sum_j b_j s_j is formed with one fp16 fma per plane (exact products, each sum rounded at 2^-11 relative; weight 7
-of a byte starts from z^ = z + (1/2) sum_j s_j, rounded once, and adds +-s_j / 2), products are exact and the sums fp32.  The
+Tolerance: W_hat = z + sum_j b_j s_j is formed with one fp16 fma per plane (exact products, each sum rounded at 2^-11 relative; above 32
+rows weight 7 of a byte starts from z^ = z + (1/2) sum_j s_j, rounded once, and adds +-s_j / 2), products are exact and the sums fp32.  The
 weights' rounding errors are independent across k: a relative error of about 2^-12 .. 2^-11 in norm, bar 1e-3; per element
 the worst-case bound of gpu_util.assert_elementwise.
 """
@@ -133,3 +133,65 @@ def test_waits_that_run_out_behind_loaders_that_are_done(q, N, K, M):
     assert int(ws.view(torch.int32)[0]) == 0
     assert hlq.rel_fro_error(y.cpu().numpy(), ref) <= TOL
     elutq.elutq_release_scratch()
+
+
+# few tokens, whose activations two warps bring in another order: clusters, whole tiles, equal shares, and (1000 rows) the order of more tokens
+@pytest.mark.parametrize("q,N,K,M", [(2, 4096, 4096, 16), (3, 28672, 2048, 9), (4, 21500, 2048, 27), (1, 4500, 1152, 32), (2, 1000, 1024, 17)])
+def test_activations_that_are_not_finite(q, N, K, M):
+    """An infinity makes its row's results infinite by the signs of its weights, a NaN or opposite infinities NaN; the other rows keep their bits."""
+    assert elutq.elutq_gemm_kernel(M, N, K, q, G) == elutq.KERNEL_TENSOR_MEMORY
+    layer = workloads.hlq_layer(77, f"tmem/inf/{q}/{N}/{K}", q, G, N, K, signed_scales=True)
+    X = synth.activations(77, f"tmem/inf/x/{M}/{K}", M, K)
+    packed = pack_layer(layer)
+    y = gemm_f32(X, packed, N, K)
+    X[0, 3] = np.inf
+    X[2, K - 1] = -np.inf
+    X[M - 2, K // 2 + 17] = np.nan
+    X[M - 1, 40], X[M - 1, K - 30] = np.inf, np.inf
+    z = gemm_f32(X, packed, N, K)
+    keep = np.ones(M, dtype=bool)
+    keep[[0, 2, M - 2, M - 1]] = False
+    assert np.array_equal(z[keep], y[keep])
+    assert np.isnan(z[M - 2]).all()
+
+    def column(k):                                           # W_hat[:, k], and how far the rebuilt one may be from it
+        w = hlq.reconstruct(layer.planes[:, :, k // G * G: (k // G + 1) * G], layer.scales[:, k // G: k // G + 1], layer.offsets[:, k // G: k // G + 1], G)[:, k % G]
+        size = np.abs(layer.offsets[:, k // G].astype(np.float64)) + np.abs(layer.scales[:, k // G].astype(np.float64)).sum(1)
+        return w, np.abs(w) > (q + 1) * 2.0 ** -11 * size
+
+    for row, k, sign in ((0, 3, 1.0), (2, K - 1, -1.0)):
+        w, sure = column(k)
+        assert np.array_equal(z[row][sure], np.where(sign * w > 0, np.inf, -np.inf)[sure])
+        assert not np.isfinite(z[row]).any()
+    (w0, sure0), (w1, sure1) = column(40), column(K - 30)
+    sure = sure0 & sure1
+    same = np.sign(w0) == np.sign(w1)
+    assert np.array_equal(z[M - 1][sure & same], np.where(w0 > 0, np.inf, -np.inf)[sure & same])
+    assert np.isnan(z[M - 1][sure & ~same]).all()
+
+
+# the fragment kernel's clusters (digits, halves at G = 64) and the rebuild of few tokens (clusters, whole tiles, equal shares)
+@pytest.mark.parametrize("q,g,N,K,M", [(3, 128, 4096, 4096, 4), (2, 64, 1300, 3648, 20), (2, 128, 4096, 4096, 16), (2, 128, 28672, 1024, 9), (4, 128, 21500, 2048, 32)])
+def test_captured_batches_read_what_is_there_at_replay(q, g, N, K, M):
+    layer = workloads.hlq_layer(78, f"tmem/graph/{q}/{g}/{N}/{K}", q, g, N, K)
+    packed = pack_layer(layer)
+    Xs = [synth.activations(78, f"tmem/graph/x/{i}/{M}/{K}", M, K) for i in range(3)]
+    eager = [gemm_f32(X, packed, N, K) for X in Xs]
+    x = x_dev(Xs[0])
+    Y = torch.zeros((2, M, N), dtype=torch.float32, device="cuda")
+    stream = torch.cuda.Stream()
+    elutq.elutq_reserve(M, N, K, stream)
+    stream.synchronize()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        for i in range(2):                                   # twice: the second begins while the first is still running
+            elutq.elutq_lut_gemm_f32(x, packed, Y[i], M, N, K, 0)
+    for X, want in zip(Xs, eager):
+        x.copy_(x_dev(X))
+        Y.fill_(float("nan"))
+        graph.replay()
+        torch.cuda.synchronize()
+        assert np.array_equal(Y[0].cpu().numpy(), want) and np.array_equal(Y[1].cpu().numpy(), want)
+    graph.reset()
+    assert elutq.elutq_device_status(stream) == 0
