@@ -192,17 +192,19 @@ int launch_copy_in(const void* src, void* dst, size_t bytes, cudaStream_t stream
 }
 
 // Two rows at G = 128: whether the fragment kernel is ahead of the look-up kernel.  Its time follows the weights, that of the look-up kernel the rows too,
-// and the more bit-planes the more it saves (us, look-up / fragment, q = 1, 2, 3, 4):
-//    6144 x 4096   7.4, 8.6, 10.7, 11.8 / 7.4, 8.3, 9.0, 10.1       57344 x 1024   9.5, 11.7, 14.7, 17.5 / 9.9, 12.4, 14.4, 16.8
-//    4096 x 14336  11.2, 13.3, 16.4, 19.3 / 9.0, 11.3, 13.6, 16.1   28672 x 4096   13.5, 17.5, 22.5, 27.2 / 15.2, 18.8, 22.3, 26.3
-//    8192 x 16384  15.6, 20.3, 26.0, 31.0 / 15.7, 19.6, 23.1, 27.6  57344 x 2048   13.2, 17.3, 22.3, 27.0 / 15.2, 19.0, 22.4, 26.5
-//   12288 x 4096   9.2, 11.2, 13.6, 15.8 / 9.4, 11.1, 12.7, 15.0   120000 x 1024   13.3, 17.5, 22.4, 27.1 / 15.1, 19.5, 23.2, 27.5
-//   16500 x 1024   6.1, 6.7, 7.8, 9.0 / 3.5, 4.3, 4.9, 6.0          40000 x 1024   8.2, 10.1, 12.6, 14.6 / 8.1, 10.2, 11.7, 13.4
-// Above 2^27 weights little is between the two from q = 3 on, and the look-up kernel is ahead below (57344 x 8192 35.1, 50.0, 67.1, 82.9 / 42.0, 56.3,
-// 67.8, 81.6; 14336 x 16384 21.3, 29.0, 38.1, 46.5 / 24.0, 30.9, 36.8, 44.4).  Up to 2^24 the fragment kernel would be ahead as well (1000 x 1024 4.6, 4.7,
-// 5.4, 5.5 / 4.4, 4.7, 5.0, 5.3; 2048 x 4096 5.9, 6.2, 7.0, 7.4 / 4.9, 5.2, 5.5, 5.9; 4096 x 4096 6.7, 7.4, 8.4, 9.6 / 5.1, 5.9, 6.5, 7.3): these stay
+// and the more bit-planes the more it saves (us, calls in a stream, look-up / fragment, q = 1, 2, 3, 4):
+//    4096 x 14336  11.8, 14.0, 17.1, 19.8 / 8.6, 10.7, 13.0, 15.4   57344 x 1024   10.1, 12.5, 15.4, 18.2 / 9.7, 12.1, 14.2, 16.8
+//    8192 x 16384  16.1, 20.8, 26.4, 31.4 / 15.2, 19.4, 23.2, 28.0  28672 x 4096   14.0, 18.2, 23.1, 27.6 / 14.5, 18.5, 22.2, 26.3
+//   12288 x 4096   9.7, 11.8, 14.0, 16.2 / 8.9, 10.7, 12.5, 14.8    57344 x 2048   13.8, 17.8, 22.7, 27.3 / 14.8, 18.8, 22.4, 26.6
+//    8192 x 8192   12.6, 15.3, 19.0, 21.9 / 10.1, 12.4, 14.6, 17.1  120000 x 1024  13.8, 18.0, 22.9, 27.5 / 14.8, 19.3, 23.1, 27.8
+//                                                                   40000 x 1024   9.3, 10.8, 13.2, 15.2 / 8.0, 9.8, 11.4, 13.3
+// (and in a graph of calls 6144 x 4096 7.9, 8.9, 10.8, 12.0 / 6.4, 7.4, 8.6, 9.7; 16500 x 1024 6.4, 7.0, 8.1, 9.1 / 3.4, 4.3, 5.0, 6.0).  At q = 1 and 2 the fragment
+// kernel is by now ahead of some calls beyond the lines (12288 x 4096 and 57344 x 1024 at q = 1).
+// Above 2^27 weights little is between the two from q = 3 on, and the look-up kernel is ahead below (57344 x 8192 35.7, 45.7, 62.1, 77.5 / 41.1, 55.8,
+// 67.4, 81.2; 14336 x 16384 21.9, 29.5, 38.2, 46.5 / 23.5, 30.6, 36.9, 44.4).  Up to 2^24 the fragment kernel would be ahead as well (in a graph of calls 1000 x 1024
+// 4.5, 4.6, 5.3, 5.5 / 2.7, 3.0, 3.3, 3.6; 2048 x 4096 6.4, 6.7, 7.5, 8.1 / 4.4, 4.8, 5.1, 5.4; 4096 x 4096 6.8, 7.6, 8.8, 7.6 / 4.2, 4.9, 5.6, 6.5): these stay
 // because tests/test_abi_host.py states the look-up kernel for 4096 x 4096, not for their time.  The offset term alone is the look-up kernel's
-// earlier, as that reads no planes (28672 x 4096, q = 4 11.5 / 13.9; 8192 x 8192 10.7 / 10.1; 8192 x 16384 13.3 / 14.9).
+// earlier, as that reads no planes (q = 4: 28672 x 4096 12.0 / 13.7; 8192 x 8192 11.3 / 10.2; 8192 x 16384 14.0 / 15.1).
 bool two_rows_on_fragments(int N, int K, int q, unsigned flags) {
     const long long weights = (long long)N * K;
     if (weights <= (1LL << 24) || weights > (1LL << 27)) return false;

@@ -34,7 +34,7 @@
 //            a call, output tile by output tile (the batch blocks of a row tile next to each other: its weights come from the L2 again), are
 //            dealt to the CTAs (one per SM) in equal contiguous runs, so no SM idles for a wave.  An output tile that several CTAs share
 //            is summed in ascending k order (bit-reproducible) by the CTA that finishes it last (a ticket, no CTA waits for another).  Few output
-//              tiles are shared by clusters of CTAs instead, whose first CTA adds up.
+//            tiles are shared by clusters of CTAs instead, whose first CTA adds up.
 //   warps    16 compute warps: warp 4 s + r takes step s (128 k) of every unit and rows 32 r .. 32 r + 31 of the tile, so each
 //            activation fragment serves two MMAs.  Four activation warps, one per step: scale the unit's activations and
 //            lay them out as B fragments, form the group sums; the first of them also loads the weights.
@@ -1001,7 +1001,10 @@ int launch_frag_qg(const GemmArgs& g, int num_sms, cudaStream_t stream) {
     if constexpr (G == 64) {
         // The height of a batch block, by the longest run of units: a unit takes u us, the first one of a taller block u0 more.  (Fitted
         // to 1100 calls, 256 to 28672 rows.  Blocks of 32 rows, whose sums do not fit the registers, are nowhere ahead: 4096 x 4096,
-        // q = 4, M = 32 23.3 us in blocks of 16, 28.3 of 32; 28672 x 8192 218 and 232.)
+        // q = 4, M = 32 23.3 us in blocks of 16, 28.3 of 32; 28672 x 8192 218 and 232.)  A cluster's longest share is as long as the equal runs would be in all but a
+        // few calls, so counting it instead changes no choice.  Since there are clusters, the choice is 2.9 % behind the better height over 400 calls of
+        // 9 to 40 rows; 60 of them lose 5 % and more, most of these with one to three units a CTA (us, taken / other height: 499 x 7744, q = 3, M = 18
+        // 12.3 / 7.6, in clusters of eight; 4264 x 576, q = 1, M = 39 7.5 / 5.2).
         const long long tiles = (long long)((g.N + kUnitRows - 1) / kUnitRows) * g.n_kc;
         auto us = [&](int rows, double u0, double u) {
             const long long units = tiles * ((g.M + rows - 1) / rows);
