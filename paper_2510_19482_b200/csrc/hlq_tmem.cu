@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
     if (tid == 0) {
         auto init = [&](int i, int n) { asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(bar(i)), "r"(n) : "memory"); };
         for (int i = 0; i < kBlocks * kMaxW; ++i) { init(kBarWFull + i, 1); init(kBarWEmpty + i, 4 * kTurns); }
-        for (int i = 0; i < kMaxX; ++i) { init(kBarXFull + i, 1); init(kBarXEmpty + i, 1); }
+        for (int i = 0; i < kMaxX; ++i) { init(kBarXFull + i, PERM > 16 ? 2 : 1); init(kBarXEmpty + i, 1); }
         for (int i = 0; i < kBlocks * kMaxSlots; ++i) { init(kBarAFull + i, 4); init(kBarAEmpty + i, 1); }
         for (int i = 0; i < kBlocks; ++i) { init(kBarDFull + i, 1); init(kBarDEmpty + i, 4 * kTurns); }
         init(kBarDrain, 1);
@@ -278,57 +278,65 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
             for (int blk = 0; blk < kBlocks; ++blk) drain(kBarWFull + blk * kMaxW, a.ws, issued[blk]);
         }
     } else if (PERM > 0 && (warp == 2 || warp == 3)) {
-        // ---- activation loaders of few tokens, which take the steps in turn: a lane takes 32 k of a token and puts k and k + 16 side by side, as the
-        // two halves of a word of weight bits lie.  (Walking instead of dividing: M = 32 3 to 5 % faster, since the divisions take the rebuild's pipes.) ---
+        // ---- activation loaders of few tokens: a lane takes 32 k of a token and puts k and k + 16 side by side, as the two halves of a word of weight
+        // bits lie.  16 tokens: the two warps take the steps in turn; 32: half of the tokens of every step each, with the loads of two steps on their way, so that
+        // a step waits for half as many (in turn 1 to 5 % slower, us, q = 1 and 2, M = 32: 28672 x 4096 22.0 and 25.5, now 21.5 and 24.8; 37888 x 2048, q = 2 16.6, now
+        // 16.3).  (Walking instead of dividing: M = 32 3 to 5 % faster, since the divisions take the rebuild's pipes.) ------------
         grid_dependency_wait();
-        const int m_lane = lane >> 2, c = lane & 3;           // (one token tile: step t is step t mod n_steps of K)
-        const __half* x = a.g.X + (size_t)m_lane * a.g.K + c * 32;
-        const uint32_t at = (uint32_t)((c >> 1) * blk_bytes + m_lane * 128 + ((4 * (c & 1) ^ m_lane) << 4));
-        constexpr int kTokens = PERM > 0 ? PERM : 16;         // = a.mp
-        int step = t0 % a.n_steps;
-        uint4 v[kTokens / 8][4];
-        auto fetch = [&](bool more) {
-            const __half* xk = x + step * 128;
-#pragma unroll
-            for (int g = 0; g < kTokens / 8; ++g) {
-                const bool there = more && m_lane + 8 * g < a.g.M;
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    v[g][e] = there ? reinterpret_cast<const uint4*>(xk + (size_t)(8 * g) * a.g.K)[e] : make_uint4(0, 0, 0, 0);
-            }
-        };
+        constexpr bool kHalves = PERM > 16;
+        constexpr int kGroups = 2, kDeep = kHalves ? 2 : 1, kStride = kHalves ? 1 : 2;      // groups of 8 tokens, steps on their way
+        const int first = kHalves ? 0 : warp - 2, m_lane = lane >> 2, c = lane & 3, m0 = (kHalves ? (warp - 2) * 16 : 0) + m_lane;
+        const __half* x = a.g.X + (size_t)m0 * a.g.K + c * 32;       // (one token tile: step t is step t mod n_steps of K)
+        const uint32_t at = (uint32_t)((c >> 1) * blk_bytes + m0 * 128 + ((4 * (c & 1) ^ m_lane) << 4));
+        int step = t0 % a.n_steps, left = t1 - t0 - first, slot = first;
+        uint32_t phase = 0;
+        uint4 v[kDeep][kGroups][4];
         auto on = [&](int by) {
             step += by;
             while (step >= a.n_steps) step -= a.n_steps;
         };
-        int left = t1 - t0 - (warp - 2), slot = warp - 2;
-        uint32_t phase = 0;
-        on(slot);
-        fetch(left > 0);
-        while (left > 0) {
-            if (!wait_warp(kBarXEmpty + slot, phase ^ 1u)) break;
-            uint8_t* dst = sX + slot * x_bytes;
+        auto fetch = [&](uint4 (&r)[kGroups][4], bool more) {
+            const __half* xk = x + step * 128;
 #pragma unroll
-            for (int g = 0; g < kTokens / 8; ++g) {
+            for (int g = 0; g < kGroups; ++g) {
+                const bool there = more && m0 + 8 * g < a.g.M;
 #pragma unroll
-                for (int e = 0; e < 2; ++e) {                 // bytes e and e + 2 of the words
-                    const uint4 lo = v[g][e], hi = v[g][e + 2];
-                    const uint4 o[2] = {make_uint4(__byte_perm(lo.x, hi.x, 0x5410), __byte_perm(lo.x, hi.x, 0x7632), __byte_perm(lo.y, hi.y, 0x5410), __byte_perm(lo.y, hi.y, 0x7632)),
-                                        make_uint4(__byte_perm(lo.z, hi.z, 0x5410), __byte_perm(lo.z, hi.z, 0x7632), __byte_perm(lo.w, hi.w, 0x5410), __byte_perm(lo.w, hi.w, 0x7632))};
-#pragma unroll
-                    for (int i = 0; i < 2; ++i) *reinterpret_cast<uint4*>(dst + (at ^ ((2 * e + i) << 4)) + g * 1024) = o[i];
-                }
+                for (int e = 0; e < 4; ++e)
+                    r[g][e] = there ? reinterpret_cast<const uint4*>(xk + (size_t)(8 * g) * a.g.K)[e] : make_uint4(0, 0, 0, 0);
             }
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar(kBarXFull + slot));
-            left -= 2;
-            on(2);
-            fetch(left > 0);
-            slot += 2;
-            if (slot >= a.xs) {
-                slot -= a.xs;
-                phase ^= 1u;
+            on(kStride);
+        };
+        on(first);
+#pragma unroll
+        for (int d = 0; d < kDeep; ++d) fetch(v[d], left > d * kStride);
+        for (bool ok = true; ok && left > 0;) {
+#pragma unroll
+            for (int d = 0; d < kDeep; ++d) {
+                if (left <= 0) break;
+                ok = wait_warp(kBarXEmpty + slot, phase ^ 1u);
+                if (!ok) break;
+                uint8_t* dst = sX + slot * x_bytes;
+#pragma unroll
+                for (int g = 0; g < kGroups; ++g) {
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {             // bytes e and e + 2 of the words
+                        const uint4 lo = v[d][g][e], hi = v[d][g][e + 2];
+                        const uint4 o[2] = {make_uint4(__byte_perm(lo.x, hi.x, 0x5410), __byte_perm(lo.x, hi.x, 0x7632), __byte_perm(lo.y, hi.y, 0x5410), __byte_perm(lo.y, hi.y, 0x7632)),
+                                            make_uint4(__byte_perm(lo.z, hi.z, 0x5410), __byte_perm(lo.z, hi.z, 0x7632), __byte_perm(lo.w, hi.w, 0x5410), __byte_perm(lo.w, hi.w, 0x7632))};
+#pragma unroll
+                        for (int i = 0; i < 2; ++i) *reinterpret_cast<uint4*>(dst + (at ^ ((2 * e + i) << 4)) + g * 1024) = o[i];
+                    }
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar(kBarXFull + slot));
+                left -= kStride;
+                fetch(v[d], left > (kDeep - 1) * kStride);
+                slot += kStride;
+                if (slot >= a.xs) {
+                    slot -= a.xs;
+                    phase ^= 1u;
+                }
             }
         }
     } else if (warp == 2) {

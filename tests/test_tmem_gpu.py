@@ -72,6 +72,13 @@ def test_equal_shares_of_few_tokens_are_one_launch(q, N, K, M):
     assert hlq.rel_fro_error(y, gemm_f32(X, packed, N, K, elutq.FLAG_LUT_ONLY)) <= TOL
 
 
+# 17 to 32 tokens, half of them each loader's, with two steps on their way: one step, two, three, tokens that end in either half, a run that begins inside
+# a tile, more steps than places in the ring
+@pytest.mark.parametrize("q,N,K,M", [(1, 4480, 128, 17), (2, 4621, 256, 24), (3, 5000, 384, 25), (4, 3001, 1152, 31), (1, 21500, 2048, 32), (4, 300, 4096, 18), (2, 38000, 640, 23)])
+def test_few_tokens_in_two_halves(q, N, K, M):
+    test_tensor_memory_kernel_matches_oracle(q, N, K, M)
+
+
 @pytest.mark.parametrize("q", [1, 2, 4])
 def test_scales_of_one_and_more(q, M=40):
     N, K = 4700, 256
