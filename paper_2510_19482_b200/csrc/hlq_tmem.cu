@@ -114,6 +114,10 @@ __device__ __forceinline__ void tmem_st16(uint32_t addr, const uint32_t (&r)[16]
                  :: "r"(addr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
                  "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]) : "memory");
 }
+__device__ __forceinline__ void tmem_st8(uint32_t addr, const uint32_t* r) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                 :: "r"(addr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory");
+}
 __device__ __forceinline__ void tmem_ld16(uint32_t (&r)[16], uint32_t addr) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
@@ -421,10 +425,10 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
         auto row_of = [&](int tile) { return ((tile + base_tile) / a.m_tiles) * kTileRowsN + blk * kBlockRows + quad * 32 + lane; };
         auto put16 = [&](int m, int n, int count, const uint32_t (&v)[16]) {
             if (!(a.g.flags & (ELUTQ_FLAG_OUT_F32 | ELUTQ_FLAG_ACCUMULATE))) {
-                __half* y = reinterpret_cast<__half*>(a.g.Y) + (size_t)m * N + n;
+                __half* y = reinterpret_cast<__half*>(a.g.Y) + (size_t)m * N + n;      // (one address that walks: see kStoreEights)
 #pragma unroll
                 for (int i = 0; i < 16; ++i)
-                    if (i < count) y[(size_t)i * N] = __float2half_rn(__uint_as_float(v[i]));
+                    if (i < count) { *y = __float2half_rn(__uint_as_float(v[i])); y += N; }
             } else {
 #pragma unroll
                 for (int i = 0; i < 16; ++i)
@@ -562,6 +566,20 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
                 if (!live) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t dst = dst0 + (uint32_t)(s.i * kSlotCols);
+                auto scale_up = [&](auto& r, int from = 0, int to = 16) {
+                    const __half2 up0 = __float2half2_rn(__int_as_float((127 + (down >> 1)) << 23));
+                    const __half2 up1 = __float2half2_rn(__int_as_float((127 + ((down + 1) >> 1)) << 23));
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        if (i < from || i >= to) continue;
+                        const __half2 t = __hmul2(__hmul2(as_half2(r[i]), up0), up1);
+                        r[i] = *reinterpret_cast<const uint32_t*>(&t);
+                    }
+                };
+                // Registers are short: at q = 4 sixteen rebuilt words at a time and an address for every token written out spilled, and a tile's end took 0.1
+                // us for 16 and 0.4 for 32 tokens.  In eights, with one address (for all q and numbers of tokens): us, 19456 x 256, q = 4, M = 32 6.05 -> 5.59, M = 16 5.38 ->
+                // 5.2, 37888 x 768, M = 32 13.4 -> 12.5; 28672 x 4096, M = 64, q = 3 34.8 -> 33.5, M = 128, q = 2 32.6 -> 31.6.  (Clusters of 32 tokens: eights spill.)
+                constexpr bool kStoreEights = PERM > 0 && Q == 4 && !(CLUSTER && PERM > 16);
 #pragma unroll
                 for (int i4 = 0; i4 < 4; ++i4) {
                     uint32_t o[16];
@@ -578,6 +596,12 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
                             }
 #pragma unroll
                             for (int p = 0; p < 4; ++p) o[4 * v + p] = *reinterpret_cast<const uint32_t*>(&acc[p]);
+                            if constexpr (kStoreEights) {
+                                if (v & 1) {
+                                    if (any_up) scale_up(o, 4 * v - 4, 4 * v + 4);
+                                    tmem_st8(dst + 16u * i4 + 4u * v - 4u, o + 4 * v - 4);
+                                }
+                            }
                         }
                     } else {
 #pragma unroll
@@ -598,16 +622,10 @@ __global__ void __launch_bounds__(kTmThreads, 1) hlq_tmem_kernel(const __grid_co
                         for (int p = 0; p < 4; ++p) o[4 * by + p] = *reinterpret_cast<const uint32_t*>(&acc[p]);
                     }
                     }
-                    if (any_up) {
-                        const __half2 up0 = __float2half2_rn(__int_as_float((127 + (down >> 1)) << 23));
-                        const __half2 up1 = __float2half2_rn(__int_as_float((127 + ((down + 1) >> 1)) << 23));
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) {
-                            const __half2 t = __hmul2(__hmul2(as_half2(o[i]), up0), up1);
-                            o[i] = *reinterpret_cast<const uint32_t*>(&t);
-                        }
+                    if constexpr (!kStoreEights) {
+                        if (any_up) scale_up(o);
+                        tmem_st16(dst + 16u * i4, o);
                     }
-                    tmem_st16(dst + 16u * i4, o);
                 }
                 asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -952,11 +970,13 @@ int launch_tmem_q(const GemmArgs& g, int num_sms, cudaStream_t stream) {
         attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = a.split > 1 ? 2 : 1;
-        // PERM is ahead where the rebuild is the bound and two warps put the activations in order in time and beside the rebuild.  us without and with it,
-        // q = 2, 3, 4: M = 16, 4096 x 4096 8.5, 9.8, 11.3 / 8.1, 9.35, 10.8; 4096 x 14336 18.0, 22.1, 26.4 / 16.7, 20.3, 25.1; 28672 x 4096 25.0, 33.0, 40.6 /
-        // 23.3, 30.0, 38.2; 57344 x 8192 74.9, 99.7, 122.6 / 69.0, 91, 115.  M = 32 9.0, 10.3, 11.8 / 8.8, 10.2, 11.4; 18.5, 22.5, 27.0 / 17.3, 21.2, 25.3; 25.3, 33.5, 40.9 /
-        // 24.2, 30.5, 38.6; 76.5, 101.8, 124.5 / 72.3, 94.7, 116.6.  M = 48, two turns of loads a step, 28672 x 4096 25.7, 33.9, 41.4 / 30.0, 34.9, 42.3.  On less than
-        // half of the SMs the next kernel's CTAs rebuild meanwhile, the activations' way is what counts: 1000 x 4096, M = 16 5.0, 5.2, 5.35 / 5.1, 5.4, 5.55.
+        // PERM is ahead where the rebuild is the bound and two warps put the activations in order in time and beside the rebuild.  us without and with it, weights
+        // from HBM, q = 1, 2, 3, 4: M = 16, 4096 x 4096 7.7, 8.6, 9.7, 11.1 / 7.4, 8.2, 9.3, 10.8; 4096 x 14336 14.6, 18.1, 22.6, 26.6 / 14.2, 16.9, 21.0, 25.7; 28672 x 4096
+        // 19.9, 24.9, 31.4, 37.8 / 19.2, 23.3, 29.7, 36.2; 57344 x 8192 59.9, 74.6, 97.3, 123.4 / 56.3, 69.6, 90.5, 116.4.  M = 32 8.2, 9.1, 10.3, 11.6 / 8.1, 9.0, 10.1, 11.3; 15.2, 18.7,
+        // 23.2, 27.2 / 14.9, 17.8, 22.0, 25.6; 20.5, 25.3, 32.8, 38.9 / 21.4, 24.8, 31.2, 38.5; 61.6, 76.1, 98.4, 124.9 / 58.7, 72.7, 92.8, 120.6.  Over 264 calls of 40 to 222 tiles and
+        // 256 to 8192 k 3 % ahead in the mean; behind at M = 32 with q = 1 and whole tiles (4 % at 28672 x 4096) and with q = 4 and two to six steps (1 to 3 %), where its
+        // results are still the more exact ones.  M = 48, two turns of loads a step, 28672 x 4096 25.7, 33.9, 41.4 / 30.0, 34.9, 42.3.  On less than
+        // half of the SMs the next kernel's CTAs rebuild meanwhile, the activations' way is what counts: 1000 x 4096, M = 16, q = 2, 3, 4 5.0, 5.2, 5.35 / 5.1, 5.4, 5.55.
         const int perm = 2 * grid <= num_sms || a.mp > 32 ? 0 : a.mp;
         auto kernel = a.split > 1 ? (perm == 16 ? hlq_tmem_kernel<Q, true, 16> : perm == 32 ? hlq_tmem_kernel<Q, true, 32> : hlq_tmem_kernel<Q, true, 0>)
                                   : (perm == 16 ? hlq_tmem_kernel<Q, false, 16> : perm == 32 ? hlq_tmem_kernel<Q, false, 32> : hlq_tmem_kernel<Q, false, 0>);
